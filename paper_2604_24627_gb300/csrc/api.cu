@@ -74,7 +74,10 @@ struct axpic_ctx {
   double* diag = nullptr;
   int32_t* photon_start = nullptr;
   float* tables = nullptr;
-  double* tally = nullptr;
+  double* tally = nullptr;       // the folded tally: 3 nbins + 6 sums
+  double* tally_rows = nullptr;  // after it: what the event kernels add to since the last fold
+  int tally_nrows = 1;
+  long tally_stride = 0;         // doubles per row
   unsigned long long* counters = nullptr;
   int* err = nullptr;
   double* scratch = nullptr;  // totals (8) + counters (kNumCounters) + info chunk
@@ -315,7 +318,9 @@ static StepArgs make_args(axpic_ctx* ctx, int64_t step, int mask) {
   A.diag = ctx->diag;
   A.photon_start = ctx->photon_start;
   A.tables = ctx->tables;
-  A.tally = ctx->tally;
+  A.tally = ctx->tally_rows;
+  A.tally_mask = ctx->tally_nrows - 1;
+  A.tally_stride = ctx->tally_stride;
   A.nbins = p.tally_nbins;
   A.inv_dE_bin = (float)(p.tally_nbins / p.tally_Emax_keV);
   A.counters = ctx->counters;
@@ -510,7 +515,14 @@ axpic_status axpic_init_plasma(axpic_ctx** out, const axpic_plasma_desc* desc, c
   ALLOC(ctx->diag, sizeof(double) * AXPIC_CELL_DIAG_LEN * (size_t)n);
   ALLOC(ctx->photon_start, sizeof(int32_t) * (size_t)n);
   ALLOC(ctx->tables, sizeof(float) * kNumTables * kTableN);
-  ALLOC(ctx->tally, sizeof(double) * (3 * (size_t)p.tally_nbins + 6));
+  ctx->tally_stride = (3 * (long)p.tally_nbins + 6 + 15) / 16 * 16;  // rows on 128-byte lines
+  ctx->tally_nrows = 1;
+  // no more rows than event CTAs can use (a small plasma keeps one)
+  while (ctx->tally_nrows < std::min(kTallyRows, (n + 127) / 128) && 2 * sizeof(double) * ctx->tally_nrows * (size_t)ctx->tally_stride <= kTallyBytes)
+    ctx->tally_nrows *= 2;
+  const size_t tally_bytes = sizeof(double) * (1 + ctx->tally_nrows) * (size_t)ctx->tally_stride;
+  ALLOC(ctx->tally, tally_bytes);
+  ctx->tally_rows = ctx->tally + ctx->tally_stride;
   ALLOC(ctx->counters, sizeof(unsigned long long) * kNumCounters * (size_t)ctx->ctr_rows);
   ALLOC(ctx->step_dev, sizeof(uint32_t) * kMaxBranches);
   ALLOC(ctx->heavy, sizeof(int32_t) * (size_t)n);
@@ -549,7 +561,7 @@ axpic_status axpic_init_plasma(axpic_ctx** out, const axpic_plasma_desc* desc, c
       (e = cudaMemsetAsync(ctx->res, 0, sizeof(double) * 4 * (size_t)n, st)) ||
       (e = cudaMemsetAsync(ctx->diag, 0, sizeof(double) * AXPIC_CELL_DIAG_LEN * (size_t)n, st)) ||
       (e = cudaMemsetAsync(ctx->photon_start, 0, sizeof(int32_t) * (size_t)n, st)) ||
-      (e = cudaMemsetAsync(ctx->tally, 0, sizeof(double) * (3 * (size_t)p.tally_nbins + 6), st)) ||
+      (e = cudaMemsetAsync(ctx->tally, 0, tally_bytes, st)) ||
       (e = cudaMemsetAsync(ctx->counters, 0, sizeof(unsigned long long) * kNumCounters * (size_t)ctx->ctr_rows, st)) ||
       (e = cudaMemsetAsync(ctx->err, 0, sizeof(int), st)) ||
       (e = cudaMemsetAsync(ctx->bits, 0, sizeof(uint32_t) * (bit_words > 0 ? bit_words : 1), st)) ||
@@ -702,6 +714,16 @@ axpic_status axpic_step_cells(axpic_ctx* ctx, int64_t step, int32_t channel_mask
   return AXPIC_OK;
 }
 
+// Adds the event kernels' tally rows to the folded tally and clears them.
+static cudaError_t fold_tally(axpic_ctx* ctx) {
+  return launch_fold_tally(ctx->tally_rows, ctx->tally_nrows, ctx->tally_stride, 3 * ctx->prm.tally_nbins + 6,
+                           ctx->tally, ctx->stream);
+}
+static cudaError_t clear_tally_rows(axpic_ctx* ctx) {
+  return cudaMemsetAsync(ctx->tally_rows, 0, sizeof(double) * ctx->tally_nrows * (size_t)ctx->tally_stride,
+                         ctx->stream);
+}
+
 static axpic_status read_err(axpic_ctx* ctx) {
   int h = 0;
   CK(cudaMemcpyAsync(&h, ctx->err, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream), "read error flag");
@@ -725,6 +747,7 @@ axpic_status axpic_tally_spectrum(axpic_ctx* ctx, int32_t nbins, double* H_out, 
   CK(launch_totals(d.ncells, to_ptrs(d.electrons), to_ptrs(d.photons), to_ptrs(d.axions), ctx->res, ctx->counters,
                    ctx->ctr_rows, ctx->scratch, ctx->scratch + 8, st),
      "totals");
+  CK(fold_tally(ctx), "fold tally");
   CK(cudaMemcpyAsync(h.data(), ctx->tally, hn * sizeof(double), cudaMemcpyDeviceToHost, st), "copy tally");
   CK(cudaMemcpyAsync(tot.data(), ctx->scratch, tot.size() * sizeof(double), cudaMemcpyDeviceToHost, st),
      "copy totals");
@@ -1041,6 +1064,9 @@ static std::vector<std::pair<void*, size_t>> state_buffers(axpic_ctx* ctx, bool 
 
 static cudaError_t copy_state(axpic_ctx* ctx, unsigned char* save, bool to_save) {
   size_t off = 0;
+  // the tally rows are not part of the state: folded before, cleared after
+  const cudaError_t te = to_save ? fold_tally(ctx) : clear_tally_rows(ctx);
+  if (te != cudaSuccess) return te;
   for (auto& b : state_buffers(ctx)) {
     if (b.second == 0) continue;
     void* dst = to_save ? (void*)(save + off) : b.first;
@@ -1288,6 +1314,7 @@ axpic_status axpic_save_state(axpic_ctx* ctx, void* host_out, uint64_t bytes) {
   uint64_t need = 0;
   if (!ctx || !host_out || axpic_state_bytes(ctx, &need) != AXPIC_OK || bytes != need)
     return ctx ? fail(ctx, AXPIC_E_INVALID, "axpic_save_state: buffer size") : AXPIC_E_INVALID;
+  CK(fold_tally(ctx), "fold tally");
   unsigned char* p = static_cast<unsigned char*>(host_out);
   for (auto& b : state_buffers(ctx, false)) {
     CK(cudaMemcpyAsync(p, b.first, b.second, cudaMemcpyDeviceToHost, ctx->stream), "copy");
@@ -1302,6 +1329,7 @@ axpic_status axpic_load_state(axpic_ctx* ctx, const void* host_in, uint64_t byte
   uint64_t need = 0;
   if (!ctx || !host_in || axpic_state_bytes(ctx, &need) != AXPIC_OK || bytes != need)
     return ctx ? fail(ctx, AXPIC_E_INVALID, "axpic_load_state: buffer size") : AXPIC_E_INVALID;
+  CK(clear_tally_rows(ctx), "clear tally rows");
   const unsigned char* p = static_cast<const unsigned char*>(host_in);
   for (auto& b : state_buffers(ctx, false)) {
     CK(cudaMemcpyAsync(b.first, p, b.second, cudaMemcpyHostToDevice, ctx->stream), "copy");
@@ -1481,7 +1509,7 @@ axpic_status axpic_step_noalloc(const axpic_plasma_desc* desc, const axpic_param
   c.xbuf = reinterpret_cast<double*>(base + kNaXbuf);
   c.photon_start = reinterpret_cast<int32_t*>(base + kNaStart);
   c.diag = reinterpret_cast<double*>(base + kNaUnused);
-  c.tally = reinterpret_cast<double*>(base + kNaUnused);
+  c.tally_rows = reinterpret_cast<double*>(base + kNaUnused);
   c.bits = reinterpret_cast<uint32_t*>(base + kNaBits);
   c.recA = reinterpret_cast<uint4*>(base + kNaRecs);
   c.heavy = reinterpret_cast<int32_t*>(base + kNaHeavy);

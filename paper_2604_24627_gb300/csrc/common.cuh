@@ -86,6 +86,15 @@ enum { ERR_CAPACITY = 1, ERR_NUMERIC = 2, ERR_TIMEOUT = 4 };
 // Rows of per-CTA event counters (CTAs share rows beyond this).
 constexpr int kCounterRows = 4096;
 
+// Rows of the emitted-spectrum tally. Every emitted axion adds to its energy
+// bin and to two per-channel totals in FP64; with one row all of a step's
+// events met on the totals' cache line and the event kernel took 3.79 ms a
+// step at 4.1 M cells, bound by that line's atomics (no tally: 0.5 ms). The
+// rows are folded into one when the tally is read or saved. At most
+// kTallyBytes of them, so that a long histogram keeps the scratch small.
+constexpr int kTallyRows = 256;
+constexpr size_t kTallyBytes = 4u << 20;
+
 // Constants folded on the host (binary64) for the binary32 record.
 struct CellConst {
   int nspecies;
@@ -387,7 +396,9 @@ struct StepArgs {
   double* diag;           // [ncells * AXPIC_CELL_DIAG_LEN]
   int32_t* photon_start;  // [ncells] photon count before absorb
   const float* tables;    // [kNumTables * kTableN]
-  double* tally;          // [3 * nbins + 6]
+  double* tally;          // tally rows: row r's [3 * nbins + 6] sums at r * tally_stride
+  int tally_mask;         // rows - 1 (rows a power of two); CTA b adds to row b & tally_mask
+  long tally_stride;      // doubles per row
   int nbins;
   float inv_dE_bin;
   unsigned long long* counters;  // [ctr_rows * kNumCounters]

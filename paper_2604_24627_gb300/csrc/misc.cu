@@ -285,6 +285,31 @@ __global__ void counters_kernel(const unsigned long long* __restrict__ ctr, int 
   if (threadIdx.x == 0) out[col] = (double)buf[0];
 }
 
+// Folds the tally rows: thread (x, y) sums rows y, y + 8, ... of entry x.
+__global__ void fold_tally_kernel(double* __restrict__ rows, int nrows, long stride, int n, double* __restrict__ tally) {
+  __shared__ double part[8][33];
+  const int i = blockIdx.x * 32 + threadIdx.x;
+  double s = 0.0;
+  if (i < n)
+    for (int r = threadIdx.y; r < nrows; r += 8) {
+      double* p = rows + (size_t)r * stride + i;
+      s += *p;
+      *p = 0.0;
+    }
+  part[threadIdx.y][threadIdx.x] = s;
+  __syncthreads();
+  if (threadIdx.y == 0 && i < n) {
+    double t = 0.0;
+    for (int y = 0; y < 8; ++y) t += part[y][threadIdx.x];
+    tally[i] += t;
+  }
+}
+
+cudaError_t launch_fold_tally(double* rows, int nrows, long stride, int n, double* tally, cudaStream_t st) {
+  fold_tally_kernel<<<(n + 31) / 32, dim3(32, 8), 0, st>>>(rows, nrows, stride, n, tally);
+  return cudaGetLastError();
+}
+
 // Alive totals: sum w and sum w E for axions and photons, electron NR
 // kinetic energy, macroparticle counts and carried energy. One warp per cell,
 // FP64 atomics once per warp.

@@ -31,6 +31,9 @@ cudaError_t launch_sample(const SampleArgs& S, cudaStream_t st);
 cudaError_t launch_rates(const float* rec, int cell, const float* E, int n, int eq_stats, float am3, float prim_mult,
                          float mu2, float* out,
                          cudaStream_t st);
+// tally[i] += sum over the rows of rows[r * stride + i], i < n, in row order;
+// the rows are cleared.
+cudaError_t launch_fold_tally(double* rows, int nrows, long stride, int n, double* tally, cudaStream_t st);
 cudaError_t launch_totals(int ncells, const SpeciesPtrs& e, const SpeciesPtrs& g, const SpeciesPtrs& a,
                           const double* res, const unsigned long long* ctr, int ctr_rows, double* out8,
                           double* out_ctr, cudaStream_t st);

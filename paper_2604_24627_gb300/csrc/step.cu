@@ -108,9 +108,10 @@ __device__ __forceinline__ float& slot_w(const SpeciesPtrs& s, long idx) {
 __device__ __noinline__ void tally_add(const StepArgs& A, int ch, float w, float E) {
   const int k = (int)floorf(E * A.inv_dE_bin);
   const double wE = (double)w * (double)E;
-  if (k >= 0 && k < A.nbins) atomicAdd(A.tally + ch * A.nbins + k, wE);
-  atomicAdd(A.tally + 3 * A.nbins + ch, (double)w);
-  atomicAdd(A.tally + 3 * A.nbins + 3 + ch, wE);
+  double* row = A.tally + (size_t)(blockIdx.x & A.tally_mask) * A.tally_stride;
+  if (k >= 0 && k < A.nbins) atomicAdd(row + ch * A.nbins + k, wE);
+  atomicAdd(row + 3 * A.nbins + ch, (double)w);
+  atomicAdd(row + 3 * A.nbins + 3 + ch, wE);
 }
 
 // ---------------------------------------------------------------- spectral records
