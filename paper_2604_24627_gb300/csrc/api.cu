@@ -743,9 +743,9 @@ axpic_status axpic_tally_spectrum(axpic_ctx* ctx, int32_t nbins, double* H_out, 
   cudaStream_t st = ctx->stream;
   const size_t hn = 3 * (size_t)nbins + 6;
   std::vector<double> h(hn), tot(8 + kNumCounters);
-  CK(cudaMemsetAsync(ctx->scratch, 0, sizeof(double) * (8 + kNumCounters), st), "memset");
   CK(launch_totals(d.ncells, to_ptrs(d.electrons), to_ptrs(d.photons), to_ptrs(d.axions), ctx->res, ctx->counters,
-                   ctx->ctr_rows, ctx->scratch, ctx->scratch + 8, st),
+                   ctx->ctr_rows, ctx->scratch, ctx->scratch + 8, ctx->scratch + 8 + kNumCounters,
+                   kInfoChunk * AXPIC_CELL_INFO_LEN / 8, st),
      "totals");
   CK(fold_tally(ctx), "fold tally");
   CK(cudaMemcpyAsync(h.data(), ctx->tally, hn * sizeof(double), cudaMemcpyDeviceToHost, st), "copy tally");
