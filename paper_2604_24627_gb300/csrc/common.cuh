@@ -196,6 +196,33 @@ __device__ __forceinline__ uint32_t word(const uint4& b, int j) {
   return j == 0 ? b.x : (j == 1 ? b.y : (j == 2 ? b.z : b.w));
 }
 
+// ---------------------------------------------------------------- sums
+// An unevaluated sum of three binary32 numbers, for sums that FP64 (1/64 of
+// the FP32 rate) would bound: TwoSum is exact, so each term loses the rounding
+// of the third member alone, 2^-72 of the sum against 2^-53 in FP64.
+struct Sum3 {
+  float a = 0.f, b = 0.f, c = 0.f;
+  __device__ __forceinline__ static float two_sum(float& s, float x) {  // s := s + x, returns the exact error
+    const float t = __fadd_rn(s, x);
+    const float u = __fsub_rn(t, s);
+    const float e = __fadd_rn(__fsub_rn(s, __fsub_rn(t, u)), __fsub_rn(x, u));
+    s = t;
+    return e;
+  }
+  __device__ __forceinline__ void add(float x) { c = __fadd_rn(c, two_sum(b, two_sum(a, x))); }
+  __device__ __forceinline__ void add_product(float w, float E) {
+    const float h = __fmul_rn(w, E);
+    add(h);
+    c = __fadd_rn(c, two_sum(b, __fmaf_rn(w, E, -h)));
+  }
+  __device__ __forceinline__ double value() const { return ((double)c + (double)b) + (double)a; }
+  // outside the range where the triple is exact (a sum or an error term that
+  // overflowed, or products whose remainders underflow)
+  __device__ __forceinline__ bool unsafe() const {
+    return !isfinite(a) || !isfinite(b) || !isfinite(c) || (a != 0.f && fabsf(a) < 0x1p-60f);
+  }
+};
+
 // ---------------------------------------------------------------- physics
 // F(s) = (1 + 1/s) ln(1 + s) - 1; below s = 0.25 its power series
 // sum_{n>=1} (-1)^(n+1) s^n / (n (n+1)) (12 terms) avoids the cancellation.

@@ -356,29 +356,6 @@ cudaError_t launch_fold_tally(double* rows, int nrows, long stride, int n, doubl
 // kernel adds the rows in a fixed order. With FP64 sums, a shuffle reduction
 // and 8 atomics on one line per cell it took 2217 us for 262,144 cells of 109
 // particles (457 MB); now 109 us (ncu), 4.3 TB/s with 32 warps an SM.
-struct Sum3 {
-  float a = 0.f, b = 0.f, c = 0.f;
-  __device__ __forceinline__ static float two_sum(float& s, float x) {  // s := s + x, returns the exact error
-    const float t = __fadd_rn(s, x);
-    const float u = __fsub_rn(t, s);
-    const float e = __fadd_rn(__fsub_rn(s, __fsub_rn(t, u)), __fsub_rn(x, u));
-    s = t;
-    return e;
-  }
-  __device__ __forceinline__ void add(float x) { c = __fadd_rn(c, two_sum(b, two_sum(a, x))); }
-  __device__ __forceinline__ void add_product(float w, float E) {
-    const float h = __fmul_rn(w, E);
-    add(h);
-    c = __fadd_rn(c, two_sum(b, __fmaf_rn(w, E, -h)));
-  }
-  __device__ __forceinline__ double value() const { return ((double)c + (double)b) + (double)a; }
-  // outside the range where the triple is exact (a sum or an error term that
-  // overflowed, or products whose remainders underflow)
-  __device__ __forceinline__ bool unsafe() const {
-    return !isfinite(a) || !isfinite(b) || !isfinite(c) || (a != 0.f && fabsf(a) < 0x1p-60f);
-  }
-};
-
 constexpr int kTotThreads = 256;
 constexpr int kTotWarps = kTotThreads / 32;
 constexpr int kTotCells = 8;  // cells a warp takes at a time

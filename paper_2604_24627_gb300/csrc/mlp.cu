@@ -1,9 +1,8 @@
 // The spectral surrogate's MLP (4 -> 64 -> 64 -> 96, tanh hidden layers) on
 // the GPU: forward, backward and Adam. Layer 1 (K = 4) runs on the CUDA
-// cores; every other product, forward and backward, is a tile GEMM on the
-// 5th-generation tensor cores: operands staged by the CTA as bfloat16 in
-// shared memory (K-major, no swizzle), one elected thread issues
-// tcgen05.mma.kind::f16 with an FP32 accumulator in tensor memory, commits to
+// cores; every other product, forward and backward, on the 5th-generation
+// tensor cores: bfloat16 operands in shared memory, one elected thread issues
+// tcgen05.mma.kind::f16 with FP32 accumulators in tensor memory, commits to
 // an mbarrier, and the CTA reads the tile back with tcgen05.ld.
 #include <cuda_bf16.h>
 
@@ -17,270 +16,449 @@
 
 #include <nvtx3/nvToolsExt.h>
 
+#include "common.cuh"
 #include "mlp.h"
 #include "tc.cuh"
 #include "surrogate.h"
 
 namespace axpic {
 
-// ---------------------------------------------------------------- tile GEMM
-// C (M x N) = A (M x K) . B (K x N) on tiles of 128 rows, split along K into
-// chunks of kc. A(m, k) = transA ? A[k * lda + m] : A[m * lda + k], and
-// B(k, n) likewise. Store mode (accumulate = 0, one K chunk): C = AB + bias,
-// then tanh when act = 1. Accumulate mode (split-K): K chunk s writes its
-// partial product to part[s][M][N]; a second kernel adds the partials to C
-// in chunk order, so the sum (and training) does not depend on scheduling.
-struct GemmArgs {
-  const float* A;
-  long lda;
-  int transA;
-  const float* B;
-  long ldb;
-  int transB;
-  float* C;
-  long ldc;
-  const float* bias;
-  int M, N, K, kc, accumulate, act;
-  float* part;  // accumulate mode: [ceil(K / kc)][M][N]
+// ---------------------------------------------------------------- the network's kernel
+// One persistent CTA takes tiles of 128 rows through the whole network, and
+// in training through the backward pass: every intermediate stays on the SM.
+// 16 warps: warp w holds rows 32 (w & 3) .. + 31 (the tensor memory lanes it
+// can read) and the column group w >> 2 of four, so a thread keeps 16 columns
+// of h1 and h2 and 24 of z of its row in registers.
+//
+// Bound by the chain of four products with their read-backs (a tile's
+// products are 0.2 us of tensor-core time), not by bytes: a row is 400 B.
+// Formed kernel by kernel (16 launches a training step, activations through
+// memory, operands staged element by element) a step of 8192 rows took
+// 268 us; fused, with one kernel summing the CTAs' gradients, 27 us (eight steps
+// and the weights read back: 2171 -> 245 us).
+//
+// Operands are bfloat16 tiles of 8 x 16-byte core matrices without swizzle.
+// The weight gradients contract over the tile's rows: their operands are the
+// same activation tiles read MN-major (a core matrix of 8 rows by 8 columns
+// serves both majors; the group strides swap roles), 128 features by 128
+// rows of which the first 64 features are real (the others read the
+// neighbouring core matrices and end in accumulator lanes nothing reads).
+constexpr int kNetRows = 128;
+constexpr int kMlpThreads = 512;
+// shared memory, bytes
+constexpr int kSH1 = 0, kSH2 = 16384, kSdZ = 32768, kSdA2 = 57344;  // training: four activation tiles
+constexpr int kSW2f = 73728, kSW3f = 81920, kSW2b = 94208, kSW3b = 102400;
+constexpr int kSSmall = 114688;                       // W1, b1, b2, b3 (FP32), then the column sums
+constexpr int kSmallFloats = 256 + 64 + 64 + 96;
+constexpr int kTrainSmem = kSSmall + 4 * kSmallFloats + 4 * 4 * kSmallFloats;
+// inference: h1, h2 and the forward weights alone
+constexpr int kFW2f = 32768, kFW3f = 40960, kFSmall = 53248;
+constexpr int kFwdSmem = kFSmall + 4 * kSmallFloats;
+// tensor memory columns (training; inference uses z's columns over z2's)
+constexpr int kTZ2 = 0, kTZ = 64, kTdH2 = 160, kTdH1 = 224, kTgW3 = 288, kTgW2 = 384, kTTrain = 512, kTFwd = 128;
+
+struct MlpArgs {
+  const float* P;   // parameters
+  const float* X;   // [n][4]
+  const float* Zt;  // training targets [n][96]
+  float* Z;         // inference output [n][96]
+  float* part;      // training: [CTAs][kMlpParams] gradients of each CTA's rows
+  double* loss;     // training: [CTAs] sums of (z - Zt)^2
+  int n;
+  float inv_n;
+  int vec;          // Zt (training) or Z (inference) rows are 16-byte aligned
   int* err;
 };
 
-constexpr int kGemmThreads = 128;
-constexpr int kGemmMaxN = 128;
-constexpr int kGemmMaxKc = 128;
+// Descriptor of an instruction with MN-major A and B.
+__host__ __device__ constexpr uint32_t mma_idesc_mn(int M, int N) { return mma_idesc(M, N) | (1u << 15) | (1u << 16); }
 
-__global__ void __launch_bounds__(kGemmThreads) gemm_tc_kernel(GemmArgs g) {
-  extern __shared__ __align__(1024) unsigned char sm[];
-  __shared__ uint64_t bar;
-  __shared__ uint32_t tmem_base;
-  __nv_bfloat16* sA = reinterpret_cast<__nv_bfloat16*>(sm);
-  __nv_bfloat16* sB = sA + 128 * g.kc;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int m0 = blockIdx.x * 128;
-  const int k0 = blockIdx.y * g.kc;
-  const uint32_t ncols = g.N <= 32 ? 32u : (g.N <= 64 ? 64u : 128u);
-  if (warp == 0) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base)),
-                 "r"(ncols));
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
-  }
-  if (tid == 0) {
-    mbar_init(&bar, 1);
-    asm volatile("fence.mbarrier_init.release.cluster;");
-  }
-  // stage A (128 x kc) and B^T (N x kc) as bfloat16, zero outside the matrix
-  for (int i = tid; i < 128 * g.kc; i += kGemmThreads) {
-    const int r = i / g.kc, k = i - r * g.kc;
-    const int m = m0 + r, kk = k0 + k;
-    float v = 0.f;
-    if (m < g.M && kk < g.K) v = g.transA ? g.A[(long)kk * g.lda + m] : g.A[(long)m * g.lda + kk];
-    sA[core_off(r, k, g.kc)] = __float2bfloat16_rn(v);
-  }
-  for (int i = tid; i < g.N * g.kc; i += kGemmThreads) {
-    const int n = i / g.kc, k = i - n * g.kc;
-    const int kk = k0 + k;
-    float v = 0.f;
-    if (kk < g.K) v = g.transB ? g.B[(long)n * g.ldb + kk] : g.B[(long)kk * g.ldb + n];
-    sB[core_off(n, k, g.kc)] = __float2bfloat16_rn(v);
-  }
-  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-  __syncthreads();
-  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-  const uint32_t tmem = tmem_base;
-  if (tid == 0) {
-    const uint32_t lbo = 128, sbo = (uint32_t)(g.kc >> 3) * 128u;
-    const uint32_t a0 = smem_u32(sA), b0 = smem_u32(sB);
-    const uint32_t idesc = mma_idesc(128, g.N);
-    for (int s = 0; s < g.kc / 16; ++s)
-      mma_bf16(tmem, mma_desc(a0 + s * 256, lbo, sbo), mma_desc(b0 + s * 256, lbo, sbo), idesc, s > 0 ? 1u : 0u);
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(&bar))
-                 : "memory");
-  }
-  const bool ok = mbar_wait(&bar, 0);
-  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-  if (!ok) {
-    // flag it, give the tensor core a second bounded wait, then free the
-    // tensor memory and return
-    if (tid == 0) atomicOr(g.err, 1);
-    mbar_wait(&bar, 0);
-  } else {
-    const int m = m0 + warp * 32 + lane;
-    for (int c0 = 0; c0 < g.N; c0 += 16) {
-      uint32_t r[16];
-      asm volatile(
-          "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-          : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-            "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-          : "r"(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)c0));
-      asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-      if (m < g.M) {
+__device__ __forceinline__ void tmem_ld8(uint32_t taddr, float* v) {
+  uint32_t r[8];
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+               : "r"(taddr));
+  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
-        for (int j = 0; j < 16; ++j) {
-          const int n = c0 + j;
-          float v = __uint_as_float(r[j]);
-          if (g.accumulate) {
-            g.part[((long)blockIdx.y * g.M + m) * g.N + n] = v;
-          } else {
-            if (g.bias) v += g.bias[n];
-            if (g.act == 1) v = act_tanh(v);
-            g.C[(long)m * g.ldc + n] = v;
-          }
-        }
-      }
+  for (int j = 0; j < 8; ++j) v[j] = __uint_as_float(r[j]);
+}
+
+// Eight values (columns j0 .. j0 + 7 of row r) as bfloat16 into one 16-byte
+// row of a core matrix of a tile of kc columns.
+__device__ __forceinline__ void store8(unsigned char* tile, int r, int j0, int kc, const float* v) {
+  uint4 u;
+  uint32_t* w = reinterpret_cast<uint32_t*>(&u);
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const __nv_bfloat162 h = __floats2bfloat162_rn(v[2 * i], v[2 * i + 1]);
+    w[i] = *reinterpret_cast<const uint32_t*>(&h);
+  }
+  *reinterpret_cast<uint4*>(reinterpret_cast<__nv_bfloat16*>(tile) + core_off(r, j0, kc)) = u;
+}
+
+// B^T tile (N rows n, K columns k) of a product with B(k, n) = W[k * ldn + n]
+// (forward) or W[n * ldk + k] (the transposed weights of the backward pass).
+template <bool TRANS>
+__device__ __forceinline__ void stage_weights(unsigned char* tile, const float* __restrict__ W, int N, int K) {
+  for (int i = threadIdx.x; i < N * (K / 8); i += kMlpThreads) {
+    float v[8];
+    int n, k0;
+    if (TRANS) {
+      n = i / (K / 8);
+      k0 = 8 * (i - n * (K / 8));
+#pragma unroll
+      for (int j = 0; j < 8; ++j) v[j] = W[n * K + k0 + j];
+    } else {
+      k0 = 8 * (i / N);
+      n = i - (i / N) * N;
+#pragma unroll
+      for (int j = 0; j < 8; ++j) v[j] = W[(k0 + j) * N + n];
+    }
+    store8(tile, n, k0, K, v);
+  }
+}
+
+// C += A . B over K/16 instructions, both K-major (A rows of kc columns).
+__device__ __forceinline__ void issue_k(uint32_t tmem, uint32_t a, uint32_t b, int N, int K) {
+  const uint32_t sbo = (uint32_t)(K >> 3) * 128u;
+  for (int s = 0; s < K / 16; ++s)
+    mma_bf16(tmem, mma_desc(a + s * 256, 128, sbo), mma_desc(b + s * 256, 128, sbo), mma_idesc(128, N), s > 0);
+}
+
+// C (features x N) (+)= A^T . B over the tile's 128 rows: A a tile of 64
+// columns, B one of N, both read MN-major (LBO: the row groups, SBO: the
+// column groups).
+__device__ __forceinline__ void issue_mn(uint32_t tmem, uint32_t a, uint32_t b, int N, bool add) {
+  const uint32_t lba = 8 * 128, lbb = (uint32_t)(N >> 3) * 128u;
+  for (int s = 0; s < kNetRows / 16; ++s)
+    mma_bf16(tmem, mma_desc(a + 2 * s * lba, lba, 128), mma_desc(b + 2 * s * lbb, lbb, 128), mma_idesc_mn(128, N),
+             add || s > 0);
+}
+
+// Sum over the warp's lanes of each of C (16 or 32) columns: lane l returns
+// column l's sum (l mod 16 for 16 columns). Recursive halving, C - 1 or C
+// shuffles.
+template <int C>
+__device__ __forceinline__ float lane_column_sums(float* v) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int o = C / 2; o; o >>= 1) {
+    const bool up = lane & o;
+#pragma unroll
+    for (int i = 0; i < o; ++i) {
+      const float give = up ? v[i] : v[i + o], keep = up ? v[i + o] : v[i];
+      v[i] = keep + __shfl_xor_sync(0xFFFFFFFFu, give, o);
     }
   }
-  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-  __syncthreads();
-  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-  if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(ncols));
+  if (C == 16) v[0] += __shfl_xor_sync(0xFFFFFFFFu, v[0], 16);
+  return v[0];
 }
 
-static size_t gemm_smem(int N, int kc) { return (size_t)(128 + N) * kc * sizeof(__nv_bfloat16); }
+template <bool TRAIN>
+__global__ void __launch_bounds__(kMlpThreads, TRAIN ? 1 : 2) mlp_kernel(MlpArgs g) {
+  extern __shared__ __align__(1024) unsigned char sm[];
+  __shared__ uint64_t bars[2];
+  __shared__ uint32_t tmem_base;
+  __shared__ double lsum[kMlpThreads / 32];
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int quad = warp & 3, grp = warp >> 2;
+  const int row = 32 * quad + lane;
+  if (warp == 0) tmem_alloc(&tmem_base, TRAIN ? kTTrain : kTFwd);
+  if (tid == 0) {
+    mbar_init(&bars[0], 1);
+    mbar_init(&bars[1], 1);
+    asm volatile("fence.mbarrier_init.release.cluster;");
+  }
+  unsigned char* const sW2f = sm + (TRAIN ? kSW2f : kFW2f);
+  unsigned char* const sW3f = sm + (TRAIN ? kSW3f : kFW3f);
+  float* const small = reinterpret_cast<float*>(sm + (TRAIN ? kSSmall : kFSmall));
+  float *const sW1 = small, *const sb1 = small + 256, *const sb2 = small + 320, *const sb3 = small + 384;
+  for (int i = tid; i < 256; i += kMlpThreads) sW1[i] = g.P[kOffW1 + i];
+  if (tid < 64) sb1[tid] = g.P[kOffB1 + tid];
+  else if (tid < 128) sb2[tid - 64] = g.P[kOffB2 + tid - 64];
+  else if (tid < 224) sb3[tid - 128] = g.P[kOffB3 + tid - 128];
+  stage_weights<false>(sW2f, g.P + kOffW2, 64, 64);
+  stage_weights<false>(sW3f, g.P + kOffW3, 96, 64);
+  if (TRAIN) {
+    stage_weights<true>(sm + kSW2b, g.P + kOffW2, 64, 64);
+    stage_weights<true>(sm + kSW3b, g.P + kOffW3, 64, 96);
+  }
+  bool ok = true;
+  // shared-memory operands and tensor-memory reads of all threads before the
+  // next products, and whether every wait so far completed
+  auto join = [&]() {
+    smem_to_async_proxy();
+    tc_fence_before();
+    ok = __syncthreads_and(ok) != 0;
+    tc_fence_after();
+  };
+  join();
+  const uint32_t tmem = tmem_base;
+  const uint32_t trow = tmem + ((uint32_t)(32 * quad) << 16);
+  const uint32_t aH1 = smem_u32(sm + kSH1), aH2 = smem_u32(sm + kSH2);
+  const uint32_t aW2f = smem_u32(sW2f), aW3f = smem_u32(sW3f);
+  const uint32_t tZ = TRAIN ? kTZ : 0;  // inference: z over z2, which has been read
+  uint32_t ph = 0, ph1 = 0;
+  // one commit of barrier b (phase parity p); the warp converges for the
+  // tensor-memory loads that follow
+  auto await = [&](int b, uint32_t& p) {
+    ok = ok && mbar_wait(&bars[b], p);
+    p ^= 1u;
+    __syncwarp();
+    tc_fence_after();
+  };
+  const int ntiles = (g.n + kNetRows - 1) / kNetRows;
+  float sgb3 = 0.f, sgb2 = 0.f, sgb1 = 0.f, sgw1[4] = {0.f, 0.f, 0.f, 0.f};
+  double loss = 0.0;
+  bool first = true;
+  for (int tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x) {
+    const long r = (long)tile * kNetRows + row;
+    const bool live = r < g.n;
+    float x[4] = {0.f, 0.f, 0.f, 0.f}, zt[24];
+    if (live) {
+#pragma unroll
+      for (int k = 0; k < 4; ++k) x[k] = g.X[r * 4 + k];
+    }
+    if (TRAIN) {
+      // the targets, long before they are needed
+      const float* t = g.Zt + r * 96 + 24 * grp;
+      if (live && g.vec) {
+#pragma unroll
+        for (int j = 0; j < 6; ++j) {
+          const float4 q = __ldg(reinterpret_cast<const float4*>(t) + j);
+          zt[4 * j] = q.x;
+          zt[4 * j + 1] = q.y;
+          zt[4 * j + 2] = q.z;
+          zt[4 * j + 3] = q.w;
+        }
+      } else {
+#pragma unroll
+        for (int j = 0; j < 24; ++j) zt[j] = live ? __ldg(t + j) : 0.f;
+      }
+    }
+    // layer 1 (K = 4) on the CUDA cores
+    float h1[16], h2[16];
+#pragma unroll
+    for (int j = 0; j < 16; ++j) {
+      const int c = 16 * grp + j;
+      float a = sb1[c];
+#pragma unroll
+      for (int k = 0; k < 4; ++k) a = fmaf(x[k], sW1[k * 64 + c], a);
+      h1[j] = act_tanh(a);
+    }
+    store8(sm + kSH1, row, 16 * grp, 64, h1);
+    store8(sm + kSH1, row, 16 * grp + 8, 64, h1 + 8);
+    join();
+    if (tid == 0 && ok) {
+      issue_k(tmem + kTZ2, aH1, aW2f, 64, 64);
+      tc_commit(&bars[0]);
+    }
+    await(0, ph);
+    tmem_ld16(trow + kTZ2 + 16 * grp, h2);
+#pragma unroll
+    for (int j = 0; j < 16; ++j) h2[j] = act_tanh(h2[j] + sb2[16 * grp + j]);
+    store8(sm + kSH2, row, 16 * grp, 64, h2);
+    store8(sm + kSH2, row, 16 * grp + 8, 64, h2 + 8);
+    join();
+    if (tid == 0 && ok) {
+      issue_k(tmem + tZ, aH2, aW3f, 96, 64);
+      tc_commit(&bars[0]);
+    }
+    await(0, ph);
+    float z[32];
+#pragma unroll
+    for (int j = 0; j < 24; j += 8) tmem_ld8(trow + tZ + 24 * grp + j, z + j);
+#pragma unroll
+    for (int j = 0; j < 24; ++j) z[j] += sb3[24 * grp + j];
+    if (!TRAIN) {
+      float* o = g.Z + r * 96 + 24 * grp;
+      if (live && ok) {
+        if (g.vec) {
+#pragma unroll
+          for (int j = 0; j < 6; ++j)
+            reinterpret_cast<float4*>(o)[j] = make_float4(z[4 * j], z[4 * j + 1], z[4 * j + 2], z[4 * j + 3]);
+        } else {
+#pragma unroll
+          for (int j = 0; j < 24; ++j) o[j] = z[j];
+        }
+      }
+      continue;  // the next tile's first join orders these reads before z2 is written again
+    }
+    // dz = 2 (z - t) / n; the loss as an exact sum of (z - t)^2
+    Sum3 sq;
+#pragma unroll
+    for (int j = 0; j < 24; ++j) {
+      const float d = live ? z[j] - zt[j] : 0.f;
+      zt[j] = d;
+      sq.add_product(d, d);
+      z[j] = 2.0f * d * g.inv_n;
+    }
+    if (sq.unsafe()) {
+      for (int j = 0; j < 24; ++j) loss += (double)zt[j] * (double)zt[j];
+    } else {
+      loss += sq.value();
+    }
+#pragma unroll
+    for (int j = 0; j < 24; j += 8) store8(sm + kSdZ, row, 24 * grp + j, 96, z + j);
+    join();
+    if (tid == 0 && ok) {
+      issue_k(tmem + kTdH2, smem_u32(sm + kSdZ), smem_u32(sm + kSW3b), 64, 96);  // dh2 = dz W3^T
+      tc_commit(&bars[0]);
+      issue_mn(tmem + kTgW3, aH2, smem_u32(sm + kSdZ), 96, !first);  // gW3 += h2^T dz
+    }
+#pragma unroll
+    for (int j = 24; j < 32; ++j) z[j] = 0.f;
+    sgb3 += lane_column_sums<32>(z);
+    await(0, ph);
+    float d[16];
+    tmem_ld16(trow + kTdH2 + 16 * grp, d);
+#pragma unroll
+    for (int j = 0; j < 16; ++j) d[j] *= 1.0f - h2[j] * h2[j];  // da2 = dh2 (1 - h2^2)
+    store8(sm + kSdA2, row, 16 * grp, 64, d);
+    store8(sm + kSdA2, row, 16 * grp + 8, 64, d + 8);
+    join();
+    if (tid == 0 && ok) {
+      issue_k(tmem + kTdH1, smem_u32(sm + kSdA2), smem_u32(sm + kSW2b), 64, 64);  // dh1 = da2 W2^T
+      tc_commit(&bars[0]);
+      issue_mn(tmem + kTgW2, aH1, smem_u32(sm + kSdA2), 64, !first);  // gW2 += h1^T da2
+      tc_commit(&bars[1]);  // gW3 and gW2: the tiles may be written again
+    }
+    sgb2 += lane_column_sums<16>(d);
+    await(0, ph);
+    tmem_ld16(trow + kTdH1 + 16 * grp, d);
+#pragma unroll
+    for (int j = 0; j < 16; ++j) d[j] *= 1.0f - h1[j] * h1[j];  // da1 = dh1 (1 - h1^2)
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      float p[16];
+#pragma unroll
+      for (int j = 0; j < 16; ++j) p[j] = x[k] * d[j];
+      sgw1[k] += lane_column_sums<16>(p);
+    }
+    sgb1 += lane_column_sums<16>(d);
+    await(1, ph1);
+    first = false;
+  }
+  ok = __syncthreads_and(ok) != 0;
+  if (!ok) {
+    // flag it and give the tensor core a second bounded wait on whatever it
+    // may still be doing before the tensor memory is released
+    if (tid == 0) atomicOr(g.err, 1);
+    mbar_wait(&bars[0], ph ^ 1u);
+    if (TRAIN) mbar_wait(&bars[1], ph1);
+  } else if (TRAIN) {
+    // the CTA's gradients: one row of partials
+    float* out = g.part + (size_t)blockIdx.x * kMlpParams;
+    if (quad < 2) {
+      float v[24];
+#pragma unroll
+      for (int j = 0; j < 24; j += 8) tmem_ld8(trow + kTgW3 + 24 * grp + j, v + j);
+#pragma unroll
+      for (int j = 0; j < 24; j += 4)
+        *reinterpret_cast<float4*>(out + kOffW3 + row * 96 + 24 * grp + j) =
+            make_float4(v[j], v[j + 1], v[j + 2], v[j + 3]);
+      tmem_ld16(trow + kTgW2 + 16 * grp, v);
+#pragma unroll
+      for (int j = 0; j < 16; j += 4)
+        *reinterpret_cast<float4*>(out + kOffW2 + row * 64 + 16 * grp + j) =
+            make_float4(v[j], v[j + 1], v[j + 2], v[j + 3]);
+    }
+    float* red = small + kSmallFloats + quad * kSmallFloats;  // gW1, gb1, gb2, gb3 of these 32 rows
+    if (lane < 24) red[384 + 24 * grp + lane] = sgb3;
+    if (lane < 16) {
+      red[320 + 16 * grp + lane] = sgb2;
+      red[256 + 16 * grp + lane] = sgb1;
+#pragma unroll
+      for (int k = 0; k < 4; ++k) red[k * 64 + 16 * grp + lane] = sgw1[k];
+    }
+    for (int o = 16; o; o >>= 1) loss += __shfl_xor_sync(0xFFFFFFFFu, loss, o);
+    if (lane == 0) lsum[warp] = loss;
+    __syncthreads();
+    for (int i = tid; i < kSmallFloats; i += kMlpThreads) {
+      const float* q = small + kSmallFloats + i;
+      const float v = ((q[0] + q[kSmallFloats]) + q[2 * kSmallFloats]) + q[3 * kSmallFloats];
+      const int o = i < 256 ? kOffW1 + i : i < 320 ? kOffB1 + i - 256 : i < 384 ? kOffB2 + i - 320 : kOffB3 + i - 384;
+      out[o] = v;
+    }
+    if (tid == 0) {
+      double s = 0.0;
+      for (int w = 0; w < kMlpThreads / 32; ++w) s += lsum[w];
+      g.loss[blockIdx.x] = s;
+    }
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  if (warp == 0) tmem_free(tmem, TRAIN ? kTTrain : kTFwd);
+}
 
-// C[m][n] += sum over s = 0, 1, ... of part[s][m][n], in that order.
-__global__ void splitk_sum_kernel(const float* __restrict__ part, int splits, int M, int N, float* __restrict__ C,
-                                  long ldc) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= M * N) return;
-  const long mn = (long)M * N;
+// ---------------------------------------------------------------- gradients and Adam
+// The CTAs' gradient rows added in CTA order (eight slices of rows per
+// parameter, then the slices in order), so training does not depend on
+// scheduling; then Adam with bias correction on the FP32 master parameters
+// (ADAM), or the gradients themselves. Block 0 also sums the loss.
+constexpr int kRedX = 32, kRedY = 8;
+
+template <bool ADAM>
+__global__ void __launch_bounds__(kRedX* kRedY) reduce_kernel(const float* __restrict__ part,
+                                                              const double* __restrict__ losses, int rows, float inv_n,
+                                                              float* __restrict__ G, float* __restrict__ P,
+                                                              float* __restrict__ M, float* __restrict__ V,
+                                                              double* __restrict__ loss, float lr, float b1, float b2,
+                                                              float eps, float c1, float c2) {
+  __shared__ float s[kRedY][kRedX];
+  const int i = blockIdx.x * kRedX + threadIdx.x;
+  const int per = (rows + kRedY - 1) / kRedY;
+  const int r0 = threadIdx.y * per, r1 = min(rows, r0 + per);
   float acc = 0.f;
-  for (int s = 0; s < splits; ++s) acc += part[s * mn + i];
-  const int m = i / N, n = i - m * N;
-  C[(long)m * ldc + n] += acc;
-}
-
-cudaError_t gemm_tc(const GemmArgs& g0, cudaStream_t st) {
-  GemmArgs g = g0;
-  if (g.M <= 0) return cudaSuccess;
-  if (g.N < 16 || g.N > kGemmMaxN || (g.N & 15) || g.K <= 0) return cudaErrorInvalidValue;
-  if (!g.accumulate) g.kc = ((g.K + 15) / 16) * 16;
-  if (g.kc < 16 || g.kc > kGemmMaxKc || (g.kc & 15)) return cudaErrorInvalidValue;
-  if (g.accumulate && (!g.part || g.M > 128)) return cudaErrorInvalidValue;
-  const dim3 grid((g.M + 127) / 128, (g.K + g.kc - 1) / g.kc);
-  gemm_tc_kernel<<<grid, kGemmThreads, gemm_smem(g.N, g.kc), st>>>(g);
-  cudaError_t e = cudaGetLastError();
-  if (e || !g.accumulate) return e;
-  splitk_sum_kernel<<<(g.M * g.N + 255) / 256, 256, 0, st>>>(g.part, (int)grid.y, g.M, g.N, g.C, g.ldc);
-  return cudaGetLastError();
-}
-
-// ---------------------------------------------------------------- element-wise pieces
-// h1 = tanh(X W1 + b1): K = 4, on the CUDA cores; one thread per output.
-__global__ void layer1_kernel(const float* __restrict__ X, const float* __restrict__ W1, const float* __restrict__ b1,
-                              float* __restrict__ H1, int n) {
-  const long i = (long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= (long)n * 64) return;
-  const int r = (int)(i >> 6), j = (int)(i & 63);
-  const float* x = X + (long)r * 4;
-  float a = b1[j];
-#pragma unroll
-  for (int k = 0; k < 4; ++k) a = fmaf(x[k], W1[k * 64 + j], a);
-  H1[i] = act_tanh(a);
-}
-
-// dz = 2 (z - t) / n per element; the loss sum (z - t)^2 / n in FP64.
-__global__ void out_grad_kernel(const float* __restrict__ Zp, const float* __restrict__ Zt, float* __restrict__ dZ,
-                                long total, float inv_n, double* loss) {
-  double acc = 0.0;
-  for (long i = (long)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (long)gridDim.x * blockDim.x) {
-    const float d = Zp[i] - Zt[i];
-    dZ[i] = 2.0f * d * inv_n;
-    acc += (double)d * (double)d;
-  }
-  for (int o = 16; o; o >>= 1) acc += __shfl_xor_sync(0xFFFFFFFFu, acc, o);
-  if ((threadIdx.x & 31) == 0 && acc != 0.0) atomicAdd(loss, acc * (double)inv_n);
-}
-
-// d = d * (1 - h^2) (tanh derivative through its output).
-__global__ void tanh_back_kernel(float* __restrict__ D, const float* __restrict__ H, long total) {
-  for (long i = (long)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (long)gridDim.x * blockDim.x)
-    D[i] *= 1.0f - H[i] * H[i];
-}
-
-// Column sums of an n x w matrix into g (bias gradients).
-__global__ void colsum_kernel(const float* __restrict__ D, int n, int w, float* __restrict__ g) {
-  const int j = blockIdx.x;
-  float acc = 0.f;
-  for (int r = threadIdx.x; r < n; r += blockDim.x) acc += D[(long)r * w + j];
-  for (int o = 16; o; o >>= 1) acc += __shfl_xor_sync(0xFFFFFFFFu, acc, o);
-  __shared__ float part[32];
-  if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = acc;
+#pragma unroll 8
+  for (int r = r0; r < r1; ++r) acc += part[(size_t)r * kMlpParams + i];
+  s[threadIdx.y][threadIdx.x] = acc;
   __syncthreads();
-  if (threadIdx.x == 0) {
-    float s = 0.f;
-    for (int k = 0; k < (int)(blockDim.x >> 5); ++k) s += part[k];
-    g[j] += s;
-  }
-}
-
-// gW1 (4 x 64) += X^T dA1: one block per output column j, K = n.
-__global__ void w1_grad_kernel(const float* __restrict__ X, const float* __restrict__ dA1, int n,
-                               float* __restrict__ gW1) {
-  const int j = blockIdx.x;
-  float acc[4] = {0.f, 0.f, 0.f, 0.f};
-  for (int r = threadIdx.x; r < n; r += blockDim.x) {
-    const float d = dA1[(long)r * 64 + j];
+  if (threadIdx.y == 0) {
+    float g = 0.f;
 #pragma unroll
-    for (int k = 0; k < 4; ++k) acc[k] = fmaf(X[(long)r * 4 + k], d, acc[k]);
+    for (int y = 0; y < kRedY; ++y) g += s[y][threadIdx.x];
+    if (ADAM) {
+      const float m = b1 * M[i] + (1.f - b1) * g;
+      const float v = b2 * V[i] + (1.f - b2) * g * g;
+      M[i] = m;
+      V[i] = v;
+      P[i] -= lr * (m / c1) / (sqrtf(v / c2) + eps);
+    } else {
+      G[i] = g;
+    }
   }
-  __shared__ float part[4][32];
-#pragma unroll
-  for (int k = 0; k < 4; ++k) {
-    float a = acc[k];
-    for (int o = 16; o; o >>= 1) a += __shfl_xor_sync(0xFFFFFFFFu, a, o);
-    if ((threadIdx.x & 31) == 0) part[k][threadIdx.x >> 5] = a;
-  }
-  __syncthreads();
-  if (threadIdx.x < 4) {
-    float s = 0.f;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) s += part[threadIdx.x][w];
-    gW1[threadIdx.x * 64 + j] += s;
+  if (blockIdx.x == 0 && threadIdx.y == 1) {
+    double l = 0.0;
+    for (int r = threadIdx.x; r < rows; r += 32) l += losses[r];
+    for (int o = 16; o; o >>= 1) l += __shfl_xor_sync(0xFFFFFFFFu, l, o);
+    if (threadIdx.x == 0) *loss = l * (double)inv_n;
   }
 }
-
-// Adam with bias correction on the FP32 master parameters.
-__global__ void adam_kernel(float* __restrict__ P, const float* __restrict__ G, float* __restrict__ M,
-                            float* __restrict__ V, int n, float lr, float b1, float b2, float eps, float c1, float c2) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  const float g = G[i];
-  const float m = b1 * M[i] + (1.f - b1) * g;
-  const float v = b2 * V[i] + (1.f - b2) * g * g;
-  M[i] = m;
-  V[i] = v;
-  P[i] -= lr * (m / c1) / (sqrtf(v / c2) + eps);
-}
+static_assert(kMlpParams % kRedX == 0, "whole blocks of parameters");
 
 // ---------------------------------------------------------------- the network
 Mlp::~Mlp() {
-  void* bufs[] = {P, G, Ma, Va, h1, h2, z, dz, dh, part, err, loss};
+  void* bufs[] = {P, G, Ma, Va, part, err, loss, losses};
   for (void* b : bufs)
     if (b) cudaFree(b);
 }
 
-cudaError_t Mlp::reserve(int n) {
-  if (n <= cap) return cudaSuccess;
-  void* bufs[] = {h1, h2, z, dz, dh, part};
-  for (void* b : bufs)
-    if (b) cudaFree(b);
-  h1 = h2 = z = dz = dh = part = nullptr;
+// The training CTAs (one an SM: a tile's buffers and all of its tensor
+// memory) and their gradient rows, made by the first training call.
+cudaError_t Mlp::reserve_train() {
+  if (part) return cudaSuccess;
   cudaError_t e;
-  // split-K partials of the weight gradients: K = n rows in chunks of 128,
-  // at most 64 x 96 outputs each
-  const size_t splits = ((size_t)n + 127) / 128;
-  if ((e = cudaMalloc(&h1, sizeof(float) * 64 * (size_t)n)) || (e = cudaMalloc(&h2, sizeof(float) * 64 * (size_t)n)) ||
-      (e = cudaMalloc(&z, sizeof(float) * 96 * (size_t)n)) || (e = cudaMalloc(&dz, sizeof(float) * 96 * (size_t)n)) ||
-      (e = cudaMalloc(&dh, sizeof(float) * 64 * (size_t)n)) ||
-      (e = cudaMalloc(&part, sizeof(float) * 64 * 96 * (splits > 0 ? splits : 1))))
-    return e;
-  cap = n;
-  return cudaSuccess;
+  if ((e = cudaMalloc(&part, sizeof(float) * kMlpParams * (size_t)sms))) return e;
+  return cudaMalloc(&losses, sizeof(double) * (size_t)sms);
 }
 
 cudaError_t Mlp::init(cudaStream_t s) {
   st = s;
   cudaError_t e;
+  int dev = 0;
+  if ((e = cudaGetDevice(&dev)) || (e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev))) return e;
   if ((e = cudaMalloc(&P, sizeof(float) * kMlpParams)) || (e = cudaMalloc(&G, sizeof(float) * kMlpParams)) ||
       (e = cudaMalloc(&Ma, sizeof(float) * kMlpParams)) || (e = cudaMalloc(&Va, sizeof(float) * kMlpParams)) ||
       (e = cudaMalloc(&err, sizeof(int))) || (e = cudaMalloc(&loss, sizeof(double))) ||
@@ -288,98 +466,63 @@ cudaError_t Mlp::init(cudaStream_t s) {
       (e = cudaMemsetAsync(Ma, 0, sizeof(float) * kMlpParams, st)) ||
       (e = cudaMemsetAsync(Va, 0, sizeof(float) * kMlpParams, st)) || (e = cudaMemsetAsync(err, 0, sizeof(int), st)))
     return e;
-  const int smem = (int)gemm_smem(kGemmMaxN, kGemmMaxKc);
-  return cudaFuncSetAttribute(gemm_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  if ((e = cudaFuncSetAttribute(mlp_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kTrainSmem))) return e;
+  return cudaFuncSetAttribute(mlp_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kFwdSmem);
 }
 
-static GemmArgs store_gemm(const float* A, int K, const float* B, long ldb, int transB, float* C, int N,
-                           const float* bias, int act, int n, int* err) {
-  GemmArgs g;
-  std::memset(&g, 0, sizeof(g));
-  g.A = A;
-  g.lda = K;
-  g.B = B;
-  g.ldb = ldb;
-  g.transB = transB;
-  g.C = C;
-  g.ldc = N;
-  g.bias = bias;
-  g.M = n;
-  g.N = N;
-  g.K = K;
-  g.act = act;
-  g.err = err;
-  return g;
-}
-
-// C (rows x cols) += A^T B with A n x rows and B n x cols (weight gradients).
-static GemmArgs wgrad_gemm(const float* A, int rows, const float* B, int cols, float* C, int n, float* part,
-                           int* err) {
-  GemmArgs g;
-  std::memset(&g, 0, sizeof(g));
-  g.A = A;
-  g.lda = rows;
-  g.transA = 1;
-  g.B = B;
-  g.ldb = cols;
-  g.C = C;
-  g.ldc = cols;
-  g.M = rows;
-  g.N = cols;
-  g.K = n;
-  g.kc = 128;
-  g.accumulate = 1;
-  g.part = part;
-  g.err = err;
-  return g;
-}
+static bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
 cudaError_t Mlp::forward(const float* X, int n, float* out) {
-  cudaError_t e;
-  if ((e = reserve(n))) return e;  // may reallocate every work buffer, z included
   if (n == 0) return cudaSuccess;
-  const long t1 = (long)n * 64;
-  layer1_kernel<<<(unsigned)((t1 + 255) / 256), 256, 0, st>>>(X, W1(), b1(), h1, n);
-  if ((e = cudaGetLastError()) || (e = gemm_tc(store_gemm(h1, 64, W2(), 64, 0, h2, 64, b2(), 1, n, err), st)) ||
-      (e = gemm_tc(store_gemm(h2, 64, W3(), 96, 0, out ? out : z, 96, b3(), 0, n, err), st)))
-    return e;
-  return cudaSuccess;
-}
-
-cudaError_t Mlp::gradients(const float* X, const float* Zt, int n) {
-  cudaError_t e;
-  // NULL: the output buffer is resolved after forward() has reserved it
-  if ((e = forward(X, n, nullptr))) return e;
-  if ((e = cudaMemsetAsync(G, 0, sizeof(float) * kMlpParams, st)) || (e = cudaMemsetAsync(loss, 0, sizeof(double), st)))
-    return e;
-  if (n == 0) return cudaSuccess;
-  const long tz = (long)n * 96, th = (long)n * 64;
-  out_grad_kernel<<<1024, 256, 0, st>>>(z, Zt, dz, tz, 1.0f / (float)n, loss);
-  // layer 3: gW3 = h2^T dz, gb3, dh2 = dz W3^T
-  if ((e = cudaGetLastError()) || (e = gemm_tc(wgrad_gemm(h2, 64, dz, 96, G + kOffW3, n, part, err), st))) return e;
-  colsum_kernel<<<96, 256, 0, st>>>(dz, n, 96, G + kOffB3);
-  if ((e = cudaGetLastError()) || (e = gemm_tc(store_gemm(dz, 96, W3(), 96, 1, dh, 64, nullptr, 0, n, err), st)))
-    return e;
-  // layer 2: da2 = dh2 (1 - h2^2), gW2 = h1^T da2, gb2, dh1 = da2 W2^T
-  tanh_back_kernel<<<1024, 256, 0, st>>>(dh, h2, th);
-  if ((e = cudaGetLastError()) || (e = gemm_tc(wgrad_gemm(h1, 64, dh, 64, G + kOffW2, n, part, err), st))) return e;
-  colsum_kernel<<<64, 256, 0, st>>>(dh, n, 64, G + kOffB2);
-  // h2 is free now: dh1 goes there
-  if ((e = cudaGetLastError()) || (e = gemm_tc(store_gemm(dh, 64, W2(), 64, 1, h2, 64, nullptr, 0, n, err), st)))
-    return e;
-  // layer 1: da1 = dh1 (1 - h1^2), gW1 = X^T da1, gb1
-  tanh_back_kernel<<<1024, 256, 0, st>>>(h2, h1, th);
-  w1_grad_kernel<<<64, 256, 0, st>>>(X, h2, n, G + kOffW1);
-  colsum_kernel<<<64, 256, 0, st>>>(h2, n, 64, G + kOffB1);
+  MlpArgs a;
+  std::memset(&a, 0, sizeof(a));
+  a.P = P;
+  a.X = X;
+  a.Z = out;
+  a.n = n;
+  a.vec = aligned16(out);
+  a.err = err;
+  const int ntiles = (n + kNetRows - 1) / kNetRows;
+  mlp_kernel<false><<<std::min(ntiles, 2 * sms), kMlpThreads, kFwdSmem, st>>>(a);
   return cudaGetLastError();
 }
 
-cudaError_t Mlp::adam(float lr) {
-  ++t;
-  const float c1 = 1.0f - powf(0.9f, (float)t), c2 = 1.0f - powf(0.999f, (float)t);
-  adam_kernel<<<(kMlpParams + 255) / 256, 256, 0, st>>>(P, G, Ma, Va, kMlpParams, lr, 0.9f, 0.999f, 1e-8f, c1, c2);
+cudaError_t Mlp::backward(const float* X, const float* Zt, int n, bool adam, float lr) {
+  cudaError_t e;
+  if (n == 0) {
+    if ((e = cudaMemsetAsync(G, 0, sizeof(float) * kMlpParams, st))) return e;
+    return cudaMemsetAsync(loss, 0, sizeof(double), st);
+  }
+  if ((e = reserve_train())) return e;
+  MlpArgs a;
+  std::memset(&a, 0, sizeof(a));
+  a.P = P;
+  a.X = X;
+  a.Zt = Zt;
+  a.part = part;
+  a.loss = losses;
+  a.n = n;
+  a.inv_n = 1.0f / (float)n;
+  a.vec = aligned16(Zt);
+  a.err = err;
+  const int grid = std::min((n + kNetRows - 1) / kNetRows, sms);
+  mlp_kernel<true><<<grid, kMlpThreads, kTrainSmem, st>>>(a);
+  if ((e = cudaGetLastError())) return e;
+  const dim3 block(kRedX, kRedY);
+  if (adam) {
+    ++t;
+    const float c1 = 1.0f - powf(0.9f, (float)t), c2 = 1.0f - powf(0.999f, (float)t);
+    reduce_kernel<true><<<kMlpParams / kRedX, block, 0, st>>>(part, losses, grid, a.inv_n, G, P, Ma, Va, loss, lr, 0.9f,
+                                                              0.999f, 1e-8f, c1, c2);
+  } else {
+    reduce_kernel<false><<<kMlpParams / kRedX, block, 0, st>>>(part, losses, grid, a.inv_n, G, P, Ma, Va, loss, 0.f, 0.f,
+                                                               0.f, 0.f, 1.f, 1.f);
+  }
   return cudaGetLastError();
 }
+
+cudaError_t Mlp::gradients(const float* X, const float* Zt, int n) { return backward(X, Zt, n, false, 0.f); }
+cudaError_t Mlp::train(const float* X, const float* Zt, int n, float lr) { return backward(X, Zt, n, true, lr); }
 
 }  // namespace axpic
 
@@ -490,8 +633,7 @@ axpic_status axpic_mlp_gradients(axpic_mlp* h, const float* X, const float* Zt, 
 axpic_status axpic_mlp_train_step(axpic_mlp* h, const float* X, const float* Zt, int32_t n, float lr,
                                   double* loss_out) {
   if (!h || n < 1 || !X || !Zt || !(lr > 0.f)) return AXPIC_E_INVALID;
-  cudaError_t e = h->m.gradients(X, Zt, n);
-  if (!e) e = h->m.adam(lr);
+  cudaError_t e = h->m.train(X, Zt, n, lr);
   if (e) return mlp_fail(h, e, "axpic_mlp_train_step");
   if (loss_out) {
     if ((e = cudaMemcpyAsync(loss_out, h->m.loss, sizeof(double), cudaMemcpyDeviceToHost, h->m.st)))
@@ -677,8 +819,7 @@ axpic_status axpic_surrogate_fit(axpic_mlp* h, int32_t ncells, int32_t x_per_cel
   for (int t = 0; t < steps && !e; ++t) {
     const int b = t % nb;
     const float lr_t = lr * (0.01f + 0.99f * 0.5f * (1.0f + cosf(3.14159265f * (float)t / (float)steps)));
-    e = h->m.gradients(dX + (size_t)b * batch * 4, dZ + (size_t)b * batch * 96, batch);
-    if (!e) e = h->m.adam(lr_t);
+    e = h->m.train(dX + (size_t)b * batch * 4, dZ + (size_t)b * batch * 96, batch, lr_t);
   }
   if (!e) e = h->m.gradients(dX, dZ, (int)n);
   double loss = 0.0;

@@ -11,29 +11,25 @@ constexpr int kMlpParams = 10720;
 struct Mlp {
   cudaStream_t st = nullptr;
   float *P = nullptr, *G = nullptr, *Ma = nullptr, *Va = nullptr;  // params, grads, Adam moments
-  float *h1 = nullptr, *h2 = nullptr, *z = nullptr, *dz = nullptr, *dh = nullptr;
-  float* part = nullptr;  // split-K partials of the weight gradients
+  float* part = nullptr;     // each training CTA's gradients
+  double* losses = nullptr;  // and its sum of squares
   int* err = nullptr;
   double* loss = nullptr;
-  int cap = 0;
+  int sms = 1;
   long t = 0;  // Adam steps taken
 
   ~Mlp();
   cudaError_t init(cudaStream_t s);
-  cudaError_t reserve(int n);
-  // z[n][96] = network(X[n][4]) (normalised outputs); out NULL: the own
-  // buffer z, taken after the work buffers are reserved for n rows (never
-  // pass z itself: reserving may reallocate it)
+  cudaError_t reserve_train();
+  // out[n][96] = network(X[n][4]) (normalised outputs)
   cudaError_t forward(const float* X, int n, float* out);
   // G = d loss / d P and *loss, loss = sum (z - Zt)^2 / n
   cudaError_t gradients(const float* X, const float* Zt, int n);
-  cudaError_t adam(float lr);
-  const float* W1() const { return P + kOffW1; }
-  const float* b1() const { return P + kOffB1; }
-  const float* W2() const { return P + kOffW2; }
-  const float* b2() const { return P + kOffB2; }
-  const float* W3() const { return P + kOffW3; }
-  const float* b3() const { return P + kOffB3; }
+  // the same gradients applied by one Adam step (G is not written)
+  cudaError_t train(const float* X, const float* Zt, int n, float lr);
+
+ private:
+  cudaError_t backward(const float* X, const float* Zt, int n, bool adam, float lr);
 };
 
 }  // namespace axpic
