@@ -325,65 +325,164 @@ struct RemapOut {
   float mW, mPx, mPy, mPz, mU2;
 };
 
-// p' = p + (s1 p + b) over the cell's electrons (Eq. affine_map with S = 1 + s1),
-// measuring in FP64 what the binary32 momenta actually received.
-__device__ __noinline__ RemapOut remap_electrons(const StepArgs& A, long ebase, int ne, float s1, float fbx, float fby,
-                                                 float fbz) {
+// Sums over the G lanes of a group (G = 8, 16, 32; lanes of the same
+// lane / G) of four values: lane i of the group returns value (2 if bit G/2
+// of i is set) + (1 if bit G/4 is). The first two steps halve the values
+// instead of adding all of them in every lane, so four FP64 sums over a warp
+// take 6 adds instead of 20; the pairs added are a butterfly's, and so are
+// the bits.
+template <int G, typename T>
+__device__ __forceinline__ T group_sum4(T a, T b, T c, T d) {
   const int lane = lane_id();
+  const bool u = lane & (G / 2), v = lane & (G / 4);
+  T k0 = u ? c : a, k1 = u ? d : b;
+  k0 += __shfl_xor_sync(kFull, u ? a : c, G / 2);
+  k1 += __shfl_xor_sync(kFull, u ? b : d, G / 2);
+  T k = v ? k1 : k0;
+  k += __shfl_xor_sync(kFull, v ? k0 : k1, G / 4);
+#pragma unroll
+  for (int o = G / 8; o; o >>= 1) k += __shfl_xor_sync(kFull, k, o);
+  return k;
+}
+
+// The affine map on one quad of electrons, p' = p + (s1 p + b) (Eq.
+// affine_map with S = 1 + s1), and what the binary32 momenta actually
+// received.
+struct RemapSums {
   float aE = 0.f, aPx = 0.f, aPy = 0.f, aPz = 0.f;
   float mW = 0.f, mPx = 0.f, mPy = 0.f, mPz = 0.f, mU2 = 0.f;
-  const int nqe = (ne + 3) >> 2;
-  // two quads per lane and pass, both loaded before either is stored; each
-  // lane still sums its quads in ascending order
-  for (int q0 = lane; q0 < nqe; q0 += 64) {
-    float4 v[2][4];
+  __device__ __forceinline__ void quad(float4* e, const float4* v, int nj, float s1, float fbx, float fby, float fbz) {
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      const int q = q0 + 32 * h;
-      if (q < nqe) {
-        const long b = ebase + 4 * q;
-#pragma unroll
-        for (int j = 0; j < 4; ++j) v[h][j] = A.e.wp[b + j];
-      }
-    }
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      const int q = q0 + 32 * h;
-      if (q >= nqe) break;
-      const long b = ebase + 4 * q;
-      const int nj = min(4, ne - 4 * q);
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        if (j >= nj) break;
-        const float w = v[h][j].x, px = v[h][j].y, py = v[h][j].z, pz = v[h][j].w;
-        const float nx = px + fmaf(s1, px, fbx);
-        const float ny = py + fmaf(s1, py, fby);
-        const float nz = pz + fmaf(s1, pz, fbz);
-        const float ddx = nx - px, ddy = ny - py, ddz = nz - pz;
-        aE += w * (ddx * (2.f * px + ddx) + ddy * (2.f * py + ddy) + ddz * (2.f * pz + ddz));
-        aPx += w * ddx;
-        aPy += w * ddy;
-        aPz += w * ddz;
-        mW += w;
-        mPx += w * nx;
-        mPy += w * ny;
-        mPz += w * nz;
-        mU2 += w * (nx * nx + ny * ny + nz * nz);
-        A.e.wp[b + j] = make_float4(w, nx, ny, nz);
-      }
+    for (int j = 0; j < 4; ++j) {
+      if (j >= nj) break;
+      const float w = v[j].x, px = v[j].y, py = v[j].z, pz = v[j].w;
+      const float nx = px + fmaf(s1, px, fbx);
+      const float ny = py + fmaf(s1, py, fby);
+      const float nz = pz + fmaf(s1, pz, fbz);
+      const float ddx = nx - px, ddy = ny - py, ddz = nz - pz;
+      aE += w * (ddx * (2.f * px + ddx) + ddy * (2.f * py + ddy) + ddz * (2.f * pz + ddz));
+      aPx += w * ddx;
+      aPy += w * ddy;
+      aPz += w * ddz;
+      mW += w;
+      mPx += w * nx;
+      mPy += w * ny;
+      mPz += w * nz;
+      mU2 += w * (nx * nx + ny * ny + nz * nz);
+      e[j] = make_float4(w, nx, ny, nz);
     }
   }
-  RemapOut o;
-  o.applied_E = warp_sum_d((double)aE) * 0.5 * kMeC2;
-  o.apx = warp_sum_d((double)aPx);
-  o.apy = warp_sum_d((double)aPy);
-  o.apz = warp_sum_d((double)aPz);
-  o.mW = warp_sum_f(mW);
-  o.mPx = warp_sum_f(mPx);
-  o.mPy = warp_sum_f(mPy);
-  o.mPz = warp_sum_f(mPz);
-  o.mU2 = warp_sum_f(mU2);
-  return o;
+  // The sums over the lane's group, for the lanes whose cell group `own` took.
+  template <int G>
+  __device__ __forceinline__ RemapOut reduce(int own) {
+    const double x = group_sum4<G>((double)aE, (double)aPx, (double)aPy, (double)aPz);
+    const float m = group_sum4<G>(mW, mPx, mPy, mPz);
+#pragma unroll
+    for (int o = G / 2; o; o >>= 1) mU2 += __shfl_xor_sync(kFull, mU2, o);
+    const int src = own * G;
+    RemapOut o;
+    o.applied_E = __shfl_sync(kFull, x, src) * 0.5 * kMeC2;
+    o.apx = __shfl_sync(kFull, x, src + G / 4);
+    o.apy = __shfl_sync(kFull, x, src + G / 2);
+    o.apz = __shfl_sync(kFull, x, src + G / 2 + G / 4);
+    o.mW = __shfl_sync(kFull, m, src);
+    o.mPx = __shfl_sync(kFull, m, src + G / 4);
+    o.mPy = __shfl_sync(kFull, m, src + G / 2);
+    o.mPz = __shfl_sync(kFull, m, src + G / 2 + G / 4);
+    o.mU2 = __shfl_sync(kFull, mU2, src);
+    return o;
+  }
+};
+
+// The remap of the warp's cells of `need` (a lane's bit: its own cell, with
+// its electrons ne and the map s1, b). G lanes a cell, 32 / G cells side by
+// side, each with at most G quads of electrons unless G is 32. A lane sums
+// its quads in ascending order, so the result does not depend on G: the
+// lanes beyond a cell's quads add zeros.
+template <int G>
+__device__ __noinline__ RemapOut remap_cells(const StepArgs& A, unsigned need, int cell, int ne, float s1, float bx,
+                                             float by, float bz) {
+  const int lane = lane_id(), gl = lane & (G - 1);
+  RemapOut mine = {};
+  // the next cell (its lane) of this lane's group; the group of this lane's cell
+  auto pick = [&](int& j, int& own) {
+    j = own = -1;
+#pragma unroll
+    for (int g = 0; g < 32 / G; ++g) {
+      const int b = __ffs(need) - 1;
+      if (lane / G == g) j = b;
+      if (b == lane) own = g;
+      need &= need - 1u;
+    }
+  };
+  if constexpr (G == 32) {
+    while (need) {
+      int j, own;
+      pick(j, own);
+      float4* const e = A.e.wp + (long)__shfl_sync(kFull, cell, j) * A.e.cap;
+      const int n = __shfl_sync(kFull, ne, j), nq = (n + 3) >> 2;
+      const float t1 = __shfl_sync(kFull, s1, j), tx = __shfl_sync(kFull, bx, j), ty = __shfl_sync(kFull, by, j),
+                  tz = __shfl_sync(kFull, bz, j);
+      RemapSums S;
+      // two quads per lane and pass, both loaded before either is stored
+      for (int q0 = lane; q0 < nq; q0 += 64) {
+        float4 v[2][4];
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+          if (q0 + 32 * h < nq)
+#pragma unroll
+            for (int k = 0; k < 4; ++k) v[h][k] = e[4 * (q0 + 32 * h) + k];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          const int q = q0 + 32 * h;
+          if (q < nq) S.quad(e + 4 * q, v[h], n - 4 * q, t1, tx, ty, tz);
+        }
+      }
+      __syncwarp();
+      const RemapOut r = S.reduce<32>(0);
+      if (own >= 0) mine = r;
+    }
+  } else {
+    // one quad a lane; the next cells' quads are loaded before these are summed
+    int j, own, n = 0;
+    float4* e = nullptr;
+    float4 v[4];
+    auto load = [&](float4*& ep, int& np, float4* vp) {
+      const int src = max(j, 0);
+      ep = A.e.wp + (long)__shfl_sync(kFull, cell, src) * A.e.cap + 4 * gl;
+      np = __shfl_sync(kFull, ne, src) - 4 * gl;  // electrons from this lane's quad on
+      if (j < 0) np = 0;
+      if (np > 0)
+#pragma unroll
+        for (int k = 0; k < 4; ++k) vp[k] = ep[k];
+    };
+    pick(j, own);
+    load(e, n, v);
+    while (true) {
+      const int src = max(j, 0), o = own;
+      const float t1 = __shfl_sync(kFull, s1, src), tx = __shfl_sync(kFull, bx, src),
+                  ty = __shfl_sync(kFull, by, src), tz = __shfl_sync(kFull, bz, src);
+      const bool more = need != 0;
+      float4* e2 = nullptr;
+      int n2 = 0;
+      float4 v2[4];
+      if (more) {
+        pick(j, own);
+        load(e2, n2, v2);
+      }
+      RemapSums S;
+      if (n > 0) S.quad(e, v, n, t1, tx, ty, tz);
+      __syncwarp();
+      const RemapOut r = S.reduce<G>(max(o, 0));
+      if (o >= 0) mine = r;
+      if (!more) break;
+      e = e2;
+      n = n2;
+#pragma unroll
+      for (int k = 0; k < 4; ++k) v[k] = v2[k];
+    }
+  }
+  return mine;
 }
 
 __device__ __forceinline__ bool nz64(double v) { return (__double_as_longlong(v) << 1) != 0; }
@@ -977,13 +1076,24 @@ __device__ __forceinline__ void fb_finish(const StepArgs& A, int cell, const FbC
 }
 
 // Thread per cell, every load issued first; a warp remaps the cells among
-// its 32 whose exchange needs an affine remap, one at a time with all lanes
-// (about one warp in twelve has one), then each thread finishes its cell. No
-// CTA barrier: the warps of a CTA never wait for one another's remaps. Five
-// CTAs an SM (96 registers; the remap path spills a little).
+// its 32 whose exchange needs an affine remap, then each thread finishes its
+// cell. No CTA barrier: the warps of a CTA never wait for one another's
+// remaps. Bound by its loads where few cells are remapped (about one warp in
+// twelve has one at 5 keV), by the FP64 sums and the chain of remaps where
+// all are.
+// * DENSE = false: a remap takes the whole warp; five CTAs an SM (96
+//   registers; the remap path spills a little). 4.1 M cells at 5 keV: 217 us
+//   with 20 FP64 adds a remap, 202 with the 6 of group_sum4; 224 with the
+//   groups below in the same kernel (more spills).
+// * DENSE = true (absorption by weight reduction, which takes energy from
+//   every axion): cells of at most 64 electrons are remapped two or four side
+//   by side, the next ones' electrons loaded meanwhile; four CTAs an SM
+//   without spills. 112,095 cells of 64 electrons, all remapped: 306 us ->
+//   125 us.
 constexpr int kFeedbackThreads = 128;
 
-__global__ void __launch_bounds__(kFeedbackThreads, 5) feedback_kernel(StepArgs A) {
+template <bool DENSE>
+__global__ void __launch_bounds__(kFeedbackThreads, DENSE ? 4 : 5) feedback_kernel(StepArgs A) {
   // a replayed graph takes its step index from the device counter: the last
   // kernel of the step advances it (no kernel of this launch reads it)
   if (A.step_dev && blockIdx.x == 0 && threadIdx.x == 0) *A.step_dev += 1u;
@@ -1006,15 +1116,16 @@ __global__ void __launch_bounds__(kFeedbackThreads, 5) feedback_kernel(StepArgs 
       xb[3] = 0.0;
     }
   }
-  // the warp remaps its cells that need it one by one, all lanes together
+  // the warp remaps its cells that need it: as many side by side as have a
+  // lane for every quad of electrons
   RemapOut mine;
-  for (unsigned m = __ballot_sync(kFull, f.need); m; m &= m - 1u) {
-    const int j = __ffs(m) - 1;
-    const int c = __shfl_sync(kFull, cell, j);
-    const RemapOut r = remap_electrons(A, (long)c * A.e.cap, __shfl_sync(kFull, f.ne, j),
-                                       __shfl_sync(kFull, (float)f.s1d, j), __shfl_sync(kFull, (float)f.bx, j),
-                                       __shfl_sync(kFull, (float)f.by, j), __shfl_sync(kFull, (float)f.bz, j));
-    if (lane == j) mine = r;
+  const unsigned need = __ballot_sync(kFull, f.need);
+  if (need) {
+    const float s1 = (float)f.s1d, bx = (float)f.bx, by = (float)f.by, bz = (float)f.bz;
+    const int nq = DENSE ? __reduce_max_sync(kFull, f.need ? (f.ne + 3) >> 2 : 0) : 32;
+    if (DENSE && nq <= 8) mine = remap_cells<8>(A, need, cell, f.ne, s1, bx, by, bz);
+    else if (DENSE && nq <= 16) mine = remap_cells<16>(A, need, cell, f.ne, s1, bx, by, bz);
+    else mine = remap_cells<32>(A, need, cell, f.ne, s1, bx, by, bz);
   }
   if (valid) {
     fb_finish(A, cell, f, f.need ? &mine : nullptr);
@@ -2152,7 +2263,10 @@ static cudaError_t launch_decide(const StepArgs& A, int phases, cudaStream_t st)
 
 static cudaError_t launch_feedback(const StepArgs& A, cudaStream_t st) {
   const int grid = (A.ncells + kFeedbackThreads - 1) / kFeedbackThreads;
-  feedback_kernel<<<grid, kFeedbackThreads, 0, st>>>(A);
+  // absorption by weight reduction takes energy from every axion: most cells
+  // are remapped every step
+  if (A.absorb_mode == 1) feedback_kernel<true><<<grid, kFeedbackThreads, 0, st>>>(A);
+  else feedback_kernel<false><<<grid, kFeedbackThreads, 0, st>>>(A);
   return cudaGetLastError();
 }
 
