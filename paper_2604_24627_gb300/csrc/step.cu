@@ -1649,6 +1649,21 @@ __device__ __forceinline__ int scan_row(const uint32_t* row, int n, uint16_t* li
   return c;
 }
 
+// The flagged slots of a staged mask row in [0, n), and its nonzero words.
+__device__ __forceinline__ int count_row(const uint32_t* row, int n, uint32_t* nz) {
+  const int nw = (n + 31) >> 5;
+  int c = 0;
+  uint32_t m = 0u;
+  for (int w = 0; w < nw; ++w) {
+    uint32_t v = row[w];
+    if (v) m |= 1u << w;
+    if (w == nw - 1 && (n & 31)) v &= (1u << (n & 31)) - 1u;
+    c += __popc(v);
+  }
+  *nz = m;
+  return c;
+}
+
 // Clears the nonzero words of a cell's global mask row.
 __device__ __forceinline__ void clear_row(uint32_t* bits, int W, int cell, uint32_t nz) {
   uint32_t* row = bits + (size_t)cell * W;
@@ -1742,13 +1757,12 @@ __device__ __forceinline__ void fill_rest(const SpeciesPtrs& sp, long base, cons
   }
 }
 
-// One cell by one lane: its absorb phase (doA), its emit phase (doE) or the
-// full step (both: the new axions of the emit phase reuse the axion slots the
-// absorb phase freed). Round trips: the first kLoad flagged axions and
-// photons together; the first kLoad tail movers together; then the stores.
-// Longer lists take further round trips. Every flagged axion is read before
-// a new axion is written over a freed slot, and axion movers before any new
-// axion is written.
+// One cell by one lane: its emit phase, or the full step (doA: the new axions
+// of the emit phase reuse the axion slots the absorb phase freed). Round
+// trips: the first kLoad flagged axions and photons together; the first kLoad
+// photon tail movers together; then the stores. Longer lists take further
+// round trips. Every flagged axion is read before a new axion is written over
+// a freed slot.
 struct LaneCell {
   int na, ng;       // in: counts at the start of the phase(s); out: final counts
   int ng0, ne;      // photons eligible for gamma->a, electrons
@@ -1756,16 +1770,16 @@ struct LaneCell {
   float wu, r_cc, r_cb, r_T;
 };
 
-__device__ __forceinline__ void cell_lane(const StepArgs& A, uint32_t step, int cell, bool doA, bool doE,
-                                          uint16_t* lA, uint16_t* lG, const uint16_t* lE, LaneCell& L,
-                                          const Cnt& cnt, Lane64& xa, Lane64& xe) {
+__device__ __forceinline__ void cell_lane(const StepArgs& A, uint32_t step, int cell, bool doA, uint16_t* lA,
+                                          uint16_t* lG, const uint16_t* lE, LaneCell& L, const Cnt& cnt, Lane64& xa,
+                                          Lane64& xe) {
   const bool bath = A.mask & (AXPIC_CH_COMPTON | AXPIC_CH_BREMS);
   const long abase = (long)cell * A.a.cap;
   const long gbase = (long)cell * A.g.cap;
   const long ebase = (long)cell * A.e.cap;
   const int nA = doA ? L.nflA : 0;
-  const int nG = doE ? L.nflG : 0;
-  const int nE = doE ? L.nflE : 0;
+  const int nG = L.nflG;
+  const int nE = L.nflE;
   AxItem ta[kLoad];
   PhItem tg[kLoad];
 #pragma unroll
@@ -1822,61 +1836,141 @@ __device__ __forceinline__ void cell_lane(const StepArgs& A, uint32_t step, int 
     }
   }
 
-  // tail movers, loaded together: the axions' unless the step reuses the
-  // freed slots, the photons' when every photon removal is known
-  const bool reuse = doA && doE;
-  FillIt fa = fill_begin(lA, reuse ? 0 : nrmA, na);
-  Mover ma[kLoad], mg[kLoad];
-  fill_load(A.a, abase, lA, reuse ? 0 : nrmA, fa, ma);
+  // photon tail movers, loaded together, when every photon removal is known
+  Mover mg[kLoad];
   const bool gFill = nG <= kLoad;
   FillIt fg = fill_begin(lG, nrmG, ng - nrmG);
   if (gFill) fill_load(A.g, gbase, lG, nrmG, fg, mg);
-  if (!reuse) {
-#pragma unroll
-    for (int t = 0; t < kLoad; ++t) mover_store(A.a, abase, ma[t]);
-    fill_rest(A.a, abase, lA, nrmA, fa);
-  }
 
-  if (doE) {
-    // new axions: gamma->a products, then thermal-bath events
-    const AxDest D{lA, reuse ? nrmA : 0, 32, reuse ? L.na : na};
-    int NP = 0;
+  // new axions: gamma->a products, then thermal-bath events
+  const AxDest D{lA, nrmA, 32, L.na};
+  int NP = 0;
 #pragma unroll
-    for (int j = 0; j < kLoad; ++j) {
-      if (Kg[j]) gamma_products(A, tg[j], abase, D, NP, Kg[j], cnt);
-      NP += Kg[j];
-    }
-    for (int i = kLoad; i < nG; ++i) {
-      const PhItem t = ph_load(A, gbase, lG[32 * i]);
-      bool removed;
-      const int K = photon_outcome(A, t, gbase, cnt, &removed);
-      if (K) gamma_products(A, t, abase, D, NP, K, cnt);
-      NP += K;
-      if (removed) lG[32 * nrmG++] = (uint16_t)t.slot;
-    }
-    for (int i = 0; i < nE; ++i) {
-      const ElItem t = el_load(A, ebase, lE[32 * i], L.wu);
-      NP += electron_events<true>(A, step, cell, t, abase, D, NP, L.r_cc, L.r_cb, L.r_T, L.wu, cnt, xe);
-    }
-    na = min(D.base - D.nholes + NP, A.a.cap);
-    if (reuse && NP < nrmA) {
-      // freed slots left over: closed from the tail (their movers lie beyond
-      // every slot a new axion took)
-      FillIt fr = fill_begin(lA + 32 * NP, nrmA - NP, na);
-      fill_rest(A.a, abase, lA + 32 * NP, nrmA - NP, fr);
-    }
-    // photon tail fill (a->gamma products included)
-    if (gFill) {
-#pragma unroll
-      for (int t = 0; t < kLoad; ++t) mover_store(A.g, gbase, mg[t]);
-    } else {
-      fg = fill_begin(lG, nrmG, ng - nrmG);
-    }
-    fill_rest(A.g, gbase, lG, nrmG, fg);
-    ng -= nrmG;
+  for (int j = 0; j < kLoad; ++j) {
+    if (Kg[j]) gamma_products(A, tg[j], abase, D, NP, Kg[j], cnt);
+    NP += Kg[j];
   }
+  for (int i = kLoad; i < nG; ++i) {
+    const PhItem t = ph_load(A, gbase, lG[32 * i]);
+    bool removed;
+    const int K = photon_outcome(A, t, gbase, cnt, &removed);
+    if (K) gamma_products(A, t, abase, D, NP, K, cnt);
+    NP += K;
+    if (removed) lG[32 * nrmG++] = (uint16_t)t.slot;
+  }
+  for (int i = 0; i < nE; ++i) {
+    const ElItem t = el_load(A, ebase, lE[32 * i], L.wu);
+    NP += electron_events<true>(A, step, cell, t, abase, D, NP, L.r_cc, L.r_cb, L.r_T, L.wu, cnt, xe);
+  }
+  na = min(D.base - D.nholes + NP, A.a.cap);
+  if (NP < nrmA) {
+    // freed slots left over: closed from the tail (their movers lie beyond
+    // every slot a new axion took)
+    FillIt fr = fill_begin(lA + 32 * NP, nrmA - NP, na);
+    fill_rest(A.a, abase, lA + 32 * NP, nrmA - NP, fr);
+  }
+  // photon tail fill (a->gamma products included)
+  if (gFill) {
+#pragma unroll
+    for (int t = 0; t < kLoad; ++t) mover_store(A.g, gbase, mg[t]);
+  } else {
+    fg = fill_begin(lG, nrmG, ng - nrmG);
+  }
+  fill_rest(A.g, gbase, lG, nrmG, fg);
+  ng -= nrmG;
   L.na = na;
   L.ng = ng;
+}
+
+// The absorb phase of a separate call by one lane: the cell's flagged axions
+// in slot order straight from its staged mask row (up to kLightAbsorb of
+// them, so no list is needed), the next one's record and momentum loaded
+// while one is decided, its position only if it converts. Words of the row
+// are cleared as they are read and take the removed slots' bits, which the
+// tail fill then follows. Weight reduction flags every axion of every cell:
+// taken by the warp one cell after the other (FP64 sums of 32 lanes for 24
+// axions, reduced by 20 adds of 1/64 rate, and three dependent round trips a
+// cell) the kernel took 341 us for 112,095 cells of 23 axions; a lane a cell
+// takes 100 us. Beyond 64 flagged axions the chain of one lane, about
+// 1 us an axion, gets longer than the warp's way through its cells.
+constexpr int kLightAbsorb = 64;
+
+__device__ __forceinline__ void absorb_lane(const StepArgs& A, int cell, uint32_t* row, LaneCell& L, const Cnt& cnt,
+                                            Lane64& xa) {
+  const bool bath = A.mask & (AXPIC_CH_COMPTON | AXPIC_CH_BREMS);
+  const long abase = (long)cell * A.a.cap, gbase = (long)cell * A.g.cap;
+  const int n = L.na, nw = (n + 31) >> 5;
+  int w = -1;
+  uint32_t v = 0u;
+  auto next = [&]() {  // the next flagged slot, or -1
+    while (v == 0u) {
+      if (++w >= nw) return -1;
+      v = row[w];
+      row[w] = 0u;
+      if (w == nw - 1 && (n & 31)) v &= (1u << (n & 31)) - 1u;  // bits beyond n never count
+    }
+    const int b = __ffs(v) - 1;
+    v &= v - 1u;
+    return 32 * w + b;
+  };
+  AxItem t;
+  float4 q;
+  t.slot = next();
+  t.x = t.y = t.z = 0.f;
+  if (t.slot >= 0) {
+    t.r = A.recA[abase + t.slot];
+    q = A.a.wp[abase + t.slot];
+  }
+  int run = 0, nrm = 0;
+  while (t.slot >= 0) {
+    t.w = q.x;
+    t.px = q.y;
+    t.py = q.z;
+    t.pz = q.w;
+    const int slot2 = next();
+    uint4 r2 = make_uint4(0, 0, 0, 0);
+    if (slot2 >= 0) {
+      r2 = A.recA[abase + slot2];
+      q = A.a.wp[abase + slot2];
+    }
+    bool removed;
+    const int K = axion_outcome(A, t, abase, bath, cnt, xa, &removed);
+    if (K > 0) {
+      const float4 u = A.a.xyz[abase + t.slot];
+      const float wprod = __uint_as_float(t.r.y);
+      const float3 pg = photon_from_axion(A, t.px, t.py, t.pz);
+      for (int k = 0; k < K; ++k) {
+        const int dst = L.ng + run + k;
+        if (dst < A.g.cap) write_particle(A.g, gbase + dst, wprod, pg.x, pg.y, pg.z, u.x, u.y, u.z);
+        else cnt.add(C_DROP, 1);
+      }
+      run += K;
+    }
+    if (removed) {
+      row[t.slot >> 5] |= 1u << (t.slot & 31);
+      ++nrm;
+    }
+    t.slot = slot2;
+    t.r = r2;
+  }
+  L.ng = min(L.ng + run, A.g.cap);
+  if (nrm == 0) return;
+  // tail fill: removed slots below ns, ascending, take the kept slots from ns on
+  const int ns = n - nrm;
+  int src = ns;
+  for (int wd = 0; 32 * wd < ns; ++wd) {
+    uint32_t h = row[wd];
+    if (32 * wd + 32 > ns && (ns & 31)) h &= (1u << (ns & 31)) - 1u;
+    for (; h; h &= h - 1u) {
+      while ((row[src >> 5] >> (src & 31)) & 1u) ++src;
+      const long d = abase + 32 * wd + __ffs(h) - 1;
+      A.a.wp[d] = A.a.wp[abase + src];
+      const float4 u = A.a.xyz[abase + src];
+      A.a.xyz[d] = make_float4(u.x, u.y, u.z, 0.f);
+      ++src;
+    }
+  }
+  L.na = ns;
 }
 
 #ifndef AXPIC_EVENT_MIN_CTAS
@@ -1972,10 +2066,11 @@ __global__ void __launch_bounds__(128, PH == 3 ? AXPIC_EVENT_FULL_MIN_CTAS : AXP
   if (valid) {
     if (staged) {
       uint32_t nzA = 0u, nzG = 0u, nzE = 0u;
-      if (PH & PH_ABSORB) L.nflA = scan_row(rA, na_start, lA, &nzA);
+      if (PH == PH_ABSORB) L.nflA = count_row(rA, na_start, &nzA);
+      else if (PH & PH_ABSORB) L.nflA = scan_row(rA, na_start, lA, &nzA);
       if (emitG) L.nflG = scan_row(rG, L.ng0, lG, &nzG);
       if (emitE) L.nflE = scan_row(rE, ne, lE, &nzE);
-      hA = L.nflA > kLight;
+      hA = L.nflA > (PH == PH_ABSORB ? kLightAbsorb : kLight);
       hE = L.nflG > kLight || L.nflE > kLightE;
       defer = PH == (PH_ABSORB | PH_EMIT) && (hA || hE);
       if (!defer) {
@@ -2014,7 +2109,7 @@ __global__ void __launch_bounds__(128, PH == 3 ? AXPIC_EVENT_FULL_MIN_CTAS : AXP
     // by event_heavy_kernel after this kernel (a warp per cell); either way
     // the new axions reuse the freed slots
     if (valid && !defer && (L.nflA | L.nflG | L.nflE))
-      cell_lane(A, step, cell, true, true, lA, lG, lE, L, cnt, xa, xe);
+      cell_lane(A, step, cell, true, lA, lG, lE, L, cnt, xa, xe);
     // the heavy cells are listed for event_heavy_kernel, from index cell0
     const unsigned hm = __ballot_sync(kFull, defer);
     if (hm) {
@@ -2024,7 +2119,7 @@ __global__ void __launch_bounds__(128, PH == 3 ? AXPIC_EVENT_FULL_MIN_CTAS : AXP
       if (defer) A.heavy[A.cell0 + base + __popc(hm & ((1u << lane) - 1u))] = cell;
     }
   } else if (PH == PH_ABSORB) {
-    if (valid && !hA && L.nflA) cell_lane(A, step, cell, true, false, lA, lG, lE, L, cnt, xa, xe);
+    if (valid && !hA && L.nflA) absorb_lane(A, cell, rA, L, cnt, xa);
     __syncwarp();
     for (unsigned hm = __ballot_sync(kFull, valid && hA); hm; hm &= hm - 1u) {
       const int j = __ffs(hm) - 1;
@@ -2044,7 +2139,7 @@ __global__ void __launch_bounds__(128, PH == 3 ? AXPIC_EVENT_FULL_MIN_CTAS : AXP
       }
     }
   } else {
-    if (valid && !hE && (L.nflG | L.nflE)) cell_lane(A, step, cell, false, true, lA, lG, lE, L, cnt, xa, xe);
+    if (valid && !hE && (L.nflG | L.nflE)) cell_lane(A, step, cell, false, lA, lG, lE, L, cnt, xa, xe);
     __syncwarp();
     for (unsigned hm = __ballot_sync(kFull, valid && hE); hm; hm &= hm - 1u) {
       const int j = __ffs(hm) - 1;
