@@ -279,7 +279,7 @@ axpic_status axpic_deposit_composition(axpic_ctx *ctx, int32_t bind_species, con
  * closed by the tail fill (the slot rule of a full step's axions). Staying
  * axions keep their slots unless the tail fill moves them. Axions beyond the
  * capacity are dropped, counted and latch AXPIC_E_CAPACITY. Asynchronous on the context's stream; the first
- * call allocates scratch (33 bytes per axion slot plus 216 per cell), later
+ * call allocates scratch (32.125 bytes per axion slot plus 64 per cell), later
  * calls allocate nothing. AXPIC_E_INVALID (nothing launched) for a grid
  * that does not match, h_cm <= 0, dt_s < 0, c dt_s >= h_cm or another
  * boundary value, or a negative mass. */

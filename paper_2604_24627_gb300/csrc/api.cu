@@ -115,8 +115,8 @@ struct axpic_ctx {
   float* sur_uni = nullptr;        // [kSrLen] the network's cell-independent quantiles
   unsigned char* sur_img = nullptr;  // the network laid out for the fused kernels
   // axion streaming scratch, made by the first axpic_stream_axions call
-  uint8_t* st_dir = nullptr;  // [ncells * axion capacity]
-  int32_t* st_cnt = nullptr;  // [ncells * 27 * 2]: counts, then group offsets
+  uint32_t* st_freed = nullptr;  // [ncells * words of the axion capacity]
+  uint16_t* st_off = nullptr;    // [ncells * kStreamOffs]
   float* st_buf = nullptr;    // [ncells * axion capacity * 8]
   double* st_stats = nullptr; // [4]
   // axion merging scratch, made by the first axpic_merge_axions call
@@ -396,7 +396,7 @@ static void free_ctx(axpic_ctx* ctx) {
                   ctx->tables, ctx->tally, ctx->counters, ctx->err, ctx->scratch, ctx->bits,
                   ctx->recA,   ctx->recG,  ctx->recE,     ctx->step_dev, ctx->sr, ctx->srtab,
                   ctx->sur_P,  ctx->sur_mu, ctx->sur_sigma, ctx->sur_trust, ctx->sur_img, ctx->sur_skip,
-                  ctx->sr_src, ctx->sur_uni, ctx->st_dir, ctx->st_cnt, ctx->st_buf, ctx->st_stats, ctx->mg_grp,
+                  ctx->sr_src, ctx->sur_uni, ctx->st_freed, ctx->st_off, ctx->st_buf, ctx->st_stats, ctx->mg_grp,
                   ctx->mg_removed, ctx->heavy, ctx->heavy_n};
   for (void* b : bufs)
     if (b) cudaFree(b);
@@ -1263,9 +1263,10 @@ static axpic_status stream_setup(axpic_ctx* ctx, int32_t nx, int32_t ny, int32_t
   if (!(kappa < 1.0f - 0x1p-20f))
     return fail(ctx, AXPIC_E_INVALID, "axpic_stream_axions: c dt must stay below the cell edge");
   const size_t slots = (size_t)d.ncells * d.axions.capacity;
-  if (!ctx->st_dir) {
-    CK(cudaMalloc((void**)&ctx->st_dir, std::max<size_t>(slots, 1)), "streaming scratch");
-    CK(cudaMalloc((void**)&ctx->st_cnt, sizeof(int32_t) * 2 * kStreamDirs * (size_t)d.ncells), "streaming scratch");
+  if (!ctx->st_freed) {
+    const size_t words = (size_t)d.ncells * ((d.axions.capacity + 31) / 32);
+    CK(cudaMalloc((void**)&ctx->st_freed, sizeof(uint32_t) * std::max<size_t>(words, 1)), "streaming scratch");
+    CK(cudaMalloc((void**)&ctx->st_off, sizeof(uint16_t) * kStreamOffs * (size_t)d.ncells), "streaming scratch");
     CK(cudaMalloc((void**)&ctx->st_buf, sizeof(float) * 8 * std::max<size_t>(slots, 1)), "streaming scratch");
     CK(cudaMalloc((void**)&ctx->st_stats, sizeof(double) * 4), "streaming scratch");
     CK(cudaMemsetAsync(ctx->st_stats, 0, sizeof(double) * 4, ctx->stream), "memset");
@@ -1280,9 +1281,8 @@ static axpic_status stream_setup(axpic_ctx* ctx, int32_t nx, int32_t ny, int32_t
   a.kappa = kappa;
   a.mu = (float)(mass_keV / kMeC2);
   a.periodic = boundary == 0;
-  a.dir = ctx->st_dir;
-  a.cnt = ctx->st_cnt;
-  a.goff = ctx->st_cnt + (size_t)kStreamDirs * d.ncells;
+  a.freed = ctx->st_freed;
+  a.goff = ctx->st_off;
   a.buf = ctx->st_buf;
   a.stats = ctx->st_stats;
   a.err = ctx->err;

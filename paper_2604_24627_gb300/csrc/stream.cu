@@ -3,12 +3,13 @@
 // sub-luminal; the transport of the axion macroparticles between steps) on
 // the cell-sorted slabs, positions being fractions of the cell.
 //
-// Two kernels, a warp per cell each (grid-stride):
-//  * stream_move_kernel moves every axion of its cell, in binary32 with each
+// Two kernels, a warp for K consecutive cells each:
+//  * stream_move_kernel moves every axion of its cells, in binary32 with each
 //    rounding fixed (the result decides the destination cell), writes the
-//    new position in place, the direction of each slot and the count per
-//    direction, and copies the leaving axions into the cell's staging rows,
-//    grouped by direction in slot order.
+//    new position in place, a bit per slot that does not stay, the first
+//    staging row of each of the 27 directions (16-bit prefix sums, 64 bytes a
+//    cell), and the leaving axions into the cell's staging rows, grouped by
+//    direction in slot order.
 //  * stream_place_kernel takes the arrivals from its neighbours' staging
 //    rows, ordered by the neighbour's position relative to it, (dz, dy, dx)
 //    ascending, then by source slot, into the slots its own leavers freed
@@ -16,9 +17,20 @@
 //    by the tail fill. Staying axions keep their slots unless the tail fill
 //    moves them. Slots beyond the capacity are dropped, counted, and latch
 //    ERR_CAPACITY.
-// The first kernel writes only its own cell's slots and rows; the second
-// reads the neighbours' rows and writes only its own slab, so neither needs
+// The first kernel writes only its own cells' slots and rows; the second
+// reads the neighbours' rows and writes only its own slabs, so neither needs
 // a barrier across cells.
+//
+// Bound by instruction issue and memory latency together; the bytes are 48 an
+// axion (32 read, 16 written) and 96 a leaver (staged, read, placed). So a
+// warp takes as many cells as keep its lanes full, an axion's records stay in
+// registers from the move to the staging, the direction ranks and counts come
+// from one match per 32 slots, an arrival finds its group by a 5-step search
+// and its slot by a bit count, and a neighbour's group is two 16-bit loads.
+// Warp instructions a cell, move + place: 912 + 1371 -> 696 + 727 with 128
+// axions in 2-D, 404 + 595 -> 156 + 253 with 13 in 3-D. Time of a call:
+// 65,536 cells of 128 249 -> 216 us, 262,144 cells of 13 in 3-D 350 -> 166 us
+// (ncu, both kernels).
 #include "stream.h"
 
 namespace axpic {
@@ -44,230 +56,502 @@ __device__ __forceinline__ float advance(float q, float d, int* shift) {
   return r;
 }
 
-__global__ void __launch_bounds__(kThreads) stream_move_kernel(StreamArgs a) {
-  __shared__ int cnt[kWarps][32];
-  __shared__ int run[kWarps][32];
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+// One axion moved: its new position in u (unchanged where it has no
+// momentum), the direction returned.
+__device__ __forceinline__ int move_axion(const StreamArgs& a, const float4& r, float4& u) {
+  // E = sqrt(p^2 + mu^2): v = p / E in units of c
+  const float en = __fsqrt_rn(__fadd_rn(
+      __fadd_rn(__fadd_rn(__fmul_rn(r.y, r.y), __fmul_rn(r.z, r.z)), __fmul_rn(r.w, r.w)), __fmul_rn(a.mu, a.mu)));
+  int sx = 0, sy = 0, sz = 0;
+  if (en > 0.f) {
+    const float k = __fdiv_rn(a.kappa, en);
+    u.w = 0.f;
+    if (a.nx > 1) u.x = advance(u.x, __fmul_rn(k, r.y), &sx);
+    if (a.ny > 1) u.y = advance(u.y, __fmul_rn(k, r.z), &sy);
+    if (a.nz > 1) u.z = advance(u.z, __fmul_rn(k, r.w), &sz);
+  }
+  return (sz + 1) * 9 + (sy + 1) * 3 + (sx + 1);
+}
+
+// Whether the neighbour of cell c in direction o lies outside an open box.
+__device__ __forceinline__ bool escapes(const StreamArgs& a, int c, int o) {
+  const int ii = c % a.nx + o % 3 - 1, jj = (c / a.nx) % a.ny + (o / 3) % 3 - 1, kk = c / (a.nx * a.ny) + o / 9 - 1;
+  return ii < 0 || ii >= a.nx || jj < 0 || jj >= a.ny || kk < 0 || kk >= a.nz;
+}
+
+__device__ __forceinline__ void count_escape(const StreamArgs& a, const float4& r) {
+  const double wd = (double)r.x;
+  const double pm = sqrt((double)r.y * r.y + (double)r.z * r.z + (double)r.w * r.w + (double)a.mu * a.mu);
+  atomicAdd(a.stats + 0, 1.0);
+  atomicAdd(a.stats + 1, wd);
+  atomicAdd(a.stats + 2, wd * pm * kMeC2);
+}
+
+// The warp's K cells as one flat range of slots: cell k's slots start at
+// off[k].
+template <int K>
+struct FlatCells {
+  int off[K + 1];
+  __device__ __forceinline__ void set(int n) {  // lanes < K hold their cell's count, the others 0
+    off[0] = 0;
+#pragma unroll
+    for (int k = 0; k < K; ++k) off[k + 1] = off[k] + __shfl_sync(kAll, n, k);
+  }
+  __device__ __forceinline__ int total() const { return off[K]; }
+  // cell of flat slot f, and the slot in it
+  __device__ __forceinline__ int cell(int f, int* slot) const {
+    int k = 0, o = 0;
+#pragma unroll
+    for (int j = 1; j < K; ++j)
+      if (f >= off[j]) k = j, o = off[j];
+    *slot = f - o;
+    return k;
+  }
+};
+
+__device__ __forceinline__ int incl_scan(int v) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int d = 1; d < 32; d <<= 1) {
+    const int t = __shfl_up_sync(kAll, v, d);
+    if (lane >= d) v += t;
+  }
+  return v;
+}
+
+// Slots a warp holds in registers from the move to the staging, passes of 32:
+// four cells together, one cell. A cell with more is read twice beyond them.
+constexpr int kHoldGroup = 4, kHoldOne = 5;
+constexpr int kGroup = 4;  // cells a warp
+constexpr int kWords = 32 / kGroup;  // words of freed bits a cell of a group has in shared memory
+static_assert(kHoldGroup <= kWords, "freed words");
+
+struct MoveShared {
+  int cnt[kGroup * 32];      // leavers per direction so far
+  int off[kGroup * 32];      // first staging row of a direction
+  uint32_t freed[32];
+};
+
+// The K cells from c0 on with n_l slots in lane k < K: all of them in R
+// register passes, or (K = 1) more than those hold.
+template <int K, int R>
+__device__ __forceinline__ void move_cells(const StreamArgs& a, int c0, int n_l, MoveShared& S) {
+  const int lane = threadIdx.x & 31;
   const unsigned lt = (1u << lane) - 1u;
-  for (int c = blockIdx.x * kWarps + wid; c < a.ncells; c += gridDim.x * kWarps) {
-    cnt[wid][lane] = 0;
-    run[wid][lane] = 0;
+  const int W = (a.s.cap + 31) >> 5;
+  FlatCells<K> F;
+  F.set(n_l);
+  const int N = F.total();
+#pragma unroll
+  for (int k = 0; k < K; ++k) S.cnt[32 * k + lane] = 0;
+  if (K > 1) S.freed[lane] = 0u;
+  __syncwarp();
+
+  // the freed bit of flat slot f, slot sl of cell k (all lanes call it)
+  auto mark = [&](int f, int k, int sl, bool fr) {
+    if (K == 1) {
+      const unsigned m = __ballot_sync(kAll, fr);
+      if (lane == 0) a.freed[(size_t)c0 * W + (f >> 5)] = m;
+    } else if (fr) {
+      atomicOr(&S.freed[kWords * k + (sl >> 5)], 1u << (sl & 31));
+    }
+  };
+  // rank of a leaver among its cell and direction, in slot order
+  auto rank = [&](bool leave, int key) {
+    const unsigned m = __match_any_sync(kAll, leave ? key : 32 * K + lane);
+    const int base = leave ? S.cnt[key] : 0;
     __syncwarp();
-    const int n = min(max(a.s.count[c], 0), a.s.cap);
-    const long base = (long)c * a.s.cap;
-    const int ci = c % a.nx, cj = (c / a.nx) % a.ny, ck = c / (a.nx * a.ny);
-    // two chunks of 32 slots per pass: both chunks' loads are issued before
-    // either is stored
-    for (int s0 = 0; s0 < n; s0 += 64) {
-      float w[2], px[2], py[2], pz[2], x[2], y[2], z[2];
+    if (leave && (m & lt) == 0) S.cnt[key] = base + __popc(m);
+    __syncwarp();
+    return base + __popc(m & lt);
+  };
+  auto staged = [&](int key, int rk) {
+    return reinterpret_cast<float4*>(a.buf) + ((size_t)(c0 + (key >> 5)) * a.s.cap + S.off[key] + rk) * 2;
+  };
+
+  // every pass's records are loaded before any is moved
+  float4 r[R], u[R];
 #pragma unroll
-      for (int hh = 0; hh < 2; ++hh) {
-        const int slot = s0 + 32 * hh + lane;
-        w[hh] = px[hh] = py[hh] = pz[hh] = x[hh] = y[hh] = z[hh] = 0.f;
-        if (slot < n) {
-          const long q = base + slot;
-          const float4 r = a.s.wp[q], u = a.s.xyz[q];
-          w[hh] = r.x, px[hh] = r.y, py[hh] = r.z, pz[hh] = r.w;
-          x[hh] = u.x, y[hh] = u.y, z[hh] = u.z;
-        }
-      }
+  for (int i = 0; i < R; ++i) {
+    const int f = 32 * i + lane;
+    if (f < N) {
+      int sl;
+      const int k = F.cell(f, &sl);
+      const long q = (long)(c0 + k) * a.s.cap + sl;
+      r[i] = a.s.wp[q];
+      u[i] = a.s.xyz[q];
+    }
+  }
+  int kr[R];  // a leaver's rank << 8 | its cell and direction, or -1
 #pragma unroll
-      for (int hh = 0; hh < 2; ++hh) {
-        const int slot = s0 + 32 * hh + lane;
-        if (slot >= n) continue;
-        const long q = base + slot;
-        // E = sqrt(p^2 + mu^2): v = p / E in units of c
-        const float en = __fsqrt_rn(__fadd_rn(
-            __fadd_rn(__fadd_rn(__fmul_rn(px[hh], px[hh]), __fmul_rn(py[hh], py[hh])), __fmul_rn(pz[hh], pz[hh])),
-            __fmul_rn(a.mu, a.mu)));
-        int sx = 0, sy = 0, sz = 0;
-        if (en > 0.f) {
-          const float k = __fdiv_rn(a.kappa, en);
-          float4 u = make_float4(x[hh], y[hh], z[hh], 0.f);
-          if (a.nx > 1) u.x = advance(x[hh], __fmul_rn(k, px[hh]), &sx);
-          if (a.ny > 1) u.y = advance(y[hh], __fmul_rn(k, py[hh]), &sy);
-          if (a.nz > 1) u.z = advance(z[hh], __fmul_rn(k, pz[hh]), &sz);
-          a.s.xyz[q] = u;
-        }
-        int o = (sz + 1) * 9 + (sy + 1) * 3 + (sx + 1);
-        if (!a.periodic) {
-          const int ii = ci + sx, jj = cj + sy, kk = ck + sz;
-          if (ii < 0 || ii >= a.nx || jj < 0 || jj >= a.ny || kk < 0 || kk >= a.nz) {
-            o = kStreamEscaped;
-            const double wd = (double)w[hh];
-            const double pm = sqrt((double)px[hh] * px[hh] + (double)py[hh] * py[hh] + (double)pz[hh] * pz[hh] +
-                                   (double)a.mu * a.mu);
-            atomicAdd(a.stats + 0, 1.0);
-            atomicAdd(a.stats + 1, wd);
-            atomicAdd(a.stats + 2, wd * pm * kMeC2);
-          }
-        }
-        a.dir[q] = (uint8_t)o;
-        atomicAdd(&cnt[wid][o], 1);
+  for (int i = 0; i < R; ++i) {
+    kr[i] = -1;
+    if (32 * i >= N) continue;
+    const int f = 32 * i + lane;
+    bool leave = false, fr = false;
+    int key = 0, k = 0, sl = 0;
+    if (f < N) {
+      k = F.cell(f, &sl);
+      const int o = move_axion(a, r[i], u[i]);
+      a.s.xyz[(long)(c0 + k) * a.s.cap + sl] = u[i];
+      fr = leave = o != kStreamStay;
+      if (leave && !a.periodic && escapes(a, c0 + k, o)) {
+        leave = false;
+        count_escape(a, r[i]);
       }
+      key = 32 * k + o;
+    }
+    mark(f, k, sl, fr);
+    const int rk = rank(leave, key);
+    if (leave) kr[i] = rk << 8 | key;
+  }
+  // slots beyond the register passes: counted now, moved and staged below
+  int held = 0;
+  if (K == 1 && N > 32 * R) {
+    held = S.cnt[lane];
+    __syncwarp();
+    for (int f0 = 32 * R; f0 < N; f0 += 32) {
+      const int f = f0 + lane;
+      bool fr = false;
+      if (f < N) {
+        const long q = (long)c0 * a.s.cap + f;
+        const float4 rr = a.s.wp[q];
+        float4 uu = a.s.xyz[q];
+        const int o = move_axion(a, rr, uu);
+        fr = o != kStreamStay;
+        if (fr && (a.periodic || !escapes(a, c0, o))) atomicAdd(&S.cnt[o], 1);
+      }
+      mark(f, 0, f, fr);
     }
     __syncwarp();
-    if (lane < kStreamDirs) a.cnt[(size_t)c * kStreamDirs + lane] = cnt[wid][lane];
-    // staging offset of each direction's group: the leavers of the lower
-    // directions (13 stays and 27 escaped hold none)
-    const int v = (lane < kStreamDirs && lane != kStreamStay) ? cnt[wid][lane] : 0;
-    int incl = v;
+  }
+  // staging offset of each direction's group: the leavers of the lower
+  // directions (those that stay and those that escape hold none)
 #pragma unroll
-    for (int d = 1; d < 32; d <<= 1) {
-      const int t = __shfl_up_sync(kAll, incl, d);
-      if (lane >= d) incl += t;
-    }
-    const int off = incl - v;
-    if (lane < kStreamDirs) a.goff[(size_t)c * kStreamDirs + lane] = off;
-    for (int s0 = 0; s0 < n; s0 += 32) {
-      const int slot = s0 + lane;
-      const int o = slot < n ? (int)a.dir[base + slot] : 31;
-      const bool leave = o < kStreamDirs && o != kStreamStay;
-      const unsigned m = __match_any_sync(kAll, o);
-      const int goff = __shfl_sync(kAll, off, o);
+  for (int k = 0; k < K; ++k) {
+    const int v = S.cnt[32 * k + lane];
+    const int e = incl_scan(v) - v;
+    S.off[32 * k + lane] = e;
+    if (K == 1 || c0 + k < a.ncells) a.goff[(size_t)(c0 + k) * kStreamOffs + lane] = (uint16_t)e;
+  }
+  if (K > 1) {
+    const int k = lane / kWords, w = lane % kWords;
+    if (32 * w < __shfl_sync(kAll, n_l, k)) a.freed[(size_t)(c0 + k) * W + w] = S.freed[lane];
+  }
+  __syncwarp();
+#pragma unroll
+  for (int i = 0; i < R; ++i) {
+    if (kr[i] < 0) continue;
+    float4* dst = staged(kr[i] & 255, kr[i] >> 8);
+    dst[0] = r[i];
+    dst[1] = u[i];
+  }
+  if (K == 1 && N > 32 * R) {
+    S.cnt[lane] = held;
+    __syncwarp();
+    for (int f0 = 32 * R; f0 < N; f0 += 32) {
+      const int f = f0 + lane;
+      bool leave = false;
+      int o = 0;
+      float4 rr, uu;
+      if (f < N) {
+        const long q = (long)c0 * a.s.cap + f;
+        rr = a.s.wp[q];
+        uu = a.s.xyz[q];
+        o = move_axion(a, rr, uu);
+        a.s.xyz[q] = uu;
+        leave = o != kStreamStay;
+        if (leave && !a.periodic && escapes(a, c0, o)) {
+          leave = false;
+          count_escape(a, rr);
+        }
+      }
+      const int rk = rank(leave, o);
       if (leave) {
-        const int pos = goff + run[wid][o] + __popc(m & lt);
-        const long q = base + slot;
-        float4* dst = reinterpret_cast<float4*>(a.buf + ((size_t)c * a.s.cap + pos) * 8);
-        dst[0] = a.s.wp[q];
-        dst[1] = a.s.xyz[q];
+        float4* dst = staged(o, rk);
+        dst[0] = rr;
+        dst[1] = uu;
       }
-      __syncwarp();
-      if (leave && (m & lt) == 0) run[wid][o] += __popc(m);  // the group's first lane
-      __syncwarp();
+    }
+  }
+  __syncwarp();
+}
+
+// A warp takes K cells (kGroup, or 1): together where their slots fit the
+// register passes, else one after the other.
+template <int K>
+__global__ void __launch_bounds__(kThreads, 3) stream_move_kernel(StreamArgs a) {
+  __shared__ MoveShared S[kWarps];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int c0 = (blockIdx.x * kWarps + wid) * K;
+  if (c0 >= a.ncells) return;
+  const int n_l = lane < K && c0 + lane < a.ncells ? min(max(a.s.count[c0 + lane], 0), a.s.cap) : 0;
+  if (K > 1 && __reduce_add_sync(kAll, (unsigned)n_l) <= 32 * kHoldGroup) {
+    move_cells<K, kHoldGroup>(a, c0, n_l, S[wid]);
+  } else {
+    for (int k = 0; k < K && c0 + k < a.ncells; ++k) {
+      const int n = __shfl_sync(kAll, n_l, k);
+      move_cells<1, kHoldOne>(a, c0 + k, lane == 0 ? n : 0, S[wid]);
     }
   }
 }
 
-__global__ void __launch_bounds__(kThreads) stream_place_kernel(StreamArgs a) {
+// Position of the k-th (0-based) set bit of a word that has more than k.
+__device__ __forceinline__ int nth_bit(uint32_t v, int k) {
+  int p = 0;
+#pragma unroll
+  for (int s = 16; s; s >>= 1) {
+    const int c = __popc((v >> p) & ((1u << s) - 1u));
+    if (k >= c) k -= c, p += s;
+  }
+  return p;
+}
+
+// Cell coordinates, stepped to the next cell without dividing again.
+struct CellAt {
+  int i, j, k;
+  __device__ __forceinline__ void next(const StreamArgs& a) {
+    if (++i == a.nx) {
+      i = 0;
+      if (++j == a.ny) j = 0, ++k;
+    }
+  }
+};
+
+constexpr int kPlace = 2;  // words of freed slots whose arrivals are loaded together
+
+template <int K>
+__global__ void __launch_bounds__(kThreads, 6) stream_place_kernel(StreamArgs a) {
+  // a cell's arrival groups, lane r the neighbour at (dz, dy, dx) = r's
+  // digits - 1: arrivals up to and with the group, the neighbour, and the
+  // staging row of arrival 0 of the cell's numbering
+  __shared__ int g_incl[kWarps][K * 32], g_src[kWarps][K * 32], g_row[kWarps][K * 32];
+  __shared__ uint32_t freed[kWarps][K * 4];
+  __shared__ int sA[kWarps][K], sH[kWarps][K];  // arrivals, freed slots
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const unsigned lt = (1u << lane) - 1u;
   const SpeciesPtrs& s = a.s;
-  for (int c = blockIdx.x * kWarps + wid; c < a.ncells; c += gridDim.x * kWarps) {
-    const int n = min(max(s.count[c], 0), s.cap);
-    const long base = (long)c * s.cap;
-    const int ci = c % a.nx, cj = (c / a.nx) % a.ny, ck = c / (a.nx * a.ny);
-    // freed slots: every slot of the cell that did not stay
-    const int H = n - a.cnt[(size_t)c * kStreamDirs + kStreamStay];
-    // arrivals: lane r (r < 27, r != 13) takes the neighbour at (dz, dy, dx)
-    // = r's digits - 1, lanes ascending in r; that neighbour's axions that
-    // moved here have the shift -(dz, dy, dx), direction 26 - r. Every
-    // lane's group is found at once; a scan orders the groups by r.
-    int m = 0, src = 0, g = 0;
-    if (lane < kStreamDirs && lane != kStreamStay) {
-      const int r = lane;
-      const int dz = r / 9 - 1, dy = (r / 3) % 3 - 1, dx = r % 3 - 1;
-      int si = ci + dx, sj = cj + dy, sk = ck + dz;
-      bool ok = !((dx && a.nx == 1) || (dy && a.ny == 1) || (dz && a.nz == 1));
+  const int c0 = (blockIdx.x * kWarps + wid) * K;
+  if (c0 >= a.ncells) return;
+  const int W = (s.cap + 31) >> 5;
+  const int n_l = lane < K && c0 + lane < a.ncells ? min(max(s.count[c0 + lane], 0), s.cap) : 0;
+  FlatCells<K> F;
+  F.set(n_l);
+  // the cells' slots as one flat range where they are few, else cell by cell
+  const bool flat = K > 1 && F.total() <= 128;
+  // the arrival groups: the neighbour's axions that moved here have the shift
+  // -(dz, dy, dx), direction 26 - r. All K cells' loads are issued together.
+  const int dz = lane / 9 - 1, dy = (lane / 3) % 3 - 1, dx = lane % 3 - 1;
+  const bool dir = lane < kStreamDirs && lane != kStreamStay && !(dx && a.nx == 1) && !(dy && a.ny == 1) &&
+                   !(dz && a.nz == 1);
+  int m[K], g[K], src[K];
+  CellAt at;
+  {
+    const int row = c0 / a.nx;
+    at.i = c0 - row * a.nx;
+    at.k = row / a.ny;
+    at.j = row - at.k * a.ny;
+  }
+#pragma unroll
+  for (int k = 0; k < K; ++k) {
+    m[k] = g[k] = src[k] = 0;
+    if (c0 + k < a.ncells && dir) {
+      int si = at.i + dx, sj = at.j + dy, sk = at.k + dz;
+      bool ok = true;
       if (a.periodic) {
-        si = (si + a.nx) % a.nx;
-        sj = (sj + a.ny) % a.ny;
-        sk = (sk + a.nz) % a.nz;
-      } else if (si < 0 || si >= a.nx || sj < 0 || sj >= a.ny || sk < 0 || sk >= a.nz) {
-        ok = false;
+        si += si < 0 ? a.nx : (si >= a.nx ? -a.nx : 0);
+        sj += sj < 0 ? a.ny : (sj >= a.ny ? -a.ny : 0);
+        sk += sk < 0 ? a.nz : (sk >= a.nz ? -a.nz : 0);
+      } else {
+        ok = si >= 0 && si < a.nx && sj >= 0 && sj < a.ny && sk >= 0 && sk < a.nz;
       }
       if (ok) {
-        src = (sk * a.ny + sj) * a.nx + si;
-        const size_t k = (size_t)src * kStreamDirs + (kStreamDirs - 1 - r);
-        m = a.cnt[k];
-        g = a.goff[k];
+        src[k] = (sk * a.ny + sj) * a.nx + si;
+        const uint16_t* o = a.goff + (size_t)src[k] * kStreamOffs + (kStreamDirs - 1 - lane);
+        g[k] = o[0];
+        m[k] = o[1];
       }
     }
-    int incl = m;
+    at.next(a);
+  }
+  if (flat) {  // at most 4 words a cell
+    const int n_k = __shfl_sync(kAll, n_l, lane >> 2);
+    if (lane < K * 4)
+      freed[wid][lane] = 32 * (lane & 3) < n_k ? a.freed[(size_t)(c0 + (lane >> 2)) * W + (lane & 3)] : 0u;
+  }
 #pragma unroll
-    for (int d = 1; d < 32; d <<= 1) {
-      const int t = __shfl_up_sync(kAll, incl, d);
-      if (lane >= d) incl += t;
-    }
-    const int A = __shfl_sync(kAll, incl, 31);
-    const int excl = incl - m;
-    // arrival t takes freed slot t (ascending) while there are any, then
-    // slot n + (t - H)
-    for (int t0 = 0; t0 < A; t0 += 32) {
-      const int t = t0 + lane;
-      int sel = 0;
+  for (int k = 0; k < K; ++k) {
+    m[k] -= g[k];
+    const int e = incl_scan(m[k]);
+    g_incl[wid][32 * k + lane] = e;
+    g_src[wid][32 * k + lane] = src[k];
+    g_row[wid][32 * k + lane] = g[k] - (e - m[k]);
+    if (lane == 31) sA[wid][k] = e;
+  }
+  __syncwarp();
+  // staging row of arrival t of cell k: the first group that ends after t
+  auto arrival = [&](int k, int t) {
+    const int* e = g_incl[wid] + 32 * k;
+    int lo = 0;
 #pragma unroll
-      for (int r = 1; r < kStreamDirs; ++r) {
-        const int e = __shfl_sync(kAll, excl, r), mr = __shfl_sync(kAll, m, r);
-        if (mr > 0 && e <= t) sel = r;
-      }
-      const int e = __shfl_sync(kAll, excl, sel);
-      const int gs = __shfl_sync(kAll, g, sel), ss = __shfl_sync(kAll, src, sel);
-      int dst = n + (t - H);
-      const int need = min(t0 + 32, H);  // freed slots of this pass: indices t0 .. need - 1
-      if (t0 < need) {
-        int run = 0;
-        for (int s0 = 0; s0 < n && run < need; s0 += 32) {
-          const int slot = s0 + lane;
-          const unsigned hm = __ballot_sync(kAll, slot < n && a.dir[base + slot] != kStreamStay);
-          const int k = t - run;
-          if (t < H && k >= 0 && k < __popc(hm)) dst = s0 + (int)__fns(hm, 0, k + 1);
-          run += __popc(hm);
-        }
-      }
-      if (t < A && dst < s.cap) {
-        const float* row = a.buf + ((size_t)ss * s.cap + gs + (t - e)) * 8;
-        const float4 u0 = reinterpret_cast<const float4*>(row)[0];
-        const float4 u1 = reinterpret_cast<const float4*>(row)[1];
-        const long q = base + dst;
-        s.wp[q] = u0;
-        s.xyz[q] = u1;
+    for (int st = 16; st; st >>= 1)
+      if (e[lo + st - 1] <= t) lo += st;
+    return reinterpret_cast<const float4*>(a.buf) +
+           ((size_t)g_src[wid][32 * k + lo] * s.cap + g_row[wid][32 * k + lo] + t) * 2;
+  };
+  // arrival t takes freed slot t (ascending) while there are any
+  if (flat) {
+    if (lane < K) {
+      const uint32_t* v = freed[wid] + 4 * lane;
+      sH[wid][lane] = __popc(v[0]) + __popc(v[1]) + __popc(v[2]) + __popc(v[3]);
+    }
+    for (int f0 = 0; f0 < F.total(); f0 += 32) {
+      const int f = f0 + lane;
+      if (f >= F.total()) continue;
+      int sl;
+      const int k = F.cell(f, &sl);
+      const uint32_t* v = freed[wid] + 4 * k;
+      const int w = sl >> 5;
+      if (!((v[w] >> (sl & 31)) & 1u)) continue;
+      int t = __popc(v[w] & ((1u << (sl & 31)) - 1u));
+      for (int j = 0; j < w; ++j) t += __popc(v[j]);
+      if (t < sA[wid][k]) {
+        const float4* x = arrival(k, t);
+        const long q = (long)(c0 + k) * s.cap + sl;
+        const float4 p0 = __ldg(x), q0 = __ldg(x + 1);
+        s.wp[q] = p0;
+        s.xyz[q] = q0;
       }
     }
-    __syncwarp();
-    // fewer arrivals than freed slots: the freed slots left over (indices A
-    // .. H - 1) below the new count ns take, in ascending order, the kept
-    // slots at or beyond ns (stayers and filled slots), in ascending order
-    if (A < H) {
-      const int ns = n - (H - A);
-      for (int j0 = 0;; j0 += 32) {
-        const int j = j0 + lane;
-        int from = -1, to = -1, runH = 0, runTo = 0, runFrom = 0;
-        for (int s0 = 0; s0 < n; s0 += 32) {
-          const int slot = s0 + lane;
-          const bool freed = slot < n && a.dir[base + slot] != kStreamStay;
-          const unsigned hm = __ballot_sync(kAll, freed);
-          const bool left = freed && runH + __popc(hm & lt) >= A;  // freed and not filled
-          const unsigned tm = __ballot_sync(kAll, left && slot < ns);
-          const unsigned fm = __ballot_sync(kAll, slot < n && slot >= ns && !left);
-          int k = j - runTo;
-          if (k >= 0 && k < __popc(tm)) to = s0 + (int)__fns(tm, 0, k + 1);
-          k = j - runFrom;
-          if (k >= 0 && k < __popc(fm)) from = s0 + (int)__fns(fm, 0, k + 1);
-          runH += __popc(hm);
-          runTo += __popc(tm);
-          runFrom += __popc(fm);
-        }
-        if (j < runTo && from >= 0 && to >= 0) {
-          const long qf = base + from, qt = base + to;
-          const float4 r = s.wp[qf], u = s.xyz[qf];
-          s.wp[qt] = r;
-          s.xyz[qt] = u;
-        }
-        if (j0 + 32 >= runTo) break;
+  } else {
+    for (int k = 0; k < K; ++k) {
+      const int n = __shfl_sync(kAll, n_l, k), A = sA[wid][k];
+      if (n == 0) {
+        if (lane == 0) sH[wid][k] = 0;
+        continue;
       }
-    }
-    const int total = n - H + A;
-    if (lane == 0) {
-      s.count[c] = min(total, s.cap);
-      if (total > s.cap) {
-        atomicAdd(a.stats + 3, (double)(total - s.cap));
-        atomicOr(a.err, ERR_CAPACITY);
+      const uint32_t* fw = a.freed + (size_t)(c0 + k) * W;
+      const long base = (long)(c0 + k) * s.cap;
+      const int nw = (n + 31) >> 5;
+      int tb = 0;
+      for (int wb = 0; wb < nw; wb += 32) {
+        const uint32_t f_l = wb + lane < nw ? fw[wb + lane] : 0u;
+        for (int w = wb; w < min(wb + 32, nw); w += kPlace) {
+          // kPlace words at a time, all loaded before any is stored
+          float4 p[kPlace], q[kPlace];
+          bool b[kPlace];
+#pragma unroll
+          for (int i = 0; i < kPlace; ++i) {
+            const uint32_t v = __shfl_sync(kAll, f_l, w - wb + i);  // wb + 32 is a multiple of kPlace
+            const int t = tb + __popc(v & lt);
+            tb += __popc(v);
+            b[i] = ((v >> lane) & 1u) && t < A;
+            if (b[i]) {
+              const float4* x = arrival(k, t);
+              p[i] = __ldg(x);
+              q[i] = __ldg(x + 1);
+            }
+          }
+#pragma unroll
+          for (int i = 0; i < kPlace; ++i)
+            if (b[i]) {
+              s.wp[base + 32 * (w + i) + lane] = p[i];
+              s.xyz[base + 32 * (w + i) + lane] = q[i];
+            }
+        }
       }
+      if (lane == 0) sH[wid][k] = tb;
     }
   }
+  __syncwarp();
+  // then slots n + (t - H): the cells' further arrivals as one flat range
+  FlatCells<K> X;
+  X.off[0] = 0;
+#pragma unroll
+  for (int k = 0; k < K; ++k) X.off[k + 1] = X.off[k] + max(sA[wid][k] - sH[wid][k], 0);
+  for (int f0 = 0; f0 < X.total(); f0 += 32) {
+    const int f = f0 + lane;
+    int e;
+    const int k = X.cell(f, &e);
+    const int dst = __shfl_sync(kAll, n_l, k) + e;
+    if (f < X.total() && dst < s.cap) {
+      const float4* x = arrival(k, sH[wid][k] + e);
+      const long q = (long)(c0 + k) * s.cap + dst;
+      const float4 p0 = __ldg(x), q0 = __ldg(x + 1);
+      s.wp[q] = p0;
+      s.xyz[q] = q0;
+    }
+  }
+  __syncwarp();
+  // fewer arrivals than freed slots: the freed slots left over (indices A
+  // .. H - 1) below the new count ns take, in ascending order, the kept slots
+  // at or beyond ns (stayers and filled slots), in ascending order
+  for (int k = 0; k < K; ++k) {
+    const int A = sA[wid][k], H = sH[wid][k];
+    const int n = __shfl_sync(kAll, n_l, k), ns = n - (H - A);
+    if (A >= H) continue;
+    const uint32_t* fw = flat ? freed[wid] + 4 * k : a.freed + (size_t)(c0 + k) * W;
+    const long base = (long)(c0 + k) * s.cap;
+    int before = 0;  // freed slots of the words before the current one
+    const int w0 = ns >> 5;
+    for (int w = 0; w < w0; ++w) before += __popc(fw[w]);
+    int moved = 0;
+    for (int w = w0; 32 * w < n; ++w) {
+      const uint32_t v = fw[w];
+      const int sl = 32 * w + lane;
+      const bool left = ((v >> lane) & 1u) && before + __popc(v & lt) >= A;  // freed and not filled
+      const bool mv = sl >= ns && sl < n && !left;
+      const unsigned mm = __ballot_sync(kAll, mv);
+      if (mv) {
+        int j = A + moved + __popc(mm & lt), d = 0;  // the freed slot it takes, of all freed slots
+        for (int p = __popc(fw[0]); j >= p; p = __popc(fw[d])) {
+          j -= p;
+          ++d;
+        }
+        const long qf = base + sl, qt = base + 32 * d + nth_bit(fw[d], j);
+        const float4 p0 = s.wp[qf], q0 = s.xyz[qf];
+        s.wp[qt] = p0;
+        s.xyz[qt] = q0;
+      }
+      moved += __popc(mm);
+      before += __popc(v);
+    }
+  }
+  if (lane < K && c0 + lane < a.ncells) {
+    const int total = n_l - sH[wid][lane] + sA[wid][lane];
+    s.count[c0 + lane] = min(total, s.cap);
+    if (total > s.cap) {
+      atomicAdd(a.stats + 3, (double)(total - s.cap));
+      atomicOr(a.err, ERR_CAPACITY);
+    }
+  }
+}
+
+template <int K>
+cudaError_t launch(const StreamArgs& a, cudaStream_t st) {
+  const int grid = (a.ncells + kWarps * K - 1) / (kWarps * K);
+  stream_move_kernel<K><<<grid, kThreads, 0, st>>>(a);
+  cudaError_t e = cudaGetLastError();
+  if (e) return e;
+  stream_place_kernel<K><<<grid, kThreads, 0, st>>>(a);
+  return cudaGetLastError();
 }
 
 }  // namespace
 
+// Cells a warp: 4, so that thinly filled cells (13 axions of 64 slots in the
+// 3-D plasma) share its lanes, or 1. A large slab may hold few axions too,
+// so with enough cells for 8 rounds of resident warps it takes 4 as well
+// (262,144 cells of about 25 in 384 slots: 250 us a call against 345); with
+// fewer, 4 cells a warp leave the last of 2 rounds nearly empty where the
+// cells are full (65,536 of 128: 235 us against 215). 4 cells a warp want
+// at least one round.
+constexpr int kRound = 152 * 48;  // resident warps
+
 cudaError_t launch_stream(const StreamArgs& a, cudaStream_t st) {
   if (a.ncells <= 0) return cudaSuccess;
-  const int grid = (a.ncells + kWarps - 1) / kWarps;
-  stream_move_kernel<<<grid, kThreads, 0, st>>>(a);
-  cudaError_t e = cudaGetLastError();
-  if (e) return e;
-  stream_place_kernel<<<grid, kThreads, 0, st>>>(a);
-  return cudaGetLastError();
+  const int rounds = a.s.cap <= 64 ? 1 : 8;
+  return a.ncells / kGroup >= rounds * kRound ? launch<kGroup>(a, st) : launch<1>(a, st);
 }
 
 }  // namespace axpic

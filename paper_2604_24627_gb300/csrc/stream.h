@@ -7,9 +7,12 @@
 
 namespace axpic {
 
-// Direction of a slot after a move: the cell shift (sx, sy, sz) in {-1, 0, 1}^3
-// as (sz + 1) 9 + (sy + 1) 3 + (sx + 1); 13 stays; 27 left an open box.
-constexpr int kStreamDirs = 27, kStreamStay = 13, kStreamEscaped = 27;
+// Direction of an axion after a move: the cell shift (sx, sy, sz) in {-1, 0, 1}^3
+// as (sz + 1) 9 + (sy + 1) 3 + (sx + 1); 13 stays.
+constexpr int kStreamDirs = 27, kStreamStay = 13;
+// 16-bit entries a cell of the staging offsets: entry d the leavers with a
+// direction below d, entry 27 all of them (64 bytes, two sectors)
+constexpr int kStreamOffs = 32;
 
 struct StreamArgs {
   SpeciesPtrs s;       // the axion slabs (positions rewritten, slots re-binned)
@@ -17,9 +20,8 @@ struct StreamArgs {
   float kappa;         // binary32(c dt / h): the cell fraction moved at |v| = c
   float mu;            // binary32(m_a c^2 / m_e c^2): the axion mass in units of the momenta
   int periodic;        // 1 periodic, 0 open
-  uint8_t* dir;        // [ncells * cap]: direction of each slot
-  int32_t* cnt;        // [ncells * 27]: slots per direction
-  int32_t* goff;       // [ncells * 27]: the direction's first row in the cell's staging rows
+  uint32_t* freed;     // [ncells * ceil(cap / 32)]: a bit per slot whose axion does not stay
+  uint16_t* goff;      // [ncells * kStreamOffs]: each direction's first row in the cell's staging rows
   float* buf;          // [ncells * cap * 8]: the cell's leaving axions, grouped by direction
   double* stats;       // [4]: escaped number, weight, weight x energy [keV]; dropped number
   int* err;            // latched error flags (ERR_CAPACITY)
