@@ -295,28 +295,68 @@ __device__ __noinline__ PhotonDecision photon_decide_slow(const StepArgs& A, int
 // u <= 1 - lb <= exp(-lambda).
 // A bound at or above the Poisson-mean cap also sends the slot to the full
 // decision, so that cap hits are counted exactly.
-// kb is the cell's A / w_ref with the margin 1.0001 (times the rate model's
-// guard margin) folded in.
-__device__ __forceinline__ bool no_conversion(float w, float p2, float c_s, float kb, float u, float lam_cap) {
+// kb is the cell's A ln 2 / w_ref with the margin 1.0001 (times the rate
+// model's guard margin) folded in. Both bounds hold in binary32 on their own:
+// s/2 to its rounding, and log2(1 + s + 5e-7), whose offset covers the
+// rounding of the sum and the approximation's absolute error near 1
+// (2^-22), the margin its relative error.
+//
+// These bounds are the decision kernel's arithmetic: one special-function
+// instruction and 12 others per conversion, three and 8 per absorption (the
+// approximations flush subnormals, so no scaling code surrounds them, and the
+// uniform is one funnel shift and one addition of the draw's word). With
+// 1 - lb - 1e-6 formed from u, a comparison to choose the bound and x formed
+// first, the kernel issued 205 warp instructions a cell at 5 keV and took
+// 1060 us for 4.1 M cells; now 170 and 933 us.
+__device__ __forceinline__ float lg2_ftz(float x) {
+  float y;
+  asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+__device__ __forceinline__ float ex2_ftz(float x) {
+  float y;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+__device__ __forceinline__ float rsqrt_ftz(float x) {
+  float y;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+// 1 + (w >> 9) 2^-23 = u + 1 - 2^-24
+__device__ __forceinline__ float one_plus(uint32_t w) { return __uint_as_float(__funnelshift_r(w, 0x7Fu, 9)); }
+constexpr float kGuardAbs = 1.2e-6f;  // covers the roundings of u and of the bounds below 1
+
+__device__ __forceinline__ bool no_conversion(float w, float p2, float c_s, float kb, uint32_t word, float lam_cap) {
   const float s = p2 * c_s;
-  const float Fb = s < 2.5f ? 0.5f * s : __logf(1.0f + s);
+  const float Fb = fminf(0.72134752f * s, lg2_ftz(s + 1.0000005f));  // F / ln 2
   const float lb = w * kb * Fb;
-  return (lb < lam_cap) & (u <= 1.0f - lb - 1e-6f);
+  return (lb < lam_cap) & (lb < (2.0f - kGuardAbs) - one_plus(word));
 }
 __device__ __forceinline__ float conversion_kb(float Acoef, float inv_wref, float gm) {
-  return Acoef * inv_wref * (1.0001f * gm);
+  return Acoef * inv_wref * (0.69314718f * 1.0001f * gm);
 }
 
 // Absorption: P_abs <= tau; x/(1-e^-x) <= 1 + x bounds the Compton-like
-// factor, (1 - e^-x) <= 1 the Bose-Einstein one. b_c, b_b: the cell's
-// coefficients with the margin 1.001 (times the guard margin) folded in; x
-// = |p| m_e c^2 / T from p2 by a reciprocal square root (p2 = 0 gives NaN,
-// which clears nothing).
-__device__ __forceinline__ bool no_absorption(float b_c, float b_b, const StepArgs& A, int mask, float x, float u) {
-  float tb = 0.f;
-  if (mask & AXPIC_CH_COMPTON) tb += b_c * x * (1.0f + x);
-  if (mask & AXPIC_CH_BREMS) tb += b_b * __expf(A.brems_am3 * __logf(x));
-  return u >= tb + 1e-6f;
+// factor, (1 - e^-x) <= 1 the Bose-Einstein one. With x = c |p|, c = m_e c^2
+// / T, tau <= b_c x (1 + x) + b_b x^(a-3) = bc1 |p| + bc2 p^2 + bb
+// (p^2)^((a-3)/2): the cell's coefficients with the margin 1.001 (times the
+// guard margin) folded in, zero for a channel that is off. p2 = 0 gives NaN,
+// which clears nothing.
+struct AbsorbBound {
+  float bc1, bc2, bb;
+};
+__device__ __forceinline__ AbsorbBound absorb_bound(float b_c, float b_b, float c, float am3) {
+  AbsorbBound b;
+  b.bc1 = b_c * c;
+  b.bc2 = b.bc1 * c;
+  b.bb = b_b * ex2_ftz(am3 * lg2_ftz(c));
+  return b;
+}
+__device__ __forceinline__ bool no_absorption(const AbsorbBound& b, float half_am3, float p2, uint32_t word) {
+  const float p = p2 * rsqrt_ftz(p2);
+  const float tb = b.bc2 * p2 + (b.bc1 * p + b.bb * ex2_ftz(half_am3 * lg2_ftz(p2)));
+  return tb <= one_plus(word) - (1.0f + kGuardAbs);
 }
 
 // ---------------------------------------------------------------- feedback
@@ -603,6 +643,10 @@ __device__ __forceinline__ void photon_full(const StepArgs& A, uint4 it) {
   atomicOr(A.bitsG + (size_t)cell * A.Wg + (it.y >> 5), 1u << (it.y & 31));
 }
 
+__device__ __forceinline__ void prefetch_l1(const void* p) {
+  asm volatile("prefetch.global.L1 [%0];" ::"l"(p));
+}
+
 // Decides full batches of 32 from the top of a list; returns what is left.
 template <bool AX>
 __device__ __forceinline__ int list_drain(const StepArgs& A, const uint4* L, int pend, int lane) {
@@ -690,23 +734,36 @@ __device__ __forceinline__ void electron_chunk(const StepArgs& A, uint32_t step,
   if (__all_sync(kFull, lane >= nc || wu > 0.f)) {
     // every cell of the chunk has a common weight: the decision is the
     // integer compare alone. Two quads per lane and pass, so that two
-    // independent Philox chains are in flight.
+    // independent Philox chains are in flight. Where the cells hold equally
+    // many electrons (they never change) a quad's cell is a multiplication by
+    // ceil(2^32 / nq), exact for the g < 32 nq <= 2^17 here.
+    const int nq0 = __shfl_sync(kFull, (n + 3) >> 2, 0);
+    const bool even = nq0 > 1 && nq0 <= 4096 && __all_sync(kFull, lane >= nc || (n + 3) >> 2 == nq0);
+    const uint32_t magic = even ? 0xFFFFFFFFu / (uint32_t)nq0 + 1u : 0u;
     for (int g0 = 0; g0 < R.total; g0 += 64) {
       int lc[2], q[2];
       uint4 r[2];
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
-        lc[h] = quad_cell(R, g0 + 32 * h + lane);
-        q[h] = g0 + 32 * h + lane - __shfl_sync(kFull, R.qoff, lc[h]);
+        const int g = g0 + 32 * h + lane;
+        if (even) {
+          lc[h] = (int)__umulhi((uint32_t)g, magic);
+          q[h] = g - lc[h] * nq0;
+        } else {
+          lc[h] = quad_cell(R, g);
+          q[h] = g - __shfl_sync(kFull, R.qoff, lc[h]);
+        }
         r[h] = philox4x32_10(make_uint4(step, A.cell_base + (uint32_t)(c0 + lc[h]), (uint32_t)q[h], S_EMIT_E << 24), A.rk);
       }
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
-        const int nn = __shfl_sync(kFull, n, lc[h]);
         const int cthr = __shfl_sync(kFull, thr, lc[h]);
-        const float cls = __shfl_sync(kFull, lsum, lc[h]);
         const uint32_t m = max(max(r[h].x, r[h].y), max(r[h].z, r[h].w));
-        if (g0 + 32 * h + lane >= R.total || (int)(m >> 9) <= cthr) continue;  // no slot of the quad emits
+        const bool emits = g0 + 32 * h + lane < R.total && (int)(m >> 9) > cthr;
+        if (!__any_sync(kFull, emits)) continue;  // the common pass: no slot of any quad emits
+        const int nn = __shfl_sync(kFull, n, lc[h]);
+        const float cls = __shfl_sync(kFull, lsum, lc[h]);
+        if (!emits) continue;
         const int cell = c0 + lc[h];
         const int nj = min(4, nn - 4 * q[h]);
         const long b = (long)cell * A.e.cap + 4 * q[h];
@@ -773,6 +830,11 @@ __device__ __forceinline__ void electron_chunk(const StepArgs& A, uint32_t step,
   }
 }
 
+// The photon and axion passes find the next pass's cells one pass ahead and
+// prefetch its slots into L1: the loads were a third of the kernel's stalls,
+// and held in registers instead they spill. 65,536 cells in 8 launches: 361
+// -> 340 us, 196,000 cells of boxes 459 -> 417 us.
+
 // Photons of a chunk present at the start of the step (gamma->a).
 template <int C>
 __device__ __forceinline__ int photon_chunk(const StepArgs& A, uint32_t step, int c0, int nc, int lane, uint4* L,
@@ -788,10 +850,15 @@ __device__ __forceinline__ int photon_chunk(const StepArgs& A, uint32_t step, in
     ap = conversion_kb(__ldg(rec + R_AP), A.inv_w_a, A.guard_margin);
   }
   const QuadRange<C> R = quad_range<C>(n, lane, nc);
+  int lcn = quad_cell(R, lane), qbn = __shfl_sync(kFull, R.qoff, lcn);
   for (int g0 = 0; g0 < R.total; g0 += 32) {
     const int g = g0 + lane;
-    const int lc = quad_cell(R, g);
-    const int qb = __shfl_sync(kFull, R.qoff, lc);
+    const int lc = lcn, qb = qbn;
+    if (g0 + 32 < R.total) {
+      lcn = quad_cell(R, g + 32);
+      qbn = __shfl_sync(kFull, R.qoff, lcn);
+      if (g + 32 < R.total) prefetch_l1(A.g.wp + (long)(c0 + lcn) * A.g.cap + 4 * (g + 32 - qbn));
+    }
     const int nn = __shfl_sync(kFull, n, lc);
     const float cs = __shfl_sync(kFull, c_s, lc);
     const float ca = __shfl_sync(kFull, ap, lc);
@@ -810,8 +877,9 @@ __device__ __forceinline__ int photon_chunk(const StepArgs& A, uint32_t step, in
       for (int j = 0; j < 4; ++j) {
         const float px = v[j].y, py = v[j].z, pz = v[j].w;
         const float p2 = px * px + py * py + pz * pz;
-        nib |= (uint32_t)((j < nj) & !no_conversion(v[j].x, p2, cs, ca, u23(word(r, j)), A.lam_cap)) << j;
+        nib |= (uint32_t)!no_conversion(v[j].x, p2, cs, ca, word(r, j), A.lam_cap) << j;
       }
+      nib &= (1u << nj) - 1u;
     }
     pend = list_append(L, pend, cell, 4 * q, nib, r, r);
     pend = list_drain<false>(A, L, pend, lane);
@@ -828,28 +896,35 @@ __device__ __forceinline__ int axion_chunk(const StepArgs& A, uint32_t step, int
   const bool bath = mask & (AXPIC_CH_COMPTON | AXPIC_CH_BREMS);
   const bool all = A.absorb_mode == 1 && bath;  // weight reduction changes every axion
   int n = 0;
-  float c_s = 0.f, apinv = 0.f, invT = 0.f, r_bc = 0.f, r_bb = 0.f;
+  const float half_am3 = 0.5f * A.brems_am3;
+  float c_s = 0.f, apinv = 0.f;
+  AbsorbBound ab = {0.f, 0.f, 0.f};
   if (lane < nc) {
     const int c = c0 + lane;
     const float* rec = A.rec + (size_t)c * kRecLen;
     n = min(max(A.a.count[c], 0), A.a.cap);
     c_s = kMeC2f * kMeC2f * __ldg(rec + R_FOURK2);
     apinv = conversion_kb(A.cc.prim_mult * __ldg(rec + R_AP), A.inv_w_gref, A.guard_margin);
-    invT = kMeC2f * __ldg(rec + R_INVT);
-    r_bc = __ldg(rec + R_BC) * (1.001f * A.guard_margin);
-    r_bb = __ldg(rec + R_BB) * (1.001f * A.guard_margin);
+    const float gm = 1.001f * A.guard_margin;
+    ab = absorb_bound((mask & AXPIC_CH_COMPTON) ? __ldg(rec + R_BC) * gm : 0.f,
+                      (mask & AXPIC_CH_BREMS) ? __ldg(rec + R_BB) * gm : 0.f, kMeC2f * __ldg(rec + R_INVT),
+                      A.brems_am3);
   }
   const QuadRange<C> R = quad_range<C>(n, lane, nc);
+  int lcn = quad_cell(R, lane), qbn = __shfl_sync(kFull, R.qoff, lcn);
   for (int g0 = 0; g0 < R.total; g0 += 32) {
     const int g = g0 + lane;
-    const int lc = quad_cell(R, g);
-    const int qb = __shfl_sync(kFull, R.qoff, lc);
+    const int lc = lcn, qb = qbn;
+    if (g0 + 32 < R.total) {
+      lcn = quad_cell(R, g + 32);
+      qbn = __shfl_sync(kFull, R.qoff, lcn);
+      if (g + 32 < R.total) prefetch_l1(A.a.wp + (long)(c0 + lcn) * A.a.cap + 4 * (g + 32 - qbn));
+    }
     const int nn = __shfl_sync(kFull, n, lc);
     const float cs = __shfl_sync(kFull, c_s, lc);
     const float cap_inv = __shfl_sync(kFull, apinv, lc);
-    const float cinvT = __shfl_sync(kFull, invT, lc);
-    const float cbc = __shfl_sync(kFull, r_bc, lc);
-    const float cbb = __shfl_sync(kFull, r_bb, lc);
+    const AbsorbBound cab = {__shfl_sync(kFull, ab.bc1, lc), __shfl_sync(kFull, ab.bc2, lc),
+                             __shfl_sync(kFull, ab.bb, lc)};
     const int cell = c0 + lc;
     const int q = g - qb;
     uint32_t nib = 0;
@@ -868,10 +943,11 @@ __device__ __forceinline__ int axion_chunk(const StepArgs& A, uint32_t step, int
         const float px = v[j].y, py = v[j].z, pz = v[j].w;
         const float p2 = (px * px + py * py + pz * pz) + A.mu2;  // E^2 (m_e c^2 units)
         bool fast = !all;
-        if (prim) fast &= no_conversion(v[j].x, p2, cs, cap_inv, u23(word(rP, j)), A.lam_cap);
-        if (bath) fast &= no_absorption(cbc, cbb, A, mask, p2 * rsqrtf(p2) * cinvT, u23(word(rA, j)));
-        nib |= (uint32_t)((j < nj) & !fast) << j;
+        if (prim) fast &= no_conversion(v[j].x, p2, cs, cap_inv, word(rP, j), A.lam_cap);
+        if (bath) fast &= no_absorption(cab, half_am3, p2, word(rA, j));
+        nib |= (uint32_t)!fast << j;
       }
+      nib &= (1u << nj) - 1u;
     }
     pend = list_append(L, pend, cell, 4 * q, nib, rP, rA);
     pend = list_drain<true>(A, L, pend, lane);
