@@ -1232,9 +1232,6 @@ __global__ void __launch_bounds__(kFeedbackThreads, DENSE ? 4 : 5) feedback_kern
 // (electrons: kLightE, each event with its own Philox block).
 constexpr int kLight = 8;
 constexpr int kLightE = 4;
-// Flagged slots and tail movers per species whose loads go out together
-// (one: more in flight cost registers, and occupancy gained more).
-constexpr int kLoad = 1;
 constexpr size_t kLaneListBytes = 3 * kLight * 32 * sizeof(uint16_t);
 
 struct EvScratch {
@@ -1252,15 +1249,20 @@ __host__ __device__ inline bool rows_staged(int acap, int gcap, int ecap) {
   return row_words(acap) <= 32 && row_words(gcap) <= 32 && row_words(ecap) <= 32;
 }
 
-__host__ __device__ inline size_t ev_scratch_bytes(int acap, int gcap, int ecap) {
-  size_t b = align16(2 * ((size_t)acap + (size_t)gcap + (size_t)ecap));
-  b = align16(b + 4 * (size_t)(row_words(acap) + row_words(gcap)));
-  b += kLaneListBytes;
+// lists: with the heavy cells' lists and bits (the full-step kernel of the
+// light cells has none)
+__host__ __device__ inline size_t ev_list_bytes(int acap, int gcap, int ecap) {
+  const size_t b = align16(2 * ((size_t)acap + (size_t)gcap + (size_t)ecap));
+  return align16(b + 4 * (size_t)(row_words(acap) + row_words(gcap)));
+}
+__host__ __device__ inline size_t ev_scratch_bytes(int acap, int gcap, int ecap, bool lists) {
+  size_t b = (lists ? ev_list_bytes(acap, gcap, ecap) : 0) + kLaneListBytes;
   if (rows_staged(acap, gcap, ecap))
     b += align16(4 * 32 * (size_t)((row_words(acap) | 1) + (row_words(gcap) | 1) + (row_words(ecap) | 1)));
   return b + 32 * 2 * sizeof(double2);
 }
 
+template <bool LISTS>
 __device__ inline EvScratch ev_carve(unsigned char* base, int acap, int gcap, int ecap) {
   EvScratch s;
   uint16_t* h = reinterpret_cast<uint16_t*>(base);
@@ -1269,11 +1271,10 @@ __device__ inline EvScratch ev_carve(unsigned char* base, int acap, int gcap, in
   s.flE = h; h += ecap;
   s.rmA = s.flA;
   s.rmG = s.flG;
-  size_t off = align16(2 * ((size_t)acap + gcap + ecap));
-  uint32_t* u = reinterpret_cast<uint32_t*>(base + off);
+  uint32_t* u = reinterpret_cast<uint32_t*>(base + align16(2 * ((size_t)acap + gcap + ecap)));
   s.rbA = u; u += row_words(acap);
   s.rbG = u;
-  off = align16(off + 4 * (size_t)(row_words(acap) + row_words(gcap)));
+  size_t off = LISTS ? ev_list_bytes(acap, gcap, ecap) : 0;
   s.lt = reinterpret_cast<uint16_t*>(base + off);
   off += kLaneListBytes;
   s.sA = row_words(acap) | 1;
@@ -1608,7 +1609,7 @@ __device__ __forceinline__ void reduce_out(const Lane64& x64, PhaseOut* out) {
 __device__ __noinline__ void absorb_warp(const StepArgs& A, int cell, unsigned char* sb, const uint32_t* row,
                                          uint32_t* clr, const Cnt cnt, int na_start, int ng_start, bool fill,
                                          PhaseOut* out) {
-  const EvScratch S = ev_carve(sb, A.a.cap, A.g.cap, A.e.cap);
+  const EvScratch S = ev_carve<true>(sb, A.a.cap, A.g.cap, A.e.cap);
   const int lane = lane_id();
   const unsigned lt = (1u << lane) - 1u;
   const bool bath = A.mask & (AXPIC_CH_COMPTON | AXPIC_CH_BREMS);
@@ -1656,7 +1657,7 @@ __device__ __noinline__ void emit_warp(const StepArgs& A, uint32_t step, int cel
                                        const uint32_t* rowG, uint32_t* clrG, const uint32_t* rowE, uint32_t* clrE,
                                        const Cnt cnt, AxDest D, int ng_tot, int ng0, int ne, float wu, float r_cc,
                                        float r_cb, float r_T, PhaseOut* out) {
-  const EvScratch S = ev_carve(sb, A.a.cap, A.g.cap, A.e.cap);
+  const EvScratch S = ev_carve<true>(sb, A.a.cap, A.g.cap, A.e.cap);
   const int lane = lane_id();
   const unsigned lt = (1u << lane) - 1u;
   const long abase = (long)cell * A.a.cap;
@@ -1751,8 +1752,7 @@ __device__ __forceinline__ void clear_row(uint32_t* bits, int W, int cell, uint3
 
 // Tail fill by one lane: the removed slots rm[0, nrm) (ascending) below
 // n_surv are refilled, in order, by the kept slots of [n_surv, n). The first
-// kLoad movers can be loaded ahead (fill_load) and written later
-// (fill_store); fill_rest moves the others.
+// mover can be loaded ahead and written later; fill_rest moves the others.
 struct FillIt {
   int h, j, i, m;  // holes, next removed entry at or past the scan, scan position, movers done
 };
@@ -1802,25 +1802,11 @@ __device__ __forceinline__ void mover_store(const SpeciesPtrs& sp, long base, co
   if (v.dst >= 0) write_particle(sp, base + v.dst, v.w, v.px, v.py, v.pz, v.x, v.y, v.z);
 }
 
-// Loads the next kLoad movers.
-__device__ __forceinline__ void fill_load(const SpeciesPtrs& sp, long base, const uint16_t* rm, int nrm, FillIt& it,
-                                          Mover* v) {
-#pragma unroll
-  for (int t = 0; t < kLoad; ++t) {
-    int src = 0, dst = -1;
-    if (it.m < it.h) {
-      src = fill_next(rm, nrm, it);
-      dst = rm[32 * it.m++];
-    }
-    v[t] = mover_load(sp, base, src, dst);
-  }
-}
-
 __device__ __forceinline__ void fill_rest(const SpeciesPtrs& sp, long base, const uint16_t* rm, int nrm, FillIt& it) {
   while (it.m < it.h) {
-    Mover v[4];
+    Mover v[2];
 #pragma unroll
-    for (int t = 0; t < 4; ++t) {
+    for (int t = 0; t < 2; ++t) {
       int src = 0, dst = -1;
       if (it.m < it.h) {
         src = fill_next(rm, nrm, it);
@@ -1829,15 +1815,18 @@ __device__ __forceinline__ void fill_rest(const SpeciesPtrs& sp, long base, cons
       v[t] = mover_load(sp, base, src, dst);
     }
 #pragma unroll
-    for (int t = 0; t < 4; ++t) mover_store(sp, base, v[t]);
+    for (int t = 0; t < 2; ++t) mover_store(sp, base, v[t]);
   }
 }
 
 // One cell by one lane: its emit phase, or the full step (doA: the new axions
 // of the emit phase reuse the axion slots the absorb phase freed). Round
-// trips: the first kLoad flagged axions and photons together; the first kLoad
-// photon tail movers together; then the stores. Longer lists take further
-// round trips. Every flagged axion is read before a new axion is written over
+// trips: the first flagged axion and photon together; the first photon tail
+// mover under the thermal-bath events. Longer lists take further round trips.
+// Each loop stands once: with the first items and
+// movers handled apart from the rest the kernel's code was half again as
+// large and stalled on instruction fetches (4.1 M cells at 5 keV: 569 us, now
+// 450; two tail movers at a time there, 529 with four). Every flagged axion is read before a new axion is written over
 // a freed slot.
 struct LaneCell {
   int na, ng;       // in: counts at the start of the phase(s); out: final counts
@@ -1856,102 +1845,65 @@ __device__ __forceinline__ void cell_lane(const StepArgs& A, uint32_t step, int 
   const int nA = doA ? L.nflA : 0;
   const int nG = L.nflG;
   const int nE = L.nflE;
-  AxItem ta[kLoad];
-  PhItem tg[kLoad];
-#pragma unroll
-  for (int j = 0; j < kLoad; ++j) ta[j] = ax_load(A, abase, j < nA ? (int)lA[32 * j] : -1);
-#pragma unroll
-  for (int j = 0; j < kLoad; ++j) tg[j] = ph_load(A, gbase, j < nG ? (int)lG[32 * j] : -1);
+  AxItem ta = ax_load(A, abase, nA > 0 ? (int)lA[0] : -1);
+  PhItem tg = ph_load(A, gbase, nG > 0 ? (int)lG[0] : -1);
 
   // absorb: a->gamma products after the photons present
-  int na = L.na, ng = L.ng, nrmA = 0;
-  if (doA) {
-    int run = 0;
-#pragma unroll
-    for (int j = 0; j < kLoad; ++j) {
-      if (ta[j].slot < 0) break;
-      bool removed;
-      const int K = axion_outcome(A, ta[j], abase, bath, cnt, xa, &removed);
-      const float wprod = __uint_as_float(ta[j].r.y);
-      const float3 pg = photon_from_axion(A, ta[j].px, ta[j].py, ta[j].pz);
-      for (int k = 0; k < K; ++k) {
-        const int dst = L.ng + run + k;
-        if (dst < A.g.cap) write_particle(A.g, gbase + dst, wprod, pg.x, pg.y, pg.z, ta[j].x, ta[j].y, ta[j].z);
-        else cnt.add(C_DROP, 1);
-      }
-      run += K;
-      if (removed) lA[32 * nrmA++] = (uint16_t)ta[j].slot;
-    }
-    for (int i = kLoad; i < nA; ++i) {
-      const AxItem t = ax_load(A, abase, lA[32 * i]);
-      bool removed;
-      const int K = axion_outcome(A, t, abase, bath, cnt, xa, &removed);
-      const float wprod = __uint_as_float(t.r.y);
-      const float3 pg = photon_from_axion(A, t.px, t.py, t.pz);
-      for (int k = 0; k < K; ++k) {
-        const int dst = L.ng + run + k;
-        if (dst < A.g.cap) write_particle(A.g, gbase + dst, wprod, pg.x, pg.y, pg.z, t.x, t.y, t.z);
-        else cnt.add(C_DROP, 1);
-      }
-      run += K;
-      if (removed) lA[32 * nrmA++] = (uint16_t)t.slot;
-    }
-    na = L.na - nrmA;
-    ng = min(L.ng + run, A.g.cap);
-  }
-
-  // emit: gamma->a decisions of the loaded photons (products after the fill)
-  int nrmG = 0, Kg[kLoad];
-#pragma unroll
-  for (int j = 0; j < kLoad; ++j) {
-    Kg[j] = 0;
-    if (tg[j].slot >= 0) {
-      bool removed;
-      Kg[j] = photon_outcome(A, tg[j], gbase, cnt, &removed);
-      if (removed) lG[32 * nrmG++] = (uint16_t)tg[j].slot;
-    }
-  }
-
-  // photon tail movers, loaded together, when every photon removal is known
-  Mover mg[kLoad];
-  const bool gFill = nG <= kLoad;
-  FillIt fg = fill_begin(lG, nrmG, ng - nrmG);
-  if (gFill) fill_load(A.g, gbase, lG, nrmG, fg, mg);
-
-  // new axions: gamma->a products, then thermal-bath events
-  const AxDest D{lA, nrmA, 32, L.na};
-  int NP = 0;
-#pragma unroll
-  for (int j = 0; j < kLoad; ++j) {
-    if (Kg[j]) gamma_products(A, tg[j], abase, D, NP, Kg[j], cnt);
-    NP += Kg[j];
-  }
-  for (int i = kLoad; i < nG; ++i) {
-    const PhItem t = ph_load(A, gbase, lG[32 * i]);
+  int ng = L.ng, nrmA = 0;
+  for (int i = 0; i < nA; ++i) {
     bool removed;
-    const int K = photon_outcome(A, t, gbase, cnt, &removed);
-    if (K) gamma_products(A, t, abase, D, NP, K, cnt);
+    const int K = axion_outcome(A, ta, abase, bath, cnt, xa, &removed);
+    if (K > 0) {
+      const float wprod = __uint_as_float(ta.r.y);
+      const float3 pg = photon_from_axion(A, ta.px, ta.py, ta.pz);
+      for (int k = 0; k < K; ++k) {
+        const int dst = ng + k;
+        if (dst < A.g.cap) write_particle(A.g, gbase + dst, wprod, pg.x, pg.y, pg.z, ta.x, ta.y, ta.z);
+        else cnt.add(C_DROP, 1);
+      }
+      ng += K;
+    }
+    if (removed) lA[32 * nrmA++] = (uint16_t)ta.slot;
+    if (i + 1 < nA) ta = ax_load(A, abase, lA[32 * (i + 1)]);
+  }
+  ng = min(ng, A.g.cap);
+
+  // emit: new axions, first the gamma->a products
+  const AxDest D{lA, nrmA, 32, L.na};
+  int NP = 0, nrmG = 0;
+  for (int i = 0; i < nG; ++i) {
+    bool removed;
+    const int K = photon_outcome(A, tg, gbase, cnt, &removed);
+    if (K) gamma_products(A, tg, abase, D, NP, K, cnt);
     NP += K;
-    if (removed) lG[32 * nrmG++] = (uint16_t)t.slot;
+    if (removed) lG[32 * nrmG++] = (uint16_t)tg.slot;
+    if (i + 1 < nG) tg = ph_load(A, gbase, lG[32 * (i + 1)]);
+  }
+  // the first photon tail mover (a->gamma products included), loaded under
+  // the thermal-bath events
+  FillIt fg = fill_begin(lG, nrmG, ng - nrmG);
+  Mover mg;
+  {
+    int src = 0, dst = -1;
+    if (fg.h > 0) {
+      src = fill_next(lG, nrmG, fg);
+      dst = lG[0];
+      fg.m = 1;
+    }
+    mg = mover_load(A.g, gbase, src, dst);
   }
   for (int i = 0; i < nE; ++i) {
     const ElItem t = el_load(A, ebase, lE[32 * i], L.wu);
     NP += electron_events<true>(A, step, cell, t, abase, D, NP, L.r_cc, L.r_cb, L.r_T, L.wu, cnt, xe);
   }
-  na = min(D.base - D.nholes + NP, A.a.cap);
+  const int na = min(D.base - D.nholes + NP, A.a.cap);
   if (NP < nrmA) {
     // freed slots left over: closed from the tail (their movers lie beyond
     // every slot a new axion took)
     FillIt fr = fill_begin(lA + 32 * NP, nrmA - NP, na);
     fill_rest(A.a, abase, lA + 32 * NP, nrmA - NP, fr);
   }
-  // photon tail fill (a->gamma products included)
-  if (gFill) {
-#pragma unroll
-    for (int t = 0; t < kLoad; ++t) mover_store(A.g, gbase, mg[t]);
-  } else {
-    fg = fill_begin(lG, nrmG, ng - nrmG);
-  }
+  mover_store(A.g, gbase, mg);
   fill_rest(A.g, gbase, lG, nrmG, fg);
   ng -= nrmG;
   L.na = na;
@@ -2082,8 +2034,9 @@ __global__ void __launch_bounds__(128, PH == 3 ? AXPIC_EVENT_FULL_MIN_CTAS : AXP
   if (lane < kNumCounters) warp_cnt[wid][lane] = 0ull;
   __syncwarp();
   const Cnt cnt{warp_cnt[wid]};
-  unsigned char* const sbase = smem + wid * ev_scratch_bytes(A.a.cap, A.g.cap, A.e.cap);
-  const EvScratch S = ev_carve(sbase, A.a.cap, A.g.cap, A.e.cap);
+  constexpr bool kLists = PH != (PH_ABSORB | PH_EMIT);
+  unsigned char* const sbase = smem + wid * ev_scratch_bytes(A.a.cap, A.g.cap, A.e.cap, kLists);
+  const EvScratch S = ev_carve<kLists>(sbase, A.a.cap, A.g.cap, A.e.cap);
   uint16_t* lA = S.lt + lane;
   uint16_t* lG = lA + 32 * kLight;
   uint16_t* lE = lG + 32 * kLight;
@@ -2293,8 +2246,8 @@ __global__ void __launch_bounds__(128) event_heavy_kernel(StepArgs A) {
   if (lane < kNumCounters) warp_cnt[wid][lane] = 0ull;
   __syncwarp();
   const Cnt cnt{warp_cnt[wid]};
-  unsigned char* const sbase = smem + wid * ev_scratch_bytes(A.a.cap, A.g.cap, A.e.cap);
-  const EvScratch S = ev_carve(sbase, A.a.cap, A.g.cap, A.e.cap);
+  unsigned char* const sbase = smem + wid * ev_scratch_bytes(A.a.cap, A.g.cap, A.e.cap, true);
+  const EvScratch S = ev_carve<true>(sbase, A.a.cap, A.g.cap, A.e.cap);
   const uint32_t step = step_of(A);
   const bool emitG = (A.mask & AXPIC_CH_PRIMAKOFF) != 0;
   const bool emitE = (A.mask & (AXPIC_CH_COMPTON | AXPIC_CH_BREMS)) != 0;
@@ -2357,7 +2310,7 @@ __global__ void __launch_bounds__(128) event_heavy_kernel(StepArgs A) {
 }
 
 // ---------------------------------------------------------------- launchers
-size_t step_smem_per_warp(int acap, int gcap, int ecap) { return ev_scratch_bytes(acap, gcap, ecap); }
+size_t step_smem_per_warp(int acap, int gcap, int ecap) { return ev_scratch_bytes(acap, gcap, ecap, true); }
 
 int resident_ctas(const void* fn, int threads, size_t dyn_smem, int max_per_sm) {
   int dev = 0, sms = 0, regs_sm = 0, smem_sm = 0, reserved = 0, threads_sm = 0, blocks_sm = 0;
@@ -2379,18 +2332,20 @@ int resident_ctas(const void* fn, int threads, size_t dyn_smem, int max_per_sm) 
 
 template <int PH>
 static cudaError_t launch_events(const StepArgs& A, int warps, cudaStream_t st) {
-  const size_t per = ev_scratch_bytes(A.a.cap, A.g.cap, A.e.cap);
+  constexpr bool full = PH == (PH_ABSORB | PH_EMIT);
+  const size_t lists = ev_scratch_bytes(A.a.cap, A.g.cap, A.e.cap, true);
+  const size_t per = ev_scratch_bytes(A.a.cap, A.g.cap, A.e.cap, !full);
   const int grid = (A.ncells + 32 * warps - 1) / (32 * warps);
-  if (PH == (PH_ABSORB | PH_EMIT)) {
+  if (full) {
     cudaError_t e = cudaMemsetAsync(A.heavy_n, 0, sizeof(int32_t), st);
     if (e) return e;
   }
   event_kernel<PH><<<grid, warps * 32, per * warps, st>>>(A);
-  if (PH == (PH_ABSORB | PH_EMIT)) {
+  if (full) {
     // persistent over the heavy list: a warp per cell, at most one warp per
     // cell of the launch and kHeavyGrid CTAs
     const int hgrid = max(1, min((A.ncells + warps - 1) / warps, kHeavyGrid));
-    event_heavy_kernel<<<hgrid, warps * 32, per * warps, st>>>(A);
+    event_heavy_kernel<<<hgrid, warps * 32, lists * warps, st>>>(A);
   }
   return cudaGetLastError();
 }
