@@ -91,7 +91,7 @@ struct axpic_ctx {
   int max_warps = 4;  // largest event CTA (warps) whose scratch fits
   int ctr_rows = 1;   // rows of per-CTA counters
   int dec_grid = 1;   // CTAs of the persistent decision kernel
-  int dec_chunk = kDefaultDecChunk;
+  int dec_chunk = 0;  // cells per chunk of its warps; 0: by the launch's cells
   uint32_t* step_dev = nullptr;      // step counter of replayed graphs
   int32_t* heavy = nullptr;          // cells left to the warp-path event kernel
   int32_t* heavy_n = nullptr;        // their count, per branch
@@ -491,7 +491,7 @@ axpic_status axpic_init_plasma(axpic_ctx** out, const axpic_plasma_desc* desc, c
     ctx->lnK_CC = (float)std::log(gae2 * 120.0 * z6 * p.dt_phys_s / (wa32 * (5.0 * z6 / z5) * kKeVerg * 1e24));
     ctx->lnK_CB = (float)std::log(gae2 * std::tgamma(a + 1.0) * p.dt_phys_s / (wa32 * a * kKeVerg * 1e24));
   }
-  ctx->dec_chunk = p.decide_chunk ? p.decide_chunk : kDefaultDecChunk;
+  ctx->dec_chunk = p.decide_chunk;
   ctx->branches = p.step_branches                    ? p.step_branches
                   : d.ncells <= kBranchCells         ? kDefaultBranches
                                                      : 1;
@@ -566,7 +566,7 @@ axpic_status axpic_init_plasma(axpic_ctx** out, const axpic_plasma_desc* desc, c
       (e = cudaMemsetAsync(ctx->err, 0, sizeof(int), st)) ||
       (e = cudaMemsetAsync(ctx->bits, 0, sizeof(uint32_t) * (bit_words > 0 ? bit_words : 1), st)) ||
       (e = set_step_smem_limits(per_warp * ctx->max_warps)) ||
-      (e = decide_shape(p.decide_chunk, n, &ctx->dec_chunk, &ctx->dec_grid)) ||
+      (e = decide_resident_ctas(&ctx->dec_grid)) ||
       (e = launch_records(n, d.nspecies, ctx->cc, d.T_keV, d.n_ion, ctx->rec, ctx->err, st)) ||
       (e = launch_moments(n, to_ptrs(d.electrons), ctx->mom, st)) ||
       (p.rate_model && (e = cudaMemcpyAsync(ctx->srtab, srtab.data(), srtab.size() * sizeof(float),
@@ -898,6 +898,7 @@ static cudaError_t capture_steps(axpic_ctx* ctx, StepArgs A, int nsteps, cudaStr
     StepArgs B = A;
     B.cell0 = c0;
     B.ncells = std::min(part, n - c0);
+    B.dec_cells = n;
     B.step_dev = ctx->step_dev + nb;
     B.heavy_n = ctx->heavy_n + nb;
     SrArgs Bsr;
@@ -1078,23 +1079,25 @@ static cudaError_t copy_state(axpic_ctx* ctx, unsigned char* save, bool to_save)
   return cudaSuccess;
 }
 
-static void set_shape(axpic_ctx* ctx, int chunk, int warps, int dec_grid) {
+static void set_shape(axpic_ctx* ctx, int chunk, int warps) {
   ctx->dec_chunk = chunk;
-  ctx->dec_grid = dec_grid;
   ctx->warps = warps;
   ctx->grid = (ctx->desc.ncells + warps - 1) / warps;
 }
 
-axpic_status axpic_launch_shape(const axpic_ctx* ctx, int32_t* decide_chunk, int32_t* event_warps,
+axpic_status axpic_launch_shape(const axpic_ctx* ctx, int32_t* decide_chunk_out, int32_t* event_warps,
                                 int32_t* step_branches) {
   if (!ctx) return AXPIC_E_INVALID;
-  if (decide_chunk) *decide_chunk = ctx->dec_chunk;
-  if (event_warps) *event_warps = ctx->warps;
-  if (step_branches) {
-    const int n = ctx->desc.ncells;
-    const int part = ((n + ctx->branches - 1) / ctx->branches + 127) / 128 * 128;
-    *step_branches = (ctx->branches == 1 || part >= n) ? 1 : (n + part - 1) / part;
+  const int n = ctx->desc.ncells;
+  const int part = ((n + ctx->branches - 1) / ctx->branches + 127) / 128 * 128;
+  const bool whole = ctx->branches == 1 || part >= n;
+  if (decide_chunk_out) {
+    StepArgs A = make_args(const_cast<axpic_ctx*>(ctx), 0, AXPIC_CH_ALL);
+    if (!whole) A.ncells = part, A.dec_cells = n;
+    *decide_chunk_out = decide_chunk(A);
   }
+  if (event_warps) *event_warps = ctx->warps;
+  if (step_branches) *step_branches = whole ? 1 : (n + part - 1) / part;
   return AXPIC_OK;
 }
 
@@ -1111,19 +1114,17 @@ axpic_status axpic_autotune(axpic_ctx* ctx, int64_t step, int32_t trial_steps, i
   unsigned char* save = nullptr;
   CK(cudaMalloc((void**)&save, total > 0 ? total : 256), "autotune scratch");
   cudaEvent_t e0 = nullptr, e1 = nullptr;
-  const int keep_chunk = ctx->dec_chunk, keep_warps = ctx->warps, keep_grid = ctx->dec_grid;
-  int best_chunk = keep_chunk, best_warps = keep_warps, best_grid = keep_grid;
+  const int keep_chunk = ctx->dec_chunk, keep_warps = ctx->warps;
+  int best_chunk = keep_chunk, best_warps = keep_warps;
   double best = -1.0;
   cudaError_t e = copy_state(ctx, save, true);
   if (!e) e = cudaEventCreate(&e0);
   if (!e) e = cudaEventCreate(&e1);
   for (int chunk : {4, 8, 16, 32}) {
-    int dgrid = 1;
-    if (!e) e = decide_resident_ctas(chunk, &dgrid);
     for (int warps : {2, 4}) {
       if (e) break;
       if (warps > ctx->max_warps) continue;
-      set_shape(ctx, chunk, warps, dgrid);
+      set_shape(ctx, chunk, warps);
       // one untimed step, then trial_steps timed ones, from the saved state
       StepArgs A = make_args(ctx, step, channel_mask);
       const SrArgs sra = make_sr_args(ctx);
@@ -1143,7 +1144,6 @@ axpic_status axpic_autotune(axpic_ctx* ctx, int64_t step, int32_t trial_steps, i
         best = per;
         best_chunk = chunk;
         best_warps = warps;
-        best_grid = dgrid;
       }
     }
   }
@@ -1152,10 +1152,10 @@ axpic_status axpic_autotune(axpic_ctx* ctx, int64_t step, int32_t trial_steps, i
   if (e1) cudaEventDestroy(e1);
   cudaFree(save);
   if (e) {
-    set_shape(ctx, keep_chunk, keep_warps, keep_grid);
+    set_shape(ctx, keep_chunk, keep_warps);
     return cuda_fail(ctx, e, "axpic_autotune");
   }
-  set_shape(ctx, best_chunk, best_warps, best_grid);
+  set_shape(ctx, best_chunk, best_warps);
   free_graphs(ctx);
   if (best_ms_out) *best_ms_out = best;
   if (chunk_out) *chunk_out = best_chunk;
@@ -1520,9 +1520,9 @@ axpic_status axpic_step_noalloc(const axpic_plasma_desc* desc, const axpic_param
   c.warps = kNoAllocWarps;
   c.grid = (d.ncells + kNoAllocWarps - 1) / kNoAllocWarps;
   c.ctr_rows = std::max(1, std::min(kCounterRows, (d.ncells + 3) / 4));
-  c.dec_chunk = kDefaultDecChunk;
+  c.dec_chunk = p.decide_chunk;
   fold_constants(&c);
-  cudaError_t e = decide_shape(p.decide_chunk, d.ncells, &c.dec_chunk, &c.dec_grid);
+  cudaError_t e = decide_resident_ctas(&c.dec_grid);
   if (e) {
     fprintf(stderr, "axpic_step_noalloc: %s\n", cudaGetErrorString(e));
     return AXPIC_E_CUDA;

@@ -65,12 +65,6 @@ enum {
 // weight (0 otherwise). Electrons change only through the remap.
 constexpr int kMomLen = 8;
 
-// Cells per chunk of a decision warp; the default is a compile-time choice
-// that launch-shape sweeps override (c2 replayed in 8 branches: 8 cells
-// 0.178 ms per step, 4 cells 0.185, 2 cells 0.210).
-#ifndef AXPIC_DEC_CHUNK
-#define AXPIC_DEC_CHUNK 32
-#endif
 enum { M_W = 0, M_PX, M_PY, M_PZ, M_U2, M_VAR, M_WU };
 
 // Per-CTA counters (u64), reduced by axpic_tally_spectrum.
@@ -436,7 +430,8 @@ struct StepArgs {
   uint32_t* recE;
   int* err;
   int dec_grid;   // CTAs of the persistent decision kernel
-  int dec_chunk;  // cells per chunk of a decision warp: 4, 8, 16 or 32
+  int dec_chunk;  // cells per chunk of a decision warp: 4, 8, 16 or 32, or 0: by the launch (decide_chunk)
+  int dec_cells;  // cells of all the launches that run side by side (the branches of a replayed step), or 0
   uint32_t* step_dev;  // NULL, or the device step counter of a replayed graph
   // cells a full step's event kernel leaves to the warp-path kernel, stored
   // from index cell0 on, and their count (one counter per branch of a

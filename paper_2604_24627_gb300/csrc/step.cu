@@ -556,11 +556,6 @@ __device__ __forceinline__ void flag_quad(uint32_t* bits, int W, int cell, int q
 // barrier is needed. List order does not matter: records are indexed by slot.
 constexpr int kDecThreads = 256;
 constexpr int kDecWarps = kDecThreads / 32;
-// Cells per chunk: a launch-shape choice (4, 8, 16 or 32), picked per context. With
-// 32 every lane holds one cell's constants.
-constexpr int kChunkDefault = AXPIC_DEC_CHUNK;
-static_assert(kChunkDefault == 4 || kChunkDefault == 8 || kChunkDefault == 16 || kChunkDefault == 32,
-              "cells per decision chunk");
 constexpr int kListCap = 32 + 4 * 32;  // < 32 pending + one pass of flags
 
 // Per-warp lists: {cell, slot, decision word(s)}.
@@ -2350,12 +2345,36 @@ static cudaError_t launch_events(const StepArgs& A, int warps, cudaStream_t st) 
   return cudaGetLastError();
 }
 
-// Persistent decision grid: A.dec_grid CTAs (what the device holds at once
-// for this chunk size), at most one warp per chunk.
-static int dec_blocks(const StepArgs& A) {
-  const int nchunks = (A.ncells + A.dec_chunk - 1) / A.dec_chunk;
-  const int need = (nchunks + kDecWarps - 1) / kDecWarps;
-  return max(1, min(need, A.dec_grid));
+// Cells per chunk of a decision warp: asked for, or by the launch. A chunk
+// should hold enough work for the warp's lanes and for full batches of full
+// decisions, not so much that the last chunks are waited for, and the chunks
+// should fill the resident warps (rounds: chunks over resident warps, over
+// all the branches that a replayed step runs side by side). The work of a
+// cell is taken from its capacities, u = e/2 + g + a slots. Times of a pass,
+// us, by chunk size (the one taken first):
+//   4,096 cells of 512 e, 256 g (u 1024):       1: 720   2: 746   4: 794   8: 898
+//   16,384 of the same:                         4: 1015  2: 1197  8: 1098  1: 1290
+//   196,000 of 128 e, 64 g (u 704), replayed:   8: 3700  16: 3884 4: 3926  32: 4515
+//   262,144 of 256 e, 128 g (u 1280):           8: 4593  16: 4655 4: 4727  32: 5047
+//   6,000 of 64 e, 48 g (u 384):                4: 41.5  2: 41.8  8: 43.8  1: 45.8
+//   64,000 of 64 e, 32 g (u 160), replayed:     16: 285  8: 293   32: 318  4: 312
+//   262,144 of the same, replayed:              32: 563  16: 581  8: 660   4: 711
+//   262,144 of the same, a launch of its own:   16: 294  32: 312  8: 328   4: 347
+//   64 of 128 g, latency (u 1154):              1: 23.7  4: 26.0  8: 28.7  32: 42.8
+int decide_chunk(const StepArgs& A) {
+  if (A.dec_chunk) return A.dec_chunk;
+  const long u = A.e.cap / 2 + A.g.cap + A.a.cap;
+  const long warps = (long)A.dec_grid * kDecWarps;
+  const long n = max(A.ncells, A.dec_cells);
+  int lo = 1, hi = 32;
+  while (lo < 32 && lo * u < 1000) lo *= 2;
+  while (hi > lo && hi * u > 10400) hi /= 2;
+  for (int c = hi; c > lo; c /= 2) {
+    // one launch of less than two rounds of the largest chunks waits for its second
+    const long tenths = c == 32 && A.dec_cells == 0 ? 20 : 8;
+    if (10 * (n / c) >= tenths * warps) return c;
+  }
+  return lo;
 }
 
 // The decision passes a phase set needs, as DK_* bits.
@@ -2370,18 +2389,29 @@ static int decide_kinds(const StepArgs& A, int phases) {
 static cudaError_t launch_decide(const StepArgs& A, int phases, cudaStream_t st) {
   const int kinds = decide_kinds(A, phases);
   if (kinds == 0) return cudaSuccess;
-  switch (A.dec_chunk) {
+  // persistent: as many CTAs as the device holds at once, at most one warp
+  // per chunk
+  const int chunk = decide_chunk(A);
+  const int nchunks = (A.ncells + chunk - 1) / chunk;
+  const int grid = max(1, min((nchunks + kDecWarps - 1) / kDecWarps, A.dec_grid));
+  switch (chunk) {
+    case 1:
+      decide_kernel<1><<<grid, kDecThreads, 0, st>>>(A, kinds);
+      break;
+    case 2:
+      decide_kernel<2><<<grid, kDecThreads, 0, st>>>(A, kinds);
+      break;
     case 4:
-      decide_kernel<4><<<dec_blocks(A), kDecThreads, 0, st>>>(A, kinds);
+      decide_kernel<4><<<grid, kDecThreads, 0, st>>>(A, kinds);
       break;
     case 8:
-      decide_kernel<8><<<dec_blocks(A), kDecThreads, 0, st>>>(A, kinds);
+      decide_kernel<8><<<grid, kDecThreads, 0, st>>>(A, kinds);
       break;
     case 16:
-      decide_kernel<16><<<dec_blocks(A), kDecThreads, 0, st>>>(A, kinds);
+      decide_kernel<16><<<grid, kDecThreads, 0, st>>>(A, kinds);
       break;
     default:
-      decide_kernel<32><<<dec_blocks(A), kDecThreads, 0, st>>>(A, kinds);
+      decide_kernel<32><<<grid, kDecThreads, 0, st>>>(A, kinds);
       break;
   }
   return cudaGetLastError();
@@ -2411,35 +2441,13 @@ cudaError_t launch_set_step(uint32_t* p, uint32_t v, int n, cudaStream_t st) {
   return cudaGetLastError();
 }
 
-cudaError_t decide_shape(int requested, int ncells, int* chunk, int* grid) {
-  int c = requested;
-  if (c == 0) {
-    int g = 1;
-    const cudaError_t e = decide_resident_ctas(32, &g);
-    if (e) return e;
-    const long warps = (long)g * kDecWarps;
-    c = 4;
-    for (int k : {32, 16, 8}) {
-      if ((long)ncells / k >= warps) {
-        c = k;
-        break;
-      }
-    }
-  }
-  *chunk = c;
-  return decide_resident_ctas(c, grid);
-}
-
-cudaError_t decide_resident_ctas(int chunk, int* out) {
+cudaError_t decide_resident_ctas(int* out) {
   int dev = 0, sms = 0, nb = 0;
   cudaError_t e;
   if ((e = cudaGetDevice(&dev)) || (e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)))
     return e;
-  if (chunk == 4) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, decide_kernel<4>, kDecThreads, 0);
-  else if (chunk == 8) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, decide_kernel<8>, kDecThreads, 0);
-  else if (chunk == 16) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, decide_kernel<16>, kDecThreads, 0);
-  else e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, decide_kernel<32>, kDecThreads, 0);
-  if (e) return e;
+  // every chunk size is bound to the same registers and shared memory
+  if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, decide_kernel<32>, kDecThreads, 0))) return e;
   *out = max(1, nb) * max(1, sms);
   return cudaSuccess;
 }
