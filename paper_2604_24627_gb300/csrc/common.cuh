@@ -190,6 +190,12 @@ __device__ __forceinline__ uint32_t word(const uint4& b, int j) {
   return j == 0 ? b.x : (j == 1 ? b.y : (j == 2 ? b.z : b.w));
 }
 
+// x^2 + y^2 + z^2 with its roundings fixed, where a tallied energy depends on
+// them: left to the compiler, the contraction varied with the code around it.
+__device__ __forceinline__ float sum_sq(float x, float y, float z) {
+  return __fmaf_rn(z, z, __fmaf_rn(x, x, __fmul_rn(y, y)));
+}
+
 // ---------------------------------------------------------------- sums
 // An unevaluated sum of three binary32 numbers, for sums that FP64 (1/64 of
 // the FP32 rate) would bound: TwoSum is exact, so each term loses the rounding

@@ -373,16 +373,16 @@ __device__ __noinline__ void totals_fp64(int ncells, const SpeciesPtrs& e, const
       for (int i = lane; i < na; i += 32) {
         const float4 r = a.wp[(long)c * a.cap + i];
         v[0] += r.x;
-        v[1] += (double)r.x * sqrtf(r.y * r.y + r.z * r.z + r.w * r.w);
+        v[1] += (double)r.x * sqrtf(sum_sq(r.y, r.z, r.w));
       }
       for (int i = lane; i < ng; i += 32) {
         const float4 r = g.wp[(long)c * g.cap + i];
         v[2] += r.x;
-        v[3] += (double)r.x * sqrtf(r.y * r.y + r.z * r.z + r.w * r.w);
+        v[3] += (double)r.x * sqrtf(sum_sq(r.y, r.z, r.w));
       }
       for (int i = lane; i < ne; i += 32) {
         const float4 r = e.wp[(long)c * e.cap + i];
-        v[4] += 0.5 * (double)r.x * (double)(r.y * r.y + r.z * r.z + r.w * r.w);
+        v[4] += 0.5 * (double)r.x * (double)sum_sq(r.y, r.z, r.w);
       }
     }
 }
@@ -423,15 +423,15 @@ __global__ void __launch_bounds__(kTotThreads) totals_kernel(int ncells, Species
         const float4 r1 = j1 < ne ? pe[j1] : z;
         if (i0 < na) {
           aw.add(ra.x);
-          aE.add_product(ra.x, sqrtf(ra.y * ra.y + ra.z * ra.z + ra.w * ra.w));
+          aE.add_product(ra.x, sqrtf(sum_sq(ra.y, ra.z, ra.w)));
         }
         if (i0 < ng) {
           gw.add(rg.x);
-          gE.add_product(rg.x, sqrtf(rg.y * rg.y + rg.z * rg.z + rg.w * rg.w));
+          gE.add_product(rg.x, sqrtf(sum_sq(rg.y, rg.z, rg.w)));
         }
         if (2 * i0 < ne) {
-          eE.add_product(r0.x, r0.y * r0.y + r0.z * r0.z + r0.w * r0.w);
-          eE.add_product(r1.x, r1.y * r1.y + r1.z * r1.z + r1.w * r1.w);
+          eE.add_product(r0.x, sum_sq(r0.y, r0.z, r0.w));
+          eE.add_product(r1.x, sum_sq(r1.y, r1.z, r1.w));
         }
       }
     }

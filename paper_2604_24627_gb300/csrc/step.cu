@@ -1497,7 +1497,7 @@ struct AxDest {
 __device__ __forceinline__ void gamma_products(const StepArgs& A, const PhItem& t, long abase, const AxDest& D,
                                                int i0, int K, const Cnt& cnt) {
   const float wprod = __uint_as_float(t.r.y);
-  const float pm = sqrtf(t.px * t.px + t.py * t.py + t.pz * t.pz);
+  const float pm = sqrtf(sum_sq(t.px, t.py, t.pz));
   const float om = pm * kMeC2f;
   // a massive axion takes E = omega and momentum beta p_gamma
   const float beta = A.mu > 0.f ? axion_beta(pm, A.mu2) : 1.0f;
