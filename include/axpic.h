@@ -461,9 +461,8 @@ axpic_status axpic_run_steps(axpic_ctx *ctx, int64_t first_step, int32_t nsteps,
  * and the branches a replayed step runs its cells as (each may be NULL).
  * A replayed step launches 4 x branches kernels (decision, event, the event
  * kernel of the cells with more flagged slots than a lane takes, feedback per
- * branch; 5 x branches with a rate model's record kernel) and one 4-byte
- * memset per branch. AXPIC_E_INVALID for a NULL context. Not part of the
- * paper's method. */
+ * branch; 5 x branches with a rate model's record kernel). AXPIC_E_INVALID
+ * for a NULL context. Not part of the paper's method. */
 axpic_status axpic_launch_shape(const axpic_ctx *ctx, int32_t *decide_chunk, int32_t *event_warps,
                                 int32_t *step_branches);
 

@@ -564,6 +564,7 @@ axpic_status axpic_init_plasma(axpic_ctx** out, const axpic_plasma_desc* desc, c
       (e = cudaMemsetAsync(ctx->tally, 0, tally_bytes, st)) ||
       (e = cudaMemsetAsync(ctx->counters, 0, sizeof(unsigned long long) * kNumCounters * (size_t)ctx->ctr_rows, st)) ||
       (e = cudaMemsetAsync(ctx->err, 0, sizeof(int), st)) ||
+      (e = cudaMemsetAsync(ctx->heavy_n, 0, sizeof(int32_t) * kMaxBranches, st)) ||
       (e = cudaMemsetAsync(ctx->bits, 0, sizeof(uint32_t) * (bit_words > 0 ? bit_words : 1), st)) ||
       (e = set_step_smem_limits(per_warp * ctx->max_warps)) ||
       (e = decide_resident_ctas(&ctx->dec_grid)) ||
@@ -883,7 +884,7 @@ static cudaError_t capture_steps(axpic_ctx* ctx, StepArgs A, int nsteps, cudaStr
   cudaError_t e;
   if (ctx->branches == 1 || part >= n) {
     for (int k = 0; k < nsteps; ++k)
-      if ((e = launch_step(PH_ALL, A, ctx->warps, gs, nullptr, sra))) return e;
+      if ((e = launch_step(PH_ALL, A, ctx->warps, gs, nullptr, sra, k > 0))) return e;
     return cudaSuccess;
   }
   for (int b = 0; b < kMaxBranches; ++b) {
@@ -910,7 +911,7 @@ static cudaError_t capture_steps(axpic_ctx* ctx, StepArgs A, int nsteps, cudaStr
     cudaStream_t bs = ctx->br_stream[nb];
     if ((e = cudaStreamWaitEvent(bs, ctx->br_ev[kMaxBranches], 0))) return e;
     for (int k = 0; k < nsteps; ++k)
-      if ((e = launch_step(PH_ALL, B, ctx->warps, bs, nullptr, sra ? &Bsr : nullptr))) return e;
+      if ((e = launch_step(PH_ALL, B, ctx->warps, bs, nullptr, sra ? &Bsr : nullptr, k > 0))) return e;
     if ((e = cudaEventRecord(ctx->br_ev[nb], bs))) return e;
   }
   for (int b = 0; b < nb; ++b)
@@ -1529,7 +1530,7 @@ axpic_status axpic_step_noalloc(const axpic_plasma_desc* desc, const axpic_param
   }
   const StepArgs A = make_args(&c, step, channel_mask);
   int h_err = 0;
-  if ((e = cudaMemsetAsync(c.err, 0, sizeof(int), st)) ||
+  if ((e = cudaMemsetAsync(c.err, 0, sizeof(int), st)) || (e = cudaMemsetAsync(c.heavy_n, 0, sizeof(int32_t), st)) ||
       (e = cudaMemsetAsync(c.counters, 0, sizeof(unsigned long long) * kNumCounters * (size_t)c.ctr_rows, st)) ||
       (e = cudaMemsetAsync(c.xbuf, 0, sizeof(double) * 4 * (size_t)d.ncells, st)) ||
       (e = cudaMemsetAsync(c.bits, 0, bit_bytes > 0 ? bit_bytes : 4, st)) ||

@@ -147,6 +147,31 @@ struct SpeciesPtrs {
   int32_t cap;
 };
 
+// ---------------------------------------------------------------- launches
+// A step is a chain of short kernels. Launched with programmatic stream
+// serialization, a kernel is set up while its predecessor ends and waits here,
+// first of all and in every thread, until the predecessor's memory is visible
+// (a no-op in a kernel launched without it). A step of 64 cells: 27.3 -> 18.0
+// us, with the memset between its kernels gone; 32 replayed steps of 65,536
+// dense cells in 8 branches: 6.77 -> 6.60 ms.
+__device__ __forceinline__ void wait_predecessor() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+template <typename... Params, typename... Args>
+cudaError_t launch_chained(bool chained, void (*kernel)(Params...), int grid, int block, size_t smem, cudaStream_t st,
+                           Args... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(block);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr = {};
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &attr;
+  cfg.numAttrs = chained ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
 // ---------------------------------------------------------------- Philox
 __device__ __forceinline__ uint4 philox4x32_10(uint4 c, uint32_t k0, uint32_t k1) {
 #pragma unroll

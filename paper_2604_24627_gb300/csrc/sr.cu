@@ -69,6 +69,7 @@ void build_sr_table(int nkt, int nne, double brems_shape, float* out) {
 // 192 record entries (consecutive threads, consecutive entries of a cell).
 constexpr int kSrTableThreads = 256;
 __global__ void __launch_bounds__(kSrTableThreads) sr_table_kernel(SrArgs a) {
+  wait_predecessor();
   __shared__ SrInterp ip[32];
   const int c0 = a.cell0 + blockIdx.x * 32;
   const int nc = min(32, a.cell0 + a.ncells - c0);
@@ -81,10 +82,9 @@ __global__ void __launch_bounds__(kSrTableThreads) sr_table_kernel(SrArgs a) {
   }
 }
 
-cudaError_t launch_sr_table(const SrArgs& a, cudaStream_t st) {
+cudaError_t launch_sr_table(const SrArgs& a, cudaStream_t st, bool chained) {
   if (a.ncells <= 0) return cudaSuccess;
-  sr_table_kernel<<<(a.ncells + 31) / 32, kSrTableThreads, 0, st>>>(a);
-  return cudaGetLastError();
+  return launch_chained(chained, sr_table_kernel, (a.ncells + 31) / 32, kSrTableThreads, 0, st, a);
 }
 
 // ---------------------------------------------------------------- surrogate model
@@ -94,6 +94,7 @@ cudaError_t launch_sr_table(const SrArgs& a, cudaStream_t st) {
 // tile that has a trusted cell; trusted cells get their rate prefactors,
 // the others the table record (a warp per cell, after the network).
 __global__ void __launch_bounds__(kNetThreads) sr_cells_kernel(SrArgs a) {
+  wait_predecessor();
   extern __shared__ __align__(1024) unsigned char sm[];
   __shared__ NetShared ns;
   __shared__ int list[kNetThreads];
@@ -167,17 +168,16 @@ __global__ void __launch_bounds__(kNetThreads) sr_cells_kernel(SrArgs a) {
 
 static int g_sr_cells_grid = 0;
 
-cudaError_t launch_sr_cells(const SrArgs& a, cudaStream_t st) {
+cudaError_t launch_sr_cells(const SrArgs& a, cudaStream_t st, bool chained) {
   if (a.ncells <= 0) return cudaSuccess;
   const int ntiles = (a.ncells + kNetThreads - 1) / kNetThreads;
   const int grid = std::max(1, std::min(ntiles, g_sr_cells_grid > 0 ? g_sr_cells_grid : ntiles));
-  sr_cells_kernel<<<grid, kNetThreads, kNetSmemBytes, st>>>(a);
-  return cudaGetLastError();
+  return launch_chained(chained, sr_cells_kernel, grid, kNetThreads, kNetSmemBytes, st, a);
 }
 
-cudaError_t launch_sr_records(int model, const SrArgs& a, cudaStream_t st) {
-  if (model == 1) return launch_sr_table(a, st);
-  if (model == 2) return launch_sr_cells(a, st);
+cudaError_t launch_sr_records(int model, const SrArgs& a, cudaStream_t st, bool chained) {
+  if (model == 1) return launch_sr_table(a, st, chained);
+  if (model == 2) return launch_sr_cells(a, st, chained);
   return cudaSuccess;
 }
 

@@ -149,14 +149,15 @@ __device__ __forceinline__ void sr_table_record_warp(const RecordArgs& a, const 
 void build_sr_table(int nkt, int nne, double brems_shape, float* out);
 
 // Rate model 1: every cell's table record.
-cudaError_t launch_sr_table(const SrArgs& a, cudaStream_t st);
+cudaError_t launch_sr_table(const SrArgs& a, cudaStream_t st, bool chained = false);
 // Rate model 2: per cell of [cell0, cell0 + ncells), from its current cell
 // record: the network's prefactors into the record's rate slots where it is
 // trusted, the table's spectral record elsewhere (src set accordingly). The
 // record's closed-form slots must be current (launch_records) before it runs.
-cudaError_t launch_sr_cells(const SrArgs& a, cudaStream_t st);
+cudaError_t launch_sr_cells(const SrArgs& a, cudaStream_t st, bool chained = false);
 // The records of rate model `model` (1 or 2) for cells [cell0, cell0 + ncells).
-cudaError_t launch_sr_records(int model, const SrArgs& a, cudaStream_t st);
+// chained: the last operation queued on st is the feedback kernel.
+cudaError_t launch_sr_records(int model, const SrArgs& a, cudaStream_t st, bool chained = false);
 cudaError_t sr_init_kernels();
 // Lays out the network (FP32 parameters P and the output model's mu, sigma
 // and S, all device) as the image of srnet.cuh in img (device, kNetImgBytes).

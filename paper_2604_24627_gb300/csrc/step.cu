@@ -965,6 +965,7 @@ __device__ __forceinline__ uint32_t step_of(const StepArgs& A) { return A.step_d
 
 template <int C>
 __global__ void __launch_bounds__(kDecThreads, AXPIC_DEC_MIN_CTAS) decide_kernel(StepArgs A, int kinds) {
+  wait_predecessor();
   __shared__ DecLists L;
   const int lane = lane_id(), wid = threadIdx.x >> 5;
   const uint32_t step = step_of(A);
@@ -1165,9 +1166,13 @@ constexpr int kFeedbackThreads = 128;
 
 template <bool DENSE>
 __global__ void __launch_bounds__(kFeedbackThreads, DENSE ? 4 : 5) feedback_kernel(StepArgs A) {
+  wait_predecessor();
   // a replayed graph takes its step index from the device counter: the last
   // kernel of the step advances it (no kernel of this launch reads it)
-  if (A.step_dev && blockIdx.x == 0 && threadIdx.x == 0) *A.step_dev += 1u;
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    if (A.step_dev) *A.step_dev += 1u;
+    *A.heavy_n = 0;  // the heavy cells' list of the next step
+  }
   const int lane = threadIdx.x & 31;
   const int cell = A.cell0 + blockIdx.x * blockDim.x + threadIdx.x;
   const bool valid = cell < A.cell0 + A.ncells;
@@ -2019,6 +2024,7 @@ __device__ __forceinline__ void absorb_lane(const StepArgs& A, int cell, uint32_
 template <int PH>
 __global__ void __launch_bounds__(128, PH == 3 ? AXPIC_EVENT_FULL_MIN_CTAS : AXPIC_EVENT_MIN_CTAS)
     event_kernel(StepArgs A) {
+  wait_predecessor();
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ unsigned long long warp_cnt[4][kNumCounters];
   const int wid = threadIdx.x >> 5;
@@ -2234,6 +2240,7 @@ __global__ void __launch_bounds__(128, PH == 3 ? AXPIC_EVENT_FULL_MIN_CTAS : AXP
 constexpr int kHeavyGrid = 152;  // one CTA on each of the 152 SMs
 
 __global__ void __launch_bounds__(128) event_heavy_kernel(StepArgs A) {
+  wait_predecessor();
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ unsigned long long warp_cnt[4][kNumCounters];
   const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -2326,23 +2333,17 @@ int resident_ctas(const void* fn, int threads, size_t dyn_smem, int max_per_sm) 
 }
 
 template <int PH>
-static cudaError_t launch_events(const StepArgs& A, int warps, cudaStream_t st) {
+static cudaError_t launch_events(const StepArgs& A, int warps, cudaStream_t st, bool chained) {
   constexpr bool full = PH == (PH_ABSORB | PH_EMIT);
   const size_t lists = ev_scratch_bytes(A.a.cap, A.g.cap, A.e.cap, true);
   const size_t per = ev_scratch_bytes(A.a.cap, A.g.cap, A.e.cap, !full);
   const int grid = (A.ncells + 32 * warps - 1) / (32 * warps);
-  if (full) {
-    cudaError_t e = cudaMemsetAsync(A.heavy_n, 0, sizeof(int32_t), st);
-    if (e) return e;
-  }
-  event_kernel<PH><<<grid, warps * 32, per * warps, st>>>(A);
-  if (full) {
-    // persistent over the heavy list: a warp per cell, at most one warp per
-    // cell of the launch and kHeavyGrid CTAs
-    const int hgrid = max(1, min((A.ncells + warps - 1) / warps, kHeavyGrid));
-    event_heavy_kernel<<<hgrid, warps * 32, lists * warps, st>>>(A);
-  }
-  return cudaGetLastError();
+  const cudaError_t e = launch_chained(chained, event_kernel<PH>, grid, warps * 32, per * warps, st, A);
+  if (e || !full) return e;
+  // persistent over the heavy list: a warp per cell, at most one warp per
+  // cell of the launch and kHeavyGrid CTAs
+  const int hgrid = max(1, min((A.ncells + warps - 1) / warps, kHeavyGrid));
+  return launch_chained(chained, event_heavy_kernel, hgrid, warps * 32, lists * warps, st, A);
 }
 
 // Cells per chunk of a decision warp: asked for, or by the launch. A chunk
@@ -2386,7 +2387,7 @@ static int decide_kinds(const StepArgs& A, int phases) {
   return k;
 }
 
-static cudaError_t launch_decide(const StepArgs& A, int phases, cudaStream_t st) {
+static cudaError_t launch_decide(const StepArgs& A, int phases, cudaStream_t st, bool chained) {
   const int kinds = decide_kinds(A, phases);
   if (kinds == 0) return cudaSuccess;
   // persistent: as many CTAs as the device holds at once, at most one warp
@@ -2394,36 +2395,24 @@ static cudaError_t launch_decide(const StepArgs& A, int phases, cudaStream_t st)
   const int chunk = decide_chunk(A);
   const int nchunks = (A.ncells + chunk - 1) / chunk;
   const int grid = max(1, min((nchunks + kDecWarps - 1) / kDecWarps, A.dec_grid));
+  auto kernel = decide_kernel<32>;
   switch (chunk) {
-    case 1:
-      decide_kernel<1><<<grid, kDecThreads, 0, st>>>(A, kinds);
-      break;
-    case 2:
-      decide_kernel<2><<<grid, kDecThreads, 0, st>>>(A, kinds);
-      break;
-    case 4:
-      decide_kernel<4><<<grid, kDecThreads, 0, st>>>(A, kinds);
-      break;
-    case 8:
-      decide_kernel<8><<<grid, kDecThreads, 0, st>>>(A, kinds);
-      break;
-    case 16:
-      decide_kernel<16><<<grid, kDecThreads, 0, st>>>(A, kinds);
-      break;
-    default:
-      decide_kernel<32><<<grid, kDecThreads, 0, st>>>(A, kinds);
-      break;
+    case 1: kernel = decide_kernel<1>; break;
+    case 2: kernel = decide_kernel<2>; break;
+    case 4: kernel = decide_kernel<4>; break;
+    case 8: kernel = decide_kernel<8>; break;
+    case 16: kernel = decide_kernel<16>; break;
+    default: break;
   }
-  return cudaGetLastError();
+  return launch_chained(chained, kernel, grid, kDecThreads, 0, st, A, kinds);
 }
 
-static cudaError_t launch_feedback(const StepArgs& A, cudaStream_t st) {
+static cudaError_t launch_feedback(const StepArgs& A, cudaStream_t st, bool chained) {
   const int grid = (A.ncells + kFeedbackThreads - 1) / kFeedbackThreads;
   // absorption by weight reduction takes energy from every axion: most cells
   // are remapped every step
-  if (A.absorb_mode == 1) feedback_kernel<true><<<grid, kFeedbackThreads, 0, st>>>(A);
-  else feedback_kernel<false><<<grid, kFeedbackThreads, 0, st>>>(A);
-  return cudaGetLastError();
+  return launch_chained(chained, A.absorb_mode == 1 ? feedback_kernel<true> : feedback_kernel<false>, grid,
+                        kFeedbackThreads, 0, st, A);
 }
 
 const char* step_kernel_names(int rate_model, int T_mode) {
@@ -2455,31 +2444,39 @@ cudaError_t decide_resident_ctas(int* out) {
 // After the temperature update of an evolved-T step the rate model's records
 // follow the new T: the table model's spectral records, or the surrogate
 // network's prefactors (the table's records where it is not trusted).
-static cudaError_t launch_records_update(const StepArgs& A, const SrArgs* sra, cudaStream_t st) {
+static cudaError_t launch_records_update(const StepArgs& A, const SrArgs* sra, cudaStream_t st, bool chained) {
   if (!sra || A.T_mode != 2) return cudaSuccess;
-  return launch_sr_records(A.rate_model, *sra, st);
+  return launch_sr_records(A.rate_model, *sra, st, chained);
 }
 
 cudaError_t launch_step(int phases, const StepArgs& A, int warps, cudaStream_t st, cudaEvent_t* ev,
-                        const SrArgs* sra) {
+                        const SrArgs* sra, bool after_step) {
   if (A.ncells == 0) return cudaSuccess;
   cudaError_t e;
-  // optional measurement: events between the kernels of a full step
+  // optional measurement: events between the kernels of a full step, which
+  // then run one by one
   auto mark = [&](int i) { return ev ? cudaEventRecord(ev[i], st) : cudaSuccess; };
+  const bool chain = !ev;
   switch (phases) {
     case PH_ABSORB:
-      if ((e = launch_decide(A, PH_ABSORB, st))) return e;
-      return launch_events<PH_ABSORB>(A, warps, st);
+      if ((e = launch_decide(A, PH_ABSORB, st, false))) return e;
+      return launch_events<PH_ABSORB>(A, warps, st, true);
     case PH_EMIT:
-      if ((e = launch_decide(A, PH_EMIT, st))) return e;
-      return launch_events<PH_EMIT>(A, warps, st);
+      if ((e = launch_decide(A, PH_EMIT, st, false))) return e;
+      return launch_events<PH_EMIT>(A, warps, st, true);
     case PH_FEEDBACK:
-      if ((e = launch_feedback(A, st))) return e;
-      return launch_records_update(A, sra, st);
+      if ((e = launch_feedback(A, st, false))) return e;
+      return launch_records_update(A, sra, st, true);
     case PH_ALL:
-      if ((e = mark(0)) || (e = launch_decide(A, PH_ABSORB | PH_EMIT, st)) || (e = mark(1))) return e;
-      if ((e = launch_events<PH_ABSORB | PH_EMIT>(A, warps, st)) || (e = mark(2))) return e;
-      if ((e = launch_feedback(A, st)) || (e = mark(3)) || (e = launch_records_update(A, sra, st)) || (e = mark(4)))
+      if ((e = mark(0)) || (e = launch_decide(A, PH_ABSORB | PH_EMIT, st, chain && after_step)) || (e = mark(1)))
+        return e;
+      // (with nothing to decide the events are the first kernel)
+      if ((e = launch_events<PH_ABSORB | PH_EMIT>(A, warps, st,
+                                                  chain && (after_step || decide_kinds(A, PH_ABSORB | PH_EMIT)))) ||
+          (e = mark(2)))
+        return e;
+      if ((e = launch_feedback(A, st, chain)) || (e = mark(3)) || (e = launch_records_update(A, sra, st, chain)) ||
+          (e = mark(4)))
         return e;
       return cudaSuccess;
     default:

@@ -12,8 +12,10 @@ size_t step_smem_per_warp(int acap, int gcap, int ecap);
 // PH_ALL step: decisions, events, feedback, and the rate model's record
 // kernel (an empty interval when there is none). sra: the record kernels'
 // arguments (rate models 1 and 2), else NULL.
+// after_step: the last operation queued on st is a kernel of another step (the
+// first kernel then overlaps its end too).
 cudaError_t launch_step(int phases, const StepArgs& A, int warps, cudaStream_t st, cudaEvent_t* ev = nullptr,
-                        const SrArgs* sra = nullptr);
+                        const SrArgs* sra = nullptr, bool after_step = false);
 constexpr int kStepKernels = 4;
 // Comma-separated names of the kernels a PH_ALL step launches, in order.
 const char* step_kernel_names(int rate_model, int T_mode);

@@ -281,6 +281,7 @@ __device__ __forceinline__ void move_cells(const StreamArgs& a, int c0, int n_l,
 // register passes, else one after the other.
 template <int K>
 __global__ void __launch_bounds__(kThreads, 3) stream_move_kernel(StreamArgs a) {
+  wait_predecessor();
   __shared__ MoveShared S[kWarps];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int c0 = (blockIdx.x * kWarps + wid) * K;
@@ -322,6 +323,7 @@ constexpr int kPlace = 2;  // words of freed slots whose arrivals are loaded tog
 
 template <int K>
 __global__ void __launch_bounds__(kThreads, 6) stream_place_kernel(StreamArgs a) {
+  wait_predecessor();
   // a cell's arrival groups, lane r the neighbour at (dz, dy, dx) = r's
   // digits - 1: arrivals up to and with the group, the neighbour, and the
   // staging row of arrival 0 of the cell's numbering
@@ -530,11 +532,9 @@ __global__ void __launch_bounds__(kThreads, 6) stream_place_kernel(StreamArgs a)
 template <int K>
 cudaError_t launch(const StreamArgs& a, cudaStream_t st) {
   const int grid = (a.ncells + kWarps * K - 1) / (kWarps * K);
-  stream_move_kernel<K><<<grid, kThreads, 0, st>>>(a);
-  cudaError_t e = cudaGetLastError();
+  const cudaError_t e = launch_chained(false, stream_move_kernel<K>, grid, kThreads, 0, st, a);
   if (e) return e;
-  stream_place_kernel<K><<<grid, kThreads, 0, st>>>(a);
-  return cudaGetLastError();
+  return launch_chained(true, stream_place_kernel<K>, grid, kThreads, 0, st, a);
 }
 
 }  // namespace
