@@ -443,7 +443,7 @@ axpic_status axpic_step_noalloc(const axpic_plasma_desc *desc, const axpic_param
 /* Runs nsteps full steps (as axpic_step with steps first_step,
  * first_step + 1, ...) by replaying CUDA graphs of 32 steps and of one step
  * (for the remainder): the decision, event and feedback kernels (and, with
- * evolved T, the rate model's record kernel), with the step index read from
+ * evolved T, the surrogate's network kernel), with the step index read from
  * device counters that the feedback kernels advance.
  * Inside a graph the cells run as step_branches independent ranges on forked
  * streams, each range with its own counter, joined at the graph's end. Both
@@ -461,7 +461,7 @@ axpic_status axpic_run_steps(axpic_ctx *ctx, int64_t first_step, int32_t nsteps,
  * and the branches a replayed step runs its cells as (each may be NULL).
  * A replayed step launches 4 x branches kernels (decision, event, the event
  * kernel of the cells with more flagged slots than a lane takes, feedback per
- * branch; 5 x branches with a rate model's record kernel). AXPIC_E_INVALID
+ * branch; 5 x branches with the surrogate's network kernel). AXPIC_E_INVALID
  * for a NULL context. Not part of the paper's method. */
 axpic_status axpic_launch_shape(const axpic_ctx *ctx, int32_t *decide_chunk, int32_t *event_warps,
                                 int32_t *step_branches);
@@ -496,8 +496,9 @@ axpic_status axpic_profile_end(axpic_ctx *ctx, double *ms_out, int32_t *steps_ou
 /* Comma-separated names of the profiled kernels of one axpic_step, in
  * launch order: decisions, events (its slot also times event_heavy_kernel,
  * launched right after it for the cells with more flagged slots than a lane
- * takes), feedback, then, with evolved T, the rate model's record kernel
- * (sr_table_kernel for the table model, sr_cells_kernel for the surrogate).
+ * takes), feedback, then, with evolved T under the surrogate model, the
+ * network kernel (sr_cells_kernel; the table model interpolates the entries
+ * it needs inside the decision and event kernels).
  * The string is static; "" for a NULL context. */
 const char *axpic_step_kernel_names(const axpic_ctx *ctx);
 
@@ -642,7 +643,8 @@ axpic_status axpic_get_cell_records(axpic_ctx *ctx, int32_t first, int32_t count
  * k = 0..31 (c * 32 + k; c = Primakoff, Compton-like, brems), the
  * quantiles x(j/32) (96 + c * 31 + j - 1), then ln(g_agg^2 dt pi^2 (hbar c)^3
  * / (T^4 keV)), ln(g_ae^2 dt 2 pi^2 (hbar c)^3 / (T^4 keV)) and T.
- * Synchronises. */
+ * Interpolated from the table for the cells' current records (the step
+ * interpolates the entries it needs and keeps none). Synchronises. */
 axpic_status axpic_get_spectral_records(axpic_ctx *ctx, int32_t first, int32_t count, float *out);
 
 /* Wait for the stream and return the first latched device error, if any. */

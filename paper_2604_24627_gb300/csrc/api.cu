@@ -360,13 +360,23 @@ static SrArgs make_sr_args(axpic_ctx* ctx) {
   return a;
 }
 
-// Rebuilds every cell's rate-model record for its current T and composition
-// (the cell records' closed-form slots must be current): the table model's
-// spectral records; under the surrogate model the network's prefactors
-// where it is trusted and the table's records elsewhere.
+// After the cell records' closed-form slots were recomputed for the current T
+// and composition: under the surrogate model the network's prefactors where it
+// is trusted, and which cells it is not trusted for. (The table's records
+// follow the cell records by themselves: the step interpolates what it needs.)
 static cudaError_t build_records(axpic_ctx* ctx, cudaStream_t st) {
-  if (!ctx->prm.rate_model) return cudaSuccess;
-  return launch_sr_records(ctx->prm.rate_model, make_sr_args(ctx), st);
+  if (ctx->prm.rate_model != 2) return cudaSuccess;
+  return launch_sr_cells(make_sr_args(ctx), st);
+}
+
+// The spectral records of cells [first, first + count) as they are read or
+// saved.
+static cudaError_t write_spectra(axpic_ctx* ctx, int first, int count) {
+  if (!ctx->sr) return cudaSuccess;
+  SrArgs a = make_sr_args(ctx);
+  a.cell0 = first;
+  a.ncells = count;
+  return launch_sr_table(a, ctx->stream);
 }
 
 static void free_events(axpic_ctx* ctx) {
@@ -1316,6 +1326,7 @@ axpic_status axpic_save_state(axpic_ctx* ctx, void* host_out, uint64_t bytes) {
   if (!ctx || !host_out || axpic_state_bytes(ctx, &need) != AXPIC_OK || bytes != need)
     return ctx ? fail(ctx, AXPIC_E_INVALID, "axpic_save_state: buffer size") : AXPIC_E_INVALID;
   CK(fold_tally(ctx), "fold tally");
+  CK(write_spectra(ctx, 0, ctx->desc.ncells), "spectral records");
   unsigned char* p = static_cast<unsigned char*>(host_out);
   for (auto& b : state_buffers(ctx, false)) {
     CK(cudaMemcpyAsync(p, b.first, b.second, cudaMemcpyDeviceToHost, ctx->stream), "copy");
@@ -1390,6 +1401,7 @@ axpic_status axpic_get_spectral_records(axpic_ctx* ctx, int32_t first, int32_t c
   if (!ctx || !out || first < 0 || count < 0 || first + count > ctx->desc.ncells) return AXPIC_E_INVALID;
   if (!ctx->sr) return fail(ctx, AXPIC_E_INVALID, "axpic_get_spectral_records: rate_model 0 keeps no records");
   if (count == 0) return AXPIC_OK;
+  CK(write_spectra(ctx, first, count), "spectral records");
   CK(cudaMemcpyAsync(out, ctx->sr + (size_t)first * kSrLen, sizeof(float) * kSrLen * count, cudaMemcpyDeviceToHost,
                      ctx->stream),
      "copy");

@@ -123,7 +123,7 @@ struct CellConst {
 //    cell-independent quantiles (uni); elsewhere (src[cell] = 1) the cell has
 //    the table's spectral record, as in rate model 1.
 struct RecordArgs {
-  float* sr;                  // [ncells * 192] spectral records
+  float* sr;                  // [ncells * 192] spectral records, written when they are read or saved
   const float* tab;           // exact table [2][nne][nkt][189]
   int nkt, nne;
   float Z;                    // the single ion species' charge

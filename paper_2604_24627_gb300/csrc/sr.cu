@@ -2,15 +2,16 @@
 //
 // Table model (rate model 1): the exact targets tabulated on the host over
 // (ln kappa/T, log10 n_e, Z) and interpolated bilinearly per cell into a
-// 192-float spectral record.
+// 192-float spectral record, of which a step interpolates the entries it
+// needs.
 //
 // Surrogate model (rate model 2): the network evaluated once per cell (its
 // inputs are the cell features; every x-dependence is in the exact shapes),
 // one tcgen05 row per cell, giving the cell's three ln-emissivity constants;
 // they become the prefactors of the closed functional forms in the cell
 // record (srnet.cuh). Cells whose (T, n_e, Z) lies outside the region where
-// the network's validated error is within the bound get the table's
-// spectral record instead, written by the same CTA. The kernel runs right
+// the network's validated error is within the bound are marked, and use the
+// table's spectral record instead. The kernel runs right
 // after the feedback kernel of every evolved-T step (the records then hold
 // the new temperature with closed-form prefactors), at set-up, and after the
 // caller changes T or the composition.
@@ -64,42 +65,46 @@ void build_sr_table(int nkt, int nne, double brems_shape, float* out) {
 }
 
 // ---------------------------------------------------------------- table model
-// A CTA takes 32 cells: warp 0 forms each cell's interpolation constants
-// (lane per cell) in shared memory, then the CTA's threads stream the 32 x
-// 192 record entries (consecutive threads, consecutive entries of a cell).
+// The records as they are read out and saved (the step interpolates the
+// entries it needs). A CTA takes 32 cells: warp 0 forms each cell's
+// interpolation constants (lane per cell) in shared memory, then the CTA's
+// threads stream the 32 x 192 record entries (consecutive threads,
+// consecutive entries of a cell); under the surrogate model only those of
+// the cells the network is not trusted for.
 constexpr int kSrTableThreads = 256;
 __global__ void __launch_bounds__(kSrTableThreads) sr_table_kernel(SrArgs a) {
-  wait_predecessor();
   __shared__ SrInterp ip[32];
+  __shared__ uint8_t has[32];
   const int c0 = a.cell0 + blockIdx.x * 32;
   const int nc = min(32, a.cell0 + a.ncells - c0);
-  if (threadIdx.x < 32 && (int)threadIdx.x < nc)
+  if (threadIdx.x < 32 && (int)threadIdx.x < nc) {
     sr_interp(a.ra, sr_cell_from(a.rec + (size_t)(c0 + threadIdx.x) * kRecLen, a.ra.k_T7), &ip[threadIdx.x]);
+    has[threadIdx.x] = a.ra.src ? a.ra.src[c0 + threadIdx.x] : 1;
+  }
   __syncthreads();
   for (int e = threadIdx.x; e < nc * kSrLen; e += kSrTableThreads) {
     const int c = e / kSrLen, o = e - c * kSrLen;
-    a.ra.sr[(size_t)(c0 + c) * kSrLen + o] = sr_table_entry(a.ra, ip[c], o);
+    if (has[c]) a.ra.sr[(size_t)(c0 + c) * kSrLen + o] = sr_table_entry(a.ra, ip[c], o);
   }
 }
 
-cudaError_t launch_sr_table(const SrArgs& a, cudaStream_t st, bool chained) {
+cudaError_t launch_sr_table(const SrArgs& a, cudaStream_t st) {
   if (a.ncells <= 0) return cudaSuccess;
-  return launch_chained(chained, sr_table_kernel, (a.ncells + 31) / 32, kSrTableThreads, 0, st, a);
+  sr_table_kernel<<<(a.ncells + 31) / 32, kSrTableThreads, 0, st>>>(a);
+  return cudaGetLastError();
 }
 
 // ---------------------------------------------------------------- surrogate model
 // A persistent grid: each CTA sets the network up once (tensor memory, the
 // weights' image in shared memory) and takes tiles of 128 consecutive cells,
 // thread t = cell t of the tile = tensor-core row t. The network runs for a
-// tile that has a trusted cell; trusted cells get their rate prefactors,
-// the others the table record (a warp per cell, after the network).
+// tile that has a trusted cell; trusted cells get their rate prefactors, the
+// others are marked for the table.
 __global__ void __launch_bounds__(kNetThreads) sr_cells_kernel(SrArgs a) {
   wait_predecessor();
   extern __shared__ __align__(1024) unsigned char sm[];
   __shared__ NetShared ns;
-  __shared__ int list[kNetThreads];
-  __shared__ int nlist;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x;
   const int ntiles = (a.ncells + kNetThreads - 1) / kNetThreads;
   const bool net = a.ra.trust != nullptr;
   if (net) net_begin(&ns, sm, a.ra.img);
@@ -116,7 +121,6 @@ __global__ void __launch_bounds__(kNetThreads) sr_cells_kernel(SrArgs a) {
   for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
     const int cell = a.cell0 + tile * kNetThreads + tid;
     const bool valid = cell < a.cell0 + a.ncells;
-    if (tid == 0) nlist = 0;
     float r[kRecLen];
 #pragma unroll
     for (int i = 0; i < kRecLen / 4; ++i) {
@@ -150,18 +154,7 @@ __global__ void __launch_bounds__(kNetThreads) sr_cells_kernel(SrArgs a) {
         o[1] = make_float4(r[4], r[5], r[6], r[7]);
       }
     }
-    if (valid) {
-      a.ra.src[cell] = trusted ? 0 : 1;
-      if (!trusted) list[atomicAdd(&nlist, 1)] = tid;
-    }
-    __syncthreads();
-    const int n = nlist;
-    for (int k = warp; k < n; k += kNetThreads / 32) {
-      const int c = a.cell0 + tile * kNetThreads + list[k];
-      const SrCellIn cc = sr_cell_from(a.rec + (size_t)c * kRecLen, a.ra.k_T7);
-      sr_table_record_warp(a.ra, cc, a.ra.sr + (size_t)c * kSrLen, lane);
-    }
-    __syncthreads();  // the list and nlist are reused by the next tile
+    if (valid) a.ra.src[cell] = trusted ? 0 : 1;
   }
   if (net) net_end(&ns);
 }
@@ -173,12 +166,6 @@ cudaError_t launch_sr_cells(const SrArgs& a, cudaStream_t st, bool chained) {
   const int ntiles = (a.ncells + kNetThreads - 1) / kNetThreads;
   const int grid = std::max(1, std::min(ntiles, g_sr_cells_grid > 0 ? g_sr_cells_grid : ntiles));
   return launch_chained(chained, sr_cells_kernel, grid, kNetThreads, kNetSmemBytes, st, a);
-}
-
-cudaError_t launch_sr_records(int model, const SrArgs& a, cudaStream_t st, bool chained) {
-  if (model == 1) return launch_sr_table(a, st, chained);
-  if (model == 2) return launch_sr_cells(a, st, chained);
-  return cudaSuccess;
 }
 
 // The persistent grid: as many CTAs as the device holds at once (worked out

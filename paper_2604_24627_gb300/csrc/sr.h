@@ -133,14 +133,6 @@ __device__ __forceinline__ bool sr_trusted(const RecordArgs& a, float T, float l
   return t[0] && t[1] && t[a.tnT] && t[a.tnT + 1];
 }
 
-// A warp writes one cell's whole table record (lane l: entries l + 32 k).
-__device__ __forceinline__ void sr_table_record_warp(const RecordArgs& a, const SrCellIn& c, float* out, int lane) {
-  SrInterp q;
-  sr_interp(a, c, &q);
-#pragma unroll
-  for (int k = 0; k < kSrLen / 32; ++k) out[lane + 32 * k] = sr_table_entry(a, q, lane + 32 * k);
-}
-
 // ---------------------------------------------------------------- host side
 // The exact table, nkt x nne x 2 nodes (ln(kappa/T) uniform on
 // [ln 0.012, ln 41], log10 n_e uniform on [23, 26], Z = 1, 2), binary64
@@ -148,16 +140,15 @@ __device__ __forceinline__ void sr_table_record_warp(const RecordArgs& a, const 
 // brackets).
 void build_sr_table(int nkt, int nne, double brems_shape, float* out);
 
-// Rate model 1: every cell's table record.
-cudaError_t launch_sr_table(const SrArgs& a, cudaStream_t st, bool chained = false);
+// The table's spectral records of cells [cell0, cell0 + ncells) into ra.sr, for
+// reading and saving: all of them, or those with src set.
+cudaError_t launch_sr_table(const SrArgs& a, cudaStream_t st);
 // Rate model 2: per cell of [cell0, cell0 + ncells), from its current cell
 // record: the network's prefactors into the record's rate slots where it is
-// trusted, the table's spectral record elsewhere (src set accordingly). The
-// record's closed-form slots must be current (launch_records) before it runs.
+// trusted (src 0; 1 elsewhere: the table). The record's closed-form slots
+// must be current (launch_records) before it runs. chained: the last operation
+// queued on st is the feedback kernel.
 cudaError_t launch_sr_cells(const SrArgs& a, cudaStream_t st, bool chained = false);
-// The records of rate model `model` (1 or 2) for cells [cell0, cell0 + ncells).
-// chained: the last operation queued on st is the feedback kernel.
-cudaError_t launch_sr_records(int model, const SrArgs& a, cudaStream_t st, bool chained = false);
 cudaError_t sr_init_kernels();
 // Lays out the network (FP32 parameters P and the output model's mu, sigma
 // and S, all device) as the image of srnet.cuh in img (device, kNetImgBytes).

@@ -119,43 +119,55 @@ __device__ __noinline__ void tally_add(const StepArgs& A, int ch, float w, float
 // record holds ln(dQ_c/dx) + x at unit coupling on 32 points of ln x (step
 // ln(400)/29, one beyond each end of [0.05, 20]); a Catmull-Rom spline in
 // ln x interpolates it, the closed factors of Eqs. prim_rate and gamma_abs
-// turn it into a rate.
+// turn it into a rate. The entries a decision needs (4 of 192 a channel) are
+// interpolated from the table where they are needed (sr_table_entry, the bits
+// of the stored record): about 1.5 slots a cell and step take a full decision,
+// and writing every cell's 768-byte record after each temperature update took
+// 287 us a step of 884,736 cells (4 steps: 2.58 -> 1.80 ms without).
+struct CellSpectrum {
+  SrInterp q;
+  const RecordArgs& a;
+  __device__ __forceinline__ float at(int o) const { return sr_table_entry(a, q, o); }
+};
+
 __device__ __forceinline__ bool sr_in_range(float x) { return x >= 0.05f && x <= 20.0f; }
 
-__device__ __forceinline__ float sr_lnL(const float* sr, int ch, float lnx) {
+__device__ __forceinline__ float sr_lnL(const CellSpectrum& sr, int ch, float lnx) {
   float u = (lnx - kSrLnXLo) * (1.0f / kSrH) + 1.0f;
   u = fminf(fmaxf(u, 1.f), 30.f);
   const int k = min((int)u, 29);
   const float f = u - (float)k;
-  const float* g = sr + ch * kSrGrid;
-  const float p0 = g[k - 1], p1 = g[k], p2 = g[k + 1], p3 = g[k + 2];
+  const int g = ch * kSrGrid + k;
+  const float p0 = sr.at(g - 1), p1 = sr.at(g), p2 = sr.at(g + 1), p3 = sr.at(g + 2);
   const float s = p1 + 0.5f * f * (p2 - p0 + f * (2.f * p0 - 5.f * p1 + 4.f * p2 - p3 + f * (3.f * (p1 - p2) + p3 - p0)));
   return s - fminf(fmaxf(__expf(lnx), 0.05f), 20.0f);  // the stored values are ln(dQ/dx) + x
 }
 
 // Gamma_{gamma->a} dt at the cell's couplings (multiplicity 1).
-__device__ __forceinline__ float sr_prim_gdt(const float* sr, float x) {
+__device__ __forceinline__ float sr_prim_gdt(const CellSpectrum& sr, float x) {
   const float lx = logf(x);
-  return expf((sr_lnL(sr, 0, lx) + sr[SR_LNKP]) - 3.f * lx) * expm1f(x);
+  return expf((sr_lnL(sr, 0, lx) + sr.q.lnKP) - 3.f * lx) * expm1f(x);
 }
 
 // Absorption tau_c = Gamma_abs,c dt (c = 1 Compton-like, 2 bremsstrahlung).
-__device__ __forceinline__ float sr_tau(const float* sr, int ch, float x, int eq_stats) {
+__device__ __forceinline__ float sr_tau(const CellSpectrum& sr, int ch, float x, int eq_stats) {
   const float lx = logf(x);
-  const float b = expf((sr_lnL(sr, ch, lx) + sr[SR_LNKA]) - 3.f * lx);
+  const float b = expf((sr_lnL(sr, ch, lx) + sr.q.lnKA) - 3.f * lx);
   return eq_stats ? b * expm1f(x) : b * expf(x);
 }
 
-// x from the record's 31 quantiles of channel c (end points 0.05 and 20),
-// linear between quantiles.
-__device__ __forceinline__ float sr_sample_x(const float* sr, int ch, float u) {
-  const float t = u * 32.f;
-  const int j = min((int)t, 31);
-  const float f = t - (float)j;
-  const float* q = sr + 96 + ch * kSrKnots;
-  const float x0 = j == 0 ? 0.05f : q[j - 1];
-  const float x1 = j == 31 ? 20.0f : q[j];
-  return fmaf(f, x1 - x0, x0);
+// Whether a cell's full decisions and emission energies take their rates from
+// its spectral record: every cell under the table model, the cells the
+// network is not trusted for under the surrogate model; the others use the
+// closed forms with the cell record's prefactors.
+__device__ __forceinline__ bool cell_has_sr(const StepArgs& A, int cell) {
+  return A.rate_model == 1 || (A.rate_model == 2 && A.ra.src[cell]);
+}
+
+__device__ __forceinline__ CellSpectrum cell_spectrum(const StepArgs& A, const float* rec) {
+  CellSpectrum s{{}, A.ra};
+  sr_interp(A.ra, sr_cell_from(rec, A.ra.k_T7), &s.q);
+  return s;
 }
 
 // ---------------------------------------------------------------- decisions
@@ -168,7 +180,7 @@ struct AxionDecision {
   bool keep, absorbed, capped, over, abs_c;
 };
 
-__device__ __forceinline__ AxionDecision axion_decide(const float* rec, const float* sr, const StepArgs& A, int mask,
+__device__ __forceinline__ AxionDecision axion_decide(const float* rec, const CellSpectrum* sr, const StepArgs& A, int mask,
                                                       float w, float px, float py, float pz, uint32_t wP,
                                                       uint32_t wA) {
   AxionDecision d;
@@ -183,7 +195,7 @@ __device__ __forceinline__ AxionDecision axion_decide(const float* rec, const fl
   const float xr = d.om * rec[R_INVT];
   const bool use_sr = sr && sr_in_range(xr);
   if (mask & AXPIC_CH_PRIMAKOFF) {
-    const float P = use_sr ? -expm1f(-A.cc.prim_mult * sr_prim_gdt(sr, xr))
+    const float P = use_sr ? -expm1f(-A.cc.prim_mult * sr_prim_gdt(*sr, xr))
                            : prim_prob(rec, d.om, A.cc.prim_mult * rec[R_AP]);
     float fac;
     const float le = cap_lambda(w * P * A.inv_w_gref, A.lam_cap, &fac, &d.capped);
@@ -195,10 +207,10 @@ __device__ __forceinline__ AxionDecision axion_decide(const float* rec, const fl
   if (d.keep && (mask & (AXPIC_CH_COMPTON | AXPIC_CH_BREMS))) {
     const float x = xr;
     const float tc = !(mask & AXPIC_CH_COMPTON) ? 0.f
-                     : use_sr                   ? sr_tau(sr, 1, x, A.eq_stats)
+                     : use_sr                   ? sr_tau(*sr, 1, x, A.eq_stats)
                                                 : tau_compton(rec, x, A.eq_stats);
     const float tb = !(mask & AXPIC_CH_BREMS) ? 0.f
-                     : use_sr                 ? sr_tau(sr, 2, x, A.eq_stats)
+                     : use_sr                 ? sr_tau(*sr, 2, x, A.eq_stats)
                                               : tau_brems(rec, x, A.brems_am3, A.eq_stats);
     const float tau = tc + tb;
     if (A.absorb_mode == 0) {
@@ -215,15 +227,6 @@ __device__ __forceinline__ AxionDecision axion_decide(const float* rec, const fl
     }
   }
   return d;
-}
-
-// The spectral record a cell's full decisions and emission energies take
-// their rates from: every cell's under the table model, the cells the
-// network is not trusted for under the surrogate model; NULL otherwise (the
-// closed forms with the cell record's prefactors).
-__device__ __forceinline__ const float* cell_sr(const StepArgs& A, int cell) {
-  if (A.rate_model == 1 || (A.rate_model == 2 && A.ra.src[cell])) return A.ra.sr + (size_t)cell * kSrLen;
-  return nullptr;
 }
 
 __device__ __forceinline__ void load_rec(const StepArgs& A, int cell, float* rec) {
@@ -246,7 +249,13 @@ __device__ __noinline__ AxionDecision axion_decide_slow(const StepArgs& A, int c
   const float4 v = A.a.wp[idx];
   float rec[kRecLen];
   load_rec(A, cell, rec);
-  AxionDecision d = axion_decide(rec, cell_sr(A, cell), A, mask, v.x, v.y, v.z, v.w, wP, wA);
+  AxionDecision d;
+  if (cell_has_sr(A, cell)) {
+    const CellSpectrum sr = cell_spectrum(A, rec);
+    d = axion_decide(rec, &sr, A, mask, v.x, v.y, v.z, v.w, wP, wA);
+  } else {
+    d = axion_decide(rec, nullptr, A, mask, v.x, v.y, v.z, v.w, wP, wA);
+  }
   d.w = v.x;
   return d;
 }
@@ -259,7 +268,7 @@ struct PhotonDecision {
   bool capped, over;
 };
 
-__device__ __forceinline__ PhotonDecision photon_decide(const float* rec, const float* sr, const StepArgs& A, float w,
+__device__ __forceinline__ PhotonDecision photon_decide(const float* rec, const CellSpectrum* sr, const StepArgs& A, float w,
                                                         float px, float py, float pz, uint32_t wd) {
   PhotonDecision d;
   const float pm = sqrtf(px * px + py * py + pz * pz);
@@ -267,7 +276,7 @@ __device__ __forceinline__ PhotonDecision photon_decide(const float* rec, const 
   const float xr = d.om * rec[R_INVT];
   // a massive axion: the rate times beta(omega), zero at and below m_a
   const float beta = A.mu > 0.f ? axion_beta(pm, A.mu2) : 1.0f;
-  const float P = sr && sr_in_range(xr) ? -expm1f(-(beta * sr_prim_gdt(sr, xr))) : prim_prob(rec, d.om, beta * rec[R_AP]);
+  const float P = sr && sr_in_range(xr) ? -expm1f(-(beta * sr_prim_gdt(*sr, xr))) : prim_prob(rec, d.om, beta * rec[R_AP]);
   float fac;
   const float le = cap_lambda(w * P * A.inv_w_a, A.lam_cap, &fac, &d.capped);
   d.K = poisson_inv(u23(wd), le);
@@ -282,7 +291,11 @@ __device__ __noinline__ PhotonDecision photon_decide_slow(const StepArgs& A, int
   const float4 v = A.g.wp[idx];
   float rec[kRecLen];
   load_rec(A, cell, rec);
-  return photon_decide(rec, cell_sr(A, cell), A, v.x, v.y, v.z, v.w, wd);
+  if (cell_has_sr(A, cell)) {
+    const CellSpectrum sr = cell_spectrum(A, rec);
+    return photon_decide(rec, &sr, A, v.x, v.y, v.z, v.w, wd);
+  }
+  return photon_decide(rec, nullptr, A, v.x, v.y, v.z, v.w, wd);
 }
 
 // Guards: cheap upper bounds that prove, without the transcendental chain,
@@ -1519,13 +1532,37 @@ __device__ __forceinline__ void gamma_products(const StepArgs& A, const PhItem& 
   }
 }
 
+// x from the 31 quantiles of channel c (end points 0.05 and 20), linear
+// between quantiles: the cell's spectral record's, or the network's for every
+// cell. Rate models 1 and 2 have their own instances of the event kernels: out
+// of line in one instance for all it cost 60 bytes of spills and 15 % of the
+// kernel (450 -> 517 us at 4.1 M cells).
+__device__ __forceinline__ float sr_sample_x(const StepArgs& A, int cell, int ch, float u) {
+  const float t = u * 32.f;
+  const int j = min((int)t, 31);
+  const float f = t - (float)j;
+  const int o = 96 + ch * kSrKnots + j;
+  float x0, x1;
+  if (cell_has_sr(A, cell)) {
+    float rec[kRecLen];
+    load_rec(A, cell, rec);
+    const CellSpectrum sr = cell_spectrum(A, rec);
+    x0 = j == 0 ? 0.05f : sr.at(o - 1);
+    x1 = j == 31 ? 20.0f : sr.at(o);
+  } else {
+    x0 = j == 0 ? 0.05f : A.ra.uni[o - 1];
+    x1 = j == 31 ? 20.0f : A.ra.uni[o];
+  }
+  return fmaf(f, x1 - x0, x0);
+}
+
 // The events of a flagged electron (thermal-bath emission), new axions i0
 // on: event k takes cos theta, phi, energy and channel from one Philox
 // block. A massive axion's event is kept when the channel uniform, rescaled
 // inside its channel's interval, is below beta(E) (thinning; every event is
 // kept when massless). Returns the kept events; WRITE = false only counts
 // them (the warp path's offsets need the counts first).
-template <bool WRITE>
+template <bool WRITE, bool SR>
 __device__ __forceinline__ int electron_events(const StepArgs& A, uint32_t step, int cell, const ElItem& t,
                                                long abase, const AxDest& D, int i0, float r_cc, float r_cb,
                                                float r_T, float wu, const Cnt& cnt, Lane64& x64) {
@@ -1543,18 +1580,13 @@ __device__ __forceinline__ int electron_events(const StepArgs& A, uint32_t step,
   const uint32_t gcell = A.cell_base + (uint32_t)cell;
   // the energies: the exact inverse CDFs (closed forms), the cell's spectral
   // record, or the network's cell-independent quantiles
-  const float* q = nullptr;
-  if (A.rate_model) {
-    q = cell_sr(A, cell);
-    if (!q) q = A.ra.uni;
-  }
   int kept = 0;
   for (int k = 0; k < K; ++k) {
     const uint4 r = philox4x32_10(make_uint4(step, gcell, (uint32_t)t.slot, (S_EV_E << 24) | (uint32_t)k), A.rk);
     const float uc = u23(r.w);
     const bool isC = uc < fracC;
-    const float E = (q ? sr_sample_x(q, isC ? 1 : 2, u23(r.z))
-                       : icdf_lookup(A.tables + (isC ? TAB_COMPTON : TAB_BREMS) * kTableN, u23(r.z))) *
+    const float E = (SR ? sr_sample_x(A, cell, isC ? 1 : 2, u23(r.z))
+                        : icdf_lookup(A.tables + (isC ? TAB_COMPTON : TAB_BREMS) * kTableN, u23(r.z))) *
                     r_T;
     float pm = E * kInvMeC2f;
     if (A.mu > 0.f) {
@@ -1653,6 +1685,7 @@ __device__ __noinline__ void absorb_warp(const StepArgs& A, int cell, unsigned c
 // Emit phase of one cell by the warp: gamma->a, the thermal-bath events (new
 // axions placed by D), then the photon tail fill (a->gamma products
 // included).
+template <bool SR>
 __device__ __noinline__ void emit_warp(const StepArgs& A, uint32_t step, int cell, unsigned char* sb,
                                        const uint32_t* rowG, uint32_t* clrG, const uint32_t* rowE, uint32_t* clrE,
                                        const Cnt cnt, AxDest D, int ng_tot, int ng0, int ne, float wu, float r_cc,
@@ -1689,10 +1722,10 @@ __device__ __noinline__ void emit_warp(const StepArgs& A, uint32_t step, int cel
     const ElItem t = el_load(A, ebase, i0 + lane < nflE ? (int)S.flE[i0 + lane] : -1, wu);
     int K = t.slot >= 0 ? (int)(t.f & 0xFF) : 0;
     if (A.mu > 0.f && K > 0)  // massive axions: the kept events, before the offsets
-      K = electron_events<false>(A, step, cell, t, abase, D, 0, r_cc, r_cb, r_T, wu, cnt, x64);
+      K = electron_events<false, SR>(A, step, cell, t, abase, D, 0, r_cc, r_cb, r_T, wu, cnt, x64);
     int tot;
     const int off = run + warp_excl_scan(K, &tot);
-    if (t.slot >= 0) electron_events<true>(A, step, cell, t, abase, D, off, r_cc, r_cb, r_T, wu, cnt, x64);
+    if (t.slot >= 0) electron_events<true, SR>(A, step, cell, t, abase, D, off, r_cc, r_cb, r_T, wu, cnt, x64);
     run += tot;
   }
   reduce_out(x64, out);
@@ -1835,6 +1868,7 @@ struct LaneCell {
   float wu, r_cc, r_cb, r_T;
 };
 
+template <bool SR>
 __device__ __forceinline__ void cell_lane(const StepArgs& A, uint32_t step, int cell, bool doA, uint16_t* lA,
                                           uint16_t* lG, const uint16_t* lE, LaneCell& L, const Cnt& cnt, Lane64& xa,
                                           Lane64& xe) {
@@ -1894,7 +1928,7 @@ __device__ __forceinline__ void cell_lane(const StepArgs& A, uint32_t step, int 
   }
   for (int i = 0; i < nE; ++i) {
     const ElItem t = el_load(A, ebase, lE[32 * i], L.wu);
-    NP += electron_events<true>(A, step, cell, t, abase, D, NP, L.r_cc, L.r_cb, L.r_T, L.wu, cnt, xe);
+    NP += electron_events<true, SR>(A, step, cell, t, abase, D, NP, L.r_cc, L.r_cb, L.r_T, L.wu, cnt, xe);
   }
   const int na = min(D.base - D.nholes + NP, A.a.cap);
   if (NP < nrmA) {
@@ -2021,7 +2055,7 @@ __device__ __forceinline__ void absorb_lane(const StepArgs& A, int cell, uint32_
 // cell's absorb phase ends before its emit phase starts. The absorb and emit
 // exchanges are added to the cell's buffer in that order, whichever way the
 // step was called.
-template <int PH>
+template <int PH, bool SR>
 __global__ void __launch_bounds__(128, PH == 3 ? AXPIC_EVENT_FULL_MIN_CTAS : AXPIC_EVENT_MIN_CTAS)
     event_kernel(StepArgs A) {
   wait_predecessor();
@@ -2139,7 +2173,7 @@ __global__ void __launch_bounds__(128, PH == 3 ? AXPIC_EVENT_FULL_MIN_CTAS : AXP
     // by event_heavy_kernel after this kernel (a warp per cell); either way
     // the new axions reuse the freed slots
     if (valid && !defer && (L.nflA | L.nflG | L.nflE))
-      cell_lane(A, step, cell, true, lA, lG, lE, L, cnt, xa, xe);
+      cell_lane<SR>(A, step, cell, true, lA, lG, lE, L, cnt, xa, xe);
     // the heavy cells are listed for event_heavy_kernel, from index cell0
     const unsigned hm = __ballot_sync(kFull, defer);
     if (hm) {
@@ -2169,7 +2203,7 @@ __global__ void __launch_bounds__(128, PH == 3 ? AXPIC_EVENT_FULL_MIN_CTAS : AXP
       }
     }
   } else {
-    if (valid && !hE && (L.nflG | L.nflE)) cell_lane(A, step, cell, false, lA, lG, lE, L, cnt, xa, xe);
+    if (valid && !hE && (L.nflG | L.nflE)) cell_lane<SR>(A, step, cell, false, lA, lG, lE, L, cnt, xa, xe);
     __syncwarp();
     for (unsigned hm = __ballot_sync(kFull, valid && hE); hm; hm &= hm - 1u) {
       const int j = __ffs(hm) - 1;
@@ -2177,7 +2211,7 @@ __global__ void __launch_bounds__(128, PH == 3 ? AXPIC_EVENT_FULL_MIN_CTAS : AXP
       PhaseOut o;
       const uint32_t* gG = emitG ? (staged ? S.rowG + j * S.sG : A.bitsG + (size_t)c * A.Wg) : nullptr;
       const uint32_t* gE = emitE ? (staged ? S.rowE + j * S.sE : A.bitsE + (size_t)c * A.We) : nullptr;
-      emit_warp(A, step, c, sbase, gG, (emitG && !staged) ? A.bitsG + (size_t)c * A.Wg : nullptr, gE,
+      emit_warp<SR>(A, step, c, sbase, gG, (emitG && !staged) ? A.bitsG + (size_t)c * A.Wg : nullptr, gE,
                 (emitE && !staged) ? A.bitsE + (size_t)c * A.We : nullptr, cnt,
                 AxDest{nullptr, 0, 1, __shfl_sync(kFull, L.na, j)}, __shfl_sync(kFull, L.ng, j),
                 __shfl_sync(kFull, L.ng0, j), __shfl_sync(kFull, ne, j), __shfl_sync(kFull, L.wu, j),
@@ -2239,6 +2273,7 @@ __global__ void __launch_bounds__(128, PH == 3 ? AXPIC_EVENT_FULL_MIN_CTAS : AXP
 // event kernel gave it; the list order does not matter.
 constexpr int kHeavyGrid = 152;  // one CTA on each of the 152 SMs
 
+template <bool SR>
 __global__ void __launch_bounds__(128) event_heavy_kernel(StepArgs A) {
   wait_predecessor();
   extern __shared__ __align__(16) unsigned char smem[];
@@ -2273,7 +2308,7 @@ __global__ void __launch_bounds__(128) event_heavy_kernel(StepArgs A) {
     PhaseOut oa, oe;
     absorb_warp(A, c, sbase, rowA, rowA, cnt, na0, ng0, false, &oa);
     const int nrmA = na0 - oa.na;
-    emit_warp(A, step, c, sbase, rowG, rowG, rowE, rowE, cnt, AxDest{S.rmA, nrmA, 1, na0}, oa.ng, ng0, ne, wu, r_cc,
+    emit_warp<SR>(A, step, c, sbase, rowG, rowG, rowE, rowE, cnt, AxDest{S.rmA, nrmA, 1, na0}, oa.ng, ng0, ne, wu, r_cc,
               r_cb, r_T, &oe);
     // freed slots left over: closed from the tail
     if (oe.np < nrmA) compact_tail(A.a, (long)c * A.a.cap, S.rmA + oe.np, S.rbA, oe.na, na0);
@@ -2338,12 +2373,14 @@ static cudaError_t launch_events(const StepArgs& A, int warps, cudaStream_t st, 
   const size_t lists = ev_scratch_bytes(A.a.cap, A.g.cap, A.e.cap, true);
   const size_t per = ev_scratch_bytes(A.a.cap, A.g.cap, A.e.cap, !full);
   const int grid = (A.ncells + 32 * warps - 1) / (32 * warps);
-  const cudaError_t e = launch_chained(chained, event_kernel<PH>, grid, warps * 32, per * warps, st, A);
+  const bool sr = A.rate_model != 0;
+  const cudaError_t e = launch_chained(chained, sr ? event_kernel<PH, true> : event_kernel<PH, false>, grid, warps * 32,
+                                       per * warps, st, A);
   if (e || !full) return e;
   // persistent over the heavy list: a warp per cell, at most one warp per
   // cell of the launch and kHeavyGrid CTAs
   const int hgrid = max(1, min((A.ncells + warps - 1) / warps, kHeavyGrid));
-  return launch_chained(chained, event_heavy_kernel, hgrid, warps * 32, lists * warps, st, A);
+  return launch_chained(chained, sr ? event_heavy_kernel<true> : event_heavy_kernel<false>, hgrid, warps * 32, lists * warps, st, A);
 }
 
 // Cells per chunk of a decision warp: asked for, or by the launch. A chunk
@@ -2416,7 +2453,6 @@ static cudaError_t launch_feedback(const StepArgs& A, cudaStream_t st, bool chai
 }
 
 const char* step_kernel_names(int rate_model, int T_mode) {
-  if (T_mode == 2 && rate_model == 1) return "decide_kernel,event_kernel,feedback_kernel,sr_table_kernel";
   if (T_mode == 2 && rate_model == 2) return "decide_kernel,event_kernel,feedback_kernel,sr_cells_kernel";
   return "decide_kernel,event_kernel,feedback_kernel";
 }
@@ -2441,12 +2477,12 @@ cudaError_t decide_resident_ctas(int* out) {
   return cudaSuccess;
 }
 
-// After the temperature update of an evolved-T step the rate model's records
-// follow the new T: the table model's spectral records, or the surrogate
-// network's prefactors (the table's records where it is not trusted).
+// After the temperature update of an evolved-T step the surrogate network's
+// prefactors follow the new T (the table's entries are interpolated where
+// they are needed).
 static cudaError_t launch_records_update(const StepArgs& A, const SrArgs* sra, cudaStream_t st, bool chained) {
-  if (!sra || A.T_mode != 2) return cudaSuccess;
-  return launch_sr_records(A.rate_model, *sra, st, chained);
+  if (!sra || A.T_mode != 2 || A.rate_model != 2) return cudaSuccess;
+  return launch_sr_cells(*sra, st, chained);
 }
 
 cudaError_t launch_step(int phases, const StepArgs& A, int warps, cudaStream_t st, cudaEvent_t* ev,
@@ -2498,11 +2534,12 @@ cudaError_t set_step_smem_limits(size_t bytes) {
   size_t* cur = dev >= 0 && dev < 64 ? &set_for[dev] : nullptr;
   if (cur && bytes <= *cur) return cudaSuccess;
   const int b = (int)bytes;
-  if ((e = cudaFuncSetAttribute(event_kernel<PH_ABSORB>, cudaFuncAttributeMaxDynamicSharedMemorySize, b)) ||
-      (e = cudaFuncSetAttribute(event_kernel<PH_EMIT>, cudaFuncAttributeMaxDynamicSharedMemorySize, b)) ||
-      (e = cudaFuncSetAttribute(event_kernel<PH_ABSORB | PH_EMIT>, cudaFuncAttributeMaxDynamicSharedMemorySize, b)) ||
-      (e = cudaFuncSetAttribute(event_heavy_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, b)))
-    return e;
+  for (const void* k :
+       {(const void*)event_kernel<PH_ABSORB, false>, (const void*)event_kernel<PH_EMIT, false>,
+        (const void*)event_kernel<PH_ABSORB | PH_EMIT, false>, (const void*)event_heavy_kernel<false>,
+        (const void*)event_kernel<PH_ABSORB, true>, (const void*)event_kernel<PH_EMIT, true>,
+        (const void*)event_kernel<PH_ABSORB | PH_EMIT, true>, (const void*)event_heavy_kernel<true>})
+    if ((e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, b))) return e;
   if (cur) *cur = bytes;
   return cudaSuccess;
 }

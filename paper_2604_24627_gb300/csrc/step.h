@@ -9,8 +9,8 @@ enum { PH_ABSORB = 1, PH_EMIT = 2, PH_FEEDBACK = 4, PH_ALL = 7 };
 
 size_t step_smem_per_warp(int acap, int gcap, int ecap);
 // ev: NULL, or kStepKernels + 1 events recorded around the kernels of a
-// PH_ALL step: decisions, events, feedback, and the rate model's record
-// kernel (an empty interval when there is none). sra: the record kernels'
+// PH_ALL step: decisions, events, feedback, and the surrogate's network
+// kernel (an empty interval when there is none). sra: that kernel's
 // arguments (rate models 1 and 2), else NULL.
 // after_step: the last operation queued on st is a kernel of another step (the
 // first kernel then overlaps its end too).
