@@ -298,8 +298,8 @@ axpic_status axpic_stream_axions(axpic_ctx *ctx, int32_t nx, int32_t ny, int32_t
  * every step rounded, the sums compensated (Kahan) in slot order;
  * the new axions take the group's first two slots at the weighted mean
  * position, the other slots are freed and closed by the tail fill. One pass;
- * a cell may stay above n_target. Asynchronous; the first call allocates 1
- * byte per axion slot. AXPIC_E_INVALID (nothing launched) for n_target < 0,
+ * a cell may stay above n_target. Asynchronous; the first call allocates 8
+ * bytes. AXPIC_E_INVALID (nothing launched) for n_target < 0,
  * more than 30 thresholds, or thresholds not finite, >= 0 and ascending. */
 axpic_status axpic_merge_axions(axpic_ctx *ctx, int32_t n_target, int32_t nedges, const float *edges_p2);
 /* Axions removed by every merge so far (host, 1 double). Synchronises. */

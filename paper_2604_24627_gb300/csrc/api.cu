@@ -120,7 +120,6 @@ struct axpic_ctx {
   float* st_buf = nullptr;    // [ncells * axion capacity * 8]
   double* st_stats = nullptr; // [4]
   // axion merging scratch, made by the first axpic_merge_axions call
-  uint8_t* mg_grp = nullptr;  // [ncells * axion capacity]
   double* mg_removed = nullptr;
   int sr_nkt = 0, sr_nne = 0, tnT = 0, tnne = 0, sur_set = 0, sur_any_trusted = 0;
   float ln_gP = 0.f, ln_gA = 0.f, lnK_CC = 0.f, lnK_CB = 0.f;
@@ -406,7 +405,7 @@ static void free_ctx(axpic_ctx* ctx) {
                   ctx->tables, ctx->tally, ctx->counters, ctx->err, ctx->scratch, ctx->bits,
                   ctx->recA,   ctx->recG,  ctx->recE,     ctx->step_dev, ctx->sr, ctx->srtab,
                   ctx->sur_P,  ctx->sur_mu, ctx->sur_sigma, ctx->sur_trust, ctx->sur_img, ctx->sur_skip,
-                  ctx->sr_src, ctx->sur_uni, ctx->st_freed, ctx->st_off, ctx->st_buf, ctx->st_stats, ctx->mg_grp,
+                  ctx->sr_src, ctx->sur_uni, ctx->st_freed, ctx->st_off, ctx->st_buf, ctx->st_stats,
                   ctx->mg_removed, ctx->heavy, ctx->heavy_n};
   for (void* b : bufs)
     if (b) cudaFree(b);
@@ -1360,9 +1359,8 @@ axpic_status axpic_merge_axions(axpic_ctx* ctx, int32_t n_target, int32_t nedges
     if (!std::isfinite(edges_p2[k]) || edges_p2[k] < 0.f || (k > 0 && !(edges_p2[k] > edges_p2[k - 1])))
       return fail(ctx, AXPIC_E_INVALID, "axpic_merge_axions: thresholds must be finite, >= 0 and ascending");
   const axpic_plasma_desc& d = ctx->desc;
-  if (!ctx->mg_grp) {
+  if (!ctx->mg_removed) {
     CK(merge_init_kernels(), "merge kernel attributes");
-    CK(cudaMalloc((void**)&ctx->mg_grp, std::max<size_t>((size_t)d.ncells * d.axions.capacity, 1)), "merge scratch");
     CK(cudaMalloc((void**)&ctx->mg_removed, sizeof(double)), "merge scratch");
     CK(cudaMemsetAsync(ctx->mg_removed, 0, sizeof(double), ctx->stream), "memset");
   }
@@ -1373,7 +1371,6 @@ axpic_status axpic_merge_axions(axpic_ctx* ctx, int32_t n_target, int32_t nedges
   a.n_target = n_target;
   a.nedges = nedges;
   for (int k = 0; k < nedges; ++k) a.edges[k] = edges_p2[k];
-  a.grp = ctx->mg_grp;
   a.removed = ctx->mg_removed;
   CK(launch_merge(a, ctx->stream), "merge kernel");
   return AXPIC_OK;

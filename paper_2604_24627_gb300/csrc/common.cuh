@@ -221,6 +221,18 @@ __device__ __forceinline__ float sum_sq(float x, float y, float z) {
   return __fmaf_rn(z, z, __fmaf_rn(x, x, __fmul_rn(y, y)));
 }
 
+// ---------------------------------------------------------------- bits
+// Position of the k-th (0-based) set bit of a word that has more than k.
+__device__ __forceinline__ int nth_bit(uint32_t v, int k) {
+  int p = 0;
+#pragma unroll
+  for (int s = 16; s; s >>= 1) {
+    const int c = __popc((v >> p) & ((1u << s) - 1u));
+    if (k >= c) k -= c, p += s;
+  }
+  return p;
+}
+
 // ---------------------------------------------------------------- sums
 // An unevaluated sum of three binary32 numbers, for sums that FP64 (1/64 of
 // the FP32 rate) would bound: TwoSum is exact, so each term loses the rounding

@@ -5,17 +5,26 @@
 // (2015), for massless particles; the method merges axions as a species of
 // the PIC code, Sec. II.A, and names no algorithm).
 //
-// A warp per cell:
-// * each slot's group (comparisons of binary32 |p|^2 with the thresholds,
-//   and the sign bits) and the group sizes;
+// A warp per cell, persistent over the cells:
+// * each slot's group (a 5-step search of its binary32 |p|^2 among the
+//   thresholds, and the sign bits), its rank in the group in slot order and
+//   the group sizes, from one match per 32 slots;
 // * the groups of three or more in a list, and their members' slots in
-//   shared memory, grouped and in slot order (a stable counting sort);
+//   shared memory, grouped and in slot order;
 // * a lane per listed group forms the binary32 compensated sums over its
 //   members in slot order, every rounding explicit (the results match the
 //   oracle bit for bit), writes the two new axions into the group's first
-//   two slots and frees the others;
+//   two slots and marks the others freed, a bit a slot;
 // * the tail fill closes the freed slots.
+// Bound by instruction issue (the lanes' sums are a third of it) and latency,
+// not by its bytes (a cell's axions read once, the merged ones written). With
+// 16 comparisons a slot, a byte a slot in memory, a second match pass and a
+// tail fill that scanned every slot with __fns it issued 2537 warp
+// instructions a cell of 128 axions and took 245 us for 65,536 of them, a fifth
+// of its stalls instruction fetches; now 1951 and 162 us (8 CTAs of 4 warps an
+// SM at 64 registers; 10 at 48 spill and take 168 us, 12 196).
 #include "merge.h"
+#include "step.h"
 
 #include <algorithm>
 
@@ -23,7 +32,8 @@ namespace axpic {
 
 namespace {
 
-constexpr int kWarpsMax = 2;  // small blocks: a cell that finishes early frees its slot
+constexpr int kWarpsMax = 4;
+constexpr int kHold = 5;  // passes of 32 slots whose groups stay in registers
 constexpr unsigned kAll = 0xFFFFFFFFu;
 constexpr int kGroupsMax = (kMergeMaxEdges + 1) * 8;
 
@@ -45,16 +55,18 @@ struct Kahan {
 // The two axions replacing the group whose m member slots, ascending, are
 // mem[0..m) of the cell at base: binary32 compensated sums in slot order,
 // then p_a and p_b on either side of P at cos theta = |P| / E. Members after
-// the first two are freed.
-__device__ void merge_group(const MergeArgs& a, long base, const uint16_t* mem, int m) {
-  const SpeciesPtrs& s = a.s;
+// the first two are freed (their bits set).
+__device__ __forceinline__ void merge_group(const SpeciesPtrs& s, long base, const uint16_t* mem, int m,
+                                            uint32_t* freed) {
   Kahan W, Px, Py, Pz, E, X, Y, Z;
   // member k + 1's fields are loaded before member k's sums (m >= 3)
-  long q = base + mem[0];
+  int slot = mem[0];
+  long q = base + slot;
   float4 r = s.wp[q], u = s.xyz[q];
   float w = r.x, px = r.y, py = r.z, pz = r.w, x = u.x, y = u.y, z = u.z;
   for (int k = 0; k < m; ++k) {
-    const long qn = base + mem[min(k + 1, m - 1)];
+    const int next = mem[min(k + 1, m - 1)];
+    const long qn = base + next;
     r = s.wp[qn];
     u = s.xyz[qn];
     const float wn = r.x, pxn = r.y, pyn = r.z, pzn = r.w, xn = u.x, yn = u.y, zn = u.z;
@@ -66,8 +78,8 @@ __device__ void merge_group(const MergeArgs& a, long base, const uint16_t* mem, 
     X.add(__fmul_rn(w, x));
     Y.add(__fmul_rn(w, y));
     Z.add(__fmul_rn(w, z));
-    if (k >= 2) a.grp[q] = kMergeFreed;
-    q = qn, w = wn, px = pxn, py = pyn, pz = pzn, x = xn, y = yn, z = zn;
+    if (k >= 2) atomicOr(&freed[slot >> 5], 1u << (slot & 31));
+    slot = next, w = wn, px = pxn, py = pyn, pz = pzn, x = xn, y = yn, z = zn;
   }
   const int sa = mem[0], sb = mem[1];
   const float pm = __fdiv_rn(E.s, W.s);
@@ -114,48 +126,95 @@ __device__ __forceinline__ void prefetch_l1(const void* p) {
   asm volatile("prefetch.global.L1 [%0];" ::"l"(p));
 }
 
-// Dynamic shared memory: cap slot indices (u16) per warp.
-__global__ void __launch_bounds__(kWarpsMax * 32, 20) merge_kernel(MergeArgs a) {
-  extern __shared__ uint16_t smem_members[];
-  __shared__ int gcnt[kWarpsMax][kGroupsMax];  // group sizes
-  __shared__ int gpos[kWarpsMax][kGroupsMax];  // next member position of a listed group
-  __shared__ uint8_t glist[kWarpsMax][kGroupsMax];
+struct MergeShared {
+  uint16_t cnt[kGroupsMax];   // group sizes
+  uint16_t start[kGroupsMax]; // first member position of a listed group
+  uint16_t run[kGroupsMax];   // members placed so far (slots beyond the registers)
+  uint8_t list[kGroupsMax];
+};
+
+// Dynamic shared memory, per warp: cap slot indices (u16), then a bit a slot.
+__host__ __device__ inline size_t warp_bytes(int cap) {
+  return ((size_t)cap * sizeof(uint16_t) + 3) / 4 * 4 + (size_t)((cap + 31) / 32) * sizeof(uint32_t);
+}
+
+__global__ void __launch_bounds__(kWarpsMax * 32, 8) merge_kernel(MergeArgs a) {
+  extern __shared__ __align__(16) unsigned char smem_warps[];
+  __shared__ MergeShared sh[kWarpsMax];
+  __shared__ float edges[32];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
   const SpeciesPtrs& s = a.s;
-  uint16_t* mem = smem_members + (size_t)wid * s.cap;
+  MergeShared& S = sh[wid];
+  uint16_t* const mem = reinterpret_cast<uint16_t*>(smem_warps + wid * warp_bytes(s.cap));
+  uint32_t* const freed = reinterpret_cast<uint32_t*>(smem_warps + (wid + 1) * warp_bytes(s.cap)) - (s.cap + 31) / 32;
   const int ngroups = (a.nedges + 1) * 8;
   const unsigned lt = (1u << lane) - 1u;
+  // the thresholds, then values that no |p|^2 reaches (comparisons with NaN fail)
+  if (threadIdx.x < 32) edges[threadIdx.x] = threadIdx.x < a.nedges ? a.edges[threadIdx.x] : __int_as_float(0x7FC00000);
+  __syncthreads();
+  // the number of thresholds at or below |p|^2, times 8, plus the octant of p
+  auto group_of = [&](const float4& r) {
+    const float px = r.y, py = r.z, pz = r.w;
+    const float p2 = __fadd_rn(__fadd_rn(__fmul_rn(px, px), __fmul_rn(py, py)), __fmul_rn(pz, pz));
+    int e = 0;
+#pragma unroll
+    for (int st = 16; st; st >>= 1)
+      if (edges[e + st - 1] <= p2) e += st;
+    return e * 8 + (px < 0.f ? 1 : 0) + (py < 0.f ? 2 : 0) + (pz < 0.f ? 4 : 0);
+  };
+  int total = 0;
   for (int c = blockIdx.x * nw + wid; c < a.ncells; c += gridDim.x * nw) {
     const int n = min(max(s.count[c], 0), s.cap);
     if (n <= a.n_target) continue;
     const long base = (long)c * s.cap;
-    for (int g = lane; g < ngroups; g += 32) gcnt[wid][g] = 0;
-    __syncwarp();
-    // each slot's group: the number of thresholds at or below |p|^2, times
-    // 8, plus the octant of p; the other fields' lines go to L1 meanwhile
-    for (int s0 = 0; s0 < n; s0 += 32) {
-      const int slot = s0 + lane;
+    for (int g = lane; g < ngroups; g += 32) S.cnt[g] = 0;
+    for (int w = lane; 32 * w < n; w += 32) freed[w] = 0u;
+    float4 r[kHold];
+#pragma unroll
+    for (int i = 0; i < kHold; ++i) {
+      const int slot = 32 * i + lane;
       if (slot < n) {
-        const long q = base + slot;
-        prefetch_l1(s.xyz + q);
-        const float4 r = s.wp[q];
-        const float px = r.y, py = r.z, pz = r.w;
-        const float p2 = __fadd_rn(__fadd_rn(__fmul_rn(px, px), __fmul_rn(py, py)), __fmul_rn(pz, pz));
-        int e = 0;
-        for (int k = 0; k < a.nedges; ++k) e += p2 >= a.edges[k] ? 1 : 0;
-        const int g = e * 8 + (px < 0.f ? 1 : 0) + (py < 0.f ? 2 : 0) + (pz < 0.f ? 4 : 0);
-        a.grp[q] = (uint8_t)g;
-        atomicAdd(&gcnt[wid][g], 1);
+        r[i] = s.wp[base + slot];
+        prefetch_l1(s.xyz + base + slot);  // read by the slot's group
       }
     }
     __syncwarp();
+    int gr[kHold];  // group | rank << 8, or -1
+#pragma unroll
+    for (int i = 0; i < kHold; ++i) {
+      gr[i] = -1;
+      if (32 * i >= n) continue;
+      const bool live = 32 * i + lane < n;
+      const int g = live ? group_of(r[i]) : kGroupsMax + lane;
+      const unsigned peers = __match_any_sync(kAll, g);
+      const int rank = (live ? S.cnt[g] : 0) + __popc(peers & lt);
+      __syncwarp();
+      if (live) {
+        if ((peers & lt) == 0) S.cnt[g] = (uint16_t)(rank + __popc(peers));
+        gr[i] = g | rank << 8;
+      }
+      __syncwarp();
+    }
+    if (n > 32 * kHold) {
+      for (int g = lane; g < ngroups; g += 32) S.run[g] = S.cnt[g];
+      __syncwarp();
+      for (int s0 = 32 * kHold; s0 < n; s0 += 32) {
+        const bool live = s0 + lane < n;
+        const int g = live ? group_of(s.wp[base + s0 + lane]) : kGroupsMax + lane;
+        const unsigned peers = __match_any_sync(kAll, g);
+        if (live && (peers & lt) == 0) S.cnt[g] += (uint16_t)__popc(peers);
+        __syncwarp();
+      }
+    }
     // the groups of three or more: a list, and each one's first member
     // position (exclusive prefix of their sizes)
     int nm = 0, run = 0;
     for (int g0 = 0; g0 < ngroups; g0 += 32) {
       const int g = g0 + lane;
-      const int m = g < ngroups ? gcnt[wid][g] : 0;
+      const int m = g < ngroups ? S.cnt[g] : 0;
       const bool listed = m >= 3;
+      const unsigned bm = __ballot_sync(kAll, listed);
+      if (bm == 0) continue;
       const int v = listed ? m : 0;
       int incl = v;
 #pragma unroll
@@ -163,79 +222,75 @@ __global__ void __launch_bounds__(kWarpsMax * 32, 20) merge_kernel(MergeArgs a) 
         const int t = __shfl_up_sync(kAll, incl, d);
         if (lane >= d) incl += t;
       }
-      const unsigned bm = __ballot_sync(kAll, listed);
       if (listed) {
-        gpos[wid][g] = run + incl - v;
-        glist[wid][nm + __popc(bm & lt)] = (uint8_t)g;
+        S.start[g] = (uint16_t)(run + incl - v);
+        S.list[nm + __popc(bm & lt)] = (uint8_t)g;
       }
       nm += __popc(bm);
       run += __shfl_sync(kAll, incl, 31);
     }
     if (nm == 0) continue;
     __syncwarp();
-    // members of listed groups in slot order: rank among the chunk's lanes
-    // of the same group, after the group's members of earlier chunks
-    for (int s0 = 0; s0 < n; s0 += 32) {
-      const int slot = s0 + lane;
-      const int g = slot < n ? a.grp[base + slot] : 0;
-      const bool take = slot < n && gcnt[wid][g] >= 3;
-      const unsigned peers = __match_any_sync(kAll, take ? g : kGroupsMax + lane);
-      const int rank = __popc(peers & lt);
-      const int p0 = take ? gpos[wid][g] : 0;
+    // members of listed groups in slot order
+#pragma unroll
+    for (int i = 0; i < kHold; ++i) {
+      if (gr[i] < 0) continue;
+      const int g = gr[i] & 255;
+      if (S.cnt[g] >= 3) mem[S.start[g] + (gr[i] >> 8)] = (uint16_t)(32 * i + lane);
+    }
+    for (int s0 = 32 * kHold; s0 < n; s0 += 32) {
+      const bool live = s0 + lane < n;
+      const int g = live ? group_of(s.wp[base + s0 + lane]) : kGroupsMax + lane;
+      const unsigned peers = __match_any_sync(kAll, g);
+      const int rank = (live ? S.run[g] : 0) + __popc(peers & lt);
       __syncwarp();
-      if (take) {
-        mem[p0 + rank] = (uint16_t)slot;
-        if (rank == 0) gpos[wid][g] = p0 + __popc(peers);
+      if (live) {
+        if ((peers & lt) == 0) S.run[g] = (uint16_t)(rank + __popc(peers));
+        if (S.cnt[g] >= 3) mem[S.start[g] + rank] = (uint16_t)(s0 + lane);
       }
       __syncwarp();
     }
+    __syncwarp();
     // a lane per listed group
     int removed = 0;
     for (int t = lane; t < nm; t += 32) {
-      const int g = glist[wid][t];
-      const int m = gcnt[wid][g];
-      merge_group(a, base, mem + (gpos[wid][g] - m), m);
+      const int g = S.list[t], m = S.cnt[g];
+      merge_group(s, base, mem + S.start[g], m, freed);
       removed += m - 2;
     }
-    __syncwarp();
-#pragma unroll
-    for (int d = 16; d; d >>= 1) removed += __shfl_xor_sync(kAll, removed, d);
+    removed = __reduce_add_sync(kAll, removed);
+    __syncwarp();  // the lanes' bits and new axions are visible
     // the tail fill: the freed slots below the new count ns take, in
     // ascending order, the kept slots at or beyond it, in ascending order
     const int ns = n - removed;
-    for (int j0 = 0;; j0 += 32) {
-      const int j = j0 + lane;
-      int from = -1, to = -1, runTo = 0, runFrom = 0;
-      for (int s0 = 0; s0 < n; s0 += 32) {
-        const int slot = s0 + lane;
-        const bool freed = slot < n && a.grp[base + slot] == kMergeFreed;
-        const unsigned tm = __ballot_sync(kAll, freed && slot < ns);
-        const unsigned fm = __ballot_sync(kAll, slot < n && slot >= ns && !freed);
-        int k = j - runTo;
-        if (k >= 0 && k < __popc(tm)) to = s0 + (int)__fns(tm, 0, k + 1);
-        k = j - runFrom;
-        if (k >= 0 && k < __popc(fm)) from = s0 + (int)__fns(fm, 0, k + 1);
-        runTo += __popc(tm);
-        runFrom += __popc(fm);
-      }
-      if (j < runTo && from >= 0 && to >= 0) {
-        const long qf = base + from, qt = base + to;
-        const float4 r = s.wp[qf], u = s.xyz[qf];
-        s.wp[qt] = r;
+    int moved = 0;
+    for (int w = ns >> 5; 32 * w < n; ++w) {
+      const int slot = 32 * w + lane;
+      const bool mv = slot >= ns && slot < n && !((freed[w] >> lane) & 1u);
+      const unsigned mm = __ballot_sync(kAll, mv);
+      if (mv) {
+        int j = moved + __popc(mm & lt), d = 0;  // it takes freed slot j of all
+        for (int p = __popc(freed[0]); j >= p; p = __popc(freed[d])) {
+          j -= p;
+          ++d;
+        }
+        const long qf = base + slot, qt = base + 32 * d + nth_bit(freed[d], j);
+        const float4 x = s.wp[qf], u = s.xyz[qf];
+        s.wp[qt] = x;
         s.xyz[qt] = u;
       }
-      if (j0 + 32 >= runTo) break;
+      moved += __popc(mm);
     }
-    if (lane == 0) {
-      s.count[c] = ns;
-      atomicAdd(a.removed, (double)removed);
-    }
+    if (lane == 0) s.count[c] = ns;
+    total += removed;
+    __syncwarp();
   }
+  if (lane == 0 && total) atomicAdd(a.removed, (double)total);
 }
 
 }  // namespace
 
-constexpr int kDynMax = 160 * 1024;  // the members' dynamic shared memory, at most
+constexpr int kDynMax = 160 * 1024;  // the warps' dynamic shared memory, at most
 
 cudaError_t merge_init_kernels() {
   return cudaFuncSetAttribute(merge_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kDynMax);
@@ -244,10 +299,13 @@ cudaError_t merge_init_kernels() {
 cudaError_t launch_merge(const MergeArgs& a, cudaStream_t st) {
   if (a.ncells <= 0) return cudaSuccess;
   if (a.s.cap > kMergeMaxCap) return cudaErrorInvalidValue;
-  // warps per CTA: as many as fit the members' shared memory, at most 2
-  const size_t per_warp = (size_t)std::max(a.s.cap, 1) * sizeof(uint16_t);
+  // warps per CTA: as many as fit the shared memory, at most 4; as many CTAs
+  // as the device holds at once
+  const size_t per_warp = std::max<size_t>(warp_bytes(a.s.cap), 4);
   const int nw = (int)std::max<size_t>(1, std::min<size_t>(kWarpsMax, kDynMax / per_warp));
-  merge_kernel<<<(a.ncells + nw - 1) / nw, nw * 32, per_warp * nw, st>>>(a);
+  const int fit = resident_ctas((const void*)merge_kernel, nw * 32, per_warp * nw);
+  if (fit <= 0) return cudaErrorUnknown;
+  merge_kernel<<<std::min((a.ncells + nw - 1) / nw, fit), nw * 32, per_warp * nw, st>>>(a);
   return cudaGetLastError();
 }
 

@@ -297,17 +297,6 @@ __global__ void __launch_bounds__(kThreads, 3) stream_move_kernel(StreamArgs a) 
   }
 }
 
-// Position of the k-th (0-based) set bit of a word that has more than k.
-__device__ __forceinline__ int nth_bit(uint32_t v, int k) {
-  int p = 0;
-#pragma unroll
-  for (int s = 16; s; s >>= 1) {
-    const int c = __popc((v >> p) & ((1u << s) - 1u));
-    if (k >= c) k -= c, p += s;
-  }
-  return p;
-}
-
 // Cell coordinates, stepped to the next cell without dividing again.
 struct CellAt {
   int i, j, k;
