@@ -475,6 +475,7 @@ struct StepArgs {
   int dec_grid;   // CTAs of the persistent decision kernel
   int dec_chunk;  // cells per chunk of a decision warp: 4, 8, 16 or 32, or 0: by the launch (decide_chunk)
   int dec_cells;  // cells of all the launches that run side by side (the branches of a replayed step), or 0
+  int ev_cells;   // cells a warp of a full step's event kernel takes
   uint32_t* step_dev;  // NULL, or the device step counter of a replayed graph
   // cells a full step's event kernel leaves to the warp-path kernel, stored
   // from index cell0 on, and their count (one counter per branch of a

@@ -1242,9 +1242,13 @@ __global__ void __launch_bounds__(kFeedbackThreads, DENSE ? 4 : 5) feedback_kern
 //   so that lanes reading their own rows hit distinct banks).
 
 // Flagged slots per species up to which one lane takes a cell's phase
-// (electrons: kLightE, each event with its own Philox block).
-constexpr int kLight = 8;
-constexpr int kLightE = 4;
+// (electrons: kLightE, each event with its own Philox block). Cells beyond go
+// to a kernel of their own in a full step, whose chain of a few long cells
+// every step waits for: with 8 and 4 a handful of 65,536 dense cells went
+// there, with 16 and 8 hardly any (32 replayed steps: 6.60 -> 6.13 ms; 16,384
+// cells, 8 steps: 1.14 -> 0.91 ms). The lists take 3 KB a warp.
+constexpr int kLight = 16;
+constexpr int kLightE = 8;
 constexpr size_t kLaneListBytes = 3 * kLight * 32 * sizeof(uint16_t);
 
 struct EvScratch {
@@ -2064,8 +2068,10 @@ __global__ void __launch_bounds__(128, PH == 3 ? AXPIC_EVENT_FULL_MIN_CTAS : AXP
   const int wid = threadIdx.x >> 5;
   const int nw = blockDim.x >> 5;
   const int lane = threadIdx.x & 31;
-  const int cell = A.cell0 + (blockIdx.x * nw + wid) * 32 + lane;
-  const bool valid = cell < A.cell0 + A.ncells;
+  // a full step's launch may give a warp fewer cells than lanes
+  const int cells = PH == (PH_ABSORB | PH_EMIT) ? A.ev_cells : 32;
+  const int cell = A.cell0 + (blockIdx.x * nw + wid) * cells + lane;
+  const bool valid = lane < cells && cell < A.cell0 + A.ncells;
   if (lane < kNumCounters) warp_cnt[wid][lane] = 0ull;
   __syncwarp();
   const Cnt cnt{warp_cnt[wid]};
@@ -2367,15 +2373,33 @@ int resident_ctas(const void* fn, int threads, size_t dyn_smem, int max_per_sm) 
   return max(1, min(nb, max_per_sm)) * max(1, sms);
 }
 
+// Cells per warp of a full step's event kernel. A lane takes a cell, and a
+// warp as long as its lane with the most flagged slots: 32 cells a warp issue
+// the least, fewer end sooner and spread over more warps. By the cells that
+// run side by side; a pass, us, with 32, 16, 8 and 4 cells a warp:
+//   4,096 dense cells (512 e, 256 g), 8 steps:    646   587   553   529
+//   9,200 cells of 24 boxes, 16 steps:            1074  990   935   899
+//   16,384 dense cells, 8 steps:                  909   835   800   869
+//   46,000 cells of 120 boxes, 16 steps:          2050  1829  1693
+//   65,536 dense cells, 32 steps:                 6129  6146  6915
+//   64,000 thin cells (64 e, 32 g), 4 steps:      260   267   279
+//   884,736 thin cells, 4 steps:                  1747  1977  2392
+static int event_cells(const StepArgs& A) {
+  const int n = max(A.ncells, A.dec_cells);
+  return n < 12288 ? 4 : n < 49152 ? 8 : 32;
+}
+
 template <int PH>
 static cudaError_t launch_events(const StepArgs& A, int warps, cudaStream_t st, bool chained) {
   constexpr bool full = PH == (PH_ABSORB | PH_EMIT);
   const size_t lists = ev_scratch_bytes(A.a.cap, A.g.cap, A.e.cap, true);
   const size_t per = ev_scratch_bytes(A.a.cap, A.g.cap, A.e.cap, !full);
-  const int grid = (A.ncells + 32 * warps - 1) / (32 * warps);
+  StepArgs B = A;
+  B.ev_cells = full ? event_cells(A) : 32;
+  const int grid = (A.ncells + B.ev_cells * warps - 1) / (B.ev_cells * warps);
   const bool sr = A.rate_model != 0;
   const cudaError_t e = launch_chained(chained, sr ? event_kernel<PH, true> : event_kernel<PH, false>, grid, warps * 32,
-                                       per * warps, st, A);
+                                       per * warps, st, B);
   if (e || !full) return e;
   // persistent over the heavy list: a warp per cell, at most one warp per
   // cell of the launch and kHeavyGrid CTAs
