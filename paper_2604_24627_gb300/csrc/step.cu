@@ -540,6 +540,33 @@ __device__ __noinline__ RemapOut remap_cells(const StepArgs& A, unsigned need, i
 
 __device__ __forceinline__ bool nz64(double v) { return (__double_as_longlong(v) << 1) != 0; }
 
+// Conversions on the integer units: an FP64 instruction, a conversion
+// included, takes 16 cycles of an SM for a warp, these a few each. The same
+// bits as the plain conversion, which takes what is subnormal, infinite or
+// not a number in binary32.
+__device__ __forceinline__ float f32_of(double x) {
+  const uint32_t hi = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x);
+  const uint32_t m = hi & 0x7FFFFFFFu;
+  if (m - 0x38100000u < 0x47F00000u - 0x38100000u) {  // 2^-126 <= |x| < 2^128: rounded to nearest even
+    uint32_t u = __funnelshift_l(lo, m - 0x38000000u, 3);
+    u += (lo & 0x1FFFFFFFu) + (u & 1u) > 0x10000000u;
+    return __uint_as_float(u | (hi & 0x80000000u));
+  }
+  return (float)x;
+}
+__device__ __forceinline__ double f64_of(float x) {
+  const uint32_t u = __float_as_uint(x), m = u & 0x7FFFFFFFu;
+  if (m - 0x00800000u < 0x7F000000u)  // normal
+    return __hiloint2double((int)((u & 0x80000000u) | ((m >> 3) + 0x38000000u)), (int)(u << 29));
+  return m ? (double)x : __hiloint2double((int)u, 0);
+}
+// |x| from the upper half of its bits, at most 2^-20 below it; 0 below
+// 2^-126, infinite from 2^128 on and where x is not a number
+__device__ __forceinline__ float abs_below(double x) {
+  const int m = __double2hiint(x) & 0x7FFFFFFF;
+  return m < 0x38100000 ? 0.f : __int_as_float(m >= 0x47F00000 ? 0x7F800000 : (m - 0x38000000) << 3);
+}
+
 // ---------------------------------------------------------------- decision records
 // A flagged slot's full decision, written by the decision kernels and read by
 // the event kernel (slot-indexed arrays, touched only for flagged slots):
@@ -1022,13 +1049,15 @@ __device__ __forceinline__ void fb_load(const StepArgs& A, int cell, FbCell& f) 
   f.rPx = rs[1];
   f.rPy = rs[2];
   f.rPz = rs[3];
-  const float* mom = A.mom + (size_t)cell * kMomLen;
-  f.W = mom[M_W];
-  f.Px = mom[M_PX];
-  f.Py = mom[M_PY];
-  f.Pz = mom[M_PZ];
-  f.U2 = mom[M_U2];
-  f.var = mom[M_VAR];
+  const float4* mom = reinterpret_cast<const float4*>(A.mom + (size_t)cell * kMomLen);
+  const float4 m0 = mom[0], m1 = mom[1];
+  static_assert(M_W == 0 && M_PZ == 3 && M_U2 == 4 && M_VAR == 5, "two loads");
+  f.W = m0.x;
+  f.Px = m0.y;
+  f.Py = m0.z;
+  f.Pz = m0.w;
+  f.U2 = m1.x;
+  f.var = m1.y;
   f.ne = min(max(A.e.count[cell], 0), A.e.cap);
   f.T = 0.0;
   f.rc[0] = f.rc[1] = f.rc[2] = f.rc[3] = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -1049,17 +1078,28 @@ __device__ __forceinline__ void fb_prepare(FbCell& f) {
   f.need = false;
   f.qE = f.qPx = f.qPy = f.qPz = f.s1d = f.bx = f.by = f.bz = f.vnd = 0.0;
   if (!(f.has_x || f.has_res)) return;
-  f.qE = f.dE + f.rE;
-  f.qPx = f.dPx + f.rPx;
-  f.qPy = f.dPy + f.rPy;
-  f.qPz = f.dPz + f.rPz;
+  f.qE = f.rE;
+  f.qPx = f.rPx;
+  f.qPy = f.rPy;
+  f.qPz = f.rPz;
+  if (f.has_x) {
+    f.qE += f.dE;
+    f.qPx += f.dPx;
+    f.qPy += f.dPy;
+    f.qPz += f.dPz;
+  }
   // Exchanges below 2^-22 of the cell's kinetic energy (or momentum spread)
   // cannot be represented by binary32 momenta; they stay pending.
   const float ekin = 0.5f * f.U2 * kMeC2f;
   const float prms = sqrtf(fmaxf(f.U2 * f.W, 0.f));
-  f.need = f.W > 0.f && (fabsf((float)f.qE) >= 2.384185791015625e-07f * ekin ||
-                         sqrtf((float)(f.qPx * f.qPx + f.qPy * f.qPy + f.qPz * f.qPz)) >=
-                             2.384185791015625e-07f * prms);
+  const float tE = 2.384185791015625e-07f * ekin, tP = 2.384185791015625e-07f * prms;
+  // Most are far below: told in binary32 with a margin of 1e-4 for the cut
+  // magnitudes and the roundings, thresholds so small that a square could
+  // underflow left to the test itself.
+  const float aE = abs_below(f.qE), ax = abs_below(f.qPx), ay = abs_below(f.qPy), az = abs_below(f.qPz);
+  if (tE >= 1e-30f && tP >= 1e-15f && 1.0001f * aE < tE && 1.0001f * sqrtf(ax * ax + ay * ay + az * az) < tP) return;
+  f.need = f.W > 0.f && (fabsf((float)f.qE) >= tE ||
+                         sqrtf((float)(f.qPx * f.qPx + f.qPy * f.qPy + f.qPz * f.qPz)) >= tP);
   if (!f.need) return;
   // Eqs. delta_def, dE_bulk, dE_th, var_new, s_def, b_def (mu = 1). Three
   // FP64 divisions and one square root (FP64 runs at a small fraction of the
@@ -1104,9 +1144,9 @@ __device__ __forceinline__ void fb_finish(const StepArgs& A, int cell, const FbC
     mom[M_PY] = r->mPy;
     mom[M_PZ] = r->mPz;
     mom[M_U2] = r->mU2;
-    mom[M_VAR] = fmaxf(0.f, r->mU2 - (r->mPx * r->mPx + r->mPy * r->mPy + r->mPz * r->mPz) / r->mW);
+    mom[M_VAR] = fmaxf(0.f, r->mU2 - sum_sq(r->mPx, r->mPy, r->mPz) / r->mW);
   }
-  if (f.has_x || f.has_res) {
+  if (f.has_x || r) {  // else the carried exchange is as it was
     double* rs = A.res + (size_t)cell * 4;
     rs[0] = nrE;
     rs[1] = nrPx;
@@ -1135,10 +1175,10 @@ __device__ __forceinline__ void fb_finish(const StepArgs& A, int cell, const FbC
   // temperature (Eqs. Te_est, Te_relax), then the record's temperature half;
   // T stays FP64, the relaxation step is formed in binary32 and added once
   if (A.T_mode == 2 && f.W > 0.f) {
-    const float Tf = (float)f.T;
+    const float Tf = f32_of(f.T);
     const float Test = (kMeC2f / 3.0f) * var_new / f.W;
     const float dT = A.relax_r * (Test - Tf);
-    double Tn = f.T + (double)dT;
+    double Tn = f.T + f64_of(dT);
     const float Tnf = Tf + dT;
     if (Tnf <= A.T_floor_f || Tnf >= A.T_ceil_f) Tn = fmin(fmax(Tn, A.T_floor), A.T_ceil);
     float rec[kRecLen];
@@ -1150,7 +1190,7 @@ __device__ __forceinline__ void fb_finish(const StepArgs& A, int cell, const FbC
       rec[4 * i + 2] = rc[i].z;
       rec[4 * i + 3] = rc[i].w;
     }
-    compute_temperature(A.cc, (float)Tn, rec);
+    compute_temperature(A.cc, f32_of(Tn), rec);
     A.T[cell] = Tn;
     // the closed-form Primakoff prefactor (the network's may be there)
     if (A.rate_model == 2) rec[R_AP] = A.cc.k_AP * rec[R_SZ];
@@ -1169,7 +1209,11 @@ __device__ __forceinline__ void fb_finish(const StepArgs& A, int cell, const FbC
 // * DENSE = false: a remap takes the whole warp; five CTAs an SM (96
 //   registers; the remap path spills a little). 4.1 M cells at 5 keV: 217 us
 //   with 20 FP64 adds a remap, 202 with the 6 of group_sum4; 224 with the
-//   groups below in the same kernel (more spills).
+//   groups below in the same kernel (more spills). The FP64 units were busy
+//   two thirds of the time: the test whether to remap first in binary32, the
+//   conversions on the integer units, an unchanged carry not written and
+//   16-byte loads take four steps of 4.1 M cells from 7.79 to 7.63 ms and of
+//   0.9 M from 1.74 to 1.71 (conversions of the remap too: 7.66, spills).
 // * DENSE = true (absorption by weight reduction, which takes energy from
 //   every axion): cells of at most 64 electrons are remapped two or four side
 //   by side, the next ones' electrons loaded meanwhile; four CTAs an SM
@@ -1191,19 +1235,15 @@ __global__ void __launch_bounds__(kFeedbackThreads, DENSE ? 4 : 5) feedback_kern
   const bool valid = cell < A.cell0 + A.ncells;
   FbCell f = {};
   if (valid) {
-    double* xb = A.xbuf + (size_t)cell * 4;
-    f.dE = xb[0];
-    f.dPx = xb[1];
-    f.dPy = xb[2];
-    f.dPz = xb[3];
+    double2* xb = reinterpret_cast<double2*>(A.xbuf + (size_t)cell * 4);
+    const double2 x0 = xb[0], x1 = xb[1];
+    f.dE = x0.x;
+    f.dPx = x0.y;
+    f.dPy = x1.x;
+    f.dPz = x1.y;
     fb_load(A, cell, f);
     fb_prepare(f);
-    if (f.has_x) {
-      xb[0] = 0.0;
-      xb[1] = 0.0;
-      xb[2] = 0.0;
-      xb[3] = 0.0;
-    }
+    if (f.has_x) xb[0] = xb[1] = make_double2(0.0, 0.0);
   }
   // the warp remaps its cells that need it: as many side by side as have a
   // lane for every quad of electrons
