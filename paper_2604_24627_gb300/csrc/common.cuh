@@ -157,11 +157,11 @@ struct SpeciesPtrs {
 __device__ __forceinline__ void wait_predecessor() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 template <typename... Params, typename... Args>
-cudaError_t launch_chained(bool chained, void (*kernel)(Params...), int grid, int block, size_t smem, cudaStream_t st,
+cudaError_t launch_chained(bool chained, void (*kernel)(Params...), int grid, dim3 block, size_t smem, cudaStream_t st,
                            Args... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(grid);
-  cfg.blockDim = dim3(block);
+  cfg.blockDim = block;
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
   cudaLaunchAttribute attr = {};
