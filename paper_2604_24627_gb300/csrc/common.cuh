@@ -151,7 +151,9 @@ struct SpeciesPtrs {
 // A step is a chain of short kernels. Launched with programmatic stream
 // serialization, a kernel is set up while its predecessor ends and waits here,
 // first of all and in every thread, until the predecessor's memory is visible
-// (a no-op in a kernel launched without it). A step of 64 cells: 27.3 -> 18.0
+// (a no-op in a kernel launched without it). What a predecessor may have
+// written is read with plain loads, which cannot move above the wait, not
+// through __ldg or __restrict__ pointers. A step of 64 cells: 27.3 -> 18.0
 // us, with the memset between its kernels gone; 32 replayed steps of 65,536
 // dense cells in 8 branches: 6.77 -> 6.60 ms.
 __device__ __forceinline__ void wait_predecessor() { asm volatile("griddepcontrol.wait;" ::: "memory"); }

@@ -99,7 +99,7 @@ __device__ __forceinline__ void store8(unsigned char* tile, int r, int j0, int k
 // B^T tile (N rows n, K columns k) of a product with B(k, n) = W[k * ldn + n]
 // (forward) or W[n * ldk + k] (the transposed weights of the backward pass).
 template <bool TRANS>
-__device__ __forceinline__ void stage_weights(unsigned char* tile, const float* __restrict__ W, int N, int K) {
+__device__ __forceinline__ void stage_weights(unsigned char* tile, const float* W, int N, int K) {
   for (int i = threadIdx.x; i < N * (K / 8); i += kMlpThreads) {
     float v[8];
     int n, k0;
@@ -226,7 +226,7 @@ __global__ void __launch_bounds__(kMlpThreads, TRAIN ? 1 : 2) mlp_kernel(MlpArgs
       if (live && g.vec) {
 #pragma unroll
         for (int j = 0; j < 6; ++j) {
-          const float4 q = __ldg(reinterpret_cast<const float4*>(t) + j);
+          const float4 q = reinterpret_cast<const float4*>(t)[j];
           zt[4 * j] = q.x;
           zt[4 * j + 1] = q.y;
           zt[4 * j + 2] = q.z;
@@ -234,7 +234,7 @@ __global__ void __launch_bounds__(kMlpThreads, TRAIN ? 1 : 2) mlp_kernel(MlpArgs
         }
       } else {
 #pragma unroll
-        for (int j = 0; j < 24; ++j) zt[j] = live ? __ldg(t + j) : 0.f;
+        for (int j = 0; j < 24; ++j) zt[j] = live ? t[j] : 0.f;
       }
     }
     // layer 1 (K = 4) on the CUDA cores
@@ -506,7 +506,7 @@ cudaError_t Mlp::backward(const float* X, const float* Zt, int n, bool adam, flo
   a.err = err;
   const int grid = std::min((n + kNetRows - 1) / kNetRows, sms);
   // chained: a training step is two short kernels behind the last step's two
-  // (8 steps of 8,192 rows: 244 -> 208 us)
+  // (8 steps of 8,192 rows: 244 -> 210 us)
   if ((e = launch_chained(true, mlp_kernel<true>, grid, kMlpThreads, kTrainSmem, st, a))) return e;
   const dim3 block(kRedX, kRedY);
   if (adam) {

@@ -77,7 +77,7 @@ struct NetShared {
 // Set-up, once per CTA (all threads; blockDim.x == 128): 64 tensor-memory
 // columns, the mbarrier, and the image copied into sm + kNetActBytes (sm:
 // kNetSmemBytes of shared memory, 1024-byte aligned).
-__device__ __forceinline__ void net_begin(NetShared* ns, unsigned char* sm, const unsigned char* __restrict__ img) {
+__device__ __forceinline__ void net_begin(NetShared* ns, unsigned char* sm, const unsigned char* img) {
   const int tid = threadIdx.x;
   if ((tid >> 5) == 0) tmem_alloc(&ns->tmem, 64);
   if (tid == 0) {
@@ -87,7 +87,7 @@ __device__ __forceinline__ void net_begin(NetShared* ns, unsigned char* sm, cons
   }
   const uint4* s = reinterpret_cast<const uint4*>(img);
   uint4* d = reinterpret_cast<uint4*>(sm + kNetActBytes);
-  for (int i = tid; i < kNetImgBytes / 16; i += kNetThreads) d[i] = __ldg(s + i);
+  for (int i = tid; i < kNetImgBytes / 16; i += kNetThreads) d[i] = s[i];
   tc_fence_before();
   __syncthreads();
   tc_fence_after();

@@ -708,9 +708,9 @@ __device__ __forceinline__ void electron_chunk(const StepArgs& A, uint32_t step,
     const int c = c0 + lane;
     const float* rec = A.rec + (size_t)c * kRecLen;
     n = min(max(A.e.count[c], 0), A.e.cap);
-    rcc = __ldg(rec + R_CC);
-    rcb = __ldg(rec + R_CB);
-    wu = __ldg(A.mom + (size_t)c * kMomLen + M_WU);
+    rcc = rec[R_CC];
+    rcb = rec[R_CB];
+    wu = A.mom[(size_t)c * kMomLen + M_WU];
     if (wu > 0.f) {
       float fac;
       bool cc = false, cb = false;
@@ -881,8 +881,8 @@ __device__ __forceinline__ int photon_chunk(const StepArgs& A, uint32_t step, in
     const float* rec = A.rec + (size_t)c * kRecLen;
     const int cnt = min(max(A.g.count[c], 0), A.g.cap);
     n = A.use_snapshot ? min(A.photon_start[c], cnt) : cnt;
-    c_s = kMeC2f * kMeC2f * __ldg(rec + R_FOURK2);
-    ap = conversion_kb(__ldg(rec + R_AP), A.inv_w_a, A.guard_margin);
+    c_s = kMeC2f * kMeC2f * rec[R_FOURK2];
+    ap = conversion_kb(rec[R_AP], A.inv_w_a, A.guard_margin);
   }
   const QuadRange<C> R = quad_range<C>(n, lane, nc);
   int lcn = quad_cell(R, lane), qbn = __shfl_sync(kFull, R.qoff, lcn);
@@ -938,11 +938,11 @@ __device__ __forceinline__ int axion_chunk(const StepArgs& A, uint32_t step, int
     const int c = c0 + lane;
     const float* rec = A.rec + (size_t)c * kRecLen;
     n = min(max(A.a.count[c], 0), A.a.cap);
-    c_s = kMeC2f * kMeC2f * __ldg(rec + R_FOURK2);
-    apinv = conversion_kb(A.cc.prim_mult * __ldg(rec + R_AP), A.inv_w_gref, A.guard_margin);
+    c_s = kMeC2f * kMeC2f * rec[R_FOURK2];
+    apinv = conversion_kb(A.cc.prim_mult * rec[R_AP], A.inv_w_gref, A.guard_margin);
     const float gm = 1.001f * A.guard_margin;
-    ab = absorb_bound((mask & AXPIC_CH_COMPTON) ? __ldg(rec + R_BC) * gm : 0.f,
-                      (mask & AXPIC_CH_BREMS) ? __ldg(rec + R_BB) * gm : 0.f, kMeC2f * __ldg(rec + R_INVT),
+    ab = absorb_bound((mask & AXPIC_CH_COMPTON) ? rec[R_BC] * gm : 0.f,
+                      (mask & AXPIC_CH_BREMS) ? rec[R_BB] * gm : 0.f, kMeC2f * rec[R_INVT],
                       A.brems_am3);
   }
   const QuadRange<C> R = quad_range<C>(n, lane, nc);

@@ -409,7 +409,7 @@ __global__ void __launch_bounds__(kThreads, 6) stream_place_kernel(StreamArgs a)
       if (t < sA[wid][k]) {
         const float4* x = arrival(k, t);
         const long q = (long)(c0 + k) * s.cap + sl;
-        const float4 p0 = __ldg(x), q0 = __ldg(x + 1);
+        const float4 p0 = x[0], q0 = x[1];
         s.wp[q] = p0;
         s.xyz[q] = q0;
       }
@@ -439,8 +439,8 @@ __global__ void __launch_bounds__(kThreads, 6) stream_place_kernel(StreamArgs a)
             b[i] = ((v >> lane) & 1u) && t < A;
             if (b[i]) {
               const float4* x = arrival(k, t);
-              p[i] = __ldg(x);
-              q[i] = __ldg(x + 1);
+              p[i] = x[0];
+              q[i] = x[1];
             }
           }
 #pragma unroll
@@ -468,7 +468,7 @@ __global__ void __launch_bounds__(kThreads, 6) stream_place_kernel(StreamArgs a)
     if (f < X.total() && dst < s.cap) {
       const float4* x = arrival(k, sH[wid][k] + e);
       const long q = (long)(c0 + k) * s.cap + dst;
-      const float4 p0 = __ldg(x), q0 = __ldg(x + 1);
+      const float4 p0 = x[0], q0 = x[1];
       s.wp[q] = p0;
       s.xyz[q] = q0;
     }
