@@ -121,6 +121,7 @@ struct axpic_ctx {
   double* st_stats = nullptr; // [4]
   // axion merging scratch, made by the first axpic_merge_axions call
   double* mg_removed = nullptr;
+  int mg_fit = 0;             // the merge kernel's largest grid
   int sr_nkt = 0, sr_nne = 0, tnT = 0, tnne = 0, sur_set = 0, sur_any_trusted = 0;
   float ln_gP = 0.f, ln_gA = 0.f, lnK_CC = 0.f, lnK_CB = 0.f;
   int64_t last_absorb_step = -1;
@@ -1360,7 +1361,7 @@ axpic_status axpic_merge_axions(axpic_ctx* ctx, int32_t n_target, int32_t nedges
       return fail(ctx, AXPIC_E_INVALID, "axpic_merge_axions: thresholds must be finite, >= 0 and ascending");
   const axpic_plasma_desc& d = ctx->desc;
   if (!ctx->mg_removed) {
-    CK(merge_init_kernels(), "merge kernel attributes");
+    CK(merge_init_kernels(d.axions.capacity, &ctx->mg_fit), "merge kernel attributes");
     CK(cudaMalloc((void**)&ctx->mg_removed, sizeof(double)), "merge scratch");
     CK(cudaMemsetAsync(ctx->mg_removed, 0, sizeof(double), ctx->stream), "memset");
   }
@@ -1372,7 +1373,7 @@ axpic_status axpic_merge_axions(axpic_ctx* ctx, int32_t n_target, int32_t nedges
   a.nedges = nedges;
   for (int k = 0; k < nedges; ++k) a.edges[k] = edges_p2[k];
   a.removed = ctx->mg_removed;
-  CK(launch_merge(a, ctx->stream), "merge kernel");
+  CK(launch_merge(a, ctx->mg_fit, ctx->stream), "merge kernel");
   return AXPIC_OK;
 }
 

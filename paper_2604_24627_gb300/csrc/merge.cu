@@ -292,20 +292,27 @@ __global__ void __launch_bounds__(kWarpsMax * 32, 8) merge_kernel(MergeArgs a) {
 
 constexpr int kDynMax = 160 * 1024;  // the warps' dynamic shared memory, at most
 
-cudaError_t merge_init_kernels() {
-  return cudaFuncSetAttribute(merge_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kDynMax);
+// warps per CTA: as many as fit the shared memory, at most 4
+static int merge_warps(int cap) {
+  const size_t per_warp = std::max<size_t>(warp_bytes(cap), 4);
+  return (int)std::max<size_t>(1, std::min<size_t>(kWarpsMax, kDynMax / per_warp));
 }
 
-cudaError_t launch_merge(const MergeArgs& a, cudaStream_t st) {
+// as many CTAs as the device holds at once; asked for once, since the
+// driver's answers take some microseconds and a merge of a thousand cells 40
+cudaError_t merge_init_kernels(int cap, int* fit) {
+  const cudaError_t e = cudaFuncSetAttribute(merge_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kDynMax);
+  if (e) return e;
+  const int nw = merge_warps(cap);
+  *fit = resident_ctas((const void*)merge_kernel, nw * 32, std::max<size_t>(warp_bytes(cap), 4) * nw);
+  return *fit > 0 ? cudaSuccess : cudaErrorUnknown;
+}
+
+cudaError_t launch_merge(const MergeArgs& a, int fit, cudaStream_t st) {
   if (a.ncells <= 0) return cudaSuccess;
   if (a.s.cap > kMergeMaxCap) return cudaErrorInvalidValue;
-  // warps per CTA: as many as fit the shared memory, at most 4; as many CTAs
-  // as the device holds at once
-  const size_t per_warp = std::max<size_t>(warp_bytes(a.s.cap), 4);
-  const int nw = (int)std::max<size_t>(1, std::min<size_t>(kWarpsMax, kDynMax / per_warp));
-  const int fit = resident_ctas((const void*)merge_kernel, nw * 32, per_warp * nw);
-  if (fit <= 0) return cudaErrorUnknown;
-  merge_kernel<<<std::min((a.ncells + nw - 1) / nw, fit), nw * 32, per_warp * nw, st>>>(a);
+  const int nw = merge_warps(a.s.cap);
+  merge_kernel<<<std::min((a.ncells + nw - 1) / nw, fit), nw * 32, std::max<size_t>(warp_bytes(a.s.cap), 4) * nw, st>>>(a);
   return cudaGetLastError();
 }
 

@@ -19,8 +19,9 @@ struct MergeArgs {
   double* removed;   // [1]: axions removed so far
 };
 
-// Sets the merge kernel's shared-memory limit; called before its first launch.
-cudaError_t merge_init_kernels();
-cudaError_t launch_merge(const MergeArgs& a, cudaStream_t st);
+// Sets the merge kernel's shared-memory limit and works out its largest grid
+// for slabs of cap slots; called before a context's first launch.
+cudaError_t merge_init_kernels(int cap, int* fit);
+cudaError_t launch_merge(const MergeArgs& a, int fit, cudaStream_t st);
 
 }  // namespace axpic
