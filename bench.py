@@ -119,9 +119,10 @@ def kernel_bytes(tot, T_mode):
         electron of remapped cells (w, p read, p written);
       the surrogate network's record kernel (evolved T): the cell record
         read (64 B), the five prefactors written (32 B, two 16-byte stores)
-        and the source byte;
-      the table's record kernel (evolved T): the cell record read (64 B) and
-        the 192-float spectral record written (768 B)."""
+        and the source byte.
+
+    The table model writes no records in a step: the decisions and events
+    interpolate the table's entries they need."""
     cells = tot["cell_steps"]
     products = tot["events_p"] + tot["events_c"] + tot["events_b"] + tot["events_pinv"]
     removed = tot["events_p"] + tot["absorbed_c"] + tot["absorbed_b"] + tot["events_pinv"]
@@ -132,7 +133,6 @@ def kernel_bytes(tot, T_mode):
         "event_kernel": parts / 8.0 + 40.0 * cells + 56.0 * products + 56.0 * removed,
         "feedback_kernel": (104.0 + (80.0 if T_mode == 2 else 0.0)) * cells + 28.0 * tot["remap_e"],
         "sr_cells_kernel": 97.0 * cells,
-        "sr_table_kernel": 832.0 * cells,
     }
 
 
