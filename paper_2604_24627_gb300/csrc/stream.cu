@@ -528,18 +528,26 @@ cudaError_t launch(const StreamArgs& a, cudaStream_t st) {
 
 }  // namespace
 
-// Cells a warp: 4, so that thinly filled cells (13 axions of 64 slots in the
-// 3-D plasma) share its lanes, or 1. A large slab may hold few axions too,
-// so with enough cells for 8 rounds of resident warps it takes 4 as well
-// (262,144 cells of about 25 in 384 slots: 250 us a call against 345); with
-// fewer, 4 cells a warp leave the last of 2 rounds nearly empty where the
-// cells are full (65,536 of 128: 235 us against 215). 4 cells a warp want
-// at least one round.
+// Cells a warp: 4, so that thinly filled cells share its lanes, or 1. 4 are
+// better up to about 32 axions a cell, 1 beyond; the host does not know the
+// counts, only the capacities. Slabs of at most 128 slots take 4 from one
+// round of resident warps on: with the usual room to grow they hold at most
+// about 40. Us a call with 4 and 1 cells a warp:
+//   95,000 cells of 13 in 76 slots, 3-D      63   113
+//   216,000 cells of 20 in 92 slots, 3-D    179   279
+//   62,500 cells of 24 in 128 slots          58    81
+//   62,500 cells of 32 in 120 slots          88    94
+//   62,500 cells of 60 in 128 slots         125   121
+//   36,000 cells of 100 in 128 slots        106    94
+// A larger slab may hold few axions too: with enough cells for 8 rounds it
+// takes 4 as well (262,144 cells of about 25 in 384 slots: 250 against 345);
+// with fewer, 4 cells a warp leave the last of 2 rounds nearly empty where
+// the cells are full (65,536 of 128: 235 against 215).
 constexpr int kRound = 152 * 48;  // resident warps
 
 cudaError_t launch_stream(const StreamArgs& a, cudaStream_t st) {
   if (a.ncells <= 0) return cudaSuccess;
-  const int rounds = a.s.cap <= 64 ? 1 : 8;
+  const int rounds = a.s.cap <= 128 ? 1 : 8;
   return a.ncells / kGroup >= rounds * kRound ? launch<kGroup>(a, st) : launch<1>(a, st);
 }
 
