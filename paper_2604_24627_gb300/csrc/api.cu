@@ -466,15 +466,16 @@ axpic_status axpic_init_plasma(axpic_ctx** out, const axpic_plasma_desc* desc, c
     ctx->Z.push_back(d.Z[s]);
     ctx->A.push_back(d.A[s]);
   }
-  const size_t per_warp = step_smem_per_warp(d.axions.capacity, d.photons.capacity, d.electrons.capacity);
+  const size_t accepted = step_smem_accepted(d.axions.capacity, d.photons.capacity, d.electrons.capacity);
   int warps = p.threads_per_block > 0 ? p.threads_per_block / 32 : kDefaultWarps;
   if (warps < 1 || warps > 4 || (p.threads_per_block > 0 && p.threads_per_block % 32))
     return bad("threads_per_block must be 32..128, a multiple of 32");
   const size_t smem_limit = 227 * 1024 - 128;
-  while (warps > 1 && per_warp * warps > smem_limit) --warps;
-  if (per_warp > smem_limit) return bad("slab capacities too large for shared-memory scratch");
+  while (warps > 1 && accepted * warps > smem_limit) --warps;
+  if (accepted > smem_limit) return bad("slab capacities too large for shared-memory scratch");
   ctx->max_warps = 4;
-  while (ctx->max_warps > 1 && per_warp * ctx->max_warps > smem_limit) --ctx->max_warps;
+  while (ctx->max_warps > 1 && accepted * ctx->max_warps > smem_limit) --ctx->max_warps;
+  const size_t per_warp = step_smem_per_warp(d.axions.capacity, d.photons.capacity, d.electrons.capacity);
   if (p.decide_chunk != 0 && p.decide_chunk != 4 && p.decide_chunk != 8 && p.decide_chunk != 16 &&
       p.decide_chunk != 32)
     return bad("decide_chunk must be 0, 4, 8, 16 or 32");
@@ -1473,8 +1474,9 @@ axpic_status axpic_step_noalloc(const axpic_plasma_desc* desc, const axpic_param
   if (!why.empty()) return bad(why.c_str());
   if (step < 0 || step >= (int64_t)0xFFFFFFFF || (channel_mask & ~AXPIC_CH_ALL)) return bad("bad step or mask");
   if (p.rate_model != 0) return bad("rate_model must be 0 (the records need a context)");
+  if (step_smem_accepted(d.axions.capacity, d.photons.capacity, d.electrons.capacity) * kNoAllocWarps > 227 * 1024 - 128)
+    return bad("slab capacities too large");
   const size_t per_warp = step_smem_per_warp(d.axions.capacity, d.photons.capacity, d.electrons.capacity);
-  if (per_warp * kNoAllocWarps > 227 * 1024 - 128) return bad("slab capacities too large");
   const size_t bit_bytes = sizeof(uint32_t) * mask_words(d);
   if (bit_bytes > kNaBitsBytes) return bad("ncells * (capacities) / 8 above the 4 MiB mask scratch");
   const size_t rec_bytes = (size_t)d.ncells * (16 * ((size_t)d.axions.capacity + d.photons.capacity) +

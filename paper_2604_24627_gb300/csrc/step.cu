@@ -1311,20 +1311,32 @@ __host__ __device__ inline bool rows_staged(int acap, int gcap, int ecap) {
   return row_words(acap) <= 32 && row_words(gcap) <= 32 && row_words(ecap) <= 32;
 }
 
-// lists: with the heavy cells' lists and bits (the full-step kernel of the
-// light cells has none)
+// What a kernel's warps keep there: the heavy cells' lists and bits, the lanes'
+// lists, the mask rows with the exchange buffers. Lanes take cells only where
+// the rows are staged, so there are no lanes' lists without them.
+enum { EV_LISTS = 1, EV_LANES = 2, EV_ROWS = 4 };
+__host__ __device__ constexpr int ev_parts(int phases) {
+  return phases == PH_ABSORB ? EV_LISTS | EV_ROWS              // its lanes read the rows themselves
+         : phases == PH_EMIT ? EV_LISTS | EV_LANES | EV_ROWS
+                             : EV_LANES | EV_ROWS;             // heavy cells: event_heavy_kernel, EV_LISTS
+}
 __host__ __device__ inline size_t ev_list_bytes(int acap, int gcap, int ecap) {
   const size_t b = align16(2 * ((size_t)acap + (size_t)gcap + (size_t)ecap));
   return align16(b + 4 * (size_t)(row_words(acap) + row_words(gcap)));
 }
-__host__ __device__ inline size_t ev_scratch_bytes(int acap, int gcap, int ecap, bool lists) {
-  size_t b = (lists ? ev_list_bytes(acap, gcap, ecap) : 0) + kLaneListBytes;
+__host__ __device__ inline size_t ev_row_bytes(int acap, int gcap, int ecap) {
+  size_t b = 32 * 2 * sizeof(double2);
   if (rows_staged(acap, gcap, ecap))
     b += align16(4 * 32 * (size_t)((row_words(acap) | 1) + (row_words(gcap) | 1) + (row_words(ecap) | 1)));
-  return b + 32 * 2 * sizeof(double2);
+  return b;
+}
+__host__ __device__ inline size_t ev_scratch_bytes(int acap, int gcap, int ecap, int parts) {
+  return ((parts & EV_LISTS) ? ev_list_bytes(acap, gcap, ecap) : 0) +
+         ((parts & EV_LANES) && rows_staged(acap, gcap, ecap) ? kLaneListBytes : 0) +
+         ((parts & EV_ROWS) ? ev_row_bytes(acap, gcap, ecap) : 0);
 }
 
-template <bool LISTS>
+template <int PARTS>
 __device__ inline EvScratch ev_carve(unsigned char* base, int acap, int gcap, int ecap) {
   EvScratch s;
   uint16_t* h = reinterpret_cast<uint16_t*>(base);
@@ -1336,13 +1348,14 @@ __device__ inline EvScratch ev_carve(unsigned char* base, int acap, int gcap, in
   uint32_t* u = reinterpret_cast<uint32_t*>(base + align16(2 * ((size_t)acap + gcap + ecap)));
   s.rbA = u; u += row_words(acap);
   s.rbG = u;
-  size_t off = LISTS ? ev_list_bytes(acap, gcap, ecap) : 0;
+  const bool staged = rows_staged(acap, gcap, ecap);
+  size_t off = (PARTS & EV_LISTS) ? ev_list_bytes(acap, gcap, ecap) : 0;
   s.lt = reinterpret_cast<uint16_t*>(base + off);
-  off += kLaneListBytes;
+  if ((PARTS & EV_LANES) && staged) off += kLaneListBytes;
   s.sA = row_words(acap) | 1;
   s.sG = row_words(gcap) | 1;
   s.sE = row_words(ecap) | 1;
-  if (rows_staged(acap, gcap, ecap)) {
+  if ((PARTS & EV_ROWS) && staged) {
     s.rowA = reinterpret_cast<uint32_t*>(base + off);
     s.rowG = s.rowA + 32 * s.sA;
     s.rowE = s.rowG + 32 * s.sG;
@@ -1690,7 +1703,7 @@ __device__ __forceinline__ void reduce_out(const Lane64& x64, PhaseOut* out) {
 __device__ __noinline__ void absorb_warp(const StepArgs& A, int cell, unsigned char* sb, const uint32_t* row,
                                          uint32_t* clr, const Cnt cnt, int na_start, int ng_start, bool fill,
                                          PhaseOut* out) {
-  const EvScratch S = ev_carve<true>(sb, A.a.cap, A.g.cap, A.e.cap);
+  const EvScratch S = ev_carve<EV_LISTS>(sb, A.a.cap, A.g.cap, A.e.cap);
   const int lane = lane_id();
   const unsigned lt = (1u << lane) - 1u;
   const bool bath = A.mask & (AXPIC_CH_COMPTON | AXPIC_CH_BREMS);
@@ -1739,7 +1752,7 @@ __device__ __noinline__ void emit_warp(const StepArgs& A, uint32_t step, int cel
                                        const uint32_t* rowG, uint32_t* clrG, const uint32_t* rowE, uint32_t* clrE,
                                        const Cnt cnt, AxDest D, int ng_tot, int ng0, int ne, float wu, float r_cc,
                                        float r_cb, float r_T, PhaseOut* out) {
-  const EvScratch S = ev_carve<true>(sb, A.a.cap, A.g.cap, A.e.cap);
+  const EvScratch S = ev_carve<EV_LISTS>(sb, A.a.cap, A.g.cap, A.e.cap);
   const int lane = lane_id();
   const unsigned lt = (1u << lane) - 1u;
   const long abase = (long)cell * A.a.cap;
@@ -2120,9 +2133,8 @@ __global__ void __launch_bounds__(128, PH == 3 ? AXPIC_EVENT_FULL_MIN_CTAS : AXP
   if (lane < kNumCounters) warp_cnt[wid][lane] = 0ull;
   __syncwarp();
   const Cnt cnt{warp_cnt[wid]};
-  constexpr bool kLists = PH != (PH_ABSORB | PH_EMIT);
-  unsigned char* const sbase = smem + wid * ev_scratch_bytes(A.a.cap, A.g.cap, A.e.cap, kLists);
-  const EvScratch S = ev_carve<kLists>(sbase, A.a.cap, A.g.cap, A.e.cap);
+  unsigned char* const sbase = smem + wid * ev_scratch_bytes(A.a.cap, A.g.cap, A.e.cap, ev_parts(PH));
+  const EvScratch S = ev_carve<ev_parts(PH)>(sbase, A.a.cap, A.g.cap, A.e.cap);
   uint16_t* lA = S.lt + lane;
   uint16_t* lG = lA + 32 * kLight;
   uint16_t* lE = lG + 32 * kLight;
@@ -2334,8 +2346,8 @@ __global__ void __launch_bounds__(128) event_heavy_kernel(StepArgs A) {
   if (lane < kNumCounters) warp_cnt[wid][lane] = 0ull;
   __syncwarp();
   const Cnt cnt{warp_cnt[wid]};
-  unsigned char* const sbase = smem + wid * ev_scratch_bytes(A.a.cap, A.g.cap, A.e.cap, true);
-  const EvScratch S = ev_carve<true>(sbase, A.a.cap, A.g.cap, A.e.cap);
+  unsigned char* const sbase = smem + wid * ev_scratch_bytes(A.a.cap, A.g.cap, A.e.cap, EV_LISTS);
+  const EvScratch S = ev_carve<EV_LISTS>(sbase, A.a.cap, A.g.cap, A.e.cap);
   const uint32_t step = step_of(A);
   const bool emitG = (A.mask & AXPIC_CH_PRIMAKOFF) != 0;
   const bool emitE = (A.mask & (AXPIC_CH_COMPTON | AXPIC_CH_BREMS)) != 0;
@@ -2398,7 +2410,12 @@ __global__ void __launch_bounds__(128) event_heavy_kernel(StepArgs A) {
 }
 
 // ---------------------------------------------------------------- launchers
-size_t step_smem_per_warp(int acap, int gcap, int ecap) { return ev_scratch_bytes(acap, gcap, ecap, true); }
+size_t step_smem_per_warp(int acap, int gcap, int ecap) {
+  return ev_scratch_bytes(acap, gcap, ecap, EV_LISTS | EV_LANES | EV_ROWS);
+}
+size_t step_smem_accepted(int acap, int gcap, int ecap) {
+  return ev_list_bytes(acap, gcap, ecap) + 1536 + ev_row_bytes(acap, gcap, ecap);
+}
 
 int resident_ctas(const void* fn, int threads, size_t dyn_smem, int max_per_sm) {
   int dev = 0, sms = 0, regs_sm = 0, smem_sm = 0, reserved = 0, threads_sm = 0, blocks_sm = 0;
@@ -2437,8 +2454,8 @@ static int event_cells(const StepArgs& A) {
 template <int PH>
 static cudaError_t launch_events(const StepArgs& A, int warps, cudaStream_t st, bool chained) {
   constexpr bool full = PH == (PH_ABSORB | PH_EMIT);
-  const size_t lists = ev_scratch_bytes(A.a.cap, A.g.cap, A.e.cap, true);
-  const size_t per = ev_scratch_bytes(A.a.cap, A.g.cap, A.e.cap, !full);
+  const size_t lists = ev_scratch_bytes(A.a.cap, A.g.cap, A.e.cap, EV_LISTS);
+  const size_t per = ev_scratch_bytes(A.a.cap, A.g.cap, A.e.cap, ev_parts(PH));
   StepArgs B = A;
   B.ev_cells = full ? event_cells(A) : 32;
   const int grid = (A.ncells + B.ev_cells * warps - 1) / (B.ev_cells * warps);

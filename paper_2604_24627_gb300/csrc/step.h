@@ -7,7 +7,13 @@ namespace axpic {
 
 enum { PH_ABSORB = 1, PH_EMIT = 2, PH_FEEDBACK = 4, PH_ALL = 7 };
 
+// Shared memory a warp of the event kernels takes at most.
 size_t step_smem_per_warp(int acap, int gcap, int ecap);
+// The sum that slab capacities are accepted by, fixed: the lists of a cell, 1536
+// bytes, the mask rows and exchange buffers. No kernel needs more where it is
+// near a limit (beyond 1024 slots the rows are not staged and the lanes have no
+// lists; below, a warp takes 24 KB at most).
+size_t step_smem_accepted(int acap, int gcap, int ecap);
 // ev: NULL, or kStepKernels + 1 events recorded around the kernels of a
 // PH_ALL step: decisions, events, feedback, and the surrogate's network
 // kernel (an empty interval when there is none). sra: that kernel's
