@@ -158,7 +158,7 @@ template <bool TRAIN>
 __global__ void __launch_bounds__(kMlpThreads, TRAIN ? 1 : 2) mlp_kernel(MlpArgs g) {
   wait_predecessor();
   extern __shared__ __align__(1024) unsigned char sm[];
-  __shared__ uint64_t bars[2];
+  __shared__ uint64_t bars[3];  // [2]: what is in flight when a wait ran out
   __shared__ uint32_t tmem_base;
   __shared__ double lsum[kMlpThreads / 32];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -168,6 +168,7 @@ __global__ void __launch_bounds__(kMlpThreads, TRAIN ? 1 : 2) mlp_kernel(MlpArgs
   if (tid == 0) {
     mbar_init(&bars[0], 1);
     mbar_init(&bars[1], 1);
+    mbar_init(&bars[2], 1);
     asm volatile("fence.mbarrier_init.release.cluster;");
   }
   unsigned char* const sW2f = sm + (TRAIN ? kSW2f : kFW2f);
@@ -201,7 +202,8 @@ __global__ void __launch_bounds__(kMlpThreads, TRAIN ? 1 : 2) mlp_kernel(MlpArgs
   const uint32_t tZ = TRAIN ? kTZ : 0;  // inference: z over z2, which has been read
   uint32_t ph = 0, ph1 = 0;
   // one commit of barrier b (phase parity p); the warp converges for the
-  // tensor-memory loads that follow
+  // tensor-memory loads that follow. ok is the thread's own from here to the
+  // next join, which alone decides whether the CTA goes on.
   auto await = [&](int b, uint32_t& p) {
     ok = ok && mbar_wait(&bars[b], p);
     p ^= 1u;
@@ -212,7 +214,7 @@ __global__ void __launch_bounds__(kMlpThreads, TRAIN ? 1 : 2) mlp_kernel(MlpArgs
   float sgb3 = 0.f, sgb2 = 0.f, sgb1 = 0.f, sgw1[4] = {0.f, 0.f, 0.f, 0.f};
   double loss = 0.0;
   bool first = true;
-  for (int tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x) {
+  for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
     const long r = (long)tile * kNetRows + row;
     const bool live = r < g.n;
     float x[4] = {0.f, 0.f, 0.f, 0.f}, zt[24];
@@ -250,7 +252,8 @@ __global__ void __launch_bounds__(kMlpThreads, TRAIN ? 1 : 2) mlp_kernel(MlpArgs
     store8(sm + kSH1, row, 16 * grp, 64, h1);
     store8(sm + kSH1, row, 16 * grp + 8, 64, h1 + 8);
     join();
-    if (tid == 0 && ok) {
+    if (!ok) break;  // all threads alike: a wait of the last tile ran out in some
+    if (tid == 0) {
       issue_k(tmem + kTZ2, aH1, aW2f, 64, 64);
       tc_commit(&bars[0]);
     }
@@ -342,11 +345,13 @@ __global__ void __launch_bounds__(kMlpThreads, TRAIN ? 1 : 2) mlp_kernel(MlpArgs
   }
   ok = __syncthreads_and(ok) != 0;
   if (!ok) {
-    // flag it and give the tensor core a second bounded wait on whatever it
-    // may still be doing before the tensor memory is released
-    if (tid == 0) atomicOr(g.err, 1);
-    mbar_wait(&bars[0], ph ^ 1u);
-    if (TRAIN) mbar_wait(&bars[1], ph1);
+    // flag it and give the tensor core a second bounded wait: for every product
+    // issued so far, before the tensor memory is released
+    if (tid == 0) {
+      atomicOr(g.err, 1);
+      tc_commit(&bars[2]);
+    }
+    mbar_poll(&bars[2], 0, kWaitPolls);
   } else if (TRAIN) {
     // the CTA's gradients: one row of partials
     float* out = g.part + (size_t)blockIdx.x * kMlpParams;

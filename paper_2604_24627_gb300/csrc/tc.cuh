@@ -37,10 +37,16 @@ __device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count));
 }
 
+// Polls of a bounded wait (a test's build gives some threads none).
+constexpr int kWaitPolls = 1 << 22;
+#ifndef AXPIC_WAIT_POLLS
+#define AXPIC_WAIT_POLLS kWaitPolls
+#endif
+
 // Bounded wait on an mbarrier phase; false when the bound ran out.
-__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity) {
+__device__ __forceinline__ bool mbar_poll(uint64_t* bar, uint32_t parity, int polls) {
   const uint32_t a = smem_u32(bar);
-  for (int it = 0; it < (1 << 22); ++it) {
+  for (int it = 0; it < polls; ++it) {
     uint32_t done = 0;
     asm volatile(
         "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
@@ -51,6 +57,9 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity) {
     if (done) return true;
   }
   return false;
+}
+__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity) {
+  return mbar_poll(bar, parity, AXPIC_WAIT_POLLS);
 }
 
 // Core-matrix layout of a rows x kc bfloat16 tile (kc a multiple of 16):
