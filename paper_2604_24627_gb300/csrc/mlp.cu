@@ -402,15 +402,17 @@ __global__ void __launch_bounds__(kMlpThreads, TRAIN ? 1 : 2) mlp_kernel(MlpArgs
 // The CTAs' gradient rows added in CTA order (eight slices of rows per
 // parameter, then the slices in order), so training does not depend on
 // scheduling; then Adam with bias correction on the FP32 master parameters
-// (ADAM), or the gradients themselves. Block 0 also sums the loss.
+// (ADAM), or the gradients themselves. Block 0 also sums the loss. After a wait
+// that ran out (*err) the rows are not whole: nothing is written.
 constexpr int kRedX = 32, kRedY = 8;
 
 template <bool ADAM>
 __global__ void __launch_bounds__(kRedX* kRedY) reduce_kernel(const float* part, const double* losses, int rows,
                                                               float inv_n, float* G, float* P, float* M, float* V,
-                                                              double* loss, float lr, float b1, float b2, float eps,
-                                                              float c1, float c2) {
+                                                              double* loss, const int* err, float lr, float b1,
+                                                              float b2, float eps, float c1, float c2) {
   wait_predecessor();  // (no pointer here is __restrict__: nothing is read before it)
+  if (*err) return;
   __shared__ float s[kRedY][kRedX];
   const int i = blockIdx.x * kRedX + threadIdx.x;
   const int per = (rows + kRedY - 1) / kRedY;
@@ -518,10 +520,10 @@ cudaError_t Mlp::backward(const float* X, const float* Zt, int n, bool adam, flo
     ++t;
     const float c1 = 1.0f - powf(0.9f, (float)t), c2 = 1.0f - powf(0.999f, (float)t);
     return launch_chained(true, reduce_kernel<true>, kMlpParams / kRedX, block, 0, st, part, losses, grid, a.inv_n, G, P,
-                          Ma, Va, loss, lr, 0.9f, 0.999f, 1e-8f, c1, c2);
+                          Ma, Va, loss, err, lr, 0.9f, 0.999f, 1e-8f, c1, c2);
   }
   return launch_chained(true, reduce_kernel<false>, kMlpParams / kRedX, block, 0, st, part, losses, grid, a.inv_n, G, P,
-                        Ma, Va, loss, 0.f, 0.f, 0.f, 0.f, 1.f, 1.f);
+                        Ma, Va, loss, err, 0.f, 0.f, 0.f, 0.f, 1.f, 1.f);
 }
 
 cudaError_t Mlp::gradients(const float* X, const float* Zt, int n) { return backward(X, Zt, n, false, 0.f); }
