@@ -637,8 +637,8 @@ axpic_status axpic_set_surrogate(axpic_ctx *ctx, axpic_mlp *m, const float *err_
 axpic_status axpic_get_cell_records(axpic_ctx *ctx, int32_t first, int32_t count, float *rec_out,
                                     uint8_t *src_out);
 /* The spectral records of cells [first, first + count) (rate models 1 and 2;
- * under model 2 only the cells the network is not trusted for have one, see
- * axpic_get_cell_records): 192 floats per cell to out (host): ln(dQ_c/dx) +
+ * under model 2 only the cells the network is not trusted for take their rates
+ * from it, see axpic_get_cell_records): 192 floats per cell to out (host): ln(dQ_c/dx) +
  * x_k at unit coupling on x_k = 0.05 e^((k - 1) h), h = ln(400) / 29,
  * k = 0..31 (c * 32 + k; c = Primakoff, Compton-like, brems), the
  * quantiles x(j/32) (96 + c * 31 + j - 1), then ln(g_agg^2 dt pi^2 (hbar c)^3

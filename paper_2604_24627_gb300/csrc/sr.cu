@@ -69,22 +69,19 @@ void build_sr_table(int nkt, int nne, double brems_shape, float* out) {
 // entries it needs). A CTA takes 32 cells: warp 0 forms each cell's
 // interpolation constants (lane per cell) in shared memory, then the CTA's
 // threads stream the 32 x 192 record entries (consecutive threads,
-// consecutive entries of a cell); under the surrogate model only those of
-// the cells the network is not trusted for.
+// consecutive entries of a cell); under the surrogate model too every cell's,
+// so that what is read or saved does not depend on what was there before.
 constexpr int kSrTableThreads = 256;
 __global__ void __launch_bounds__(kSrTableThreads) sr_table_kernel(SrArgs a) {
   __shared__ SrInterp ip[32];
-  __shared__ uint8_t has[32];
   const int c0 = a.cell0 + blockIdx.x * 32;
   const int nc = min(32, a.cell0 + a.ncells - c0);
-  if (threadIdx.x < 32 && (int)threadIdx.x < nc) {
+  if (threadIdx.x < 32 && (int)threadIdx.x < nc)
     sr_interp(a.ra, sr_cell_from(a.rec + (size_t)(c0 + threadIdx.x) * kRecLen, a.ra.k_T7), &ip[threadIdx.x]);
-    has[threadIdx.x] = a.ra.src ? a.ra.src[c0 + threadIdx.x] : 1;
-  }
   __syncthreads();
   for (int e = threadIdx.x; e < nc * kSrLen; e += kSrTableThreads) {
     const int c = e / kSrLen, o = e - c * kSrLen;
-    if (has[c]) a.ra.sr[(size_t)(c0 + c) * kSrLen + o] = sr_table_entry(a.ra, ip[c], o);
+    a.ra.sr[(size_t)(c0 + c) * kSrLen + o] = sr_table_entry(a.ra, ip[c], o);
   }
 }
 

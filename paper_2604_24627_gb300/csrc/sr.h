@@ -141,7 +141,7 @@ __device__ __forceinline__ bool sr_trusted(const RecordArgs& a, float T, float l
 void build_sr_table(int nkt, int nne, double brems_shape, float* out);
 
 // The table's spectral records of cells [cell0, cell0 + ncells) into ra.sr, for
-// reading and saving: all of them, or those with src set.
+// reading and saving.
 cudaError_t launch_sr_table(const SrArgs& a, cudaStream_t st);
 // Rate model 2: per cell of [cell0, cell0 + ncells), from its current cell
 // record: the network's prefactors into the record's rate slots where it is
