@@ -125,10 +125,10 @@ typedef struct {
   int32_t diag_enable;      /* 1: feedback writes per-cell diagnostics */
   int32_t threads_per_block;/* threads per CTA of the event kernel (32..128, one
                                warp per cell); 0: default 128 */
-  int32_t decide_chunk;     /* cells per chunk of a decision warp: 4, 8, 16 or
-                               32; 0: 1 to 32 by the launch's cells and the
-                               slabs' capacities (launch shape, see
-                               axpic_autotune) */
+  int32_t decide_chunk;     /* cells per chunk of a decision warp: 1, 2, 4, 8,
+                               16 or 32; 0: one of them by the launch's cells
+                               and the slabs' capacities (launch shape, see
+                               axpic_launch_shape and axpic_autotune) */
   int32_t rate_model;       /* 0: closed forms (default); 1: exact FP32 table:
                                the full decisions' Primakoff and absorption
                                rates and the emission energies from per-cell

@@ -476,9 +476,8 @@ axpic_status axpic_init_plasma(axpic_ctx** out, const axpic_plasma_desc* desc, c
   ctx->max_warps = 4;
   while (ctx->max_warps > 1 && accepted * ctx->max_warps > smem_limit) --ctx->max_warps;
   const size_t per_warp = step_smem_per_warp(d.axions.capacity, d.photons.capacity, d.electrons.capacity);
-  if (p.decide_chunk != 0 && p.decide_chunk != 4 && p.decide_chunk != 8 && p.decide_chunk != 16 &&
-      p.decide_chunk != 32)
-    return bad("decide_chunk must be 0, 4, 8, 16 or 32");
+  if (p.decide_chunk < 0 || p.decide_chunk > 32 || (p.decide_chunk & (p.decide_chunk - 1)))
+    return bad("decide_chunk must be 0 or a power of two up to 32");
   if (p.step_branches < 0 || p.step_branches > kMaxBranches || (p.step_branches & (p.step_branches - 1)))
     return bad("step_branches must be 0 or a power of two up to 8");
   if (p.rate_model < 0 || p.rate_model > 2) return bad("rate_model must be 0, 1 or 2");
