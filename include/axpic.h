@@ -466,15 +466,20 @@ axpic_status axpic_run_steps(axpic_ctx *ctx, int64_t first_step, int32_t nsteps,
 axpic_status axpic_launch_shape(const axpic_ctx *ctx, int32_t *decide_chunk, int32_t *event_warps,
                                 int32_t *step_branches);
 
-/* Picks the launch shape (cells per decision chunk, 4/8/16/32, and warps per
- * event CTA, 2 or 4) by timing trial_steps steps of the context's own state
- * for each shape (CUDA events, after one untimed step), with the step index
- * `step` and channel_mask. The context's device state (the slabs and counts
+/* Looks for a better launch shape than the one in use (by default a rule's:
+ * decide_chunk 0) among 4, 8, 16 and 32 cells per decision chunk and 2 and 4
+ * warps per event CTA, by timing trial_steps steps of the context's own state
+ * for each (CUDA events, after one untimed step), with the step index `step`
+ * and channel_mask: as axpic_step launches them and, where axpic_run_steps has
+ * branches, replayed too. The fastest replaces the shape in use only if it is
+ * at least 1 % faster in each of these forms; its cells per chunk are then
+ * fixed for both (axpic_launch_shape reports what is in use). The context's
+ * device state (the slabs and counts
  * of the three species, T, rates, moments, exchange and carried buffers,
  * tallies and counters) is saved to scratch first and restored after every
  * trial, so the state afterwards is bit for bit what it was. Needs device
- * memory for one copy of that state. Synchronises. Writes the best shape's
- * ms per step to *best_ms_out (may be NULL) and its parameters to
+ * memory for one copy of that state. Synchronises. Writes the fastest of the
+ * timed shapes' ms per step to *best_ms_out (may be NULL) and its parameters to
  * *chunk_out and *warps_out (may be NULL). AXPIC_E_INVALID for
  * trial_steps < 1. Not part of the paper's method. */
 axpic_status axpic_autotune(axpic_ctx *ctx, int64_t step, int32_t trial_steps, int32_t channel_mask,

@@ -883,6 +883,13 @@ axpic_status axpic_profile_end(axpic_ctx* ctx, double* ms_out, int32_t* steps_ou
   return AXPIC_OK;
 }
 
+// Cells of a replayed step's branch: whole event CTAs (128 cells), or all cells
+// where there is one branch.
+static int branch_cells(const axpic_ctx* ctx) {
+  const int n = ctx->desc.ncells;
+  return ctx->branches == 1 ? n : ((n + ctx->branches - 1) / ctx->branches + 127) / 128 * 128;
+}
+
 // The steps a replayed graph holds (nsteps of them). With several branches
 // the cells are split into ranges of whole event CTAs (128 cells); each
 // range's kernels run nsteps steps on a stream forked from gs, reading and
@@ -890,9 +897,9 @@ axpic_status axpic_profile_end(axpic_ctx* ctx, double* ms_out, int32_t* steps_ou
 // independent, so the results are those of one launch over all cells.
 static cudaError_t capture_steps(axpic_ctx* ctx, StepArgs A, int nsteps, cudaStream_t gs, const SrArgs* sra) {
   const int n = ctx->desc.ncells;
-  const int part = ((n + ctx->branches - 1) / ctx->branches + 127) / 128 * 128;
+  const int part = branch_cells(ctx);
   cudaError_t e;
-  if (ctx->branches == 1 || part >= n) {
+  if (part >= n) {
     for (int k = 0; k < nsteps; ++k)
       if ((e = launch_step(PH_ALL, A, ctx->warps, gs, nullptr, sra, k > 0))) return e;
     return cudaSuccess;
@@ -926,6 +933,15 @@ static cudaError_t capture_steps(axpic_ctx* ctx, StepArgs A, int nsteps, cudaStr
   }
   for (int b = 0; b < nb; ++b)
     if ((e = cudaStreamWaitEvent(gs, ctx->br_ev[b], 0))) return e;
+  return cudaSuccess;
+}
+
+static cudaError_t graph_setup(axpic_ctx* ctx) {
+  if (ctx->graph_stream) return cudaSuccess;
+  cudaError_t e;
+  if ((e = cudaStreamCreateWithFlags(&ctx->graph_stream, cudaStreamNonBlocking))) return e;
+  for (auto& ev : ctx->graph_ev)
+    if ((e = cudaEventCreateWithFlags(&ev, cudaEventDisableTiming))) return e;
   return cudaSuccess;
 }
 
@@ -978,11 +994,7 @@ axpic_status axpic_run_steps(axpic_ctx* ctx, int64_t first_step, int32_t nsteps,
     return fail(ctx, AXPIC_E_INVALID, "axpic_run_steps: step range outside [0, 2^32 - 1)");
   if (channel_mask & ~AXPIC_CH_ALL) return fail(ctx, AXPIC_E_INVALID, "axpic_run_steps: unknown channel bits");
   if (nsteps == 0 || ctx->desc.ncells == 0) return AXPIC_OK;
-  if (!ctx->graph_stream) {
-    CK(cudaStreamCreateWithFlags(&ctx->graph_stream, cudaStreamNonBlocking), "stream create");
-    CK(cudaEventCreateWithFlags(&ctx->graph_ev[0], cudaEventDisableTiming), "event create");
-    CK(cudaEventCreateWithFlags(&ctx->graph_ev[1], cudaEventDisableTiming), "event create");
-  }
+  CK(graph_setup(ctx), "graph stream");
   cudaStream_t gs = ctx->graph_stream;
   // ordered after the work already queued on the context's stream
   CK(cudaEventRecord(ctx->graph_ev[0], ctx->stream), "event record");
@@ -1024,11 +1036,7 @@ axpic_status axpic_run_steps_streamed(axpic_ctx* ctx, int64_t first_step, int32_
     ctx->sgraphs.clear();
     ctx->stream_sig = sig;
   }
-  if (!ctx->graph_stream) {
-    CK(cudaStreamCreateWithFlags(&ctx->graph_stream, cudaStreamNonBlocking), "stream create");
-    CK(cudaEventCreateWithFlags(&ctx->graph_ev[0], cudaEventDisableTiming), "event create");
-    CK(cudaEventCreateWithFlags(&ctx->graph_ev[1], cudaEventDisableTiming), "event create");
-  }
+  CK(graph_setup(ctx), "graph stream");
   cudaStream_t gs = ctx->graph_stream;
   CK(cudaEventRecord(ctx->graph_ev[0], ctx->stream), "event record");
   CK(cudaStreamWaitEvent(gs, ctx->graph_ev[0], 0), "stream wait");
@@ -1100,8 +1108,8 @@ axpic_status axpic_launch_shape(const axpic_ctx* ctx, int32_t* decide_chunk_out,
                                 int32_t* step_branches) {
   if (!ctx) return AXPIC_E_INVALID;
   const int n = ctx->desc.ncells;
-  const int part = ((n + ctx->branches - 1) / ctx->branches + 127) / 128 * 128;
-  const bool whole = ctx->branches == 1 || part >= n;
+  const int part = branch_cells(ctx);
+  const bool whole = part >= n;
   if (decide_chunk_out) {
     StepArgs A = make_args(const_cast<axpic_ctx*>(ctx), 0, AXPIC_CH_ALL);
     if (!whole) A.ncells = part, A.dec_cells = n;
@@ -1112,6 +1120,50 @@ axpic_status axpic_launch_shape(const axpic_ctx* ctx, int32_t* decide_chunk_out,
   return AXPIC_OK;
 }
 
+// Times trial_steps steps of the shape in use from the saved state, after one
+// untimed: as axpic_step launches them, or replayed (as axpic_run_steps does
+// where it has branches). The state is restored.
+static cudaError_t time_shape(axpic_ctx* ctx, int64_t step, int32_t trial_steps, int32_t mask, bool replay,
+                              unsigned char* save, cudaEvent_t e0, cudaEvent_t e1, double* ms_per_step) {
+  cudaError_t e = cudaSuccess;
+  const SrArgs sra = make_sr_args(ctx);
+  const SrArgs* sp = ctx->prm.rate_model ? &sra : nullptr;
+  cudaGraphExec_t ex[2] = {nullptr, nullptr};  // the untimed step, the timed ones
+  cudaStream_t st = replay ? ctx->graph_stream : ctx->stream;
+  if (replay) {
+    StepArgs A = make_args(ctx, step, mask);
+    A.step_dev = ctx->step_dev;
+    for (int i = 0; i < 2 && !e; ++i) {
+      cudaGraph_t g = nullptr;
+      if ((e = cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal))) break;
+      e = capture_steps(ctx, A, i ? trial_steps : 1, st, sp);
+      const cudaError_t ce = cudaStreamEndCapture(st, &g);
+      if (!e) e = ce;
+      if (!e) e = cudaGraphInstantiate(&ex[i], g, 0);
+      if (g) cudaGraphDestroy(g);
+    }
+    if (!e) e = launch_set_step(ctx->step_dev, (uint32_t)step, kMaxBranches, st);
+    if (!e) e = cudaGraphLaunch(ex[0], st);
+    if (!e) e = cudaEventRecord(e0, st);
+    if (!e) e = cudaGraphLaunch(ex[1], st);
+  } else {
+    e = launch_step(PH_ALL, make_args(ctx, step, mask), ctx->warps, st, nullptr, sp);
+    if (!e) e = cudaEventRecord(e0, st);
+    for (int32_t k = 0; k < trial_steps && !e; ++k)
+      e = launch_step(PH_ALL, make_args(ctx, step + 1 + k, mask), ctx->warps, st, nullptr, sp);
+  }
+  float ms = 0.f;
+  if (!e) e = cudaEventRecord(e1, st);
+  if (!e) e = cudaEventSynchronize(e1);
+  if (!e) e = cudaEventElapsedTime(&ms, e0, e1);
+  for (cudaGraphExec_t x : ex)
+    if (x) cudaGraphExecDestroy(x);
+  if (!e) e = copy_state(ctx, save, false);
+  if (!e) e = cudaStreamSynchronize(ctx->stream);  // before a trial on the other stream
+  *ms_per_step = ms / trial_steps;
+  return e;
+}
+
 axpic_status axpic_autotune(axpic_ctx* ctx, int64_t step, int32_t trial_steps, int32_t channel_mask,
                             double* best_ms_out, int32_t* chunk_out, int32_t* warps_out) {
   AXPIC_RANGE("axpic_autotune");
@@ -1119,6 +1171,8 @@ axpic_status axpic_autotune(axpic_ctx* ctx, int64_t step, int32_t trial_steps, i
   if (trial_steps < 1 || step < 0 || step + (int64_t)trial_steps >= (int64_t)0xFFFFFFFF)
     return fail(ctx, AXPIC_E_INVALID, "axpic_autotune: trial_steps < 1 or step range outside [0, 2^32 - 1)");
   if (channel_mask & ~AXPIC_CH_ALL) return fail(ctx, AXPIC_E_INVALID, "axpic_autotune: unknown channel bits");
+  const bool branched = branch_cells(ctx) < ctx->desc.ncells;
+  if (branched) CK(graph_setup(ctx), "graph stream");
   CK(cudaStreamSynchronize(ctx->stream), "synchronize");
   size_t total = 0;
   for (auto& b : state_buffers(ctx)) total += (b.second + 255) & ~size_t(255);
@@ -1127,48 +1181,58 @@ axpic_status axpic_autotune(axpic_ctx* ctx, int64_t step, int32_t trial_steps, i
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   const int keep_chunk = ctx->dec_chunk, keep_warps = ctx->warps;
   int best_chunk = keep_chunk, best_warps = keep_warps;
-  double best = -1.0;
+  double best_ms = -1.0, best = -1.0;
   cudaError_t e = copy_state(ctx, save, true);
+  if (!e) e = cudaStreamSynchronize(ctx->stream);
   if (!e) e = cudaEventCreate(&e0);
   if (!e) e = cudaEventCreate(&e1);
-  for (int chunk : {4, 8, 16, 32}) {
+  // ms by single steps and by replay; the shape in use, then the others, then
+  // the shape in use again
+  double now[2] = {-1.0, -1.0};
+  auto trial = [&](double* ms) {
+    ms[1] = 0.0;
+    if (!e) e = time_shape(ctx, step, trial_steps, channel_mask, false, save, e0, e1, &ms[0]);
+    if (!e && branched) e = time_shape(ctx, step, trial_steps, channel_mask, true, save, e0, e1, &ms[1]);
+  };
+  auto trial_now = [&]() {
+    double ms[2];
+    set_shape(ctx, keep_chunk, keep_warps);
+    trial(ms);
+    for (int i = 0; i < 2; ++i)
+      if (now[i] < 0.0 || ms[i] < now[i]) now[i] = ms[i];
+  };
+  struct Shape { int chunk, warps; double ms[2]; };
+  std::vector<Shape> tried;
+  trial_now();
+  for (int chunk : {4, 8, 16, 32})
     for (int warps : {2, 4}) {
-      if (e) break;
-      if (warps > ctx->max_warps) continue;
+      if (e || warps > ctx->max_warps) continue;
+      Shape t{chunk, warps, {0.0, 0.0}};
       set_shape(ctx, chunk, warps);
-      // one untimed step, then trial_steps timed ones, from the saved state
-      StepArgs A = make_args(ctx, step, channel_mask);
-      const SrArgs sra = make_sr_args(ctx);
-      const SrArgs* sp = ctx->prm.rate_model ? &sra : nullptr;
-      if ((e = launch_step(PH_ALL, A, ctx->warps, ctx->stream, nullptr, sp)) || (e = cudaEventRecord(e0, ctx->stream)))
-        break;
-      for (int32_t k = 0; k < trial_steps && !e; ++k) {
-        A = make_args(ctx, step + 1 + k, channel_mask);
-        e = launch_step(PH_ALL, A, ctx->warps, ctx->stream, nullptr, sp);
-      }
-      float ms = 0.f;
-      if (e || (e = cudaEventRecord(e1, ctx->stream)) || (e = cudaEventSynchronize(e1)) ||
-          (e = cudaEventElapsedTime(&ms, e0, e1)) || (e = copy_state(ctx, save, false)))
-        break;
-      const double per = ms / trial_steps;
-      if (best < 0.0 || per < best) {
-        best = per;
-        best_chunk = chunk;
-        best_warps = warps;
-      }
+      trial(t.ms);
+      tried.push_back(t);
+    }
+  trial_now();
+  // the slower form's time against the shape in use decides
+  for (const Shape& t : tried) {
+    const double r = std::max(t.ms[0] / now[0], branched ? t.ms[1] / now[1] : 0.0);
+    if (best < 0.0 || r < best) {
+      best = r;
+      best_ms = t.ms[0];
+      best_chunk = t.chunk;
+      best_warps = t.warps;
     }
   }
-  if (!e) e = cudaStreamSynchronize(ctx->stream);
   if (e0) cudaEventDestroy(e0);
   if (e1) cudaEventDestroy(e1);
   cudaFree(save);
-  if (e) {
-    set_shape(ctx, keep_chunk, keep_warps);
-    return cuda_fail(ctx, e, "axpic_autotune");
+  set_shape(ctx, keep_chunk, keep_warps);
+  if (e) return cuda_fail(ctx, e, "axpic_autotune");
+  if (best >= 0.0 && best < 0.99) {
+    set_shape(ctx, best_chunk, best_warps);
+    free_graphs(ctx);
   }
-  set_shape(ctx, best_chunk, best_warps);
-  free_graphs(ctx);
-  if (best_ms_out) *best_ms_out = best;
+  if (best_ms_out) *best_ms_out = best_ms;
   if (chunk_out) *chunk_out = best_chunk;
   if (warps_out) *warps_out = best_warps;
   return AXPIC_OK;

@@ -131,8 +131,9 @@ class AxionPlasma:
         return _lib.axpic_launch_shape(self.ctx)
 
     def autotune(self, step, trial_steps=3, mask=_lib.CH_ALL):
-        """Times the launch shapes on this state (restored afterwards) and keeps
-        the fastest; returns (ms per step, decide_chunk, event warps)."""
+        """Times the launch shapes on this state (restored afterwards); the
+        fastest replaces the one in use if it is faster than that. Returns
+        its (ms per step, decide_chunk, event warps)."""
         return _lib.axpic_autotune(self.ctx, step, trial_steps, mask)
 
     def tally(self):

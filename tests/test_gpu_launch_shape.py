@@ -1,5 +1,6 @@
-"""Launch shapes: what axpic_launch_shape reports can be asked for (needs a
-GB300)."""
+"""Launch shapes: what axpic_launch_shape reports can be asked for, and tuning
+replaces a shape by a faster one only (needs a GB300)."""
+import numpy as np
 import pytest
 
 torch = pytest.importorskip("torch")
@@ -34,3 +35,22 @@ def test_other_chunks_are_refused(chunk):
     with pytest.raises(_lib.AxpicError) as e:
         make(2, base_params(decide_chunk=chunk))
     assert "INVALID" in str(e.value)
+
+
+def test_tuning_leaves_no_slower_shape():
+    """4,096 cells of 512 electrons and 256 photons: the rule takes 1 cell a
+    chunk, which none of the shapes that the tuner tries comes near (a step 7 %
+    slower at 4, 26 % at 8). And a shape slower than a tried one is replaced."""
+    kw = dict(T=np.full(4096, 3.0), caps=(512, 384, 384), counts=(512, 256, 16))
+    prm = base_params(dt_phys_s=8.8e11, g_ae=1e-13, w_a=1e12, tally_enable=0, diag_enable=0)
+    pl = make(4096, prm, **kw)
+    assert pl.launch_shape()[0] == 1
+    before = pl.launch_shape()
+    ms, chunk, warps = pl.autotune(0, 8)
+    assert ms > 0 and chunk in (4, 8, 16, 32) and warps in (2, 4)
+    assert pl.launch_shape() == before
+    pl.close()
+    pl = make(4096, dict(prm, decide_chunk=32), **kw)  # 128 warps' work at once: far too few
+    pl.autotune(0, 8)
+    assert pl.launch_shape()[0] in (4, 8)
+    pl.close()
