@@ -2015,9 +2015,15 @@ __device__ __forceinline__ void cell_lane(const StepArgs& A, uint32_t step, int 
 // taken by the warp one cell after the other (FP64 sums of 32 lanes for 24
 // axions, reduced by 20 adds of 1/64 rate, and three dependent round trips a
 // cell) the kernel took 341 us for 112,095 cells of 23 axions; a lane a cell
-// takes 100 us. Beyond 64 flagged axions the chain of one lane, about
-// 1 us an axion, gets longer than the warp's way through its cells.
+// takes 100 us. A warp lasts as long as its longest lane and, after that, each
+// of its heavy cells. With both in one warp it paid twice: where half of its
+// cells are heavy or more, those with more than kFewAbsorb axions flagged go
+// the warp's way as well. A call of absorption, us, 112,095 cells by the axions
+// sampled a cell: all by the warp, by each cell's own number, with this rule:
+//   60: 648, 377, 376   64: 669, 498, 502   70: 756, 893, 753   80: 785, 780, 767
+// (from 4 or 8 heavy cells on, 64: 642 and 555, 70: 734 and 733).
 constexpr int kLightAbsorb = 64;
+constexpr int kHeavyHalf = 16, kFewAbsorb = 16;
 
 __device__ __forceinline__ void absorb_lane(const StepArgs& A, int cell, uint32_t* row, LaneCell& L, const Cnt& cnt,
                                             Lane64& xa) {
@@ -2246,6 +2252,7 @@ __global__ void __launch_bounds__(128, PH == 3 ? AXPIC_EVENT_FULL_MIN_CTAS : AXP
       if (defer) A.heavy[A.cell0 + base + __popc(hm & ((1u << lane) - 1u))] = cell;
     }
   } else if (PH == PH_ABSORB) {
+    if (__popc(__ballot_sync(kFull, hA)) >= kHeavyHalf) hA = hA || L.nflA > kFewAbsorb;
     if (valid && !hA && L.nflA) absorb_lane(A, cell, rA, L, cnt, xa);
     __syncwarp();
     for (unsigned hm = __ballot_sync(kFull, valid && hA); hm; hm &= hm - 1u) {
