@@ -2007,26 +2007,39 @@ __device__ __forceinline__ void cell_lane(const StepArgs& A, uint32_t step, int 
 }
 
 // The absorb phase of a separate call by one lane: the cell's flagged axions
-// in slot order straight from its staged mask row (up to kLightAbsorb of
-// them, so no list is needed), the next one's record and momentum loaded
-// while one is decided, its position only if it converts. Words of the row
-// are cleared as they are read and take the removed slots' bits, which the
-// tail fill then follows. Weight reduction flags every axion of every cell:
-// taken by the warp one cell after the other (FP64 sums of 32 lanes for 24
-// axions, reduced by 20 adds of 1/64 rate, and three dependent round trips a
-// cell) the kernel took 341 us for 112,095 cells of 23 axions; a lane a cell
-// takes 100 us. A warp lasts as long as its longest lane and, after that, each
-// of its heavy cells. With both in one warp it paid twice: where half of its
-// cells are heavy or more, those with more than kFewAbsorb axions flagged go
-// the warp's way as well. A call of absorption, us, 112,095 cells by the axions
-// sampled a cell: all by the warp, by each cell's own number, with this rule:
-//   60: 648, 377, 376   64: 669, 498, 502   70: 756, 893, 753   80: 785, 780, 767
-// (from 4 or 8 heavy cells on, 64: 642 and 555, 70: 734 and 733).
-constexpr int kLightAbsorb = 64;
-constexpr int kHeavyHalf = 16, kFewAbsorb = 16;
+// in slot order straight from its staged mask row (any number of them, so no
+// list is needed), the next one's record and momentum loaded while one is
+// decided. Its position is loaded with them where most flagged axions convert
+// (ahead), else only if it converts. Words of the row are cleared as they are
+// read and take the removed slots' bits, which the tail fill then follows.
+//
+// Which cells (by the cell's own count and the launch's cells, so that the sums'
+// order does not depend on the cells beside it):
+// * Weight reduction flags every axion of every cell. A lane takes 0.7 to 0.9 us
+//   an axion, the warp 4 us a cell, 6 beyond 32 axions: 5 axions a cell of
+//   the warp, at most kManyAbsorb. A call of absorption, us, all cells by the
+//   warp / with a limit of 64 / with this one:
+//     cells   axions 24            60             70             140
+//     1        20   29   17     24   56   19    26   20   20     35   25   25
+//     16       73   35   36    101   71   72   120  112   83    167  155  155
+//     4,000   137   41   41    193   83   84   231  225   96    326  314  179
+//     112,000 423  154  155    650  359  359   762  741  412   1156 1119  798
+//   (without kManyAbsorb 4,000 cells of 1,000 axions with conversions take
+//   1865 instead of 1855 and 64 cells of 300 427 instead of 515.)
+// * Otherwise only axions with an event are flagged, and lanes that write
+//   products at places of their own take 3.7 us an axion in a full warp: up to
+//   kFewAbsorb, as many as the lists held at first (20,000 cells of 120 axions,
+//   a third of them flagged: 205 us by lists of 8, 331 with a limit of 64, 186
+//   now; limits of 4 and 12 lose 5 to 50 % where most cells have 5 to 8).
+constexpr int kFewAbsorb = 8, kManyAbsorb = 256, kWarpAxions = 5;
 
-__device__ __forceinline__ void absorb_lane(const StepArgs& A, int cell, uint32_t* row, LaneCell& L, const Cnt& cnt,
-                                            Lane64& xa) {
+__host__ __device__ constexpr int absorb_limit(bool all, int ncells) {
+  const int few = ncells < kManyAbsorb ? kWarpAxions * ncells : kManyAbsorb;
+  return !all || few < kFewAbsorb ? kFewAbsorb : few < kManyAbsorb ? few : kManyAbsorb;
+}
+
+__device__ __forceinline__ void absorb_lane(const StepArgs& A, int cell, uint32_t* row, bool ahead, LaneCell& L,
+                                            const Cnt& cnt, Lane64& xa) {
   const bool bath = A.mask & (AXPIC_CH_COMPTON | AXPIC_CH_BREMS);
   const long abase = (long)cell * A.a.cap, gbase = (long)cell * A.g.cap;
   const int n = L.na, nw = (n + 31) >> 5;
@@ -2044,12 +2057,13 @@ __device__ __forceinline__ void absorb_lane(const StepArgs& A, int cell, uint32_
     return 32 * w + b;
   };
   AxItem t;
-  float4 q;
+  float4 q, u;
   t.slot = next();
   t.x = t.y = t.z = 0.f;
   if (t.slot >= 0) {
     t.r = A.recA[abase + t.slot];
     q = A.a.wp[abase + t.slot];
+    if (ahead) u = A.a.xyz[abase + t.slot];
   }
   int run = 0, nrm = 0;
   while (t.slot >= 0) {
@@ -2059,14 +2073,16 @@ __device__ __forceinline__ void absorb_lane(const StepArgs& A, int cell, uint32_
     t.pz = q.w;
     const int slot2 = next();
     uint4 r2 = make_uint4(0, 0, 0, 0);
+    float4 u2;
     if (slot2 >= 0) {
       r2 = A.recA[abase + slot2];
       q = A.a.wp[abase + slot2];
+      if (ahead) u2 = A.a.xyz[abase + slot2];
     }
     bool removed;
     const int K = axion_outcome(A, t, abase, bath, cnt, xa, &removed);
     if (K > 0) {
-      const float4 u = A.a.xyz[abase + t.slot];
+      if (!ahead) u = A.a.xyz[abase + t.slot];
       const float wprod = __uint_as_float(t.r.y);
       const float3 pg = photon_from_axion(A, t.px, t.py, t.pz);
       for (int k = 0; k < K; ++k) {
@@ -2082,24 +2098,39 @@ __device__ __forceinline__ void absorb_lane(const StepArgs& A, int cell, uint32_
     }
     t.slot = slot2;
     t.r = r2;
+    u = u2;
   }
   L.ng = min(L.ng + run, A.g.cap);
   if (nrm == 0) return;
-  // tail fill: removed slots below ns, ascending, take the kept slots from ns on
+  // tail fill: removed slots below ns, ascending, take the kept slots from ns
+  // on, four at a time, all loaded before any is stored
   const int ns = n - nrm;
-  int src = ns;
-  for (int wd = 0; 32 * wd < ns; ++wd) {
-    uint32_t h = row[wd];
-    if (32 * wd + 32 > ns && (ns & 31)) h &= (1u << (ns & 31)) - 1u;
-    for (; h; h &= h - 1u) {
-      while ((row[src >> 5] >> (src & 31)) & 1u) ++src;
-      const long d = abase + 32 * wd + __ffs(h) - 1;
-      A.a.wp[d] = A.a.wp[abase + src];
-      const float4 u = A.a.xyz[abase + src];
-      A.a.xyz[d] = make_float4(u.x, u.y, u.z, 0.f);
-      ++src;
+  int src = ns, wd = -1;
+  uint32_t h = 0u;
+  auto hole = [&]() {  // the next removed slot below ns, or -1
+    while (h == 0u) {
+      if (32 * ++wd >= ns) return -1;
+      h = row[wd];
+      if (32 * wd + 32 > ns) h &= (1u << (ns & 31)) - 1u;
     }
-  }
+    const int b = __ffs(h) - 1;
+    h &= h - 1u;
+    return 32 * wd + b;
+  };
+  int dst;
+  do {
+    Mover m[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      dst = hole();
+      if (dst >= 0)
+        while ((row[src >> 5] >> (src & 31)) & 1u) ++src;
+      m[i] = mover_load(A.a, abase, src, dst);
+      if (dst >= 0) ++src;
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) mover_store(A.a, abase, m[i]);
+  } while (dst >= 0);
   L.na = ns;
 }
 
@@ -2203,7 +2234,7 @@ __global__ void __launch_bounds__(128, PH == 3 ? AXPIC_EVENT_FULL_MIN_CTAS : AXP
       else if (PH & PH_ABSORB) L.nflA = scan_row(rA, na_start, lA, &nzA);
       if (emitG) L.nflG = scan_row(rG, L.ng0, lG, &nzG);
       if (emitE) L.nflE = scan_row(rE, ne, lE, &nzE);
-      hA = L.nflA > (PH == PH_ABSORB ? kLightAbsorb : kLight);
+      hA = L.nflA > kLight;
       hE = L.nflG > kLight || L.nflE > kLightE;
       defer = PH == (PH_ABSORB | PH_EMIT) && (hA || hE);
       if (!defer) {
@@ -2252,8 +2283,9 @@ __global__ void __launch_bounds__(128, PH == 3 ? AXPIC_EVENT_FULL_MIN_CTAS : AXP
       if (defer) A.heavy[A.cell0 + base + __popc(hm & ((1u << lane) - 1u))] = cell;
     }
   } else if (PH == PH_ABSORB) {
-    if (__popc(__ballot_sync(kFull, hA)) >= kHeavyHalf) hA = hA || L.nflA > kFewAbsorb;
-    if (valid && !hA && L.nflA) absorb_lane(A, cell, rA, L, cnt, xa);
+    const bool all = A.absorb_mode == 1 && (mask & (AXPIC_CH_COMPTON | AXPIC_CH_BREMS));  // every axion is flagged
+    if (staged) hA = L.nflA > absorb_limit(all, A.ncells);
+    if (valid && !hA && L.nflA) absorb_lane(A, cell, rA, !all, L, cnt, xa);
     __syncwarp();
     for (unsigned hm = __ballot_sync(kFull, valid && hA); hm; hm &= hm - 1u) {
       const int j = __ffs(hm) - 1;

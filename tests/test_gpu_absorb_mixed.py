@@ -1,7 +1,6 @@
-"""The absorb phase of a separate call where a warp's cells are mostly heavy
-(more than 64 axions flagged): the lighter ones among them, on both sides of
-the 16 axions up to which a lane still takes them, against the oracle; and one
-heavy cell less than half of a warp (needs a GB300)."""
+"""The absorb phase of a separate call where about half of a warp's cells have
+more than 64 axions flagged and the others any number up to that, against the
+oracle (needs a GB300)."""
 import numpy as np
 import pytest
 
