@@ -278,8 +278,8 @@ axpic_status axpic_deposit_composition(axpic_ctx *ctx, int32_t bind_species, con
  * closed by the tail fill (the slot rule of a full step's axions). Staying
  * axions keep their slots unless the tail fill moves them. Axions beyond the
  * capacity are dropped, counted and latch AXPIC_E_CAPACITY. Asynchronous on the context's stream; the first
- * call allocates scratch (32.125 bytes per axion slot plus 64 per cell), later
- * calls allocate nothing. AXPIC_E_INVALID (nothing launched) for a grid
+ * call allocates scratch (32 bytes per axion slot, 64 + 4 ceil(capacity / 32)
+ * per cell and 16 KiB), later calls allocate nothing. AXPIC_E_INVALID (nothing launched) for a grid
  * that does not match, h_cm <= 0, dt_s < 0, c dt_s >= h_cm or another
  * boundary value, or a negative mass. */
 axpic_status axpic_stream_axions(axpic_ctx *ctx, int32_t nx, int32_t ny, int32_t nz, double h_cm, double dt_s,

@@ -118,7 +118,7 @@ struct axpic_ctx {
   uint32_t* st_freed = nullptr;  // [ncells * words of the axion capacity]
   uint16_t* st_off = nullptr;    // [ncells * kStreamOffs]
   float* st_buf = nullptr;    // [ncells * axion capacity * 8]
-  double* st_stats = nullptr; // [4]
+  double* st_stats = nullptr; // [kStreamRows * kStreamRow]
   // axion merging scratch, made by the first axpic_merge_axions call
   double* mg_removed = nullptr;
   int mg_fit = 0;             // the merge kernel's largest grid
@@ -1343,8 +1343,8 @@ static axpic_status stream_setup(axpic_ctx* ctx, int32_t nx, int32_t ny, int32_t
     CK(cudaMalloc((void**)&ctx->st_freed, sizeof(uint32_t) * std::max<size_t>(words, 1)), "streaming scratch");
     CK(cudaMalloc((void**)&ctx->st_off, sizeof(uint16_t) * kStreamOffs * (size_t)d.ncells), "streaming scratch");
     CK(cudaMalloc((void**)&ctx->st_buf, sizeof(float) * 8 * std::max<size_t>(slots, 1)), "streaming scratch");
-    CK(cudaMalloc((void**)&ctx->st_stats, sizeof(double) * 4), "streaming scratch");
-    CK(cudaMemsetAsync(ctx->st_stats, 0, sizeof(double) * 4, ctx->stream), "memset");
+    CK(cudaMalloc((void**)&ctx->st_stats, sizeof(double) * kStreamRows * kStreamRow), "streaming scratch");
+    CK(cudaMemsetAsync(ctx->st_stats, 0, sizeof(double) * kStreamRows * kStreamRow, ctx->stream), "memset");
   }
   StreamArgs a;
   std::memset(&a, 0, sizeof(a));
@@ -1454,8 +1454,11 @@ axpic_status axpic_stream_stats(axpic_ctx* ctx, double* out) {
   if (!ctx || !out) return AXPIC_E_INVALID;
   for (int i = 0; i < 4; ++i) out[i] = 0.0;
   if (!ctx->st_stats) return AXPIC_OK;
-  CK(cudaMemcpyAsync(out, ctx->st_stats, sizeof(double) * 4, cudaMemcpyDeviceToHost, ctx->stream), "copy");
+  double rows[kStreamRows * kStreamRow];
+  CK(cudaMemcpyAsync(rows, ctx->st_stats, sizeof(rows), cudaMemcpyDeviceToHost, ctx->stream), "copy");
   CK(cudaStreamSynchronize(ctx->stream), "synchronize");
+  for (int r = 0; r < kStreamRows; ++r)
+    for (int i = 0; i < 4; ++i) out[i] += rows[r * kStreamRow + i];
   return AXPIC_OK;
 }
 

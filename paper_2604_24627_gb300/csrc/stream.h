@@ -14,6 +14,10 @@ constexpr int kStreamDirs = 27, kStreamStay = 13;
 // direction below d, entry 27 all of them (64 bytes, two sectors)
 constexpr int kStreamOffs = 32;
 
+// rows of the escape and drop sums, added up when they are read, and doubles per
+// row (a 128-byte line)
+constexpr int kStreamRows = 128, kStreamRow = 16;
+
 struct StreamArgs {
   SpeciesPtrs s;       // the axion slabs (positions rewritten, slots re-binned)
   int ncells, nx, ny, nz;
@@ -23,7 +27,7 @@ struct StreamArgs {
   uint32_t* freed;     // [ncells * ceil(cap / 32)]: a bit per slot whose axion does not stay
   uint16_t* goff;      // [ncells * kStreamOffs]: each direction's first row in the cell's staging rows
   float* buf;          // [ncells * cap * 8]: the cell's leaving axions, grouped by direction
-  double* stats;       // [4]: escaped number, weight, weight x energy [keV]; dropped number
+  double* stats;       // [kStreamRows * kStreamRow], each row's first 4: escaped number, weight, weight x energy [keV]; dropped number
   int* err;            // latched error flags (ERR_CAPACITY)
 };
 
