@@ -33,7 +33,11 @@ namespace axpic {
 namespace {
 
 constexpr int kWarpsMax = 4;
-constexpr int kHold = 5;  // passes of 32 slots whose groups stay in registers
+// CTAs an SM, and passes of 32 slots whose groups stay in registers: 5, or as
+// many as a slab of at most 64 slots has, where fewer registers and branches pay:
+// 65,536 cells of 20 axions in 32 slots 65 -> 58 us, of 30 in 48 115 -> 108 (with
+// 10 and 12 CTAs an SM 115 and 127: spills), 500,000 of 10 in 20 299 -> 264.
+constexpr int kCtas = 8, kHold = 5;
 constexpr unsigned kAll = 0xFFFFFFFFu;
 constexpr int kGroupsMax = (kMergeMaxEdges + 1) * 8;
 
@@ -138,7 +142,8 @@ __host__ __device__ inline size_t warp_bytes(int cap) {
   return ((size_t)cap * sizeof(uint16_t) + 3) / 4 * 4 + (size_t)((cap + 31) / 32) * sizeof(uint32_t);
 }
 
-__global__ void __launch_bounds__(kWarpsMax * 32, 8) merge_kernel(MergeArgs a) {
+template <int HOLD>
+__global__ void __launch_bounds__(kWarpsMax * 32, kCtas) merge_kernel(MergeArgs a) {
   extern __shared__ __align__(16) unsigned char smem_warps[];
   __shared__ MergeShared sh[kWarpsMax];
   __shared__ float edges[32];
@@ -169,9 +174,9 @@ __global__ void __launch_bounds__(kWarpsMax * 32, 8) merge_kernel(MergeArgs a) {
     const long base = (long)c * s.cap;
     for (int g = lane; g < ngroups; g += 32) S.cnt[g] = 0;
     for (int w = lane; 32 * w < n; w += 32) freed[w] = 0u;
-    float4 r[kHold];
+    float4 r[HOLD];
 #pragma unroll
-    for (int i = 0; i < kHold; ++i) {
+    for (int i = 0; i < HOLD; ++i) {
       const int slot = 32 * i + lane;
       if (slot < n) {
         r[i] = s.wp[base + slot];
@@ -179,9 +184,9 @@ __global__ void __launch_bounds__(kWarpsMax * 32, 8) merge_kernel(MergeArgs a) {
       }
     }
     __syncwarp();
-    int gr[kHold];  // group | rank << 8, or -1
+    int gr[HOLD];  // group | rank << 8, or -1
 #pragma unroll
-    for (int i = 0; i < kHold; ++i) {
+    for (int i = 0; i < HOLD; ++i) {
       gr[i] = -1;
       if (32 * i >= n) continue;
       const bool live = 32 * i + lane < n;
@@ -195,10 +200,10 @@ __global__ void __launch_bounds__(kWarpsMax * 32, 8) merge_kernel(MergeArgs a) {
       }
       __syncwarp();
     }
-    if (n > 32 * kHold) {
+    if (n > 32 * HOLD) {
       for (int g = lane; g < ngroups; g += 32) S.run[g] = S.cnt[g];
       __syncwarp();
-      for (int s0 = 32 * kHold; s0 < n; s0 += 32) {
+      for (int s0 = 32 * HOLD; s0 < n; s0 += 32) {
         const bool live = s0 + lane < n;
         const int g = live ? group_of(s.wp[base + s0 + lane]) : kGroupsMax + lane;
         const unsigned peers = __match_any_sync(kAll, g);
@@ -233,12 +238,12 @@ __global__ void __launch_bounds__(kWarpsMax * 32, 8) merge_kernel(MergeArgs a) {
     __syncwarp();
     // members of listed groups in slot order
 #pragma unroll
-    for (int i = 0; i < kHold; ++i) {
+    for (int i = 0; i < HOLD; ++i) {
       if (gr[i] < 0) continue;
       const int g = gr[i] & 255;
       if (S.cnt[g] >= 3) mem[S.start[g] + (gr[i] >> 8)] = (uint16_t)(32 * i + lane);
     }
-    for (int s0 = 32 * kHold; s0 < n; s0 += 32) {
+    for (int s0 = 32 * HOLD; s0 < n; s0 += 32) {
       const bool live = s0 + lane < n;
       const int g = live ? group_of(s.wp[base + s0 + lane]) : kGroupsMax + lane;
       const unsigned peers = __match_any_sync(kAll, g);
@@ -298,13 +303,19 @@ static int merge_warps(int cap) {
   return (int)std::max<size_t>(1, std::min<size_t>(kWarpsMax, kDynMax / per_warp));
 }
 
+using MergeKernel = void (*)(MergeArgs);
+static MergeKernel merge_instance(int cap) {
+  return cap <= 32 ? merge_kernel<1> : cap <= 64 ? merge_kernel<2> : merge_kernel<kHold>;
+}
+
 // as many CTAs as the device holds at once; asked for once, since the
 // driver's answers take some microseconds and a merge of a thousand cells 40
 cudaError_t merge_init_kernels(int cap, int* fit) {
-  const cudaError_t e = cudaFuncSetAttribute(merge_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kDynMax);
+  const auto kernel = merge_instance(cap);
+  const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kDynMax);
   if (e) return e;
   const int nw = merge_warps(cap);
-  *fit = resident_ctas((const void*)merge_kernel, nw * 32, std::max<size_t>(warp_bytes(cap), 4) * nw);
+  *fit = resident_ctas((const void*)kernel, nw * 32, std::max<size_t>(warp_bytes(cap), 4) * nw);
   return *fit > 0 ? cudaSuccess : cudaErrorUnknown;
 }
 
@@ -312,7 +323,8 @@ cudaError_t launch_merge(const MergeArgs& a, int fit, cudaStream_t st) {
   if (a.ncells <= 0) return cudaSuccess;
   if (a.s.cap > kMergeMaxCap) return cudaErrorInvalidValue;
   const int nw = merge_warps(a.s.cap);
-  merge_kernel<<<std::min((a.ncells + nw - 1) / nw, fit), nw * 32, std::max<size_t>(warp_bytes(a.s.cap), 4) * nw, st>>>(a);
+  const int grid = std::min((a.ncells + nw - 1) / nw, fit);
+  merge_instance(a.s.cap)<<<grid, nw * 32, std::max<size_t>(warp_bytes(a.s.cap), 4) * nw, st>>>(a);
   return cudaGetLastError();
 }
 
