@@ -1283,9 +1283,10 @@ axpic_status axpic_set_surrogate(axpic_ctx* ctx, axpic_mlp* m, const float* err_
       }
   cudaStream_t st = ctx->stream;
   CK(cudaStreamSynchronize(st), "synchronize");
+  uint8_t* map = nullptr;  // (a call that fails here leaves the old network in use)
+  CK(cudaMalloc((void**)&map, trust.size()), "trust map");
   if (ctx->sur_trust) cudaFree(ctx->sur_trust);
-  ctx->sur_trust = nullptr;
-  CK(cudaMalloc((void**)&ctx->sur_trust, trust.size()), "trust map");
+  ctx->sur_trust = map;
   CK(cudaMemcpyAsync(ctx->sur_P, P.data(), sizeof(float) * P.size(), cudaMemcpyHostToDevice, st), "params");
   CK(cudaMemcpyAsync(ctx->sur_mu, mu.data(), sizeof(float) * 96, cudaMemcpyHostToDevice, st), "norm");
   CK(cudaMemcpyAsync(ctx->sur_sigma, sigma.data(), sizeof(float) * 96, cudaMemcpyHostToDevice, st), "norm");
@@ -1324,6 +1325,11 @@ axpic_status axpic_get_cell_records(axpic_ctx* ctx, int32_t first, int32_t count
   return AXPIC_OK;
 }
 
+// Device memory of at least one byte, unless *p has it already.
+static cudaError_t make_once(void** p, size_t bytes) {
+  return *p ? cudaSuccess : cudaMalloc(p, std::max<size_t>(bytes, 1));
+}
+
 // Validates the streaming parameters, makes the scratch on first use and fills
 // the kernels' arguments (nothing is launched).
 static axpic_status stream_setup(axpic_ctx* ctx, int32_t nx, int32_t ny, int32_t nz, double h_cm, double dt_s,
@@ -1338,13 +1344,14 @@ static axpic_status stream_setup(axpic_ctx* ctx, int32_t nx, int32_t ny, int32_t
   if (!(kappa < 1.0f - 0x1p-20f))
     return fail(ctx, AXPIC_E_INVALID, "axpic_stream_axions: c dt must stay below the cell edge");
   const size_t slots = (size_t)d.ncells * d.axions.capacity;
-  if (!ctx->st_freed) {
+  if (!ctx->st_stats) {  // the last one made: a call after one that failed makes what is missing
     const size_t words = (size_t)d.ncells * ((d.axions.capacity + 31) / 32);
-    CK(cudaMalloc((void**)&ctx->st_freed, sizeof(uint32_t) * std::max<size_t>(words, 1)), "streaming scratch");
-    CK(cudaMalloc((void**)&ctx->st_off, sizeof(uint16_t) * kStreamOffs * (size_t)d.ncells), "streaming scratch");
-    CK(cudaMalloc((void**)&ctx->st_buf, sizeof(float) * 8 * std::max<size_t>(slots, 1)), "streaming scratch");
-    CK(cudaMalloc((void**)&ctx->st_stats, sizeof(double) * kStreamRows * kStreamRow), "streaming scratch");
-    CK(cudaMemsetAsync(ctx->st_stats, 0, sizeof(double) * kStreamRows * kStreamRow, ctx->stream), "memset");
+    const size_t stats = sizeof(double) * kStreamRows * kStreamRow;
+    CK(make_once((void**)&ctx->st_freed, sizeof(uint32_t) * words), "streaming scratch");
+    CK(make_once((void**)&ctx->st_off, sizeof(uint16_t) * kStreamOffs * (size_t)d.ncells), "streaming scratch");
+    CK(make_once((void**)&ctx->st_buf, sizeof(float) * 8 * slots), "streaming scratch");
+    CK(make_once((void**)&ctx->st_stats, stats), "streaming scratch");
+    CK(cudaMemsetAsync(ctx->st_stats, 0, stats, ctx->stream), "memset");
   }
   StreamArgs a;
   std::memset(&a, 0, sizeof(a));

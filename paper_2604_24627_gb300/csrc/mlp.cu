@@ -455,9 +455,9 @@ Mlp::~Mlp() {
 // The training CTAs (one an SM: a tile's buffers and all of its tensor
 // memory) and their gradient rows, made by the first training call.
 cudaError_t Mlp::reserve_train() {
-  if (part) return cudaSuccess;
-  cudaError_t e;
-  if ((e = cudaMalloc(&part, sizeof(float) * kMlpParams * (size_t)sms))) return e;
+  if (losses) return cudaSuccess;
+  cudaError_t e;  // (part may be there from a call that failed)
+  if (!part && (e = cudaMalloc(&part, sizeof(float) * kMlpParams * (size_t)sms))) return e;
   return cudaMalloc(&losses, sizeof(double) * (size_t)sms);
 }
 
