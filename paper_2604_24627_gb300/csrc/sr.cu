@@ -66,17 +66,19 @@ void build_sr_table(int nkt, int nne, double brems_shape, float* out) {
 
 // ---------------------------------------------------------------- table model
 // The records as they are read out and saved (the step interpolates the
-// entries it needs). A CTA takes 32 cells: warp 0 forms each cell's
-// interpolation constants (lane per cell) in shared memory, then the CTA's
-// threads stream the 32 x 192 record entries (consecutive threads,
-// consecutive entries of a cell); under the surrogate model too every cell's,
-// so that what is read or saved does not depend on what was there before.
-constexpr int kSrTableThreads = 256;
+// entries it needs). A CTA takes 4 cells: a lane each forms their
+// interpolation constants in shared memory, then the CTA's threads stream the
+// 4 x 192 record entries (consecutive threads, consecutive entries of a cell),
+// three a thread: few cells are what is read (40: 27 us with 32 cells a CTA,
+// 24 entries a thread; now 19, and 13 for the copy alone). Under the surrogate
+// model too every cell's, so that what is read or saved does not depend on what
+// was there before.
+constexpr int kSrTableThreads = 256, kSrTableCells = 4;
 __global__ void __launch_bounds__(kSrTableThreads) sr_table_kernel(SrArgs a) {
-  __shared__ SrInterp ip[32];
-  const int c0 = a.cell0 + blockIdx.x * 32;
-  const int nc = min(32, a.cell0 + a.ncells - c0);
-  if (threadIdx.x < 32 && (int)threadIdx.x < nc)
+  __shared__ SrInterp ip[kSrTableCells];
+  const int c0 = a.cell0 + blockIdx.x * kSrTableCells;
+  const int nc = min(kSrTableCells, a.cell0 + a.ncells - c0);
+  if ((int)threadIdx.x < nc)
     sr_interp(a.ra, sr_cell_from(a.rec + (size_t)(c0 + threadIdx.x) * kRecLen, a.ra.k_T7), &ip[threadIdx.x]);
   __syncthreads();
   for (int e = threadIdx.x; e < nc * kSrLen; e += kSrTableThreads) {
@@ -87,7 +89,7 @@ __global__ void __launch_bounds__(kSrTableThreads) sr_table_kernel(SrArgs a) {
 
 cudaError_t launch_sr_table(const SrArgs& a, cudaStream_t st) {
   if (a.ncells <= 0) return cudaSuccess;
-  sr_table_kernel<<<(a.ncells + 31) / 32, kSrTableThreads, 0, st>>>(a);
+  sr_table_kernel<<<(a.ncells + kSrTableCells - 1) / kSrTableCells, kSrTableThreads, 0, st>>>(a);
   return cudaGetLastError();
 }
 
