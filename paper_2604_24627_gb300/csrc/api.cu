@@ -75,7 +75,7 @@ struct axpic_ctx {
   int32_t* photon_start = nullptr;
   float* tables = nullptr;
   double* tally = nullptr;       // the folded tally: 3 nbins + 6 sums
-  double* tally_rows = nullptr;  // after it: what the event kernels add to since the last fold
+  double* tally_rows = nullptr;  // what the event kernels add to since the last fold: rows after it, or itself where one is enough
   int tally_nrows = 1;
   long tally_stride = 0;         // doubles per row
   unsigned long long* counters = nullptr;
@@ -91,6 +91,7 @@ struct axpic_ctx {
   int max_warps = 4;  // largest event CTA (warps) whose scratch fits
   int ctr_rows = 1;   // rows of per-CTA counters
   int dec_grid = 1;   // CTAs of the persistent decision kernel
+  int tot_grid = 1;   // and, at most, of the totals kernel (asked for once: the driver's answers take some microseconds)
   int dec_chunk = 0;  // cells per chunk of its warps; 0: by the launch's cells
   uint32_t* step_dev = nullptr;      // step counter of replayed graphs
   int32_t* heavy = nullptr;          // cells left to the warp-path event kernel
@@ -527,12 +528,14 @@ axpic_status axpic_init_plasma(axpic_ctx** out, const axpic_plasma_desc* desc, c
   ALLOC(ctx->tables, sizeof(float) * kNumTables * kTableN);
   ctx->tally_stride = (3 * (long)p.tally_nbins + 6 + 15) / 16 * 16;  // rows on 128-byte lines
   ctx->tally_nrows = 1;
-  // no more rows than event CTAs can use (a small plasma keeps one)
-  while (ctx->tally_nrows < std::min(kTallyRows, (n + 127) / 128) && 2 * sizeof(double) * ctx->tally_nrows * (size_t)ctx->tally_stride <= kTallyBytes)
+  // no more rows than event CTAs can use (a small plasma keeps one, and so does
+  // one without a tally)
+  while (p.tally_enable && ctx->tally_nrows < std::min(kTallyRows, (n + 127) / 128) && 2 * sizeof(double) * ctx->tally_nrows * (size_t)ctx->tally_stride <= kTallyBytes)
     ctx->tally_nrows *= 2;
-  const size_t tally_bytes = sizeof(double) * (1 + ctx->tally_nrows) * (size_t)ctx->tally_stride;
+  const int extra = ctx->tally_nrows > 1 ? ctx->tally_nrows : 0;
+  const size_t tally_bytes = sizeof(double) * (1 + extra) * (size_t)ctx->tally_stride;
   ALLOC(ctx->tally, tally_bytes);
-  ctx->tally_rows = ctx->tally + ctx->tally_stride;
+  ctx->tally_rows = ctx->tally + (extra ? ctx->tally_stride : 0);
   ALLOC(ctx->counters, sizeof(unsigned long long) * kNumCounters * (size_t)ctx->ctr_rows);
   ALLOC(ctx->step_dev, sizeof(uint32_t) * kMaxBranches);
   ALLOC(ctx->heavy, sizeof(int32_t) * (size_t)n);
@@ -577,7 +580,7 @@ axpic_status axpic_init_plasma(axpic_ctx** out, const axpic_plasma_desc* desc, c
       (e = cudaMemsetAsync(ctx->heavy_n, 0, sizeof(int32_t) * kMaxBranches, st)) ||
       (e = cudaMemsetAsync(ctx->bits, 0, sizeof(uint32_t) * (bit_words > 0 ? bit_words : 1), st)) ||
       (e = set_step_smem_limits(per_warp * ctx->max_warps)) ||
-      (e = decide_resident_ctas(&ctx->dec_grid)) ||
+      (e = decide_resident_ctas(&ctx->dec_grid)) || (e = totals_resident_ctas(&ctx->tot_grid)) ||
       (e = launch_records(n, d.nspecies, ctx->cc, d.T_keV, d.n_ion, ctx->rec, ctx->err, st)) ||
       (e = launch_moments(n, to_ptrs(d.electrons), ctx->mom, st)) ||
       (p.rate_model && (e = cudaMemcpyAsync(ctx->srtab, srtab.data(), srtab.size() * sizeof(float),
@@ -727,10 +730,12 @@ axpic_status axpic_step_cells(axpic_ctx* ctx, int64_t step, int32_t channel_mask
 
 // Adds the event kernels' tally rows to the folded tally and clears them.
 static cudaError_t fold_tally(axpic_ctx* ctx) {
+  if (ctx->tally_rows == ctx->tally) return cudaSuccess;
   return launch_fold_tally(ctx->tally_rows, ctx->tally_nrows, ctx->tally_stride, 3 * ctx->prm.tally_nbins + 6,
                            ctx->tally, ctx->stream);
 }
 static cudaError_t clear_tally_rows(axpic_ctx* ctx) {
+  if (ctx->tally_rows == ctx->tally) return cudaSuccess;  // (the one row is about to be loaded)
   return cudaMemsetAsync(ctx->tally_rows, 0, sizeof(double) * ctx->tally_nrows * (size_t)ctx->tally_stride,
                          ctx->stream);
 }
@@ -756,7 +761,7 @@ axpic_status axpic_tally_spectrum(axpic_ctx* ctx, int32_t nbins, double* H_out, 
   std::vector<double> h(hn), tot(8 + kNumCounters);
   CK(launch_totals(d.ncells, to_ptrs(d.electrons), to_ptrs(d.photons), to_ptrs(d.axions), ctx->res, ctx->counters,
                    ctx->ctr_rows, ctx->scratch, ctx->scratch + 8, ctx->scratch + 8 + kNumCounters,
-                   kInfoChunk * AXPIC_CELL_INFO_LEN / 8, st),
+                   kInfoChunk * AXPIC_CELL_INFO_LEN / 8, ctx->tot_grid, st),
      "totals");
   CK(fold_tally(ctx), "fold tally");
   CK(cudaMemcpyAsync(h.data(), ctx->tally, hn * sizeof(double), cudaMemcpyDeviceToHost, st), "copy tally");

@@ -306,7 +306,8 @@ __global__ void __launch_bounds__(kColThreads) columns_kernel(const unsigned lon
 }
 
 // Folds the tally rows: thread (x, y) sums rows y, y + 32, ... of entry x,
-// its loads issued together.
+// its loads issued together; no more threads than rows (8 rows of 60,006 entries:
+// a tally of 1,000 cells 184 -> 133 us without the idle ones).
 constexpr int kFoldY = 32;
 __global__ void __launch_bounds__(32 * kFoldY) fold_tally_kernel(double* __restrict__ rows, int nrows, long stride,
                                                                  int n, double* __restrict__ tally) {
@@ -332,13 +333,13 @@ __global__ void __launch_bounds__(32 * kFoldY) fold_tally_kernel(double* __restr
   __syncthreads();
   if (threadIdx.y == 0 && i < n) {
     double t = 0.0;
-    for (int y = 0; y < kFoldY; ++y) t += part[y][threadIdx.x];
+    for (int y = 0; y < (int)blockDim.y; ++y) t += part[y][threadIdx.x];
     tally[i] += t;
   }
 }
 
 cudaError_t launch_fold_tally(double* rows, int nrows, long stride, int n, double* tally, cudaStream_t st) {
-  fold_tally_kernel<<<(n + 31) / 32, dim3(32, kFoldY), 0, st>>>(rows, nrows, stride, n, tally);
+  fold_tally_kernel<<<(n + 31) / 32, dim3(32, min(nrows, kFoldY)), 0, st>>>(rows, nrows, stride, n, tally);
   return cudaGetLastError();
 }
 
@@ -455,13 +456,16 @@ __global__ void __launch_bounds__(kTotThreads) totals_kernel(int ncells, Species
   }
 }
 
+cudaError_t totals_resident_ctas(int* out) {
+  *out = resident_ctas((const void*)totals_kernel, kTotThreads, 0);
+  return *out > 0 ? cudaSuccess : cudaErrorUnknown;
+}
+
 cudaError_t launch_totals(int ncells, const SpeciesPtrs& e, const SpeciesPtrs& g, const SpeciesPtrs& a,
                           const double* res, const unsigned long long* ctr, int ctr_rows, double* out8,
-                          double* out_ctr, double* part, int max_parts, cudaStream_t st) {
+                          double* out_ctr, double* part, int max_parts, int fit, cudaStream_t st) {
   int grid = 0;
   if (ncells > 0) {
-    const int fit = resident_ctas((const void*)totals_kernel, kTotThreads, 0);
-    if (fit <= 0) return cudaErrorUnknown;
     grid = (ncells + kTotWarps * kTotCells - 1) / (kTotWarps * kTotCells);
     grid = min(min(grid, fit), max_parts);
     totals_kernel<<<grid, kTotThreads, 0, st>>>(ncells, e, g, a, res, part);

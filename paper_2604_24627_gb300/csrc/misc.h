@@ -34,10 +34,13 @@ cudaError_t launch_rates(const float* rec, int cell, const float* E, int n, int 
 // tally[i] += sum over the rows of rows[r * stride + i], i < n, in row order;
 // the rows are cleared.
 cudaError_t launch_fold_tally(double* rows, int nrows, long stride, int n, double* tally, cudaStream_t st);
+// CTAs of the totals kernel that the current device holds at once.
+cudaError_t totals_resident_ctas(int* out);
 // The tally's totals: out8 (8 doubles) the particle sums, out_ctr the counters'
-// column sums; part: scratch of 8 max_parts doubles.
+// column sums; part: scratch of 8 max_parts doubles; fit: the largest grid
+// (totals_resident_ctas).
 cudaError_t launch_totals(int ncells, const SpeciesPtrs& e, const SpeciesPtrs& g, const SpeciesPtrs& a,
                           const double* res, const unsigned long long* ctr, int ctr_rows, double* out8,
-                          double* out_ctr, double* part, int max_parts, cudaStream_t st);
+                          double* out_ctr, double* part, int max_parts, int fit, cudaStream_t st);
 
 }  // namespace axpic
