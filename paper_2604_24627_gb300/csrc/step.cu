@@ -2010,7 +2010,7 @@ __device__ __forceinline__ void cell_lane(const StepArgs& A, uint32_t step, int 
 // in slot order straight from its staged mask row (any number of them, so no
 // list is needed), the next one's record and momentum loaded while one is
 // decided. Its position is loaded with them where most flagged axions convert
-// (ahead), else only if it converts. Words of the row are cleared as they are
+// (AHEAD), else only if it converts. Words of the row are cleared as they are
 // read and take the removed slots' bits, which the tail fill then follows.
 //
 // Which cells (by the cell's own count and the launch's cells, so that the sums'
@@ -2038,8 +2038,9 @@ __host__ __device__ constexpr int absorb_limit(bool all, int ncells) {
   return !all || few < kFewAbsorb ? kFewAbsorb : few < kManyAbsorb ? few : kManyAbsorb;
 }
 
-__device__ __forceinline__ void absorb_lane(const StepArgs& A, int cell, uint32_t* row, bool ahead, LaneCell& L,
-                                            const Cnt& cnt, Lane64& xa) {
+template <bool AHEAD>
+__device__ __forceinline__ void absorb_lane(const StepArgs& A, int cell, uint32_t* row, LaneCell& L, const Cnt& cnt,
+                                            Lane64& xa) {
   const bool bath = A.mask & (AXPIC_CH_COMPTON | AXPIC_CH_BREMS);
   const long abase = (long)cell * A.a.cap, gbase = (long)cell * A.g.cap;
   const int n = L.na, nw = (n + 31) >> 5;
@@ -2063,7 +2064,7 @@ __device__ __forceinline__ void absorb_lane(const StepArgs& A, int cell, uint32_
   if (t.slot >= 0) {
     t.r = A.recA[abase + t.slot];
     q = A.a.wp[abase + t.slot];
-    if (ahead) u = A.a.xyz[abase + t.slot];
+    if (AHEAD) u = A.a.xyz[abase + t.slot];
   }
   int run = 0, nrm = 0;
   while (t.slot >= 0) {
@@ -2077,12 +2078,12 @@ __device__ __forceinline__ void absorb_lane(const StepArgs& A, int cell, uint32_
     if (slot2 >= 0) {
       r2 = A.recA[abase + slot2];
       q = A.a.wp[abase + slot2];
-      if (ahead) u2 = A.a.xyz[abase + slot2];
+      if (AHEAD) u2 = A.a.xyz[abase + slot2];
     }
     bool removed;
     const int K = axion_outcome(A, t, abase, bath, cnt, xa, &removed);
     if (K > 0) {
-      if (!ahead) u = A.a.xyz[abase + t.slot];
+      if (!AHEAD) u = A.a.xyz[abase + t.slot];
       const float wprod = __uint_as_float(t.r.y);
       const float3 pg = photon_from_axion(A, t.px, t.py, t.pz);
       for (int k = 0; k < K; ++k) {
@@ -2285,7 +2286,10 @@ __global__ void __launch_bounds__(128, PH == 3 ? AXPIC_EVENT_FULL_MIN_CTAS : AXP
   } else if (PH == PH_ABSORB) {
     const bool all = A.absorb_mode == 1 && (mask & (AXPIC_CH_COMPTON | AXPIC_CH_BREMS));  // every axion is flagged
     if (staged) hA = L.nflA > absorb_limit(all, A.ncells);
-    if (valid && !hA && L.nflA) absorb_lane(A, cell, rA, !all, L, cnt, xa);
+    if (valid && !hA && L.nflA) {
+      if (all) absorb_lane<false>(A, cell, rA, L, cnt, xa);
+      else absorb_lane<true>(A, cell, rA, L, cnt, xa);
+    }
     __syncwarp();
     for (unsigned hm = __ballot_sync(kFull, valid && hA); hm; hm &= hm - 1u) {
       const int j = __ffs(hm) - 1;
