@@ -360,7 +360,8 @@ axpic_status axpic_emit(axpic_ctx *ctx, int64_t step, int32_t channel_mask);
 axpic_status axpic_feedback(axpic_ctx *ctx, int64_t step);
 
 /* One step, absorb -> emit -> feedback: the three calls above enqueued
- * together (identical results). */
+ * together (the same events and particles, new axions in other slots; sums of
+ * the exchange may differ in their last bits). */
 axpic_status axpic_step(axpic_ctx *ctx, int64_t step, int32_t channel_mask);
 /* One full step, as axpic_step, over the cells [first_cell, first_cell +
  * ncells) only. Cells are independent within a step (every operator is

@@ -1,24 +1,27 @@
 // The per-cell step: absorb -> emit -> feedback (Sec. II.D-II.J).
 //
-// A step is three kernels:
+// A step is four kernels (five with an evolved temperature under the surrogate
+// model, sr.cu), each started while its predecessor ends:
 //  * decide_kernel: persistent warps over chunks of consecutive cells, lane
-//    per quad of consecutive slots (float4 loads from the SoA slabs, one
+//    per quad of consecutive slots (16-byte records {w, p} of the slabs, one
 //    Philox4x32-10 block per quad and stream, word j for slot 4q+j). Each
 //    slot gets a cheap exact test that proves "no event this step"; slots it
 //    cannot clear are flagged in a per-cell bit mask and their full decision
 //    is taken from per-warp lists, 32 at a time, into slot-indexed records.
 //    This kernel carries almost all the per-particle work.
-//  * event_kernel: one warp per cell. It reads the bit masks and the records
-//    of the flagged slots, writes products and refills removed slots at
-//    offsets from warp prefix sums, so the output order is the deterministic
-//    one of the method's definition, and accumulates the FP64 exchange
-//    (Delta E, Delta P).
-//  * feedback_kernel: thread per cell for the temperature update; the rare
-//    cells whose exchange needs an affine remap are remapped by the CTA's
-//    warps side by side.
-// The separate API calls run the same kernels with a subset of the passes;
-// the exchange passes through an FP64 per-cell buffer in the same summation
-// order, so results do not depend on how a step is called.
+//  * event_kernel: a lane per cell, 4, 8 or 32 cells a warp. It reads the bit
+//    masks and the records of the flagged slots, writes products and refills
+//    removed slots in the deterministic order of the method's definition, and
+//    accumulates the FP64 exchange (Delta E, Delta P). Cells with more flagged
+//    slots than a lane takes are listed for
+//  * event_heavy_kernel: a warp per listed cell, offsets from warp prefix sums.
+//  * feedback_kernel: thread per cell for the temperature update; the cells
+//    whose exchange needs an affine remap are remapped by their warp.
+// The separate API calls run the same kernels with a subset of the passes (the
+// event kernel's warps take their own heavy cells). The exchange passes through
+// an FP64 per-cell buffer; a lane adds its events in slot order and a warp by
+// halves, so the two ways differ in a sum's last bits. Which way a cell takes
+// depends, in a full step, on its own flagged slots alone.
 #include <mutex>
 
 #include "common.cuh"
@@ -32,12 +35,6 @@ constexpr unsigned kFull = 0xFFFFFFFFu;
 __device__ __forceinline__ int lane_id() { return threadIdx.x & 31; }
 
 __device__ __forceinline__ int warp_sum_i(int v) {
-#pragma unroll
-  for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(kFull, v, o);
-  return v;
-}
-
-__device__ __forceinline__ float warp_sum_f(float v) {
 #pragma unroll
   for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(kFull, v, o);
   return v;
@@ -59,12 +56,6 @@ __device__ __forceinline__ int warp_excl_scan(int v, int* total) {
   }
   *total = __shfl_sync(kFull, x, 31);
   return x - v;
-}
-
-// Plain (coherent) 128-bit load: slabs are also written by this kernel.
-__device__ __forceinline__ float4 ld4(const float* p) { return *reinterpret_cast<const float4*>(p); }
-__device__ __forceinline__ float f4(const float4& v, int j) {
-  return j == 0 ? v.x : (j == 1 ? v.y : (j == 2 ? v.z : v.w));
 }
 
 __device__ __forceinline__ bool bit(const uint32_t* b, int i) { return (b[i >> 5] >> (i & 31)) & 1u; }
@@ -1272,11 +1263,12 @@ __global__ void __launch_bounds__(kFeedbackThreads, DENSE ? 4 : 5) feedback_kern
 
 
 // ---------------------------------------------------------------- event kernel
-// Warp w takes cells [32 w, 32 w + 32), lane l cell 32 w + l. Most cells
-// have a handful of flagged slots: the lane then takes the cell alone, so the
-// per-cell scans, counts and stores are shared by 32 cells per instruction.
-// A cell with more flagged slots in a phase than a lane takes is done by the
-// whole warp for that phase.
+// A warp takes consecutive cells, one a lane (32; 4 or 8 in a full step of few
+// cells). Most cells have a handful of flagged slots: the lane then takes the
+// cell alone, so the per-cell scans, counts and stores are shared by the warp's
+// cells per instruction. A cell with more flagged slots in a phase than a lane
+// takes is done by the whole warp: in a separate call after the lanes, in a full
+// step by event_heavy_kernel.
 //
 // Per-warp shared scratch:
 //   flagged-slot lists of one heavy cell (u16, full capacities; the removed
