@@ -123,8 +123,8 @@ typedef struct {
   double tally_Emax_keV;    /* histogram range [0, Emax) (80 keV) */
   int32_t tally_enable;     /* 1: step calls accumulate the emitted spectrum */
   int32_t diag_enable;      /* 1: feedback writes per-cell diagnostics */
-  int32_t threads_per_block;/* threads per CTA of the event kernel (32..128, one
-                               warp per cell); 0: default 128 */
+  int32_t threads_per_block;/* threads per CTA of the event kernels (32..128, a
+                               multiple of 32); 0: default 128 */
   int32_t decide_chunk;     /* cells per chunk of a decision warp: 1, 2, 4, 8,
                                16 or 32; 0: one of them by the launch's cells
                                and the slabs' capacities (launch shape, see
