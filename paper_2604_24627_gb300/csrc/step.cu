@@ -2500,11 +2500,14 @@ static cudaError_t launch_events(const StepArgs& A, int warps, cudaStream_t st, 
   // persistent over the heavy list: a warp per cell, at most one warp per
   // cell of the launch and kHeavyGrid CTAs
   const int hgrid = max(1, min((A.ncells + warps - 1) / warps, kHeavyGrid));
-  // as much shared memory as the event kernel where that is more: in a replay the
-  // branches' kernels share the SMs, and an SM that splits its memory otherwise for
-  // one of them waits for the others to end (65,536 dense cells in 8 branches: 133
-  // us a step, 141 with the lists alone, 137 with lists and event scratch)
-  const size_t lists = max(per, ev_scratch_bytes(A.a.cap, A.g.cap, A.e.cap, EV_LISTS));
+  // in a replay the branches' kernels share the SMs, and an SM that splits its
+  // memory otherwise for one of them waits for the others to end: as much shared
+  // memory as the event kernel where that is more (65,536 dense cells in 8
+  // branches: 133 us a step, 141 with the lists alone, 137 with lists and event
+  // scratch). A launch of its own leaves the rest to L1 (20,000 hot cells, all
+  // heavy: 612 us a step, 650 with the event kernel's size).
+  size_t lists = ev_scratch_bytes(A.a.cap, A.g.cap, A.e.cap, EV_LISTS);
+  if (A.dec_cells) lists = max(lists, per);
   return launch_chained(chained, sr ? event_heavy_kernel<true> : event_heavy_kernel<false>, hgrid, warps * 32, lists * warps, st, A);
 }
 
