@@ -134,6 +134,11 @@ constexpr int kGroup = 4;  // cells a warp
 constexpr int kWords = 32 / kGroup;  // words of freed bits a cell of a group has in shared memory
 static_assert(kHoldGroup <= kWords, "freed words");
 
+// The box that an instance is for: four cells a warp spill with an open one's code
+// (62,500 cells of 60 131 us without it, 133 with; open 156), one cell does not, and
+// was slower without (10,000 of 400 129 and 137 us).
+enum { BOX_PERIODIC, BOX_OPEN, BOX_EITHER };
+
 struct MoveShared {
   int cnt[kGroup * 32];      // leavers per direction so far
   int off[kGroup * 32];      // first staging row of a direction
@@ -142,11 +147,12 @@ struct MoveShared {
 
 // The K cells from c0 on with n_l slots in lane k < K: all of them in R
 // register passes, or (K = 1) more than those hold.
-template <int K, int R>
+template <int K, int R, int BOX>
 __device__ __forceinline__ void move_cells(const StreamArgs& a, int c0, int n_l, MoveShared& S) {
   const int lane = threadIdx.x & 31;
   const unsigned lt = (1u << lane) - 1u;
   const int W = (a.s.cap + 31) >> 5;
+  const bool open = BOX == BOX_EITHER ? !a.periodic : BOX == BOX_OPEN;
   FlatCells<K> F;
   F.set(n_l);
   const int N = F.total();
@@ -203,7 +209,7 @@ __device__ __forceinline__ void move_cells(const StreamArgs& a, int c0, int n_l,
       const int o = move_axion(a, r[i], u[i]);
       a.s.xyz[(long)(c0 + k) * a.s.cap + sl] = u[i];
       fr = leave = o != kStreamStay;
-      if (leave && !a.periodic && escapes(a, c0 + k, o)) {
+      if (open && leave && escapes(a, c0 + k, o)) {
         leave = false;
         count_escape(a, r[i]);
       }
@@ -227,7 +233,7 @@ __device__ __forceinline__ void move_cells(const StreamArgs& a, int c0, int n_l,
         float4 uu = a.s.xyz[q];
         const int o = move_axion(a, rr, uu);
         fr = o != kStreamStay;
-        if (fr && (a.periodic || !escapes(a, c0, o))) atomicAdd(&S.cnt[o], 1);
+        if (fr && (!open || !escapes(a, c0, o))) atomicAdd(&S.cnt[o], 1);
       }
       mark(f, 0, f, fr);
     }
@@ -269,7 +275,7 @@ __device__ __forceinline__ void move_cells(const StreamArgs& a, int c0, int n_l,
         o = move_axion(a, rr, uu);
         a.s.xyz[q] = uu;
         leave = o != kStreamStay;
-        if (leave && !a.periodic && escapes(a, c0, o)) {
+        if (open && leave && escapes(a, c0, o)) {
           leave = false;
           count_escape(a, rr);
         }
@@ -287,7 +293,7 @@ __device__ __forceinline__ void move_cells(const StreamArgs& a, int c0, int n_l,
 
 // A warp takes K cells (kGroup, or 1): together where their slots fit the
 // register passes, else one after the other.
-template <int K>
+template <int K, int BOX>
 __global__ void __launch_bounds__(kThreads, 3) stream_move_kernel(StreamArgs a) {
   wait_predecessor();
   __shared__ MoveShared S[kWarps];
@@ -296,11 +302,11 @@ __global__ void __launch_bounds__(kThreads, 3) stream_move_kernel(StreamArgs a) 
   if (c0 >= a.ncells) return;
   const int n_l = lane < K && c0 + lane < a.ncells ? min(max(a.s.count[c0 + lane], 0), a.s.cap) : 0;
   if (K > 1 && __reduce_add_sync(kAll, (unsigned)n_l) <= 32 * kHoldGroup) {
-    move_cells<K, kHoldGroup>(a, c0, n_l, S[wid]);
+    move_cells<K, kHoldGroup, BOX>(a, c0, n_l, S[wid]);
   } else {
     for (int k = 0; k < K && c0 + k < a.ncells; ++k) {
       const int n = __shfl_sync(kAll, n_l, k);
-      move_cells<1, kHoldOne>(a, c0 + k, lane == 0 ? n : 0, S[wid]);
+      move_cells<1, kHoldOne, BOX>(a, c0 + k, lane == 0 ? n : 0, S[wid]);
     }
   }
 }
@@ -529,7 +535,9 @@ __global__ void __launch_bounds__(kThreads, 6) stream_place_kernel(StreamArgs a)
 template <int K>
 cudaError_t launch(const StreamArgs& a, cudaStream_t st) {
   const int grid = (a.ncells + kWarps * K - 1) / (kWarps * K);
-  const cudaError_t e = launch_chained(false, stream_move_kernel<K>, grid, kThreads, 0, st, a);
+  constexpr int periodic = K == 1 ? BOX_EITHER : BOX_PERIODIC, open = K == 1 ? BOX_EITHER : BOX_OPEN;
+  const cudaError_t e = launch_chained(false, a.periodic ? stream_move_kernel<K, periodic> : stream_move_kernel<K, open>,
+                                       grid, kThreads, 0, st, a);
   if (e) return e;
   return launch_chained(true, stream_place_kernel<K>, grid, kThreads, 0, st, a);
 }
